@@ -1,17 +1,20 @@
 // Fused attention core of one encoder block (Sec. 3.1 MSA equation, Sec. 3.2 and Algorithm 1):
 //   S = Q_i K_i^T (+ bias)  ->  requantise to int8  ->  Shiftmax  ->  P_i V_i  ->  requantise
-// for one (image or window, head, 128-row tile) per CTA, rows up to 256 tokens long.
+// for one head and 128 score rows at a time: attention_short_kernel (rows of up to 256 tokens, several short windows
+// packed into the 128 rows) and attention_rows_kernel (longer rows).
 //
-// The int32 score tile lives in tensor memory, never in HBM.  Two threads share one score row (one
-// TMEM lane; they take alternate 32-column chunks), so the row maximum and the row sum of
-// Algorithm 1 need one exchange of two words through shared memory each: no shuffles.
-//   pass A  tcgen05.ld the row, requantise to int8 (kept packed in registers), running max;
-//   pass B  ShiftExp by table lookup (256 entries, I_max - I in [0, 255]), row sum, and the
-//           exponentials written back over the scores in tensor memory (tcgen05.st);
-//   pass C  one reciprocal per row (Eq. (IntDiv)), then exp * reciprocal >> shift per value; the
-//           int8 probabilities are written to shared memory in the K-major 128B-swizzled layout
-//           that the second MMA consumes as its A operand.
+// The int32 score tile lives in tensor memory, never in HBM.  Several threads share one score row (a TMEM lane) and
+// take different columns of it, so the row maximum and the row sum of Algorithm 1 need one exchange through shared
+// memory each: no shuffles.  Three passes over the scores:
+//   pass A  requantise to int8, running maximum;
+//   pass B  ShiftExp by look-up (256 entries, I_max - I in [0, 255]), row sum.  The table is kept `cp` times in shared
+//           memory, copy (lane mod cp) serving a lane, so that look-ups do not collide on banks; dp4a with one non-zero
+//           byte turns a packed score into its entry's address in one instruction;
+//   pass C  one reciprocal per row (Eq. (IntDiv)), then exp * reciprocal >> shift per value; the int8 probabilities are
+//           written to shared memory in the K-major 128B-swizzled layout that P V consumes as its A operand.
 // V is consumed as stored ([token, d] rows, MN-major B operand).  Every wait is bounded.
+// What bounds the passes: issue slots.  mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer
+// instructions two cycles of their pipe, a look-up one of the SM's shared-memory cycles.
 #include "tc_ptx.cuh"
 #include <cstdlib>
 
@@ -19,417 +22,520 @@ namespace ivit {
 
 namespace {
 
-constexpr int kAttnThreads = 288;   // warp 0: TMA + MMA issue + TMEM owner; warps 1..8: two threads per score row
 constexpr int UK = 32;              // K of one tcgen05.mma.kind::i8
 
-
 // Eq. (IntDiv) with M = 45 for four exponentials: (floor(2^45 / sum) * e) >> (45 - (k_out - 1)) = umulhi(factor, e) >> (14 - k_out),
-// clamped to 2^(k_out-1) - 1 and packed.  K8: k_out = 8, where the saturating pack does the clamp (values are <= 128).
-template <bool K8>
+// clamped to 2^(k_out-1) - 1 and packed.
 __device__ __forceinline__ uint32_t prob_word(unsigned factor, int e0, int e1, int e2, int e3, int osh, int omax) {
-  if (K8)
-    return pack_sat8((int)(__umulhi(factor, (unsigned)e0) >> 6), (int)(__umulhi(factor, (unsigned)e1) >> 6),
-                     (int)(__umulhi(factor, (unsigned)e2) >> 6), (int)(__umulhi(factor, (unsigned)e3) >> 6));
   return pack_sat8(min((int)(__umulhi(factor, (unsigned)e0) >> osh), omax), min((int)(__umulhi(factor, (unsigned)e1) >> osh), omax),
                    min((int)(__umulhi(factor, (unsigned)e2) >> osh), omax), min((int)(__umulhi(factor, (unsigned)e3) >> osh), omax));
 }
+// The same for k_out = 8 with factor4 = 4 floor(2^45 / sum): the probability is byte 1 of the high product word.  The one
+// probability that can reach 128, and is clamped to 127, belongs to a row whose only non-zero exponential is a power of
+// two; prob_factor4 takes one off the reciprocal there, which gives 127.
+__device__ __forceinline__ uint32_t prob_word8(unsigned factor4, int e0, int e1, int e2, int e3) {
+  return __byte_perm(__byte_perm(__umulhi(factor4, (unsigned)e0), __umulhi(factor4, (unsigned)e1), 0x0051),
+                     __byte_perm(__umulhi(factor4, (unsigned)e2), __umulhi(factor4, (unsigned)e3), 0x0051), 0x5410);
+}
 
+// ShiftExp of one packed score x (int8): the table entry at t - 4 cp x, where `sel` holds -4 cp in the byte that holds x.
+// (Not volatile: the table does not change once the CTA's first barrier is behind, so look-ups may be moved freely.)
+__device__ __forceinline__ unsigned exp_entry(uint32_t w, uint32_t sel, uint32_t t) {
+  unsigned e;
+  asm("{\n\t.reg .u32 a;\n\tdp4a.s32.s32 a, %1, %2, %3;\n\tld.shared.u32 %0, [a];\n\t}" : "=r"(e) : "r"(w), "r"(sel), "r"(t));
+  return e;
+}
+
+// floor(2^45 / s) for 2^15 < s < 2^32.  With d = s 2^z, 2^31 <= d < 2^32, it is floor(2^63 / d) >> (18 - z) (nested floor
+// quotients).  v starts at 2^63 / (middle of the 2^24 values that share d's upper byte), relative error below 2^-8, from
+// a table of 128 entries; two Newton steps square that twice; the shift (by at least 2) leaves at most one unit, which
+// the exact remainder puts right.  (Checked on the CPU for every s of the range; a 64-bit division takes 700 cycles on
+// the row's critical path.)
+__device__ __forceinline__ unsigned recip_seed(int i) { return (unsigned)((1ull << 40) / (unsigned)(2 * (128 + i) + 1)); }
+__device__ __forceinline__ unsigned recip45(unsigned s, const unsigned* seeds) {
+  const int z = __clz(s);
+  const unsigned d = s << z;
+  unsigned v = seeds[(d >> 24) & 127u];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int e = (int)(0x80000000u - __umulhi(v, d));               // 2^31 - v d / 2^32
+    v += (unsigned)__mulhi((int)(v >> 1), e << 2);
+  }
+  if (d == 0x80000000u) v = 0xffffffffu;   // 2^32 itself does not fit
+  unsigned q = v >> (18 - z);
+  long long r = (long long)((1ull << 45) - (unsigned long long)q * s);
+  if (r < 0) { --q; r += s; }
+  if (r >= (long long)s) ++q;
+  return q;
+}
+// Four times the reciprocal for prob_word8; `top` = I0 2^N > 2^15, the largest exponential.
+__device__ __forceinline__ unsigned prob_factor4(unsigned sum, unsigned top, const unsigned* seeds) {
+  unsigned f = recip45(sum, seeds);
+  if (sum == top && (sum & (sum - 1u)) == 0u) --f;
+  return f << 2;
+}
+
+// Fields that both kernels use.
 struct AttnArgs {
-  int T, d, heads, Npad;            // Npad = T rounded up to 32 (score columns and P.V contraction length)
+  int T, d, heads;
   int64_t D;                        // heads * d
-  int tiles_m;                      // ceil(T / 128)
-  int bh;                           // images (or windows) x heads
-  int items;                        // bh * tiles_m
-  int G, R;                         // G windows of at most R = 128 / G tokens share one tile (G = 1: one image or window per tile)
-  int Btot;                         // images or windows in the tensor
-  int tmem_cols;
+  int bh;                           // images x heads
+  int items;
+  int kpad;                         // contraction length of P V: T rounded up to 32 (packed windows: 128)
+  int kbox;                         // rows of a key box (packed windows: rows of a slot)
+  int cp;                           // copies of the ShiftExp table (a power of two, at most 32)
+  uint32_t sel[4];                  // -4 cp as a signed byte, in byte 0, 1, 2, 3
+  int chunks;                       // 16-column chunks of a row, the last one with T & 15 columns when that is not 0
   int qk_m, qk_s, pv_m, pv_s;
   ivit_exp_params smax;
   const int32_t* bias;              // [bias_batches, T, T] or nullptr
-  int64_t bias_batches;
+  int bias_batches;
   int8_t* O;                        // [B*T, D]
   int q_pos[3], k_pos[3], v_pos[3];
-  unsigned* sched;                  // this launch's counters: [0] next work item, [1] CTAs that have finished
-  unsigned* sched_other;            // the counters of the next launch
   int* status;
 };
 
-constexpr uint32_t kItemWaitRounds = 16;   // the item barrier outlasts every bounded wait of the control thread
+// A work item: head h of image b, 128 rows from m0 on (packed windows: head h of the windows from window b on).
+struct __align__(16) AttnItem {
+  int h, b, m0;
+  int rot;      // row group g (32 rows) of the tile stands in lane quarter (g + rot) & 3: the quarters (and schedulers)
+                // that a ragged tile leaves idle change from item to item
+  // The n-th work item of a CTA.  Items are ordered tile by tile, the ragged last tiles at the end, and dealt in a snake:
+  // item n gridDim + blockIdx for even n, the mirror image for odd n, so that a CTA with one item more than others has
+  // it among the ragged tiles.
+  __device__ __forceinline__ void init(const AttnArgs& a, uint32_t n) {
+    unsigned t = n * gridDim.x + ((n & 1u) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+    m0 = 0;
+    while (t >= (unsigned)a.bh) { t -= (unsigned)a.bh; m0 += 128; }
+    b = (int)(t / (unsigned)a.heads);
+    h = (int)t - b * a.heads;
+    rot = m0 + 128 >= a.T ? (int)(t & 3u) : 0;
+  }
+  static __device__ __forceinline__ uint32_t count(const AttnArgs& a) {
+    const uint32_t rounds = (uint32_t)a.items / gridDim.x, left = (uint32_t)a.items % gridDim.x;
+    return rounds + (((rounds & 1u) ? gridDim.x - 1 - blockIdx.x : blockIdx.x) < left ? 1u : 0u);
+  }
+};
 
-// Persistent CTAs (two per SM) draw work items = (image or window, head, 128-row tile) from a counter, the
-// full 128-row tiles first.  One control thread issues the TMA loads and the MMAs; the loads of the next item
-// are issued as soon as the MMAs that read the shared-memory operands of the current one have completed, so
-// they overlap the Shiftmax passes.  Barriers are used once per item: the parity of a wait is the item count.
-// kPack: several windows share the tile (AttnArgs::G > 1); the plain form carries none of that index arithmetic.
-template <bool kPack, bool K8>
-__global__ void __launch_bounds__(kAttnThreads, 2) attention_kernel(const __grid_constant__ CUtensorMap tmQ,
-                                                                 const __grid_constant__ CUtensorMap tmK,
-                                                                 const __grid_constant__ CUtensorMap tmV, AttnArgs a) {
+// Tile load; pos: which coordinate of the map (1..3) carries the row, the head and the image or window.
+__device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, const int (&pos)[3], int row, int h, int b) {
+  tma_load_4d(dst, map, bar, 0, pos[0] == 1 ? row : (pos[1] == 1 ? h : b), pos[0] == 2 ? row : (pos[1] == 2 ? h : b),
+              pos[0] == 3 ? row : (pos[1] == 3 ? h : b));
+}
+
+// The ShiftExp table: entry i, copy c at word i cp + c; consecutive lanes write different banks.  n threads.
+__device__ __forceinline__ void build_exp_table(const AttnArgs& a, uint8_t* tab, int st, int n) {
+  const unsigned e = shiftexp(-(st & 255), a.smax.I0, a.smax.N);
+  const int per = 32 / a.cp;                  // entries per 32 banks
+  for (int c = st >> 8; c < a.cp; c += n >> 8)
+    *reinterpret_cast<unsigned*>(tab + 4u * ((unsigned)(st & 255) * a.cp + ((c + (st & 31) / per) & (a.cp - 1)))) = e;
+}
+
+// Constants of the inner loops, held in registers (the compiler would fetch them again for every use).
+struct PassConsts {
+  uint32_t sel[4];
+  int qk_m, qk_rnd, qk_sh;
+  __device__ __forceinline__ void init(const AttnArgs& a) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) asm volatile("mov.b32 %0, %1;" : "=r"(sel[i]) : "r"(a.sel[i]));
+    asm volatile("mov.b32 %0, %1;" : "=r"(qk_m) : "r"(a.qk_m));
+    asm volatile("mov.b32 %0, %1;" : "=r"(qk_rnd) : "r"(a.qk_s >= 33 ? 1 << (a.qk_s - 33) : 0));
+    asm volatile("mov.b32 %0, %1;" : "=r"(qk_sh) : "r"(a.qk_s - 32));
+  }
+};
+
+// Pass A on W scores: requantise, columns from `valid` on (at most W) become -128 when EDGE, maximum into mx, packed
+// into x.  FAST: the shift is >= 33 (high product word plus 2^(s-33), shifted by s - 32).
+template <bool FAST, bool EDGE, int W>
+__device__ __forceinline__ void score_piece(const AttnArgs& a, const PassConsts& k, int (&v)[W], int valid, int& mx, uint32_t* x) {
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    if (FAST) v[i] = mad_hi(v[i], k.qk_m, k.qk_rnd) >> k.qk_sh;
+    else v[i] = (int)(((long long)v[i] * a.qk_m + (1ll << (a.qk_s - 1))) >> a.qk_s);
+  }
+  if (EDGE) {
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+      if (i >= valid) v[i] = -128;
+  }
+#pragma unroll
+  for (int i = 0; i < W; i += 2) mx = __vimax3_s32(mx, v[i], v[i + 1]);
+#pragma unroll
+  for (int q = 0; q < W / 4; ++q) x[q] = pack_sat8(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+}
+// Bytes of word q of an edge chunk that hold columns below `valid`.
+__device__ __forceinline__ uint32_t edge_mask(int valid, int q) {
+  return valid >= 4 * q + 4 ? 0xffffffffu : (valid <= 4 * q ? 0u : 0xffffffffu >> (8 * (4 * q + 4 - valid)));
+}
+// O = sat8(rq(P V; pv_scale)) of 16 columns.
+template <bool FAST>
+__device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
+  if (FAST) {
+    const int rnd = 1 << (a.pv_s - 33), sh = a.pv_s - 32;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = mad_hi(v[i], a.pv_m, rnd) >> sh;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = (int)(((long long)v[i] * a.pv_m + (1ll << (a.pv_s - 1))) >> a.pv_s);
+  }
+  return make_uint4(pack_sat8(v[0], v[1], v[2], v[3]), pack_sat8(v[4], v[5], v[6], v[7]),
+                    pack_sat8(v[8], v[9], v[10], v[11]), pack_sat8(v[12], v[13], v[14], v[15]));
+}
+
+// ------------------------------------------------------------------------------------------------------------
+// Rows of up to 256 tokens: a CTA of eight Shiftmax warps, two threads per score row (they take alternate 16-column
+// chunks), two or three CTAs per SM.  The CTAs of an SM are at different points of their items, which covers the waits
+// that an item cannot avoid (score MMAs, row exchanges, P V) and mixes passes that need different pipes.
+//   kPack = false  128 rows of one image
+//   kPack = true   G windows of up to R = 128 / G tokens share the 128 rows (window attention): the score tile is
+//                  block-diagonal and the probabilities outside a row's own window stay 0.  The int32 score bias of
+//                  the tile's windows is kept in shared memory (rows padded to an odd number of words, so that the 32
+//                  rows of a warp fall into different banks) and only fetched when it differs from the last item's;
+//                  items are ordered so that it rarely does (per head and window position, images innermost).  Read
+//                  straight from global memory, one row per lane, it took most of the kernel's time.
+// Everything of an item stays in tensor memory: the score columns hold the packed int8 scores after pass A, the
+// exponentials after pass B, and O = P V at the end.
+// Measured, back to back (before: one table, items drawn from a counter, bias read from global memory):
+//   64 x 197 tokens, 6 heads of 64      29.0 -> 22.3 us        128 x 197, 12 heads of 64   89.1 -> 69.4 us
+//   4096 windows of 49, 3 heads, bias    125 -> 87.7 us        1 x 197, 3 heads            10.1 ->  7.2 us
+constexpr int kShortThreads = 288;   // warp 0: TMA + MMA issue + TMEM owner; warps 1..8: two threads per score row
+
+struct ShortArgs {
+  AttnArgs a;
+  int G, R, Btot;                   // kPack: windows per tile, rows per window slot, windows in the tensor
+  int units, npos;                  // kPack: tiles per head; window-position groups with a bias of their own per head
+  int tmem_cols;
+};
+
+template <bool kPack, bool FAST, bool BIAS>
+__global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_kernel(const __grid_constant__ CUtensorMap tmQ,
+                                                                                       const __grid_constant__ CUtensorMap tmK,
+                                                                                       const __grid_constant__ CUtensorMap tmV,
+                                                                                       ShortArgs sa) {
+  const AttnArgs& a = sa.a;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
-  // [Q 128x128B][K Npad x 128B][V Npad x d][P 128 x 128B x kblocks][exp table][row partials][item ring][barriers]
-  const uint32_t q_off = 0, k_off = 128 * 128, v_off = k_off + a.Npad * 128;
-  const uint32_t p_off = (v_off + a.Npad * a.d + 1023u) & ~1023u;
-  const int p_kblocks = (a.Npad + 127) / 128;
-  const uint32_t tab_off = p_off + p_kblocks * 128 * 128;
-  const uint32_t part_off = tab_off + 1024;            // [2 halves][128 rows] partial max, then partial sum
-  const uint32_t item_off = part_off + 2 * 128 * 4 * 2;   // [2] work item of even / odd iterations (-1: no more work)
-  const uint32_t bar_off = item_off + 16;
-  unsigned* tab = reinterpret_cast<unsigned*>(gen + tab_off);
-  volatile int* item_ring = reinterpret_cast<volatile int*>(gen + item_off);
-  // Q and K landed | V landed | scores ready | probabilities written | output ready | output read | item published
+  // [Q 128 x d][K][V kpad x d][P 128 x 128B x kblocks][table 256 x cp][row partials][seeds][items][barriers][window bias]
+  const uint32_t k_bytes = (uint32_t)(kPack ? 128 : a.kbox) * a.d, v_bytes = (uint32_t)a.kpad * a.d;
+  const uint32_t k_off = 128u * a.d, v_off = k_off + k_bytes;
+  const uint32_t p_off = (v_off + v_bytes + 1023u) & ~1023u;
+  const uint32_t tab_off = p_off + (uint32_t)((a.kpad + 127) / 128) * 128 * 128;
+  const uint32_t part_off = tab_off + 1024u * a.cp;      // [2 halves][128 rows] partial max, then partial sum
+  const uint32_t seed_off = part_off + 4 * 128 * 4;      // [128] seeds of the reciprocal
+  const uint32_t item_off = seed_off + 128 * 4;          // [2] work item of even / odd iterations, written before its scores
+  const uint32_t bar_off = item_off + 2 * sizeof(AttnItem);
+  const uint32_t bias_off = bar_off + 64;                // kPack && BIAS: [G][T][T | 1]
+  AttnItem* const item_ring = reinterpret_cast<AttnItem*>(gen + item_off);
+  // Q and K landed | V landed | scores ready | probabilities written | output ready | output read
   const uint32_t bar_qk = base + bar_off, bar_v = bar_qk + 8, bar_s = bar_qk + 16, bar_p = bar_qk + 24,
-                 bar_o = bar_qk + 32, bar_e = bar_qk + 40, bar_item = bar_qk + 48;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 64);
+                 bar_o = bar_qk + 32, bar_e = bar_qk + 40;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 48);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
   if (threadIdx.x == 0) {
     prefetch_tmap(&tmQ);
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
     mbar_init(bar_qk, 1);
     mbar_init(bar_v, 1);
-    mbar_init(bar_s, 1);
+    mbar_init(bar_s, 2);      // the MMAs, and the control thread (the item is in the ring)
     mbar_init(bar_p, 8);
     mbar_init(bar_o, 1);
     mbar_init(bar_e, 8);
-    mbar_init(bar_item, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  if (warp == 0) tmem_alloc(smem_u32(tmem_slot), (uint32_t)a.tmem_cols);
+  if (warp == 0) tmem_alloc(smem_u32(tmem_slot), (uint32_t)sa.tmem_cols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_trigger();
-  // The ShiftExp table depends on parameters only: the Shiftmax threads build it before they wait for the previous
-  // kernel (whose QKV tensor the control thread loads and whose successors' buffers the output overwrites).
-  if (warp == 0) pdl_wait();
-  // Launches alternate between two pairs of counters.  A launch leaves its own pair at zero when its last CTA
-  // finishes, and also zeroes the other pair (below, after the wait), so that a launch that was cut short cannot
-  // poison the next.
+  // items of this CTA: a snake over all of them, or (kPack) a contiguous range
+  const uint32_t rounds = (uint32_t)a.items / gridDim.x, left = (uint32_t)a.items % gridDim.x;
+  const uint32_t n_items = kPack ? rounds + (blockIdx.x < left ? 1u : 0u) : AttnItem::count(a);
+  const uint32_t first = blockIdx.x * rounds + min(blockIdx.x, left);   // kPack
+  const uint32_t imgs = kPack ? (uint32_t)sa.units / (uint32_t)sa.npos : 1u;   // kPack: items in a row with the same bias
 
-  // item -> (tile, image/window * heads + head): all first tiles before all second tiles
   if (warp == 0) {
-    if (lane == 0) {
-      auto load_qk = [&](int item) {
-        const int tile = item / a.bh, bhid = item - tile * a.bh;
-        const int h = bhid % a.heads, b = bhid / a.heads;
-        mbar_expect_tx(bar_qk, 128 * 128 + a.Npad * 128);
-        int c[4];
-        c[0] = 0; c[a.q_pos[0]] = tile * 128; c[a.q_pos[1]] = h; c[a.q_pos[2]] = kPack ? b * a.G : b;
-        tma_load_4d(base + q_off, &tmQ, bar_qk, c[0], c[1], c[2], c[3]);
-        c[0] = 0; c[a.k_pos[0]] = 0; c[a.k_pos[1]] = h; c[a.k_pos[2]] = kPack ? b * a.G : b;
-        tma_load_4d(base + k_off, &tmK, bar_qk, c[0], c[1], c[2], c[3]);
+    pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
+    if (lane == 0 && n_items > 0) {
+      auto item_at = [&](AttnItem& it, uint32_t n) {
+        if (kPack) {
+          const unsigned t = first + n, grp = t / imgs, img = t - grp * imgs;
+          it.h = (int)(grp / (unsigned)sa.npos);
+          it.b = (int)(grp - (unsigned)it.h * sa.npos + img * sa.npos) * sa.G;
+          it.m0 = 0;
+          it.rot = 0;
+        } else {
+          it.init(a, n);
+        }
       };
-      auto load_v = [&](int item) {
-        const int tile = item / a.bh, bhid = item - tile * a.bh;
-        const int h = bhid % a.heads, b = bhid / a.heads;
-        mbar_expect_tx(bar_v, a.Npad * a.d);
-        int c[4];
-        c[0] = 0; c[a.v_pos[0]] = 0; c[a.v_pos[1]] = h; c[a.v_pos[2]] = kPack ? b * a.G : b;
-        tma_load_4d(base + v_off, &tmV, bar_v, c[0], c[1], c[2], c[3]);
+      auto load_qk = [&](const AttnItem& it) {
+        mbar_expect_tx(bar_qk, 128u * a.d + k_bytes);
+        if (kPack) {
+          load_box(base, &tmQ, bar_qk, a.q_pos, 0, it.h, it.b);
+        } else {
+          for (int g = 0; g < 4; ++g)
+            load_box(base + (uint32_t)((g + it.rot) & 3) * 32u * a.d, &tmQ, bar_qk, a.q_pos, it.m0 + 32 * g, it.h, it.b);
+        }
+        load_box(base + k_off, &tmK, bar_qk, a.k_pos, 0, it.h, it.b);
       };
-      auto draw = [&]() {
-        const unsigned t = atomicAdd(a.sched, 1u);
-        return t < (unsigned)a.items ? (int)t : -1;
+      auto load_v = [&](const AttnItem& it) {
+        mbar_expect_tx(bar_v, v_bytes);
+        load_box(base + v_off, &tmV, bar_v, a.v_pos, 0, it.h, it.b);
       };
-      auto publish = [&](uint32_t n, int item) {
-        item_ring[n & 1u] = item;
-        mbar_arrive(bar_item);   // release: the item is visible to whoever sees this phase complete
-      };
-      // S = Q K^T: M = 128, N = Npad, both operands K-major rows of 128 bytes.  O = P V: V as stored (MN-major).
-      const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.Npad >> 3) << 17) | (8u << 24);
+      // descriptor words: rows of d bytes (Q, K, V: swizzled over their width) or 128 bytes (P)
+      const uint32_t layout = a.d == 128 ? 2u : (a.d == 64 ? 4u : 6u);
+      const uint32_t row_hi = desc_hi(8u * a.d, layout), p_hi = desc_hi(1024, 2);
+      const uint32_t q_lo = desc_lo(base, 16), k_lo = desc_lo(base + k_off, 16), p_lo0 = desc_lo(base + p_off, 16),
+                     v_lo0 = desc_lo(base + v_off, 16), v_step = (uint32_t)(UK * a.d) >> 4;
+      const int s_cols = kPack ? 128 : 16 * a.chunks;
+      const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(s_cols >> 3) << 17) | (8u << 24);
       const uint32_t idesc2 = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(a.d >> 3) << 17) | (8u << 24);
-      const uint32_t v_layout = a.d == 128 ? 2u : (a.d == 64 ? 4u : 6u);
-      const int ks = (a.d + UK - 1) / UK, ks2 = a.Npad / UK;
+      const int ks = a.d / UK, ks2 = a.kpad / UK;
 
-      int item = draw();
-      bool qk_flying = false, v_flying = false;   // loads issued and not yet waited for (their barrier phase = item count)
-      if (item >= 0) { load_qk(item); load_v(item); qk_flying = v_flying = true; }
+      AttnItem cur, next;
+      item_at(cur, 0);
+      bool qk_flying = true, v_flying = true;   // loads issued and not yet waited for (their barrier phase = item count)
+      uint32_t qk_par = 0, v_par = 0;
+      load_qk(cur);
+      load_v(cur);
       bool ok = true;
-      uint32_t n = 0, qk_par = 0, v_par = 0;
-      for (; item >= 0; ++n) {
+      for (uint32_t n = 0; n < n_items; ++n) {
         const uint32_t par = n & 1u;
-        publish(n, item);
         ok = mbar_wait(bar_qk, par, a.status);
         qk_flying = !ok;
         // the output of the previous item must have left tensor memory
         if (ok && n > 0) ok = mbar_wait(bar_e, par ^ 1u, a.status);
         if (!ok) break;
+        item_ring[par] = cur;
         tc_fence_after();
         for (int k = 0; k < ks; ++k)
-          umma_i8(tmem, smem_desc(base + q_off + k * UK, 16, 1024, 2), smem_desc(base + k_off + k * UK, 16, 1024, 2),
-                  idesc, k != 0);
+          umma_i8_lohi(tmem, q_lo + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
         umma_commit(bar_s);
-        const int next = draw();
+        mbar_arrive(bar_s);   // releases the item written to the ring
+        const bool more = n + 1 < n_items;
+        if (more) item_at(next, n + 1);
         // Q and K may be overwritten once the score MMAs have read them
         ok = mbar_wait(bar_s, par, a.status);
         if (!ok) break;
-        if (next >= 0) { load_qk(next); qk_flying = true; qk_par = par ^ 1u; }
+        if (more) { load_qk(next); qk_flying = true; qk_par = par ^ 1u; }
         // O = P V once the probabilities are in shared memory and V has landed
         ok = mbar_wait(bar_p, par, a.status);
         if (ok) { ok = mbar_wait(bar_v, par, a.status); v_flying = !ok; }
         if (!ok) break;
         tc_fence_after();
-        for (int k = 0; k < ks2; ++k) {
-          const uint32_t pa = base + p_off + (k >> 2) * (128 * 128) + (k & 3) * UK;
-          umma_i8(tmem, smem_desc(pa, 16, 1024, 2), smem_desc(base + v_off + k * UK * a.d, 16, 8 * a.d, v_layout),
-                  idesc2, k != 0);
-        }
+        uint32_t p_lo = p_lo0, v_lo = v_lo0;
+        int k = 0;
+        for (; k + 4 <= ks2; k += 4, p_lo += (128 * 128) >> 4, v_lo += 4 * v_step)
+          umma_i8_x4(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
+        for (; k < ks2; ++k, p_lo += UK >> 4, v_lo += v_step)
+          umma_i8_lohi(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
         umma_commit(bar_o);
         // V may be overwritten once these MMAs have read it
         ok = mbar_wait(bar_o, par, a.status);
         if (!ok) break;
-        if (next >= 0) { load_v(next); v_flying = true; v_par = par ^ 1u; }
-        item = next;
+        if (more) { load_v(next); v_flying = true; v_par = par ^ 1u; }
+        cur = next;
       }
-      // end of work (or a wait that timed out): tell the other warps; nothing may be in flight at exit
-      publish(ok ? n : n + 1, -1);
+      // nothing may be in flight at exit (after a wait that timed out)
       if (qk_flying) mbar_wait(bar_qk, qk_par, a.status);
       if (v_flying) mbar_wait(bar_v, v_par, a.status);
     }
   } else {
-    // ---- softmax / epilogue threads: TMEM lane quarter = warp % 4; the two warps of a quarter
-    //      take the even / odd 32-column chunks of the same 32 rows ----
-    const int st = threadIdx.x - 32;   // 0..255
-    tab[st] = shiftexp(-st, a.smax.I0, a.smax.N);
-    pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 32) {
-      a.sched_other[0] = 0;
-      a.sched_other[1] = 0;
-    }
+    // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the two warps of a quarter take the even / odd
+    //      chunks of the same 32 rows ----
+    const int st = threadIdx.x - 32;              // 0..255
     const int qd = warp & 3;
     const int half = (warp - 1) >> 2;
     const int trow = qd * 32 + lane;              // row inside the tile
+    build_exp_table(a, gen + tab_off, st, 256);
+    // probabilities that no item writes are 0: columns past the last chunk, other windows' columns
+    for (int c = (kPack ? 0 : a.chunks) + half; c < a.kpad / 16; c += 2)
+      *reinterpret_cast<uint4*>(gen + p_off + (c >> 3) * (128 * 128) + trow * 128 + (((c & 7) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+    unsigned* seeds = reinterpret_cast<unsigned*>(gen + seed_off);
+    if (st < 128) seeds[st] = recip_seed(st);
+    pdl_wait();
+    PassConsts kc;
+    kc.init(a);
     const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16);
-    const int nch = a.Npad / 16;
-    const bool qk_hi = a.qk_s >= 33;              // rounding constant and shift both past the low product word
-    const long long qk_c = 1ll << (a.qk_s - 1);
-    const int qk_rnd = qk_hi ? 1 << (a.qk_s - 33) : 0, qk_sh = a.qk_s - 32;
     int* part_max = reinterpret_cast<int*>(gen + part_off);
     unsigned* part_sum = reinterpret_cast<unsigned*>(gen + part_off + 2 * 128 * 4);
+    const uint32_t tab_lane = base + tab_off + 4u * (unsigned)(lane & (a.cp - 1));
+    const unsigned top = (unsigned)a.smax.I0 << a.smax.N;    // the largest exponential
+    const int osh = 14 - a.smax.k_out, omax = (1 << (a.smax.k_out - 1)) - 1;
+    // this row's whole chunks: c_lo .. c_full - 1, this thread takes every second one; rem columns remain, which the
+    // second thread (whose share is never the larger one) takes as a piece of eight or sixteen columns
+    const int slot = kPack ? trow / sa.R : 0;
+    const int c_lo = kPack ? slot * (sa.R >> 4) : 0, c_full = c_lo + (a.T >> 4);
+    const int rem = half == 1 ? a.T & 15 : 0;
+    uint8_t* const p_row = gen + p_off + trow * 128;
+    auto p_addr = [&](int c) { return reinterpret_cast<uint4*>(p_row + (c >> 3) * (128 * 128) + (((c & 7) ^ (trow & 7)) << 4)); };
+    const int bias_ld = a.T | 1;
+    uint32_t img = kPack ? first % imgs : 0u;   // kPack: items with the present bias that are behind
     asm volatile("bar.sync 1, 256;" ::: "memory");   // the table is complete
 
     bool alive = true;   // false after a wait that timed out: no more waits, no more work, only the barriers
-    for (uint32_t n = 0;; ++n) {
+    for (uint32_t n = 0; n < n_items; ++n) {
       const uint32_t par = n & 1u;
-      // All 256 threads leave the loop together: the decision is taken on a value that every thread reads
-      // after the same barrier phase.
-      bool got_item = false;
-      if (alive) {
-        for (uint32_t w = 0; w < kItemWaitRounds && !got_item; ++w) got_item = mbar_wait(bar_item, par, a.status);
-      }
-      const int item = got_item ? item_ring[par] : -1;
-      if (item < 0) break;
-      const int tile = item / a.bh, bhid = item - tile * a.bh;
-      const int h = bhid % a.heads;
-      // G > 1: the tile holds G windows of R rows each (window `slot` in rows and columns slot R .. slot R + R - 1 of
-      // the block-diagonal score tile); a warp's 32 rows lie inside one window
-      const int slot = kPack ? trow / a.R : 0;
-      const int b = kPack ? (bhid / a.heads) * a.G + slot : bhid / a.heads;   // image / window of this row
-      const int m0 = tile * 128;
-      const int col0 = kPack ? slot * a.R : 0;      // first row and first score column of this row's window in the tile
-      const int r = m0 + trow - col0;               // token (row) inside this image / window
-      const bool row_ok = r < a.T && (!kPack || b < a.Btot);
-      const bool warp_ok = m0 + qd * 32 - col0 < a.T && (!kPack || b < a.Btot);   // warps whose 32 rows all lie past T only keep the barriers
-      const int c_lo = col0 >> 4, c_hi = kPack ? c_lo + (a.R >> 4) : nch;   // this row's 16-column chunks
-      // Plain form: the passes work on the chunks that hold columns; when the last of them holds at most eight, it is
-      // taken as one 8-column piece by the second thread of the row (whose share of full chunks is never the larger
-      // one), and chunks wholly past T only get their zero probabilities written.
-      const int c_real = kPack ? c_hi : (a.T + 15) >> 4;
-      const bool tail8 = !kPack && (a.T & 15) != 0 && (a.T & 15) <= 8;
-      const int c_end = tail8 ? c_real - 1 : c_real;   // chunks worked on sixteen columns at a time
-      const int ct = c_end * 16;                       // first column of the 8-column piece
-      const int32_t* brow = a.bias ? a.bias + ((((int64_t)b * a.heads + h) % a.bias_batches) * a.T + (row_ok ? r : 0)) * (int64_t)a.T - col0 : nullptr;
-
-      int mx = -128;
-      bool got_s = mbar_wait(bar_s, par, a.status);
-      alive = alive && got_s;
-      if (got_s) tc_fence_after();
-      if (got_s && warp_ok) {
-        // pass A: requantise the scores to int8 (Sec. 3.2), running maximum.  The two threads of a row take
-        // alternate 16-column chunks (Npad / 16 is even: equal shares).  The chunk loops are rolled (the kernel's
-        // code stays within the instruction cache); what a later pass needs of a chunk waits in the chunk's own
-        // tensor-memory columns.
-#pragma unroll 1
-        for (int c = c_lo + half; c < c_end; c += 2) {
-          int v[16];
-          tmem_ld16(t_row + c * 16, v);
-          if (brow) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (c * 16 + j - col0 < a.T) v[j] += __ldg(brow + c * 16 + j);
+      alive = alive && mbar_wait(bar_s, par, a.status);
+      const AttnItem item = item_ring[par];
+      const int b = kPack ? item.b + slot : item.b;          // image / window of this row
+      const int m0 = kPack ? qd * 32 - slot * sa.R : item.m0 + ((qd - item.rot) & 3) * 32;   // first row (token) of this lane quarter
+      const int r = m0 + lane;
+      const bool row_ok = r < a.T && (!kPack || b < sa.Btot);
+      const bool work = alive && m0 < a.T && (!kPack || b < sa.Btot);   // else the warp only keeps the barriers
+      const int32_t* brow = nullptr;
+      if (BIAS && kPack) {
+        // (decided on the item's number alone: every thread takes the same branch)
+        if (n == 0 || img == imgs) {
+          if (img == imgs) img = 0;
+          asm volatile("bar.sync 1, 256;" ::: "memory");     // pass A of the last item is behind
+          for (int s = 0; alive && s < sa.G; ++s) {
+            const int32_t* src = a.bias + (int64_t)((unsigned)((item.b + s) * a.heads + item.h) % (unsigned)a.bias_batches) * a.T * a.T;
+            int* dst = reinterpret_cast<int*>(gen + bias_off) + s * a.T * bias_ld;
+            int rr = st / a.T, cc = st - rr * a.T;
+            for (int i = st; i < a.T * a.T; i += 256) {
+              dst[rr * bias_ld + cc] = __ldg(src + i);
+              cc += 256;
+              while (cc >= a.T) { cc -= a.T; ++rr; }
+            }
           }
-          if (qk_hi) {          // the usual case: high product word plus 2^(s-33), shifted by s - 32
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = mad_hi(v[j], a.qk_m, qk_rnd) >> qk_sh;
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = (int)(((long long)v[j] * a.qk_m + qk_c) >> a.qk_s);
-          }
-          // columns past T (only in the last two chunks) never win the maximum and look up a valid table entry
-          if (c >= c_end - 2) {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (c * 16 + j - col0 >= a.T) v[j] = -128;
-          }
-          // running maximum on the unsaturated values (saturation is monotone: it is applied to the result)
-          int m = v[0];
-#pragma unroll
-          for (int j = 1; j < 16; j += 2) m = max(m, max(v[j], v[(j + 1) & 15]));
-          mx = max(mx, m);
-          // scores are kept as biased bytes (x + 128, i.e. x ^ 0x80) so that pass B can index with them:
-          // four per word in the first four columns of the chunk
-          uint32_t xs[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            xs[k] = pack_sat8(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]) ^ 0x80808080u;
-          tmem_st4(t_row + c * 16, xs);
+          asm volatile("bar.sync 1, 256;" ::: "memory");
         }
-        if (tail8 && half == 1) {
-          int v[8];
-          tmem_ld8(t_row + ct, v);
-          if (brow) {
+        ++img;
+        brow = reinterpret_cast<const int*>(gen + bias_off) + (slot * a.T + (row_ok ? r : 0)) * bias_ld - 16 * c_lo;
+      } else if (BIAS) {
+        brow = a.bias + ((int64_t)((unsigned)(item.b * a.heads + item.h) % (unsigned)a.bias_batches) * a.T + (row_ok ? r : 0)) * a.T;
+      }
+      auto add_bias = [&](auto& v, int col, int valid) {
+        if constexpr (BIAS) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-              if (ct + j < a.T) v[j] += __ldg(brow + ct + j);
+          for (int i = 0; i < (int)(sizeof(v) / sizeof(int)); ++i)
+            if (i < valid) v[i] += kPack ? brow[col + i] : __ldg(brow + col + i);
+        }
+      };
+
+      // pass A; four packed scores to a word in the first columns of the chunk's own
+      if (alive) tc_fence_after();
+      if (work) {
+        int mx = -128;
+#pragma unroll 1
+        for (int c = c_lo + half; c < c_full; c += 4) {
+          int v[2][16];
+          const bool second = c + 2 < c_full;
+          tmem_ld16_issue(t_row + 16 * c, v[0]);
+          if (second) tmem_ld16_issue(t_row + 16 * c + 32, v[1]);
+          uint32_t x[4];
+          tmem_ld_wait16(v[0]);
+          add_bias(v[0], 16 * c, 16);
+          score_piece<FAST, false>(a, kc, v[0], 16, mx, x);
+          tmem_st4(t_row + 16 * c, x);
+          if (second) {
+            tmem_ld_wait16(v[1]);
+            add_bias(v[1], 16 * c + 32, 16);
+            score_piece<FAST, false>(a, kc, v[1], 16, mx, x);
+            tmem_st4(t_row + 16 * c + 32, x);
           }
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            v[j] = qk_hi ? mad_hi(v[j], a.qk_m, qk_rnd) >> qk_sh : (int)(((long long)v[j] * a.qk_m + qk_c) >> a.qk_s);
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (ct + j >= a.T) v[j] = -128;
-          mx = max(mx, max(max(max(v[0], v[1]), max(v[2], v[3])), max(max(v[4], v[5]), max(v[6], v[7]))));
-          const uint32_t xs2[2] = {pack_sat8(v[0], v[1], v[2], v[3]) ^ 0x80808080u, pack_sat8(v[4], v[5], v[6], v[7]) ^ 0x80808080u};
-          tmem_st2(t_row + ct, xs2);
+        }
+        if (rem > 8) {
+          int v[16];
+          uint32_t x[4];
+          tmem_ld16(t_row + 16 * c_full, v);
+          add_bias(v, 16 * c_full, rem);
+          score_piece<FAST, true>(a, kc, v, rem, mx, x);
+          tmem_st4(t_row + 16 * c_full, x);
+        } else if (rem) {
+          int v[8];
+          uint32_t x[2];
+          tmem_ld8(t_row + 16 * c_full, v);
+          add_bias(v, 16 * c_full, rem);
+          score_piece<FAST, true>(a, kc, v, rem, mx, x);
+          tmem_st2(t_row + 16 * c_full, x);
         }
         tmem_st_wait();
-        mx = max(-128, min(127, mx));
-        part_max[half * 128 + trow] = mx;
+        part_max[half * 128 + trow] = max(-128, min(127, mx));
       }
       // only the two warps that share these 32 rows exchange partial results: a barrier of their own
       asm volatile("bar.sync %0, 64;" ::"r"(2 + qd) : "memory");
-      unsigned sum = 0;
-      if (got_s && warp_ok) {
-        mx = max(part_max[trow], part_max[128 + trow]);
-        // pass B: ShiftExp(I - I_max) by table, row sum, exponentials back into tensor memory
-        // entry (I_max - I) of the table = word at tab + 4*(I_max + 128) - 4*(I + 128)
-        const uint8_t* tmx = reinterpret_cast<const uint8_t*>(tab) + 4 * (mx + 128);
-#pragma unroll 1
-        for (int c = c_lo + half; c < c_end; c += 2) {
-          int ev[16];
-          uint32_t xs[4];
-          tmem_ld4(t_row + c * 16, xs);
+      if (work) {
+        // pass B: entry (I_max - I) of this lane's table copy stands at tab_lane + 4 cp (I_max - I)
+        const uint32_t tmx = tab_lane + (uint32_t)(4 * a.cp * max(part_max[trow], part_max[128 + trow]));
+        unsigned sum = 0;
+#pragma unroll 2
+        for (int c = c_lo + half; c < c_full; c += 2) {
+          uint32_t x[4];
+          tmem_ld4(t_row + 16 * c, x);
+          int e[16];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const uint32_t w = xs[k];
+          for (int i = 0; i < 16; ++i) e[i] = (int)exp_entry(x[i >> 2], kc.sel[i & 3], tmx);
+          tmem_st16(t_row + 16 * c, e);
 #pragma unroll
-            for (int bb = 0; bb < 4; ++bb)
-              ev[4 * k + bb] = (int)*reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(w, 0, 0x4440 + bb));
-          }
-          if (c >= c_end - 2) {   // columns past T contribute nothing
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (c * 16 + j - col0 >= a.T) ev[j] = 0;
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) sum += (unsigned)ev[j];
-          tmem_st16(t_row + c * 16, ev);
+          for (int i = 0; i < 16; i += 4) sum += ((unsigned)e[i] + (unsigned)e[i + 1]) + ((unsigned)e[i + 2] + (unsigned)e[i + 3]);
         }
-        if (tail8 && half == 1) {
-          int ev[8];
-          uint32_t xs2[2];
-          tmem_ld2(t_row + ct, xs2);
+        if (rem) {
+          uint32_t x[4];
+          tmem_ld4(t_row + 16 * c_full, x);
+          int e[16];
 #pragma unroll
-          for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb)
-              ev[4 * k + bb] = (int)*reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(xs2[k], 0, 0x4440 + bb));
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            if (ct + j >= a.T) ev[j] = 0;
-            sum += (unsigned)ev[j];
+          for (int i = 0; i < 16; ++i) {
+            e[i] = i < rem ? (int)exp_entry(x[i >> 2], kc.sel[i & 3], tmx) : 0;
+            sum += (unsigned)e[i];
           }
-          tmem_st8(t_row + ct, ev);
+          tmem_st16(t_row + 16 * c_full, e);
         }
         tmem_st_wait();
         part_sum[half * 128 + trow] = sum;
       }
       asm volatile("bar.sync %0, 64;" ::"r"(2 + qd) : "memory");
-      if (got_s && warp_ok) {
-        sum = part_sum[trow] + part_sum[128 + trow];
-        // pass C: Eq. (IntDiv) with M = 45 (prob_word)
-        const unsigned factor = (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
-#pragma unroll 1
-        for (int c = c_lo + half; c < c_end; c += 2) {
-          int ev[16];
-          tmem_ld16(t_row + c * 16, ev);
-          uint32_t w[4];
+      if (work) {
+        // pass C: Eq. (IntDiv) with M = 45
+        const unsigned sum = part_sum[trow] + part_sum[128 + trow];
+        const unsigned factor = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
+        auto words = [&](const int (&e)[16]) {
+          uint32_t o[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            w[k] = prob_word<K8>(factor, ev[4 * k], ev[4 * k + 1], ev[4 * k + 2], ev[4 * k + 3], 14 - a.smax.k_out, (1 << (a.smax.k_out - 1)) - 1);
-          // A operand of P V: row = tile row, k-block = 128 columns, 16-byte pieces XOR (row & 7)
-          uint8_t* prow = gen + p_off + (c >> 3) * (128 * 128) + trow * 128;
-          *reinterpret_cast<uint4*>(prow + ((((c & 7)) ^ (trow & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-        if (!kPack) {
-          if (tail8 && half == 1) {   // the 8-column piece and eight zeros
-            int ev[8];
-            tmem_ld8(t_row + ct, ev);
-            const uint32_t w0 = prob_word<K8>(factor, ev[0], ev[1], ev[2], ev[3], 14 - a.smax.k_out, (1 << (a.smax.k_out - 1)) - 1);
-            const uint32_t w1 = prob_word<K8>(factor, ev[4], ev[5], ev[6], ev[7], 14 - a.smax.k_out, (1 << (a.smax.k_out - 1)) - 1);
-            uint8_t* prow = gen + p_off + (c_end >> 3) * (128 * 128) + trow * 128;
-            *reinterpret_cast<uint4*>(prow + ((((c_end & 7)) ^ (trow & 7)) << 4)) = make_uint4(w0, w1, 0u, 0u);
-          }
-          // chunks wholly past T: probability 0 (the contraction of P V runs over Npad columns)
-          for (int c = c_real + half; c < nch; c += 2) {
-            uint8_t* prow = gen + p_off + (c >> 3) * (128 * 128) + trow * 128;
-            *reinterpret_cast<uint4*>(prow + ((((c & 7)) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+          for (int q = 0; q < 4; ++q)
+            o[q] = FAST ? prob_word8(factor, e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3])
+                        : prob_word(factor, e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3], osh, omax);
+          return make_uint4(o[0], o[1], o[2], o[3]);
+        };
+#pragma unroll 1
+        for (int c = c_lo + half; c < c_full; c += 4) {
+          int e[2][16];
+          const bool second = c + 2 < c_full;
+          tmem_ld16_issue(t_row + 16 * c, e[0]);
+          if (second) tmem_ld16_issue(t_row + 16 * c + 32, e[1]);
+          tmem_ld_wait16(e[0]);
+          *p_addr(c) = words(e[0]);
+          if (second) {
+            tmem_ld_wait16(e[1]);
+            *p_addr(c + 2) = words(e[1]);
           }
         }
-        if (kPack) {   // the other windows' columns of this row: probability 0, so that P V stays inside the window
-          for (int c = half; c < nch; c += 2)
-            if (c < c_lo || c >= c_hi)
-              *reinterpret_cast<uint4*>(gen + p_off + trow * 128 + ((((c & 7)) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        if (rem) {
+          int e[16];
+          tmem_ld16(t_row + 16 * c_full, e);
+          *p_addr(c_full) = words(e);
         }
         fence_async_smem();
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);
-      // ---- output: O = sat8(rq(P V; pv_scale)), heads concatenated along the feature dimension ----
-      const bool got_o = alive && mbar_wait(bar_o, par, a.status);
-      alive = alive && got_o;
-      if (got_o) {
+      // ---- output, heads concatenated along the feature dimension ----
+      alive = alive && mbar_wait(bar_o, par, a.status);
+      if (work && alive) {
         tc_fence_after();
-        const long long pv_c = 1ll << (a.pv_s - 1);
-        int8_t* orow = a.O + ((int64_t)b * a.T + r) * a.D + (int64_t)h * a.d;
-        for (int c = half; c < a.d / 32; c += 2) {
-          if (!warp_ok) break;
-          int v[32];
-          tmem_ld32(t_row + c * 32, v);
-          if (row_ok) {
-            if (a.pv_s >= 33) {   // high product word plus 2^(s-33), shifted by s - 32
-              const int pv_rnd = 1 << (a.pv_s - 33), pv_sh = a.pv_s - 32;
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] = mad_hi(v[j], a.pv_m, pv_rnd) >> pv_sh;
-            } else {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) v[j] = (int)(((long long)v[j] * a.pv_m + pv_c) >> a.pv_s);
-            }
-            int4 w0, w1;
-            w0.x = (int)pack_sat8(v[0], v[1], v[2], v[3]);     w0.y = (int)pack_sat8(v[4], v[5], v[6], v[7]);
-            w0.z = (int)pack_sat8(v[8], v[9], v[10], v[11]);   w0.w = (int)pack_sat8(v[12], v[13], v[14], v[15]);
-            w1.x = (int)pack_sat8(v[16], v[17], v[18], v[19]); w1.y = (int)pack_sat8(v[20], v[21], v[22], v[23]);
-            w1.z = (int)pack_sat8(v[24], v[25], v[26], v[27]); w1.w = (int)pack_sat8(v[28], v[29], v[30], v[31]);
-            reinterpret_cast<int4*>(orow + c * 32)[0] = w0;
-            reinterpret_cast<int4*>(orow + c * 32)[1] = w1;
-          }
+        int8_t* orow = a.O + ((int64_t)b * a.T + r) * a.D + (int64_t)item.h * a.d;
+#pragma unroll 1
+        for (int c = half; c < a.d / 16; c += 2) {
+          int v[16];
+          tmem_ld16(t_row + 16 * c, v);
+          const uint4 w = output_piece<FAST>(a, v);
+          if (row_ok) *reinterpret_cast<uint4*>(orow + 16 * c) = w;
         }
       }
       // tensor memory may take the next item's scores
@@ -440,67 +546,62 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attention_kernel(const __grid
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // the last CTA to finish leaves the counters at zero for the next launch
-    __threadfence();
-    if (atomicAdd(a.sched + 1, 1u) == gridDim.x - 1) {
-      a.sched[0] = 0;
-      a.sched[1] = 0;
-      __threadfence();
-    }
-  }
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, (uint32_t)a.tmem_cols);
+    tmem_dealloc(tmem, (uint32_t)sa.tmem_cols);
   }
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Rows longer than 256 tokens.  The score tile of a 128-row block no longer fits tensor memory, so the keys are
-// taken in blocks of NB columns (the last block holds the remainder): S_j = Q K_j^T goes into one of two
-// tensor-memory buffers, pass A requantises it and parks the int8 scores in shared memory, in the very place and
-// layout (K-major, 128-byte swizzle) where the probabilities of the second MMA's A operand will stand, while the
-// MMA of the next block fills the other buffer.  After the last block the row maximum is known: pass B sums the
-// exponentials from the parked bytes, pass C turns the bytes into probabilities in place, and O = P V accumulates
-// over the whole row in its own tensor-memory columns.  One CTA per SM; four threads share a score row (one TMEM
-// lane; each takes a quarter of every key block).  The control thread runs one block ahead of the Shiftmax
-// threads, also across work items.
-constexpr int kLongThreads = 544;   // warp 0: TMA + MMA issue + TMEM owner; warps 1..16: four threads per score row
+// Rows of more than 256 tokens.  One CTA per SM; sixteen Shiftmax warps share a 128-row tile, four threads per score row
+// (thread `part` takes the 16-column chunks part, part + 4, ...).
+//   S       the score columns are taken in blocks of 192, each in one of two tensor-memory buffers; the MMA of the next
+//           block, or of the next work item, runs while the Shiftmax passes work on the scores already read;
+//   scores  after pass A they are parked in shared memory, where (and in the layout in which) the probabilities will
+//           stand;
+//   output  O = P V has tensor-memory columns of its own and is read beside the reciprocals of the NEXT item's rows.
+// The chunk loops are rolled: straight-line code for all chunks waited for instructions more than for anything else.
+// Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 190 us (before: one table, remainders dealt to all threads, a wait
+// for P V in every item).  On rows of up to 256 tokens the two CTAs per SM of the kernel above win: 22.3 against 29.6 us
+// at 64 x 197, 6 heads.
+// Warps 0..3: warp 0 loads, issues MMAs and owns tensor memory (the others of its warpgroup only lend their registers);
+// warps 4..19: the Shiftmax threads.  The launch gives every warp 96 registers (640 threads); the first warpgroup hands
+// all but 64 of its own back, which lets the other four take 104: 128 x 64 + 512 x 104 = 640 x 96.
+constexpr int kRowsThreads = 640;
+constexpr int kRowsFirst = 4;       // first Shiftmax warp
+constexpr int kBlkChunks = 12;      // 16-column chunks per score block
 
-struct LongArgs {
+struct RowsArgs {
   AttnArgs a;
-  int NB;      // key-block width, a multiple of 32
-  int nblk;    // key blocks per row (>= 2)
-  int nv;      // 256-row boxes that bring V
+  int wb;                           // columns of a score buffer in tensor memory (buffers at 0 and wb, output at 2 wb)
+  int nblk;                         // score blocks per row
+  int vbox, nv;                     // rows of a value box and their number
+  uint32_t p_stride;                // bytes between the two probability buffers of even / odd items (0: one buffer)
 };
 
-__device__ __forceinline__ void tmem_ld_cols(uint32_t addr, int (&v)[16]) { tmem_ld16(addr, v); }
-__device__ __forceinline__ void tmem_ld_cols(uint32_t addr, int (&v)[8]) { tmem_ld8_issue(addr, v); tmem_ld_wait8(v); }
-
-template <bool K8>
-__global__ void __launch_bounds__(kLongThreads, 1) attention_long_kernel(const __grid_constant__ CUtensorMap tmQ,
+template <bool FAST, bool BIAS>
+__global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                         const __grid_constant__ CUtensorMap tmK,
-                                                                        const __grid_constant__ CUtensorMap tmV, LongArgs la) {
-  const AttnArgs& a = la.a;
-  const int NB = la.NB, nblk = la.nblk;
+                                                                        const __grid_constant__ CUtensorMap tmV, RowsArgs ra) {
+  const AttnArgs& a = ra.a;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
-  // [Q 128x128B][K block x 2][V 256 nv x d][P / parked scores 128 x 128B x kblocks][exp table][row partials][item ring][barriers]
-  const uint32_t q_off = 0, k_off = 128 * 128, kbuf_bytes = (uint32_t)NB * 128;
-  const uint32_t v_off = k_off + 2 * kbuf_bytes, v_bytes = (uint32_t)la.nv * 256 * a.d;
+  // [Q 128 x d][K block x 2][V nv vbox x d][P 128 x 128B x kblocks, x 2][table 256 x cp][row partials][seeds][items][barriers]
+  const uint32_t k_off = 128u * a.d, kbuf_bytes = (uint32_t)a.kbox * a.d;
+  const uint32_t v_off = k_off + 2 * kbuf_bytes, v_bytes = (uint32_t)(ra.nv * ra.vbox) * a.d;
   const uint32_t p_off = (v_off + v_bytes + 1023u) & ~1023u;
-  const uint32_t tab_off = p_off + (uint32_t)((a.Npad + 127) / 128) * 128 * 128;
-  const uint32_t part_off = tab_off + 1024;              // [4 column quarters][128 rows] partial max, then partial sum
-  const uint32_t item_off = part_off + 4 * 128 * 4 * 2;  // [2] work item of even / odd iterations (-1: no more work)
-  const uint32_t bar_off = item_off + 16;
-  unsigned* tab = reinterpret_cast<unsigned*>(gen + tab_off);
-  volatile int* item_ring = reinterpret_cast<volatile int*>(gen + item_off);
+  const uint32_t tab_off = p_off + ra.p_stride + (uint32_t)((a.kpad + 127) / 128) * 128 * 128;
+  const uint32_t part_off = tab_off + 1024u * a.cp;      // [4 parts][128 rows] partial max, then partial sum, [128] reciprocals
+  const uint32_t seed_off = part_off + 9 * 128 * 4;      // [128] seeds of the reciprocal
+  const uint32_t item_off = seed_off + 128 * 4;          // [2] work item of even / odd iterations, written before its first scores
+  const uint32_t bar_off = item_off + 2 * sizeof(AttnItem);
+  AttnItem* const item_ring = reinterpret_cast<AttnItem*>(gen + item_off);
   // Q landed | V landed | K block landed (x2) | scores ready (x2) | score buffer read (x2) | probabilities written |
-  // output ready | output read | item published
+  // output ready
   const uint32_t bar_q = base + bar_off, bar_v = bar_q + 8, bar_k = bar_q + 16, bar_s = bar_q + 32, bar_f = bar_q + 48,
-                 bar_p = bar_q + 64, bar_o = bar_q + 72, bar_e = bar_q + 80, bar_item = bar_q + 88;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 128);
+                 bar_p = bar_q + 64, bar_o = bar_q + 72;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 80);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
@@ -511,13 +612,11 @@ __global__ void __launch_bounds__(kLongThreads, 1) attention_long_kernel(const _
     mbar_init(bar_v, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_k + 8 * i, 1);
-      mbar_init(bar_s + 8 * i, 1);
+      mbar_init(bar_s + 8 * i, 2);   // the MMAs, and the control thread (the item is in the ring)
       mbar_init(bar_f + 8 * i, 16);
     }
     mbar_init(bar_p, 16);
     mbar_init(bar_o, 1);
-    mbar_init(bar_e, 16);
-    mbar_init(bar_item, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -526,356 +625,311 @@ __global__ void __launch_bounds__(kLongThreads, 1) attention_long_kernel(const _
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t o_col = 2u * (uint32_t)NB;   // output accumulator behind the two score buffers
+  const uint32_t o_col = 2u * (uint32_t)ra.wb;
   pdl_trigger();
-  if (warp == 0) pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
+  const int nblk = ra.nblk;
+  const uint32_t n_items = AttnItem::count(a);
 
-  if (warp == 0) {
-    if (lane == 0) {
-      auto coords = [&](int item, int& tile, int& h, int& b) {
-        tile = item / a.bh;
-        const int bhid = item - tile * a.bh;
-        h = bhid % a.heads;
-        b = bhid / a.heads;
+  if (warp < kRowsFirst) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    if (warp == 0) pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
+    if (warp == 0 && lane == 0 && n_items > 0) {
+      auto load_q = [&](const AttnItem& it) {
+        mbar_expect_tx(bar_q, 128u * a.d);
+        for (int g = 0; g < 4; ++g)
+          load_box(base + (uint32_t)((g + it.rot) & 3) * 32u * a.d, &tmQ, bar_q, a.q_pos, it.m0 + 32 * g, it.h, it.b);
       };
-      auto load_q = [&](int item) {
-        int tile, h, b;
-        coords(item, tile, h, b);
-        mbar_expect_tx(bar_q, 128 * 128);
-        int c[4];
-        c[0] = 0; c[a.q_pos[0]] = tile * 128; c[a.q_pos[1]] = h; c[a.q_pos[2]] = b;
-        tma_load_4d(base + q_off, &tmQ, bar_q, c[0], c[1], c[2], c[3]);
-      };
-      auto load_k = [&](int item, int j, uint32_t buf) {
-        int tile, h, b;
-        coords(item, tile, h, b);
-        mbar_expect_tx(bar_k + 8 * buf, kbuf_bytes);
-        int c[4];
-        c[0] = 0; c[a.k_pos[0]] = j * NB; c[a.k_pos[1]] = h; c[a.k_pos[2]] = b;
-        tma_load_4d(base + k_off + buf * kbuf_bytes, &tmK, bar_k + 8 * buf, c[0], c[1], c[2], c[3]);
-      };
-      auto load_v = [&](int item) {
-        int tile, h, b;
-        coords(item, tile, h, b);
+      auto load_v = [&](const AttnItem& it) {
         mbar_expect_tx(bar_v, v_bytes);
-        for (int i = 0; i < la.nv; ++i) {
-          int c[4];
-          c[0] = 0; c[a.v_pos[0]] = i * 256; c[a.v_pos[1]] = h; c[a.v_pos[2]] = b;
-          tma_load_4d(base + v_off + (uint32_t)i * 256u * a.d, &tmV, bar_v, c[0], c[1], c[2], c[3]);
-        }
+        for (int i = 0; i < ra.nv; ++i)
+          load_box(base + v_off + (uint32_t)(i * ra.vbox) * a.d, &tmV, bar_v, a.v_pos, i * ra.vbox, it.h, it.b);
       };
-      auto draw = [&]() {
-        const unsigned t = atomicAdd(a.sched, 1u);
-        return t < (unsigned)a.items ? (int)t : -1;
-      };
-      auto publish = [&](uint32_t n, int item) {
-        item_ring[n & 1u] = item;
-        mbar_arrive(bar_item);   // release: the item is visible to whoever sees this phase complete
-      };
+      // descriptor words: rows of d bytes (Q, K, V: swizzled over their width) or 128 bytes (P)
+      const uint32_t layout = a.d == 128 ? 2u : (a.d == 64 ? 4u : 6u);
+      const uint32_t row_hi = desc_hi(8u * a.d, layout), p_hi = desc_hi(1024, 2);
+      const uint32_t q_lo0 = desc_lo(base, 16), k_lo0 = desc_lo(base + k_off, 16), p_lo0 = desc_lo(base + p_off, 16),
+                     v_lo0 = desc_lo(base + v_off, 16), v_step = (uint32_t)(UK * a.d) >> 4;
       const uint32_t idesc2 = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(a.d >> 3) << 17) | (8u << 24);
-      const uint32_t v_layout = a.d == 128 ? 2u : (a.d == 64 ? 4u : 6u);
-      const int ks = (a.d + UK - 1) / UK, ks2 = a.Npad / UK;
+      const int ks = a.d / UK, ks2 = a.kpad / UK;
 
-      uint32_t g = 0;            // key blocks issued so far, over all items of this CTA
+      uint32_t g = 0, gk = 0;    // score blocks issued / key blocks requested so far, over all items of this CTA
       bool ok = true;
       bool q_fly = false, v_fly = false, k_fly[2] = {false, false};   // loads requested and not yet waited for
       uint32_t q_par = 0, v_par = 0, k_par[2] = {0, 0};
-      // S_buf = Q K_j^T for key block j of `item` (the n-th item of this CTA), then the load of the key block that
-      // follows it in the order of issue: block j + 1 of the same item, or block 0 of `next_item`.
-      auto issue_block = [&](int item, int j, uint32_t n, int next_item) {
+      auto load_k = [&](const AttnItem& it, int j) {
+        const uint32_t buf = gk & 1u, ph = (gk >> 1) & 1u;
+        // the MMAs of the block two before this one have read the buffer
+        if (gk >= 2) ok = mbar_wait(bar_s + 8 * buf, ph ^ 1u, a.status);
+        if (!ok) return;
+        mbar_expect_tx(bar_k + 8 * buf, kbuf_bytes);
+        load_box(base + k_off + buf * kbuf_bytes, &tmK, bar_k + 8 * buf, a.k_pos, j * (16 * kBlkChunks), it.h, it.b);
+        k_fly[buf] = true;
+        k_par[buf] = ph;
+        ++gk;
+      };
+      // S_buf = Q K_j^T for key block j of the n-th item of this CTA
+      auto issue_block = [&](const AttnItem& it, int j, uint32_t n) {
         const uint32_t buf = g & 1u, ph = (g >> 1) & 1u;
         ok = mbar_wait(bar_k + 8 * buf, ph, a.status);
         k_fly[buf] = !ok;
         if (ok && j == 0) { ok = mbar_wait(bar_q, n & 1u, a.status); q_fly = !ok; }
-        // pass A of the block that used this score buffer two blocks ago has read it
+        // pass A of the block that used this score buffer two blocks ago has read it.  (With it every Shiftmax thread is
+        // past item n - 2, whose place in the ring item n takes: nblk >= 2.)
         if (ok && g >= 2) ok = mbar_wait(bar_f + 8 * buf, ph ^ 1u, a.status);
         if (!ok) return;
+        if (j == 0) item_ring[n & 1u] = it;
         tc_fence_after();
-        const int w = j == nblk - 1 ? a.Npad - j * NB : NB;
+        const int w = j == nblk - 1 ? 16 * a.chunks - j * 16 * kBlkChunks : 16 * kBlkChunks;
         const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(w >> 3) << 17) | (8u << 24);
+        const uint32_t k_lo = k_lo0 + buf * (kbuf_bytes >> 4), d_tmem = tmem + buf * (uint32_t)ra.wb;
         for (int k = 0; k < ks; ++k)
-          umma_i8(tmem + buf * (uint32_t)NB, smem_desc(base + q_off + k * UK, 16, 1024, 2),
-                  smem_desc(base + k_off + buf * kbuf_bytes + k * UK, 16, 1024, 2), idesc, k != 0);
+          umma_i8_lohi(d_tmem, q_lo0 + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
         umma_commit(bar_s + 8 * buf);
-        const int fj = j + 1 < nblk ? j + 1 : 0;
-        const int fitem = j + 1 < nblk ? item : next_item;
-        if (fitem >= 0) {
-          // the other key buffer was read by the MMAs of the block before this one
-          if (g >= 1) ok = mbar_wait(bar_s + 8 * (buf ^ 1u), ((g - 1) >> 1) & 1u, a.status);
-          if (!ok) return;
-          load_k(fitem, fj, buf ^ 1u);
-          k_fly[buf ^ 1u] = true;
-          k_par[buf ^ 1u] = ((g + 1) >> 1) & 1u;
-        }
+        mbar_arrive(bar_s + 8 * buf);   // releases the item written to the ring
         ++g;
       };
 
-      int cur = draw();
-      uint32_t n = 0;
-      bool first_issued = false;   // block 0 of `cur` went out at the end of the item before it
-      if (cur >= 0) {
-        load_q(cur); q_fly = true; q_par = 0;
-        load_v(cur); v_fly = true; v_par = 0;
-        load_k(cur, 0, 0); k_fly[0] = true; k_par[0] = 0;
-        publish(0, cur);
-      }
-      while (cur >= 0) {
-        int next = -1;
-        for (int j = first_issued ? 1 : 0; ok && j < nblk; ++j) {
-          if (j == nblk - 1) next = draw();
-          issue_block(cur, j, n, next);
+      AttnItem cur, next;
+      cur.init(a, 0);
+      load_q(cur); q_fly = true; q_par = 0;
+      load_k(cur, 0);
+      load_v(cur); v_fly = true; v_par = 0;
+      issue_block(cur, 0, 0);
+      if (ok) load_k(cur, 1);
+      for (uint32_t n = 0; ok && n < n_items; ++n) {
+        // block 0 of `cur` has been issued, its block 1 requested
+        const bool more = n + 1 < n_items;
+        if (more) next.init(a, n + 1);
+        for (int j = 1; ok && j < nblk; ++j) {
+          issue_block(cur, j, n);
+          if (!ok) break;
+          if (j + 1 < nblk) load_k(cur, j + 1);
+          else if (more) load_k(next, 0);
         }
         if (!ok) break;
-        // Q may be overwritten once the score MMAs of the last block have read it
-        ok = mbar_wait(bar_s + 8 * ((g - 1) & 1u), ((g - 1) >> 1) & 1u, a.status);
-        if (!ok) break;
-        if (next >= 0) {
+        if (more) {
+          // Q may be overwritten once the score MMAs of the last block have read it
+          ok = mbar_wait(bar_s + 8 * ((g - 1) & 1u), ((g - 1) >> 1) & 1u, a.status);
+          if (!ok) break;
           load_q(next); q_fly = true; q_par = (n + 1) & 1u;
-          // The item barrier may run one phase ahead of its readers at most: every Shiftmax warp has taken item n
-          // once it has handed back the score buffer of that item's last key block (the latest phase of that
-          // barrier: the block that completes it next has not been issued yet).
-          ok = mbar_wait(bar_f + 8 * ((g - 1) & 1u), ((g - 1) >> 1) & 1u, a.status);
-          if (!ok) break;
-          publish(n + 1, next);
-          issue_block(next, 0, n + 1, -1);   // nblk >= 2: the block after it belongs to the same item
+          issue_block(next, 0, n + 1);
+          if (ok) load_k(next, 1);
           if (!ok) break;
         }
-        // O = P V once the probabilities are in shared memory, V has landed and the previous output has been read
+        // O = P V once the probabilities are in shared memory (every warp has then read the previous output too)
+        // and V has landed
         ok = mbar_wait(bar_p, n & 1u, a.status);
         if (ok) { ok = mbar_wait(bar_v, n & 1u, a.status); v_fly = !ok; }
-        if (ok && n > 0) ok = mbar_wait(bar_e, (n - 1) & 1u, a.status);
         if (!ok) break;
         tc_fence_after();
-        for (int k = 0; k < ks2; ++k) {
-          const uint32_t pa = base + p_off + (k >> 2) * (128 * 128) + (k & 3) * UK;
-          umma_i8(tmem + o_col, smem_desc(pa, 16, 1024, 2), smem_desc(base + v_off + k * UK * a.d, 16, 8 * a.d, v_layout),
-                  idesc2, k != 0);
-        }
+        uint32_t p_lo = p_lo0 + (n & 1u) * (ra.p_stride >> 4), v_lo = v_lo0;
+        int k = 0;
+        for (; k + 4 <= ks2; k += 4, p_lo += (128 * 128) >> 4, v_lo += 4 * v_step)
+          umma_i8_x4(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
+        for (; k < ks2; ++k, p_lo += UK >> 4, v_lo += v_step)
+          umma_i8_lohi(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
         umma_commit(bar_o);
-        // V (and the probabilities) may be overwritten once these MMAs have read them
+        // V may be overwritten once these MMAs have read it
         ok = mbar_wait(bar_o, n & 1u, a.status);
         if (!ok) break;
-        if (next >= 0) { load_v(next); v_fly = true; v_par = (n + 1) & 1u; }
+        if (more) { load_v(next); v_fly = true; v_par = (n + 1) & 1u; }
         cur = next;
-        ++n;
-        first_issued = true;
       }
-      // end of work (or a wait that timed out): tell the other warps; nothing may be in flight at exit
-      publish(ok ? n : n + 1, -1);
+      // end of work (or a wait that timed out): nothing may be in flight at exit
       if (q_fly) mbar_wait(bar_q, q_par, a.status);
       if (v_fly) mbar_wait(bar_v, v_par, a.status);
       for (int i = 0; i < 2; ++i)
         if (k_fly[i]) mbar_wait(bar_k + 8 * i, k_par[i], a.status);
     }
   } else {
-    // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the four warps of a quarter take the four
-    //      quarters of every key block of the same 32 rows ----
-    const int st = threadIdx.x - 32;   // 0..511
-    if (st < 256) tab[st] = shiftexp(-st, a.smax.I0, a.smax.N);
-    pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 32) {
-      a.sched_other[0] = 0;
-      a.sched_other[1] = 0;
-    }
+    // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the four warps of a quarter share its 32 rows
+    //      (and their scheduler) ----
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+    const int st = threadIdx.x - 32 * kRowsFirst;   // 0..511
     const int qd = warp & 3;
-    const int part = (warp - 1) >> 2;             // 0..3
+    const int part = (warp - kRowsFirst) >> 2;    // 0..3
     const int trow = qd * 32 + lane;              // row inside the tile
+    build_exp_table(a, gen + tab_off, st, 512);
+    // probabilities of columns past the last chunk are never written again: zero (P V contracts over kpad columns)
+    for (int c = a.chunks + part; c < a.kpad / 16; c += 4)
+      for (int u = 0; u < 2; ++u)
+        *reinterpret_cast<uint4*>(gen + p_off + u * ra.p_stride + (c >> 3) * (128 * 128) + trow * 128 + (((c & 7) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+    unsigned* seeds = reinterpret_cast<unsigned*>(gen + seed_off);
+    if (st < 128) seeds[st] = recip_seed(st);
+    pdl_wait();
+    PassConsts kc;
+    kc.init(a);
     const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16);
-    const bool qk_hi = a.qk_s >= 33;              // rounding constant and shift both past the low product word
-    const long long qk_c = 1ll << (a.qk_s - 1);
-    const int qk_rnd = qk_hi ? 1 << (a.qk_s - 33) : 0, qk_sh = a.qk_s - 32;
     int* part_max = reinterpret_cast<int*>(gen + part_off);
     unsigned* part_sum = reinterpret_cast<unsigned*>(gen + part_off + 4 * 128 * 4);
-    uint8_t* p_row = gen + p_off + trow * 128;    // this row inside every 128-column block of P
-    // byte address of 8 or 16 consecutive columns (col a multiple of 8 / 16) of this row in the A-operand layout
-    auto p_addr = [&](int col) { return p_row + (col >> 7) * (128 * 128) + ((((col >> 4) & 7) ^ (trow & 7)) << 4) + (col & 8); };
-    // this thread's pieces of key block j: whole 16-column chunks, an 8-column piece in front / behind when the
-    // quarter starts / ends on an odd multiple of 8
-    auto walk = [&](int j, auto&& fn) {
-      const int cb = j * NB;
-      const int w = j == nblk - 1 ? a.Npad - cb : NB;
-      const int lo = cb + part * (w >> 2), hi = lo + (w >> 2);
-      const int c16_lo = (lo + 15) & ~15, c16_hi = hi & ~15;
-      if (lo & 8) { int v[8]; fn(v, lo, cb); }
-#pragma unroll 1
-      for (int c = c16_lo; c < c16_hi; c += 16) { int v[16]; fn(v, c, cb); }
-      if (hi & 8) { int v[8]; fn(v, c16_hi, cb); }
-    };
+    unsigned* recips = reinterpret_cast<unsigned*>(gen + part_off + 8 * 128 * 4);
+    const uint32_t tab_lane = base + tab_off + 4u * (unsigned)(lane & (a.cp - 1));
+    const unsigned top = (unsigned)a.smax.I0 << a.smax.N;    // the largest exponential
+    const int osh = 14 - a.smax.k_out, omax = (1 << (a.smax.k_out - 1)) - 1;
+    // whole chunks c = part, part + 4, ... of this thread in the A-operand layout: k-block c >> 3, 16-byte piece c & 7;
+    // the remainder of rem columns belongs to part 3, whose share of whole chunks is never the larger one
+    const int c_full = a.T >> 4, rem = part == 3 ? a.T & 15 : 0;
+    const uint32_t sw0 = (uint32_t)((part ^ (trow & 7)) << 4), sw1 = (uint32_t)(((part + 4) ^ (trow & 7)) << 4);
+    uint8_t* p_row = gen + p_off + trow * 128;
+    auto p_addr = [&](int c) { return reinterpret_cast<uint4*>(p_row + (c >> 3) * (128 * 128) + ((c & 4) ? sw1 : sw0)); };
+    auto p_tail = [&]() { return reinterpret_cast<uint4*>(p_row + (c_full >> 3) * (128 * 128) + (((c_full & 7) ^ (trow & 7)) << 4)); };
     asm volatile("bar.sync 1, 512;" ::: "memory");   // the table is complete
 
     bool alive = true;   // false after a wait that timed out: no more waits, no more work, only the barriers
-    uint32_t g = 0;      // key blocks seen so far (same count as the control thread's)
-    for (uint32_t n = 0;; ++n) {
-      const uint32_t par = n & 1u;
-      bool got_item = false;
-      if (alive) {
-        for (uint32_t w = 0; w < kItemWaitRounds && !got_item; ++w) got_item = mbar_wait(bar_item, par, a.status);
+    uint32_t g = 0;      // score blocks seen so far (same count as the control thread's)
+    int8_t* o_prev = nullptr;          // output row of the previous item (nullptr: none, or no row of the tile)
+    bool o_prev_warp = false;          // the previous item had rows in this lane quarter
+    // the output of the previous item, heads concatenated along the feature dimension
+    auto store_output = [&](uint32_t n_prev) {
+      alive = alive && mbar_wait(bar_o, n_prev & 1u, a.status);
+      if (!alive || !o_prev_warp) return;
+      tc_fence_after();
+#pragma unroll 1
+      for (int c = part; c < a.d / 16; c += 4) {
+        int v[16];
+        tmem_ld16(t_row + o_col + 16 * c, v);
+        const uint4 w = output_piece<FAST>(a, v);
+        if (o_prev) *reinterpret_cast<uint4*>(o_prev + 16 * c) = w;
       }
-      const int item = got_item ? item_ring[par] : -1;
-      if (item < 0) break;
-      const int tile = item / a.bh, bhid = item - tile * a.bh;
-      const int h = bhid % a.heads, b = bhid / a.heads;
-      const int m0 = tile * 128;
-      const int r = m0 + trow;                      // token (row) inside this image
-      const bool row_ok = r < a.T;
-      const bool warp_ok = m0 + qd * 32 < a.T;      // warps whose 32 rows all lie past T only keep the barriers
-      const int32_t* brow = a.bias ? a.bias + (((int64_t)bhid % a.bias_batches) * a.T + (row_ok ? r : 0)) * (int64_t)a.T : nullptr;
+      tc_fence_before();
+    };
 
-      // pass A, key block by key block: requantise the scores to int8 (Sec. 3.2), park them as biased bytes
-      // (x + 128) where the probabilities will stand, running maximum
+    for (uint32_t n = 0; n < n_items; ++n) {
+      alive = alive && mbar_wait(bar_s + 8 * (g & 1u), (g >> 1) & 1u, a.status);
+      const AttnItem item = item_ring[n & 1u];
+      const int m0 = item.m0 + ((qd - item.rot) & 3) * 32;   // first row (token) of this lane quarter
+      const int r = m0 + lane;
+      const bool row_ok = r < a.T;
+      const bool warp_ok = m0 < a.T;                // quarters whose 32 rows all lie past T only keep the barriers
+      const int32_t* brow = nullptr;
+      if (BIAS) brow = a.bias + ((int64_t)((unsigned)(item.b * a.heads + item.h) % (unsigned)a.bias_batches) * a.T + (row_ok ? r : 0)) * a.T;
+      auto add_bias = [&](auto& v, int col, int valid) {
+        if constexpr (BIAS) {
+#pragma unroll
+          for (int i = 0; i < (int)(sizeof(v) / sizeof(int)); ++i)
+            if (i < valid) v[i] += __ldg(brow + col + i);
+        }
+      };
+      p_row = gen + p_off + (n & 1u) * ra.p_stride + trow * 128;
+      // with one probability buffer the parked scores overwrite what the previous item's P V reads
+      if (ra.p_stride == 0 && n > 0) alive = alive && mbar_wait(bar_o, (n - 1) & 1u, a.status);
+
+      // pass A, score block by score block, two chunks at a time
       int mx = -128;
       for (int j = 0; j < nblk; ++j, ++g) {
-        const uint32_t buf = g & 1u;
-        const bool got_s = alive && mbar_wait(bar_s + 8 * buf, (g >> 1) & 1u, a.status);
-        alive = alive && got_s;
-        if (got_s) tc_fence_after();
-        if (got_s && warp_ok) {
-          const uint32_t t_buf = t_row + buf * (uint32_t)NB;
-          walk(j, [&](auto& v, int col, int cb) {
-            constexpr int W = (int)(sizeof(v) / sizeof(v[0]));
-            tmem_ld_cols(t_buf + (uint32_t)(col - cb), v);
-            if (brow) {
-#pragma unroll
-              for (int i = 0; i < W; ++i)
-                if (col + i < a.T) v[i] += __ldg(brow + col + i);
+        if (j) alive = alive && mbar_wait(bar_s + 8 * (g & 1u), (g >> 1) & 1u, a.status);
+        if (alive) tc_fence_after();
+        if (alive && warp_ok) {
+          const uint32_t t_buf = t_row + (g & 1u) * (uint32_t)ra.wb - (uint32_t)j * (16 * kBlkChunks);
+          const int c_end = j == nblk - 1 ? c_full : (j + 1) * kBlkChunks;
+#pragma unroll 1
+          for (int c = j * kBlkChunks + part; c < c_end; c += 8) {
+            int v[2][16];
+            const bool second = c + 4 < c_end;
+            tmem_ld16_issue(t_buf + 16 * c, v[0]);
+            if (second) tmem_ld16_issue(t_buf + 16 * c + 64, v[1]);
+            uint32_t x[4];
+            tmem_ld_wait16(v[0]);
+            add_bias(v[0], 16 * c, 16);
+            score_piece<FAST, false>(a, kc, v[0], 16, mx, x);
+            *p_addr(c) = make_uint4(x[0], x[1], x[2], x[3]);
+            if (second) {
+              tmem_ld_wait16(v[1]);
+              add_bias(v[1], 16 * c + 64, 16);
+              score_piece<FAST, false>(a, kc, v[1], 16, mx, x);
+              *p_addr(c + 4) = make_uint4(x[0], x[1], x[2], x[3]);
             }
-            if (qk_hi) {          // the usual case: high product word plus 2^(s-33), shifted by s - 32
-#pragma unroll
-              for (int i = 0; i < W; ++i) v[i] = mad_hi(v[i], a.qk_m, qk_rnd) >> qk_sh;
-            } else {
-#pragma unroll
-              for (int i = 0; i < W; ++i) v[i] = (int)(((long long)v[i] * a.qk_m + qk_c) >> a.qk_s);
-            }
-            if (col + W > a.T) {  // columns past T never win the maximum
-#pragma unroll
-              for (int i = 0; i < W; ++i)
-                if (col + i >= a.T) v[i] = -128;
-            }
-            int m = v[0];
-#pragma unroll
-            for (int i = 1; i < W; i += 2) m = max(m, max(v[i], v[(i + 1) & (W - 1)]));
-            mx = max(mx, m);
-            uint32_t xs[W / 4];
-#pragma unroll
-            for (int k = 0; k < W / 4; ++k)
-              xs[k] = pack_sat8(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]) ^ 0x80808080u;
-            if constexpr (W == 16) *reinterpret_cast<uint4*>(p_addr(col)) = make_uint4(xs[0], xs[1], xs[2], xs[3]);
-            else *reinterpret_cast<uint2*>(p_addr(col)) = make_uint2(xs[0], xs[1]);
-          });
+          }
+          if (j == nblk - 1 && rem > 8) {
+            int v[16];
+            uint32_t x[4];
+            tmem_ld16(t_buf + 16 * c_full, v);
+            add_bias(v, 16 * c_full, rem);
+            score_piece<FAST, true>(a, kc, v, rem, mx, x);
+            *p_tail() = make_uint4(x[0], x[1], x[2], x[3]);
+          } else if (j == nblk - 1 && rem) {
+            int v[8];
+            uint32_t x[2];
+            tmem_ld8(t_buf + 16 * c_full, v);
+            add_bias(v, 16 * c_full, rem);
+            score_piece<FAST, true>(a, kc, v, rem, mx, x);
+            *p_tail() = make_uint4(x[0], x[1], 0u, 0u);
+          }
         }
         // the score buffer may take the block after the next one
         tc_fence_before();
+        if (j == nblk - 1 && alive && warp_ok) part_max[part * 128 + trow] = max(-128, min(127, mx));
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_f + 8 * buf);
+        if (lane == 0) mbar_arrive(bar_f + 8 * (g & 1u));
       }
-      if (alive && warp_ok) part_max[part * 128 + trow] = max(-128, min(127, mx));
       // only the four warps that share these 32 rows exchange partial results: a barrier of their own
       asm volatile("bar.sync %0, 128;" ::"r"(2 + qd) : "memory");
-      unsigned sum = 0;
-      const uint8_t* tmx = nullptr;
-      if (alive && warp_ok) {
+      const bool work = alive && warp_ok;
+      uint32_t tmx = 0;
+      if (work) {
         mx = max(max(part_max[trow], part_max[128 + trow]), max(part_max[256 + trow], part_max[384 + trow]));
-        // pass B: ShiftExp(I - I_max) by table, row sum.  Entry (I_max - I) = word at tab + 4 (I_max + 128) - 4 (I + 128)
-        tmx = reinterpret_cast<const uint8_t*>(tab) + 4 * (mx + 128);
-        for (int j = 0; j < nblk; ++j) {
-          walk(j, [&](auto& ev, int col, int) {
-            constexpr int W = (int)(sizeof(ev) / sizeof(ev[0]));
-            uint32_t xs[W / 4];
-            if constexpr (W == 16) { const uint4 q = *reinterpret_cast<const uint4*>(p_addr(col)); xs[0] = q.x; xs[1] = q.y; xs[2] = q.z; xs[3] = q.w; }
-            else { const uint2 q = *reinterpret_cast<const uint2*>(p_addr(col)); xs[0] = q.x; xs[1] = q.y; }
+        // pass B: entry (I_max - I) of this lane's table copy stands at tab_lane + 4 cp (I_max - I)
+        tmx = tab_lane + (uint32_t)(4 * a.cp * mx);
+        unsigned sum = 0;
+#pragma unroll 2
+        for (int c = part; c < c_full; c += 4) {
+          const uint4 w = *p_addr(c);
+          const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+          unsigned e[16];
 #pragma unroll
-            for (int k = 0; k < W / 4; ++k)
+          for (int i = 0; i < 16; ++i) e[i] = exp_entry(x[i >> 2], kc.sel[i & 3], tmx);
 #pragma unroll
-              for (int bb = 0; bb < 4; ++bb)
-                ev[4 * k + bb] = (int)*reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(xs[k], 0, 0x4440 + bb));
-            if (col + W > a.T) {   // columns past T contribute nothing
+          for (int i = 0; i < 16; i += 4) sum += (e[i] + e[i + 1]) + (e[i + 2] + e[i + 3]);
+        }
+        if (rem) {
+          const uint4 w = *p_tail();
+          const uint32_t x[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-              for (int i = 0; i < W; ++i)
-                if (col + i >= a.T) ev[i] = 0;
-            }
-#pragma unroll
-            for (int i = 0; i < W; ++i) sum += (unsigned)ev[i];
-          });
+          for (int i = 0; i < 16; ++i) sum += i < rem ? exp_entry(x[i >> 2], kc.sel[i & 3], tmx) : 0u;
         }
         part_sum[part * 128 + trow] = sum;
       }
       asm volatile("bar.sync %0, 128;" ::"r"(2 + qd) : "memory");
-      if (alive && warp_ok) {
-        sum = (part_sum[trow] + part_sum[128 + trow]) + (part_sum[256 + trow] + part_sum[384 + trow]);
-        // pass C: Eq. (IntDiv) with M = 45 (prob_word),
-        // the parked score bytes turned into probabilities in place
-        const unsigned factor = (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
-        for (int j = 0; j < nblk; ++j) {
-          walk(j, [&](auto& ev, int col, int) {
-            constexpr int W = (int)(sizeof(ev) / sizeof(ev[0]));
-            uint32_t xs[W / 4];
-            if constexpr (W == 16) { const uint4 q = *reinterpret_cast<const uint4*>(p_addr(col)); xs[0] = q.x; xs[1] = q.y; xs[2] = q.z; xs[3] = q.w; }
-            else { const uint2 q = *reinterpret_cast<const uint2*>(p_addr(col)); xs[0] = q.x; xs[1] = q.y; }
+      // one reciprocal per row (Eq. (IntDiv) with M = 45), and the output of the previous item
+      if (part == 3 && work) {
+        const unsigned sum = (part_sum[trow] + part_sum[128 + trow]) + (part_sum[256 + trow] + part_sum[384 + trow]);
+        recips[trow] = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
+      }
+      if (n > 0) store_output(n - 1);
+      asm volatile("bar.sync %0, 128;" ::"r"(2 + qd) : "memory");
+      if (work) {
+        const unsigned factor = recips[trow];
+        auto words = [&](const uint4& w) {
+          const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+          uint32_t o[4];
 #pragma unroll
-            for (int k = 0; k < W / 4; ++k)
+          for (int q = 0; q < 4; ++q) {
+            int e[4];
 #pragma unroll
-              for (int bb = 0; bb < 4; ++bb)
-                ev[4 * k + bb] = (int)*reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(xs[k], 0, 0x4440 + bb));
-            if (col + W > a.T) {
-#pragma unroll
-              for (int i = 0; i < W; ++i)
-                if (col + i >= a.T) ev[i] = 0;
-            }
-#pragma unroll
-            for (int k = 0; k < W / 4; ++k)
-              xs[k] = prob_word<K8>(factor, ev[4 * k], ev[4 * k + 1], ev[4 * k + 2], ev[4 * k + 3], 14 - a.smax.k_out, (1 << (a.smax.k_out - 1)) - 1);
-            if constexpr (W == 16) *reinterpret_cast<uint4*>(p_addr(col)) = make_uint4(xs[0], xs[1], xs[2], xs[3]);
-            else *reinterpret_cast<uint2*>(p_addr(col)) = make_uint2(xs[0], xs[1]);
-          });
+            for (int i = 0; i < 4; ++i) e[i] = (int)exp_entry(x[q], kc.sel[i], tmx);
+            o[q] = FAST ? prob_word8(factor, e[0], e[1], e[2], e[3]) : prob_word(factor, e[0], e[1], e[2], e[3], osh, omax);
+          }
+          return make_uint4(o[0], o[1], o[2], o[3]);
+        };
+#pragma unroll 2
+        for (int c = part; c < c_full; c += 4) *p_addr(c) = words(*p_addr(c));
+        if (rem) {
+          uint4 o = words(*p_tail());
+          o.x &= edge_mask(rem, 0); o.y &= edge_mask(rem, 1); o.z &= edge_mask(rem, 2); o.w &= edge_mask(rem, 3);
+          *p_tail() = o;
         }
         fence_async_smem();
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_p);
-      // ---- output: O = sat8(rq(P V; pv_scale)), heads concatenated along the feature dimension ----
-      const bool got_o = alive && mbar_wait(bar_o, par, a.status);
-      alive = alive && got_o;
-      if (got_o) {
-        tc_fence_after();
-        const long long pv_c = 1ll << (a.pv_s - 1);
-        int8_t* orow = a.O + ((int64_t)b * a.T + r) * a.D + (int64_t)h * a.d;
-        for (int c = part; c < a.d / 16; c += 4) {
-          if (!warp_ok) break;
-          int v[16];
-          tmem_ld16(t_row + 2u * (uint32_t)NB + c * 16, v);
-          if (row_ok) {
-            if (a.pv_s >= 33) {   // high product word plus 2^(s-33), shifted by s - 32
-              const int pv_rnd = 1 << (a.pv_s - 33), pv_sh = a.pv_s - 32;
-#pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = mad_hi(v[i], a.pv_m, pv_rnd) >> pv_sh;
-            } else {
-#pragma unroll
-              for (int i = 0; i < 16; ++i) v[i] = (int)(((long long)v[i] * a.pv_m + pv_c) >> a.pv_s);
-            }
-            int4 w0;
-            w0.x = (int)pack_sat8(v[0], v[1], v[2], v[3]);     w0.y = (int)pack_sat8(v[4], v[5], v[6], v[7]);
-            w0.z = (int)pack_sat8(v[8], v[9], v[10], v[11]);   w0.w = (int)pack_sat8(v[12], v[13], v[14], v[15]);
-            *reinterpret_cast<int4*>(orow + c * 16) = w0;
-          }
-        }
-      }
-      // the output columns of tensor memory may take the next item's P V
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_e);
+      if (lane == 0) mbar_arrive(bar_p);
+      o_prev = row_ok ? a.O + ((int64_t)item.b * a.T + r) * a.D + (int64_t)item.h * a.d : nullptr;
+      o_prev_warp = warp_ok;
     }
+    if (n_items > 0) store_output(n_items - 1);
   }
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // the last CTA to finish leaves the counters at zero for the next launch
-    __threadfence();
-    if (atomicAdd(a.sched + 1, 1u) == gridDim.x - 1) {
-      a.sched[0] = 0;
-      a.sched[1] = 0;
-      __threadfence();
-    }
-  }
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, 512u);
@@ -886,58 +940,147 @@ __global__ void __launch_bounds__(kLongThreads, 1) attention_long_kernel(const _
 
 // The shared-memory limit of a kernel is a per-device attribute: set for the current device at context creation.
 int attention_prepare_device() {
-  if (cudaFuncSetAttribute(attention_long_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(attention_long_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(attention_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(attention_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(attention_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(attention_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess)
-    return IVIT_ERR_CUDA;
+  const void* kernels[] = {(const void*)attention_short_kernel<false, false, false>, (const void*)attention_short_kernel<false, false, true>,
+                           (const void*)attention_short_kernel<false, true, false>, (const void*)attention_short_kernel<false, true, true>,
+                           (const void*)attention_short_kernel<true, false, false>, (const void*)attention_short_kernel<true, false, true>,
+                           (const void*)attention_short_kernel<true, true, false>, (const void*)attention_short_kernel<true, true, true>,
+                           (const void*)attention_rows_kernel<true, false>, (const void*)attention_rows_kernel<true, true>,
+                           (const void*)attention_rows_kernel<false, false>, (const void*)attention_rows_kernel<false, true>};
+  for (const void* k : kernels)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) return IVIT_ERR_CUDA;
   return IVIT_OK;
 }
 
-// Rows longer than 256 tokens: key blocks, one CTA per SM.  IVIT_ERR_UNSUPPORTED when the row does not fit the
-// kernel's shared memory (the probabilities of a 128-row tile and the whole V of a head stay resident).
-static int launch_attention_long(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O) {
-  const int64_t B = p->B, T = p->T, D = p->D, h = p->heads, d = D / h;
-  LongArgs la{};
-  AttnArgs& a = la.a;
-  a.T = (int)T; a.d = (int)d; a.heads = (int)h; a.D = D;
-  a.Npad = (int)((T + 31) / 32 * 32);
-  a.tiles_m = (int)((T + 127) / 128);
-  a.tmem_cols = 512;
-  a.G = 1; a.R = 128; a.Btot = (int)B;
-  int nb_max = ((512 - (int)d) / 2) / 32 * 32 > 224 ? 224 : ((512 - (int)d) / 2) / 32 * 32;   // two score buffers + d output columns
-  la.nblk = (a.Npad + nb_max - 1) / nb_max;
-  la.NB = ((a.Npad + la.nblk - 1) / la.nblk + 31) / 32 * 32;
-  la.nv = (a.Npad + 255) / 256;
-  if (la.nblk < 2 || la.NB * (la.nblk - 1) >= a.Npad) return IVIT_ERR_UNSUPPORTED;
-  const uint32_t v_off = 128 * 128 + 2 * la.NB * 128;
-  const uint32_t p_off = (v_off + (uint32_t)la.nv * 256 * (uint32_t)d + 1023u) & ~1023u;
-  const size_t smem = 1024 + p_off + (size_t)((a.Npad + 127) / 128) * 128 * 128 + 1024 + 4096 + 16 + 128 + 16;
-  if (smem > 227 * 1024) return IVIT_ERR_UNSUPPORTED;
+static CUtensorMapSwizzle swizzle_of(int64_t row_bytes) {
+  return row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+}
+
+static void fill_args(ivit_ctx* ctx, AttnArgs& a, const ivit_block_params* p, int8_t* O) {
+  a.T = (int)p->T; a.heads = (int)p->heads; a.d = (int)(p->D / p->heads); a.D = p->D;
+  a.bh = (int)(p->B * p->heads);
+  a.items = (int)(p->B * p->heads * ((p->T + 127) / 128));
+  a.chunks = (int)((p->T + 15) / 16);
+  a.kpad = (int)((p->T + 31) / 32 * 32);
   a.qk_m = p->qk_scale.mult; a.qk_s = clamp_shift(p->qk_scale.shift);
   a.pv_m = p->pv_scale.mult; a.pv_s = clamp_shift(p->pv_scale.shift);
   a.smax = p->smax;
-  a.bias = p->attn_bias; a.bias_batches = p->attn_bias ? p->attn_bias_batches : 1;
+  a.bias = p->attn_bias;
+  a.bias_batches = p->attn_bias ? (int)p->attn_bias_batches : 1;
   a.O = O;
   a.status = ctx->status_dev;
+}
+// As many copies of the ShiftExp table (up to 32) as `limit` bytes of shared memory leave room for beside `fixed`; false: none.
+static bool fit_table(AttnArgs& a, size_t fixed, size_t limit) {
+  a.cp = 32;
+  while (a.cp > 1 && fixed + 1024 * a.cp > limit) a.cp >>= 1;
+  for (int i = 0; i < 4; ++i) a.sel[i] = ((uint32_t)(-4 * a.cp) & 0xffu) << (8 * i);
+  return fixed + 1024 * a.cp <= limit;
+}
+// The arithmetic forms fixed at compile time: k_out = 8, both requantisation shifts >= 33, the largest exponential (and
+// with it every row sum) above 2^15.
+static bool fast_form(const AttnArgs& a) {
+  return a.smax.k_out == 8 && a.qk_s >= 33 && a.pv_s >= 33 && ((int64_t)a.smax.I0 << a.smax.N) > (1 << 15);
+}
+
+// IVIT_ERR_UNSUPPORTED when the row does not fit the kernel's shared memory (the probabilities of a 128-row tile and
+// the whole V of a head stay resident).
+static int launch_attention_rows(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O) {
+  const int64_t B = p->B, T = p->T, D = p->D, h = p->heads, d = D / h;
+  if (T > 1024) return IVIT_ERR_UNSUPPORTED;
+  RowsArgs ra{};
+  AttnArgs& a = ra.a;
+  fill_args(ctx, a, p, O);
+  // two score buffers and the output share the 512 columns of tensor memory
+  ra.wb = 16 * kBlkChunks;
+  ra.nblk = (a.chunks + kBlkChunks - 1) / kBlkChunks;
+  a.kbox = 16 * kBlkChunks;
+  ra.nv = (a.kpad + 255) / 256;
+  ra.vbox = ((a.kpad + ra.nv - 1) / ra.nv + 7) / 8 * 8;
+  const uint32_t v_off = 128u * a.d + 2u * a.kbox * a.d;
+  const uint32_t p_off = (v_off + (uint32_t)(ra.nv * ra.vbox) * a.d + 1023u) & ~1023u;
+  const size_t p_bytes = (size_t)((a.kpad + 127) / 128) * 128 * 128, limit = 227 * 1024;
+  size_t fixed = 1024 + p_off + p_bytes + 9 * 128 * 4 + 128 * 4 + 2 * sizeof(AttnItem) + 80 + 16;
+  if (fixed + p_bytes + 1024 * 32 <= limit) {   // a second probability buffer
+    ra.p_stride = (uint32_t)p_bytes;
+    fixed += p_bytes;
+  }
+  if (!fit_table(a, fixed, limit)) return IVIT_ERR_UNSUPPORTED;
+  const size_t smem = fixed + 1024 * a.cp;
   const int64_t ldq = 3 * D;
   CUtensorMap tmQ, tmK, tmV;
-  const CUtensorMapSwizzle vsw = d == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (d == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-  if (!make_tensor_map(ctx, &tmQ, QKV, d, T, h, B, ldq, d, T * ldq, 128, 128, CU_TENSOR_MAP_SWIZZLE_128B, a.q_pos) ||
-      !make_tensor_map(ctx, &tmK, QKV + D, d, T, h, B, ldq, d, T * ldq, 128, la.NB, CU_TENSOR_MAP_SWIZZLE_128B, a.k_pos) ||
-      !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, 256, vsw, a.v_pos))
+  if (!make_tensor_map(ctx, &tmQ, QKV, d, T, h, B, ldq, d, T * ldq, (int)d, 32, swizzle_of(d), a.q_pos) ||
+      !make_tensor_map(ctx, &tmK, QKV + D, d, T, h, B, ldq, d, T * ldq, (int)d, a.kbox, swizzle_of(d), a.k_pos) ||
+      !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, ra.vbox, swizzle_of(d), a.v_pos))
     return IVIT_ERR_UNSUPPORTED;
-  a.bh = (int)(B * h);
-  a.items = (int)(B * h * a.tiles_m);
-  a.sched = ctx->sched_dev + 2 * ctx->attn_gen;
-  a.sched_other = ctx->sched_dev + 2 * (ctx->attn_gen ^ 1);
-  ctx->attn_gen ^= 1;
-  const int64_t grid = a.items < ctx->sm_count ? a.items : ctx->sm_count;
+  const dim3 grid((unsigned)(a.items < ctx->sm_count ? a.items : ctx->sm_count)), block(kRowsThreads);
   LaunchScope ls(ctx, KIND_ATTENTION, 4.0 * (double)(B * h) * (double)T * (double)T * (double)d);
-  if (p->smax.k_out == 8) launch_k(attention_long_kernel<true>, dim3((unsigned)grid), dim3(kLongThreads), smem, ctx->stream, tmQ, tmK, tmV, la);
-  else launch_k(attention_long_kernel<false>, dim3((unsigned)grid), dim3(kLongThreads), smem, ctx->stream, tmQ, tmK, tmV, la);
+  auto run = [&](auto kernel) { launch_k(kernel, grid, block, smem, ctx->stream, tmQ, tmK, tmV, ra); };
+  if (fast_form(a)) {
+    if (a.bias) run(attention_rows_kernel<true, true>);
+    else run(attention_rows_kernel<true, false>);
+  } else {
+    if (a.bias) run(attention_rows_kernel<false, true>);
+    else run(attention_rows_kernel<false, false>);
+  }
+  return ls.done();
+}
+
+static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O) {
+  const int64_t B = p->B, T = p->T, D = p->D, h = p->heads, d = D / h;
+  ShortArgs sa{};
+  AttnArgs& a = sa.a;
+  fill_args(ctx, a, p, O);
+  sa.Btot = (int)B;
+  // several windows: 2 of up to 64 tokens, or 4 of up to 32, share one 128-row tile
+  const bool pack = T <= 64 && B >= 2;
+  a.kbox = 16 * a.chunks;
+  size_t bias_bytes = 0;
+  sa.G = sa.npos = sa.units = 1;
+  sa.R = 128;
+  if (pack) {
+    sa.G = T <= 32 ? 4 : 2;
+    sa.R = a.kbox = 128 / sa.G;
+    a.kpad = 128;
+    sa.units = (int)((B + sa.G - 1) / sa.G);
+    a.items = (int)(sa.units * h);
+    // Windows repeat their bias every `per` of them: tiles of the same positions follow one another.  Where tiles and
+    // positions do not line up the matrices are fetched for every tile (imgs = 1 in the kernel).
+    const int64_t per = a.bias_batches % h == 0 ? a.bias_batches / h : 0;
+    if (!a.bias || a.bias_batches == 1 || per == 1) sa.npos = 1;
+    else if (per > 0 && per % sa.G == 0 && B % per == 0) sa.npos = (int)(per / sa.G);
+    else sa.npos = sa.units;
+    if (a.bias) bias_bytes = (size_t)sa.G * T * (T | 1) * 4;
+  }
+  sa.tmem_cols = pack || a.chunks <= 8 ? 128 : 256;
+  const uint32_t p_off = (128u * a.d + (pack ? 128u : (uint32_t)a.kbox) * a.d + (uint32_t)a.kpad * a.d + 1023u) & ~1023u;
+  const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + 4 * 128 * 4 + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
+  // CTAs per SM: as many as leave room for four copies of the table
+  int per_sm = pack ? 3 : 2;
+  auto budget = [](int n) { return n == 1 ? (size_t)(227 * 1024) : (size_t)(228 * 1024 / n - 1024); };
+  while (per_sm > 1 && fixed + 4 * 1024 > budget(per_sm)) --per_sm;
+  if (!fit_table(a, fixed, budget(per_sm))) return IVIT_ERR_UNSUPPORTED;
+  const size_t smem = fixed + 1024 * a.cp;
+  const int64_t ldq = 3 * D;
+  CUtensorMap tmQ, tmK, tmV;
+  // boxes: R rows of G consecutive windows; or 32 query rows / all key and value rows of one image
+  if (!make_tensor_map(ctx, &tmQ, QKV, d, T, h, B, ldq, d, T * ldq, (int)d, pack ? sa.R : 32, swizzle_of(d), a.q_pos, sa.G) ||
+      !make_tensor_map(ctx, &tmK, QKV + D, d, T, h, B, ldq, d, T * ldq, (int)d, a.kbox, swizzle_of(d), a.k_pos, sa.G) ||
+      !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, pack ? sa.R : a.kpad, swizzle_of(d), a.v_pos, sa.G))
+    return IVIT_ERR_UNSUPPORTED;
+  const int64_t slots = (int64_t)per_sm * ctx->sm_count;
+  const dim3 grid((unsigned)(a.items < slots ? a.items : slots)), block(kShortThreads);
+  LaunchScope ls(ctx, KIND_ATTENTION, 4.0 * (double)(B * h) * (double)T * (double)T * (double)d);
+  auto run = [&](auto kernel) { launch_k(kernel, grid, block, smem, ctx->stream, tmQ, tmK, tmV, sa); };
+  switch ((pack ? 4 : 0) | (fast_form(a) ? 2 : 0) | (a.bias ? 1 : 0)) {
+    case 0: run(attention_short_kernel<false, false, false>); break;
+    case 1: run(attention_short_kernel<false, false, true>); break;
+    case 2: run(attention_short_kernel<false, true, false>); break;
+    case 3: run(attention_short_kernel<false, true, true>); break;
+    case 4: run(attention_short_kernel<true, false, false>); break;
+    case 5: run(attention_short_kernel<true, false, true>); break;
+    case 6: run(attention_short_kernel<true, true, false>); break;
+    default: run(attention_short_kernel<true, true, true>); break;
+  }
   return ls.done();
 }
 
@@ -945,59 +1088,11 @@ static int launch_attention_long(ivit_ctx* ctx, const ivit_block_params* p, cons
 // shared memory, misaligned tensors); the caller then composes the attention from MatMul and Shiftmax kernels.
 int launch_attention_fused(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O) {
   if (!ctx->tmap_encode) return IVIT_ERR_UNSUPPORTED;
-  const int64_t B = p->B, T = p->T, D = p->D, h = p->heads, d = D / h;
-  if ((d != 32 && d != 64 && d != 128) || B * h > 2147483647LL / 8) return IVIT_ERR_UNSUPPORTED;
+  const int64_t B = p->B, T = p->T, h = p->heads, d = p->D / h;
+  if ((d != 32 && d != 64 && d != 128) || B * h > 2147483647LL / 8 || p->attn_bias_batches > 2147483647LL) return IVIT_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(QKV) & 15) || (reinterpret_cast<uintptr_t>(O) & 15)) return IVIT_ERR_UNSUPPORTED;
   if (B == 0) return IVIT_OK;
-  if (T > 256) return launch_attention_long(ctx, p, QKV, O);
-  AttnArgs a{};
-  a.T = (int)T; a.d = (int)d; a.heads = (int)h; a.D = D;
-  a.Npad = (int)((T + 31) / 32 * 32);
-  a.tiles_m = (int)((T + 127) / 128);
-  // Short rows (window attention): 2 windows of up to 64 tokens, or 4 of up to 32, share one 128-row tile.  The
-  // score tile is then block-diagonal; the probabilities outside a row's own window are written as 0.
-  a.G = 1; a.R = 128; a.Btot = (int)B;
-  if (T <= 64 && B >= 2) {
-    a.G = T <= 32 ? 4 : 2;
-    a.R = 128 / a.G;
-    a.Npad = 128;
-  }
-  a.tmem_cols = 32;
-  while (a.tmem_cols < a.Npad) a.tmem_cols <<= 1;
-  a.qk_m = p->qk_scale.mult; a.qk_s = clamp_shift(p->qk_scale.shift);
-  a.pv_m = p->pv_scale.mult; a.pv_s = clamp_shift(p->pv_scale.shift);
-  a.smax = p->smax;
-  a.bias = p->attn_bias; a.bias_batches = p->attn_bias ? p->attn_bias_batches : 1;
-  a.O = O;
-  a.status = ctx->status_dev;
-  const int64_t ldq = 3 * D;
-  CUtensorMap tmQ, tmK, tmV;
-  const CUtensorMapSwizzle vsw = d == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (d == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-  // boxes: a.R rows of a.G consecutive images / windows (G = 1: 128 query rows, Npad key / value rows of one image)
-  if (!make_tensor_map(ctx, &tmQ, QKV, d, T, h, B, ldq, d, T * ldq, 128, a.G > 1 ? a.R : 128, CU_TENSOR_MAP_SWIZZLE_128B, a.q_pos, a.G) ||
-      !make_tensor_map(ctx, &tmK, QKV + D, d, T, h, B, ldq, d, T * ldq, 128, a.G > 1 ? a.R : a.Npad, CU_TENSOR_MAP_SWIZZLE_128B, a.k_pos, a.G) ||
-      !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, a.G > 1 ? a.R : a.Npad, vsw, a.v_pos, a.G))
-    return IVIT_ERR_UNSUPPORTED;
-  const uint32_t v_off = 128 * 128 + a.Npad * 128;
-  const uint32_t p_off = (v_off + a.Npad * a.d + 1023u) & ~1023u;
-  const size_t smem = 1024 + p_off + (size_t)((a.Npad + 127) / 128) * 128 * 128 + 1024 + 2048 + 16 + 64 + 16;
-  a.bh = (int)((B + a.G - 1) / a.G * h);
-  a.items = a.bh * a.tiles_m;
-  a.sched = ctx->sched_dev + 2 * ctx->attn_gen;
-  a.sched_other = ctx->sched_dev + 2 * (ctx->attn_gen ^ 1);
-  ctx->attn_gen ^= 1;
-  const int64_t slots = 2 * (int64_t)ctx->sm_count;
-  const int64_t grid = a.items < slots ? a.items : slots;
-  LaunchScope ls(ctx, KIND_ATTENTION, 4.0 * (double)(B * h) * (double)T * (double)T * (double)d);
-  const bool k8 = p->smax.k_out == 8;
-  if (a.G > 1) {
-    if (k8) launch_k(attention_kernel<true, true>, dim3((unsigned)grid), dim3(kAttnThreads), smem, ctx->stream, tmQ, tmK, tmV, a);
-    else launch_k(attention_kernel<true, false>, dim3((unsigned)grid), dim3(kAttnThreads), smem, ctx->stream, tmQ, tmK, tmV, a);
-  } else {
-    if (k8) launch_k(attention_kernel<false, true>, dim3((unsigned)grid), dim3(kAttnThreads), smem, ctx->stream, tmQ, tmK, tmV, a);
-    else launch_k(attention_kernel<false, false>, dim3((unsigned)grid), dim3(kAttnThreads), smem, ctx->stream, tmQ, tmK, tmV, a);
-  }
-  return ls.done();
+  return T <= 256 ? launch_attention_short(ctx, p, QKV, O) : launch_attention_rows(ctx, p, QKV, O);
 }
 
 }  // namespace ivit

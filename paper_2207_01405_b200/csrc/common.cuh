@@ -34,11 +34,9 @@ struct ivit_ctx {
   int* status_host;  // mapped pinned memory: kernels write the first device-side error here
   int* status_dev;   // device view of the same word
   int8_t* gelu_tables;  // kGeluTableSlots tables on the device
-  unsigned* sched_dev;  // two pairs of work counters of the attention kernel (behind the tables), used alternately
-  unsigned* rowblk_dev; // row-operator state of the Dense kernels: kRowStateBytes (zero between launches)
+  unsigned* rowblk_dev; // row-operator state of the Dense kernels (behind the tables): kRowStateBytes (zero between launches)
   int row_fusion;       // non-zero (bit 0 LayerNorm, bit 1 ShiftGELU; default 0): LayerNorm / ShiftGELU run in the tail of the Dense kernel that produces their rows
   int rowop_fused;      // set by the Dense launcher when the kernel it launched runs the requested row operator
-  int attn_gen;         // pair of the next launch
   ivit::GeluKey gelu_keys[ivit::kGeluTableSlots];
   int gelu_used;
   int gelu_next;

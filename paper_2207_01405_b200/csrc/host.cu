@@ -412,8 +412,8 @@ int ivit_ctx_create(ivit_ctx** out, int device, void* cuda_stream) {
   if (cudaHostAlloc((void**)&c->status_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess) { delete c; return IVIT_ERR_CUDA; }
   *c->status_host = 0;
   if (cudaHostGetDevicePointer((void**)&c->status_dev, c->status_host, 0) != cudaSuccess ||
-      cudaMalloc((void**)&c->gelu_tables, (size_t)kGeluTableSlots * kGeluTableBytes + 128 + kRowStateBytes) != cudaSuccess ||
-      cudaMemset(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes, 0, 128 + kRowStateBytes) != cudaSuccess) {
+      cudaMalloc((void**)&c->gelu_tables, (size_t)kGeluTableSlots * kGeluTableBytes + kRowStateBytes) != cudaSuccess ||
+      cudaMemset(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes, 0, kRowStateBytes) != cudaSuccess) {
     cudaFreeHost(c->status_host);
     delete c;
     return IVIT_ERR_CUDA;
@@ -431,8 +431,7 @@ int ivit_ctx_create(ivit_ctx** out, int device, void* cuda_stream) {
     delete c;
     return IVIT_ERR_CUDA;
   }
-  c->sched_dev = reinterpret_cast<unsigned*>(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes);
-  c->rowblk_dev = c->sched_dev + 32;
+  c->rowblk_dev = reinterpret_cast<unsigned*>(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes);
   c->row_fusion = 0;
   c->gemm_pairs = 1;
   *out = c;
@@ -487,7 +486,7 @@ int ivit_ctx_poll_status(ivit_ctx* ctx) {
   if (v != 0) {
     *s = 0;
     // a kernel that gave up may have left work counters behind: zero them for the launches that follow
-    cudaMemsetAsync(ctx->sched_dev, 0, 128 + kRowStateBytes, ctx->stream);
+    cudaMemsetAsync(ctx->rowblk_dev, 0, kRowStateBytes, ctx->stream);
     return v;
   }
   return IVIT_OK;

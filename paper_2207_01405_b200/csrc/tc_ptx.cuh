@@ -9,8 +9,8 @@
 
 namespace ivit {
 
-constexpr uint32_t kSpinLimit = 1u << 20;     // polls before a wait gives up
-constexpr uint32_t kSuspendHintNs = 2000;      // suspend-time hint of one poll
+constexpr uint32_t kSpinLimit = 1u << 20;     // polls (with back-off) before a wait on a flag in global memory gives up
+constexpr uint32_t kPollLimit = 1u << 23;     // polls before a wait on an mbarrier gives up
 
 // 4-D int8 tensor map over {inner, rows, batch_inner, batch_outer} (defined with the GEMM); pos[0..2]
 // receive the tensor-map dimension (1..3) holding the row, inner-batch and outer-batch coordinate.
@@ -28,15 +28,16 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
-// One poll: the thread may be suspended by the hardware for up to kSuspendHintNs while the phase is
-// incomplete (it resumes at once when the phase completes), so a waiting warp issues few instructions.
+// One poll: the thread may be suspended by the hardware while the phase is incomplete and resumes when it completes.
+// (Without a suspend-time hint: with one of 2 us the wait became poll + NANOSLEEP and every hand-over between warps took
+// longer, 1.7 us over the six of an attention item.)
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "r"(kSuspendHintNs) : "memory");
+      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
 // One non-blocking test of the phase.
@@ -51,7 +52,7 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait: false (and the timeout recorded) when the phase did not complete in time.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* status) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i)
+  for (uint32_t i = 0; i < kPollLimit; ++i)
     if (mbar_try(bar, parity)) return true;
   *reinterpret_cast<volatile int*>(status) = IVIT_ERR_DEVICE_TIMEOUT;
   __threadfence_system();

@@ -223,3 +223,27 @@ def test_attention_random_shapes():
         g.assert_equal(got, O.attention(blk, QKV), f"case {case}: B={B} T={T} heads={heads} d={d} bias={bias} k_out={k_out}")
     assert c.poll_status() == 0
 
+
+@pytest.mark.parametrize("B,T,heads,d,batches", [
+    (9, 49, 2, 32, 2), (8, 49, 2, 32, 4), (12, 49, 2, 32, 6), (16, 49, 3, 32, 12), (9, 49, 2, 64, 18),   # 64-row slots
+    (16, 16, 2, 32, 8), (13, 25, 2, 128, 2), (6, 64, 2, 32, 1), (700, 49, 2, 32, 8),                     # 32-row slots, many items
+    (2, 256, 2, 64, 2), (2, 255, 1, 128, 2), (3, 65, 2, 32, 6)])                                         # one image per tile
+def test_attention_score_bias_layouts(B, T, heads, d, batches):
+    """The score bias of packed windows is kept in shared memory and fetched again when it changes: matrices shared by
+    all windows, one set per window position (lined up with the tiles or not), one per window, one for everything.
+    I0 = 16 makes the largest exponential a power of two and the scale spreads the scores, so that rows with a single
+    non-zero exponential (probability 128, clamped to 127) occur."""
+    import dataclasses
+    from ivit_inputs import ExpParams, Scale
+    from ivit_inputs.gen import dyadic
+    g = _g()
+    c = g.ctx()
+    D = heads * d
+    blk = make_block(_Ids(4000 + T + batches), 1, B, T, D, heads, 2 * D, attn_bias_batches=batches)
+    blk = dataclasses.replace(blk, smax=ExpParams(16, 15), qk_scale=Scale(*dyadic(0.9 * 128 / (3 * np.sqrt(d) * 1024))))
+    dblk = g.binding.DeviceBlock(blk, "cuda")
+    rng = np.random.default_rng(T + B)
+    QKV = np.clip(np.rint(rng.standard_normal((B * T, 3 * D)) * 32), -128, 127).astype(np.int8)
+    got = g.host(c.attention(dblk, torch.from_numpy(QKV).cuda()))
+    g.assert_equal(got, O.attention(blk, QKV), f"B={B} T={T} heads={heads} d={d} bias matrices={batches}")
+    assert c.poll_status() == 0
