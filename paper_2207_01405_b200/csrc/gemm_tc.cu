@@ -240,7 +240,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   volatile uint32_t* rop_flag = tmem_slot + 2;                                // row operator: a flag the CTA agrees on
   uint8_t* rop_smem = gen_base + bars_off + 1024;   // ROP == 1: LayerNorm constants; ROP == 2: table rows, per warp
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // (read from lane 0, so that the compiler knows it to be the same in all lanes)
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   // this CTA's (with PAIR: this CTA pair's) contiguous range of tiles
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;      // PAIR: 0 = the CTA that issues the MMAs of the pair
   const int poff = (int)rank * BM;                          // this CTA's 128 channels inside the pair's 256
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   __syncthreads();
   if (PAIR) cluster_sync_all();   // the other CTA's barriers are initialised before anything arrives on them
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   // set-up done (barriers, tensor memory, descriptor prefetch): let the next kernel be scheduled, then wait
   // for the previous kernel's results before touching global memory
   pdl_trigger();
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    {
       int issued = 0;            // k-blocks issued so far, over all tiles of this CTA
       int s = 0, wrap = 0;       // ring slot of the next k-block and how often the ring has wrapped
       bool ok = true;
@@ -322,12 +323,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       // PAIR: both CTAs load (their 128 weight rows, their half of the activation rows); the bytes of both are
       // counted by the stage barrier of CTA rank 0, which alone arms it
       auto arm = [&](uint32_t bar, uint32_t bytes) {
-        if (!PAIR) mbar_expect_tx(bar, bytes);
-        else if (rank == 0) mbar_expect_tx(bar, 2u * bytes);
+        if (!PAIR) mbar_expect_tx_w(bar, bytes);
+        else if (rank == 0) mbar_expect_tx_w(bar, 2u * bytes);
       };
       auto load = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
-        if (PAIR) tma_load_4d_pair(dst, map, mapa_rank0(bar), c0, c1, c2, c3);
-        else tma_load_4d(dst, map, bar, c0, c1, c2, c3);
+        if (PAIR) tma_load_4d_pair_w(dst, map, mapa_rank0(bar), c0, c1, c2, c3);
+        else tma_load_4d_w(dst, map, bar, c0, c1, c2, c3);
       };
       // Dense orientation: the P operand is the weight matrix, which no kernel writes.  The weight k-blocks of the
       // first tile are requested before the wait for the previous kernel (whose last CTAs may still be running
@@ -350,13 +351,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         if (a.q_resident && q0 != cur_q) {
           // new activation row block: its k-blocks come in beside this tile's weight k-blocks, once every MMA
           // on the old block is done
-          if (qi > 0 && !mbar_wait(qrese, (qi - 1) & 1, a.status)) { ok = false; break; }
+          if (qi > 0 && !mbar_wait_warp(qrese, (qi - 1) & 1, a.status)) { ok = false; break; }
           bring_q = true;
           cur_q = q0;
           ++qi;
         }
         for (int kb = 0; kb < kblocks; ++kb) {
-          if (wrap > 0 && !mbar_wait(empty0 + 8 * s, (wrap & 1) ^ 1, a.status)) { ok = false; break; }
+          if (wrap > 0 && !mbar_wait_warp(empty0 + 8 * s, (wrap & 1) ^ 1, a.status)) { ok = false; break; }
           const uint32_t sp = base + s * stage_bytes, sq = sp + BM * BK;
           const bool early = t == t_begin && kb < pre;   // barrier armed and weights requested before the wait
           if (!early) arm(full0 + 8 * s, stage_bytes + (bring_q ? a.q_stage_bytes : 0));
@@ -377,7 +378,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0 && rank == 0) {   // PAIR: CTA rank 0 issues for both CTAs
+    if (rank == 0) {   // PAIR: CTA rank 0 issues for both CTAs
       // instruction descriptor: D = S32, A = B = signed 8 bit, A K-major, M = 128 (PAIR: 256 over both CTAs), N = BN,
       // no saturation
       const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a.q_mn << 16) |
@@ -409,44 +410,44 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           last_of_q = t + 1 >= t_end || ti.q0(a) != cur_q;
         }
         // the epilogue must have drained this buffer (its use two tiles ago)
-        if (it >= 2 && !mbar_wait(acce0 + 8 * buf, ((it >> 1) & 1) ^ 1, a.status)) { ok = false; break; }
+        if (it >= 2 && !mbar_wait_warp(acce0 + 8 * buf, ((it >> 1) & 1) ^ 1, a.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(buf * a.BN);
         for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(full0 + 8 * s, wrap & 1, a.status)) { ok = false; break; }
+          if (!mbar_wait_warp(full0 + 8 * s, wrap & 1, a.status)) { ok = false; break; }
           tc_fence_after();
           // low descriptor words of this stage's P tile and of the Q tile (resident, or behind P in the stage)
           const uint32_t p_lo = p_lo0 + (uint32_t)s * stage16;
           const uint32_t q_lo = a.q_resident ? q_lo0 + (uint32_t)kb * qstage16 : p_lo + ((BM * BK) >> 4);
           if (kb != kblocks - 1 || tail_steps == BK / UMMA_K) {
-            if (PAIR) umma_i8_x4_pair(d_tmem, p_lo, p_hi, q_lo, q_hi, idesc, kb != 0, UMMA_K >> 4, q_kstep16);
-            else umma_i8_x4(d_tmem, p_lo, p_hi, q_lo, q_hi, idesc, kb != 0, UMMA_K >> 4, q_kstep16);
+            if (PAIR) umma_i8_x4_pair_w(d_tmem, p_lo, p_hi, q_lo, q_hi, idesc, kb != 0, UMMA_K >> 4, q_kstep16);
+            else umma_i8_x4_w(d_tmem, p_lo, p_hi, q_lo, q_hi, idesc, kb != 0, UMMA_K >> 4, q_kstep16);
           } else {
             uint32_t pl = p_lo, ql = q_lo;
             for (int k = 0; k < tail_steps; ++k) {
-              if (PAIR) umma_i8_pair(d_tmem, pl, p_hi, ql, q_hi, idesc, (kb | k) != 0);
-              else umma_i8_lohi(d_tmem, pl, p_hi, ql, q_hi, idesc, (kb | k) != 0);
+              if (PAIR) umma_i8_pair_w(d_tmem, pl, p_hi, ql, q_hi, idesc, (kb | k) != 0);
+              else umma_i8_lohi_w(d_tmem, pl, p_hi, ql, q_hi, idesc, (kb | k) != 0);
               pl += UMMA_K >> 4;
               ql += q_kstep16;
             }
           }
           // the stage may be refilled once these MMAs have read it (PAIR: in both CTAs)
-          if (PAIR) umma_commit_pair(empty0 + 8 * s);
-          else umma_commit(empty0 + 8 * s);
+          if (PAIR) umma_commit_pair_w(empty0 + 8 * s);
+          else umma_commit_w(empty0 + 8 * s);
           ++consumed;
           if (++s == a.stages) { s = 0; ++wrap; }
         }
         if (ok) {   // accumulator of this tile complete (PAIR: told to the epilogue warps of both CTAs)
-          if (PAIR) umma_commit_pair(accf0 + 8 * buf);
-          else umma_commit(accf0 + 8 * buf);
+          if (PAIR) umma_commit_pair_w(accf0 + 8 * buf);
+          else umma_commit_w(accf0 + 8 * buf);
         }
-        if (ok && last_of_q) umma_commit(qrese);   // the resident tile may be replaced once these MMAs are done
+        if (ok && last_of_q) umma_commit_w(qrese);   // the resident tile may be replaced once these MMAs are done
       }
       if (!ok) {
         // drain: copies that were issued but never consumed (only after a timeout)
         const int issued = *issued_slot;
         for (int j = consumed; j < issued; ++j) {
-          mbar_wait(full0 + 8 * s, wrap & 1, a.status);
+          mbar_wait_warp(full0 + 8 * s, wrap & 1, a.status);
           if (++s == a.stages) { s = 0; ++wrap; }
         }
       }
@@ -532,10 +533,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       if (pf_t < t_end) {
         if (pf_ti.p0() + c_first < a.P) {
           const uint32_t sl = pf_g & 1u;
-          if (lane == 0) {
-            mbar_expect_tx(my_resf + 8u * sl, 1024u);
-            tma_load_4d(my_res + 1024u * sl, &tmR, my_resf + 8u * sl, pf_ti.p0() + c_first, pf_ti.q0(a) + 32 * pf_ck, 0, 0);
-          }
+          mbar_expect_tx_w(my_resf + 8u * sl, 1024u);
+          tma_load_4d_w(my_res + 1024u * sl, &tmR, my_resf + 8u * sl, pf_ti.p0() + c_first, pf_ti.q0(a) + 32 * pf_ck, 0, 0);
           rpend |= 1u << sl;
         }
         ++pf_g;
@@ -583,7 +582,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       }
       if (dense && t + 1 < t_end) fetch_channel(ti.p0());
 
-      if (ok) ok = mbar_wait(accf0 + 8 * buf, (it >> 1) & 1, a.status);
+      if (ok) ok = mbar_wait_warp(accf0 + 8 * buf, (it >> 1) & 1, a.status);
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(qd * 32) << 16) + (uint32_t)(buf * a.BN);
       const int cols_left = a.Q - tc.q0;
@@ -695,9 +694,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (tma_out) {
             const uint32_t sl = g & 1u;
             // the store that used this slot two chunks ago must have read it; the residual bytes must be here
-            if (lane == 0) tma_store_wait_read1();
+            tma_store_wait_read1();   // (every lane: only the one that issued the stores has any to wait for)
             if (tma_res && c_any) {
-              if (ok) ok = mbar_wait(my_resf + 8u * sl, (rpar >> sl) & 1u, a.status);
+              if (ok) ok = mbar_wait_warp(my_resf + 8u * sl, (rpar >> sl) & 1u, a.status);
               if (ok) { rpar ^= 1u << sl; rpend &= ~(1u << sl); }
             }
             __syncwarp();
@@ -766,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (tma_out) {
             fence_async_smem();
             __syncwarp();
-            if (lane == 0 && c_any) tma_store_4d(&tmO, my_out + 1024u * (g & 1u), tc.p0 + c_first, tc.q0 + 32 * ck, 0, 0);
+            if (c_any) tma_store_4d_w(&tmO, my_out + 1024u * (g & 1u), tc.p0 + c_first, tc.q0 + 32 * ck, 0, 0);
             // every lane is past its reads of this slot's residual bytes: fetch those of two chunks on
             if (tma_res) pf_fetch();
             ++g;
@@ -826,12 +825,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         ++tiles_in_q;
         if (t + 1 >= t_end || ti.q0(a) != tc.q0) {
           // this warp's last tile of the row block: see the stores complete, release them, count the tiles
+          tma_store_wait_all();
+          asm volatile("fence.proxy.async;" ::: "memory");
+          __threadfence();
+          __syncwarp();
           if (lane == 0) {
             unsigned* q_state = a.rop.counters;
             const unsigned qblk = (unsigned)tc.q0 / (unsigned)a.BN;
-            tma_store_wait_all();
-            asm volatile("fence.proxy.async;" ::: "memory");
-            __threadfence();
             unsigned* cnt = q_state + 32 + qblk * kRowStateStride;
             const unsigned old = atomicAdd(cnt, (unsigned)tiles_in_q);
             if (old + (unsigned)tiles_in_q == (unsigned)(a.tiles_p * kEpiWarps)) {
@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         }
       }
     }
-    if (tma_out && lane == 0) tma_store_wait_all();
+    if (tma_out) tma_store_wait_all();
     // only after a timeout: residual bytes fetched for chunks that were never worked on may be in flight
     if (tma_res && !ok && lane == 0)
       for (uint32_t sl = 0; sl < 2; ++sl)
