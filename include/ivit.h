@@ -122,9 +122,7 @@ uint64_t ivit_ctx_table_generation(const ivit_ctx* ctx);
  * qualifies (default), 1 = force the CUDA-core (dp4a) kernels everywhere.
  * Both are bit-exact; the switch exists for testing and measurement. */
 int ivit_ctx_set_gemm_engine(ivit_ctx* ctx, int engine);
-/* Where the row operators run.  Default: in layers of few rows (one wave of small tiles) LayerNorm runs in front of the
- * MMAs of the Dense layer that reads its output, inside the model forwards ShiftGELU too; elsewhere every operator is a
- * kernel of its own.  8: back to the default.  1: inside ivit_block_forward and the model forwards, LayerNorm 2, ShiftGELU
+/* Row-operator fusion (off by default).  1: inside ivit_block_forward and the model forwards, LayerNorm 2, ShiftGELU
  * (Algorithm 2 with its row maximum) and the LayerNorm 1 of the following block run inside the Dense kernel that
  * produces their input rows, where the shapes allow it: the kernel's warps count the finished channel tiles of every
  * block of rows and, after their last tile, run the operator on slices of the completed rows.  0: every operator

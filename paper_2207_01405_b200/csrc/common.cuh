@@ -36,7 +36,6 @@ struct ivit_ctx {
   int8_t* gelu_tables;  // kGeluTableSlots tables on the device
   unsigned* rowblk_dev; // row-operator state of the Dense kernels (behind the tables): kRowStateBytes (zero between launches)
   int row_fusion;       // non-zero (bit 0 LayerNorm, bit 1 ShiftGELU; default 0): LayerNorm / ShiftGELU run in the tail of the Dense kernel that produces their rows
-  int row_prologue;     // non-zero (default): in layers of few rows LayerNorm / ShiftGELU run in front of the MMAs of the Dense layer that reads them
   int rowop_fused;      // set by the Dense launcher when the kernel it launched runs the requested row operator
   ivit::GeluKey gelu_keys[ivit::kGeluTableSlots];
   int gelu_used;
@@ -242,9 +241,8 @@ int launch_gemm_simt(ivit_ctx* ctx, const GemmProblem& g);
 // Returns IVIT_ERR_UNSUPPORTED when the shape does not qualify for the tensor-core kernel.
 int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g);
 int launch_gemm(ivit_ctx* ctx, const GemmProblem& g);
-// Dense layers of one wave of small tiles; pro: row operator applied to the input rows first (1 = I-LayerNorm, 2 =
-// ShiftGELU, constants in g.epi.rop, g.A the operator's input).  IVIT_ERR_UNSUPPORTED when the layer does not qualify.
-int launch_gemm_small(ivit_ctx* ctx, const GemmProblem& g, int pro);
+// Dense layers of one wave of small tiles.  IVIT_ERR_UNSUPPORTED when the layer does not qualify.
+int launch_gemm_small(ivit_ctx* ctx, const GemmProblem& g);
 int gemm_small_prepare_device();
 // Per-device kernel attributes (shared-memory limits) of the tensor-core kernels, for the current device.
 int gemm_tc_prepare_device();

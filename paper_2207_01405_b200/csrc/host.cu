@@ -128,28 +128,12 @@ void want_layernorm(GemmProblem& g, const ivit_scale& gamma, const int32_t* beta
   g.epi.rop.ld_ln = ld;
 }
 
-// Dense layer on LayerNorm(X): one kernel where the layer is one wave of small tiles (launch_gemm_small), else two.
-int ln_dense(ivit_ctx* ctx, const int8_t* X, int64_t ldx, const ivit_scale& gamma, const int32_t* beta, int M_ln, int8_t* A, GemmProblem g) {
-  if (ctx->row_prologue && ctx->gemm_engine == 0) {
-    const int8_t* a = g.A;
-    const int64_t lda = g.lda;
-    g.A = X; g.lda = ldx;
-    want_layernorm(g, gamma, beta, M_ln, nullptr, 0);
-    const int rc = launch_gemm_small(ctx, g, 1);
-    if (rc != IVIT_ERR_UNSUPPORTED) return rc;
-    g.A = a; g.lda = lda;
-    g.epi.rop = RowOpArgs{};
-  }
-  const int rc = launch_layernorm(ctx, X, IVIT_I8, ldx, to_dev(gamma), beta, M_ln, A, g.lda, g.M, g.K);
-  return rc ? rc : launch_gemm(ctx, g);
-}
-
 // One encoder block.  a_ready: LayerNorm 1 of X already sits in the workspace (the previous block's last Dense
 // layer produced it); next: the block that follows on Y with the same shape, or nullptr - its LayerNorm 1 is then
 // run in the tail of this block's last Dense layer, where that is possible.  *a_next_ready tells the caller whether
 // it was.  Row operators that a Dense kernel cannot take on run as kernels of their own, with the same result.
 int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_t* Y, char* ws, bool a_ready = false,
-               const ivit_block_params* next = nullptr, bool* a_next_ready = nullptr, bool in_model = false) {
+               const ivit_block_params* next = nullptr, bool* a_next_ready = nullptr) {
   const BlockWs w = block_ws(p);
   const int64_t M = p->B * p->T, D = p->D, H = p->H;
   int8_t* A = reinterpret_cast<int8_t*>(ws + w.A);
@@ -161,8 +145,9 @@ int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_
   int rc;
   if (a_next_ready) *a_next_ready = false;
   // X^ = MSA(LayerNorm(X)) + X
-  const GemmProblem qkv = linear_problem(A, D, p->Wqkv, D, p->bqkv, p->qkv_scale, nullptr, 0, 1, none, QKV, 3 * D, IVIT_I8, 0, 0, M, 3 * D, D);
-  if ((rc = a_ready ? launch_gemm(ctx, qkv) : ln_dense(ctx, X, D, p->ln1_gamma, p->ln1_beta, p->M_ln, A, qkv))) return rc;
+  if (!a_ready && (rc = launch_layernorm(ctx, X, IVIT_I8, D, to_dev(p->ln1_gamma), p->ln1_beta, p->M_ln, A, D, M, D))) return rc;
+  if ((rc = launch_gemm(ctx, linear_problem(A, D, p->Wqkv, D, p->bqkv, p->qkv_scale, nullptr, 0, 1, none, QKV, 3 * D,
+                                            IVIT_I8, 0, 0, M, 3 * D, D)))) return rc;
   if ((rc = attention_impl(ctx, p, QKV, O, ws, w))) return rc;
   // output projection + residual; LayerNorm 2 of its rows in the kernel's tail
   GemmProblem proj = linear_problem(O, D, p->Wo, D, p->bo, p->o_scale, X, D, M, p->res1_scale, Xh, D, IVIT_I8, 0, 0, M, D, D);
@@ -170,15 +155,13 @@ int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_
   ctx->rowop_fused = 0;
   if ((rc = launch_gemm(ctx, proj))) return rc;
   // Y = MLP(LayerNorm(X^)) + X^
-  const bool ln2_done = ctx->rowop_fused != 0;
-  auto run_fc1 = [&](const GemmProblem& g) {
-    return ln2_done ? launch_gemm(ctx, g) : ln_dense(ctx, Xh, D, p->ln2_gamma, p->ln2_beta, p->M_ln, A, g);
-  };
+  if (!ctx->rowop_fused &&
+      (rc = launch_layernorm(ctx, Xh, IVIT_I8, D, to_dev(p->ln2_gamma), p->ln2_beta, p->M_ln, A, D, M, D))) return rc;
   GemmProblem fc1 = linear_problem(A, D, p->W1, D, p->b1, p->fc1_scale, nullptr, 0, 1, none, G, H, IVIT_I8, 0, 0, M, H, D);
   if (p->gelu_static_max) {
     // static-maximum ShiftGELU variant: element-wise, applied to the requantised value inside the FC1 epilogue
     if ((rc = gelu_static_row(ctx, p->gelu, p->gelu_post, &fc1.epi.act_table))) return rc;
-    if ((rc = run_fc1(fc1))) return rc;
+    if ((rc = launch_gemm(ctx, fc1))) return rc;
   } else {
     // Algorithm 2 needs the maximum of a token's whole MLP row: ShiftGELU of a block of rows runs once all the
     // channel tiles of those rows are stored, in the FC1 kernel's tail
@@ -187,14 +170,7 @@ int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_
       fc1.epi.rop.kind = 2;
     }
     ctx->rowop_fused = 0;
-    if ((rc = run_fc1(fc1))) return rc;
-    if (!ctx->rowop_fused && in_model && ctx->row_prologue && ctx->gemm_engine == 0) {
-      // inside a model forward ShiftGELU may run in front of FC2's MMAs (ivit_block_forward keeps it a kernel of its own)
-      GemmProblem g = linear_problem(G, H, p->W2, H, p->b2, p->fc2_scale, Xh, D, M, p->res2_scale, Y, D, IVIT_I8, 0, 0, M, D, H);
-      if ((rc = gelu_table_for(ctx, p->gelu, p->gelu_post, &g.epi.rop.table))) return rc;
-      rc = launch_gemm_small(ctx, g, 2);
-      if (rc != IVIT_ERR_UNSUPPORTED) return rc;
-    }
+    if ((rc = launch_gemm(ctx, fc1))) return rc;
     if (!ctx->rowop_fused && (rc = launch_shiftgelu(ctx, G, H, p->gelu, p->gelu_post, G, H, M, H))) return rc;
   }
   GemmProblem fc2 = linear_problem(G, H, p->W2, H, p->b2, p->fc2_scale, Xh, D, M, p->res2_scale, Y, D, IVIT_I8, 0, 0, M, D, H);
@@ -395,7 +371,7 @@ int host_forward(ivit_ctx* ctx, const int8_t* image_host, int32_t* logits_host, 
 namespace ivit {
 int launch_gemm(ivit_ctx* ctx, const GemmProblem& g) {
   if (ctx->gemm_engine == 0) {
-    int rc = g.epi.rop.kind && ctx->row_fusion ? IVIT_ERR_UNSUPPORTED : launch_gemm_small(ctx, g, 0);
+    int rc = g.epi.rop.kind && ctx->row_fusion ? IVIT_ERR_UNSUPPORTED : launch_gemm_small(ctx, g);
     if (rc != IVIT_ERR_UNSUPPORTED) return rc;
     rc = launch_gemm_tc(ctx, g);
     if (rc != IVIT_ERR_UNSUPPORTED) return rc;
@@ -459,7 +435,6 @@ int ivit_ctx_create(ivit_ctx** out, int device, void* cuda_stream) {
   }
   c->rowblk_dev = reinterpret_cast<unsigned*>(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes);
   c->row_fusion = 0;
-  c->row_prologue = 1;
   c->gemm_pairs = 1;
   *out = c;
   return IVIT_OK;
@@ -528,7 +503,6 @@ int ivit_ctx_set_row_fusion(ivit_ctx* ctx, int enable) {
   if (!ctx) return IVIT_ERR_INVALID_ARG;
   // 1: every row operator; 2: I-LayerNorm only, 4: ShiftGELU only (for measurements)
   ctx->row_fusion = enable == 1 ? 3 : (enable == 2 ? 1 : (enable == 4 ? 2 : 0));
-  ctx->row_prologue = enable == 8;
   for (int i = 0; i < 2; ++i) host_graph_drop(ctx, i);
   return IVIT_OK;
 }
@@ -789,15 +763,15 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
   bool a_ready = false;   // LayerNorm 1 of the next block already produced by the previous block's last Dense layer
   for (int64_t l = 0; l < p->depth; ++l) {
     const ivit_block_params* next = l + 1 < p->depth ? &p->blocks[l + 1] : nullptr;
-    if ((rc = block_impl(ctx, &p->blocks[l], X, Y, ws + w.block, a_ready, next, &a_ready, true))) return rc;
+    if ((rc = block_impl(ctx, &p->blocks[l], X, Y, ws + w.block, a_ready, next, &a_ready))) return rc;
     int8_t* t = X; X = Y; Y = t;
   }
   if (tokens && cudaMemcpyAsync(tokens, X, (size_t)(B * T * D), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
     return IVIT_ERR_CUDA;
   // final LayerNorm on the class-token rows, then the classifier (int32 logits, not saturated)
-  return ln_dense(ctx, X, T * D, p->lnf_gamma, p->lnf_beta, p->blocks[0].M_ln, Z,
-                  linear_problem(Z, D, p->Whead, D, p->bhead, p->head_scale, nullptr, 0, 1, none, logits, p->classes, IVIT_I32, 0, 0, B,
-                                 p->classes, D));
+  if ((rc = launch_layernorm(ctx, X, IVIT_I8, T * D, to_dev(p->lnf_gamma), p->lnf_beta, p->blocks[0].M_ln, Z, D, B, D))) return rc;
+  return launch_gemm(ctx, linear_problem(Z, D, p->Whead, D, p->bhead, p->head_scale, nullptr, 0, 1, none, logits,
+                                         p->classes, IVIT_I32, 0, 0, B, p->classes, D));
 }
 
 size_t ivit_vit_host_workspace_bytes(const ivit_vit_params* p) {
@@ -920,11 +894,11 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
       if (l + 1 == st->depth && s + 1 == p->n_stages && !sh) next = &fin;
       if (sh) {
         if ((rc = launch_gather_rows(ctx, cur, C, st->shift_index, rows, C, third, C))) return rc;
-        if ((rc = block_impl(ctx, &st->blocks[l], third, other, wsb, false, nullptr, nullptr, true))) return rc;
+        if ((rc = block_impl(ctx, &st->blocks[l], third, other, wsb, false, nullptr, nullptr))) return rc;
         if ((rc = launch_gather_rows(ctx, other, C, st->unshift_index, rows, C, cur, C))) return rc;
         a_ready = false;
       } else {
-        if ((rc = block_impl(ctx, &st->blocks[l], cur, other, wsb, a_ready, next, &a_ready, true))) return rc;
+        if ((rc = block_impl(ctx, &st->blocks[l], cur, other, wsb, a_ready, next, &a_ready))) return rc;
         int8_t* t = cur; cur = other; other = t;
       }
     }
@@ -933,18 +907,13 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
       if ((rc = launch_gather_rows(ctx, cur, C, st->merge_index, rows, C, other, C))) return rc;
       rows /= 4;
       res /= 2;
-      const GemmProblem merge = linear_problem(third, 4 * C, st->Wmerge, 4 * C, nullptr, st->merge_scale, nullptr, 0, 1, none, cur, 2 * C,
-                                               IVIT_I8, 0, 0, rows, 2 * C, 4 * C);
-      if (!(ctx->row_fusion & 1)) {
-        if ((rc = ln_dense(ctx, other, 4 * C, st->merge_ln_gamma, st->merge_ln_beta, p->M_ln, third, merge))) return rc;
-        a_ready = false;
-        continue;
-      }
       if ((rc = launch_layernorm(ctx, other, IVIT_I8, 4 * C, to_dev(st->merge_ln_gamma), st->merge_ln_beta, p->M_ln, third,
                                  4 * C, rows, 4 * C))) return rc;
       // ... followed by LayerNorm 1 of the next stage's first block (into the block workspace, where it expects it)
       const ivit_block_params* nb = &p->stages[s + 1].blocks[0];
-      if ((rc = dense_then_layernorm(ctx, merge, nb->ln1_gamma, nb->ln1_beta, nb->M_ln, reinterpret_cast<int8_t*>(wsb)))) return rc;
+      if ((rc = dense_then_layernorm(ctx, linear_problem(third, 4 * C, st->Wmerge, 4 * C, nullptr, st->merge_scale, nullptr, 0, 1,
+                                                          none, cur, 2 * C, IVIT_I8, 0, 0, rows, 2 * C, 4 * C),
+                                     nb->ln1_gamma, nb->ln1_beta, nb->M_ln, reinterpret_cast<int8_t*>(wsb)))) return rc;
       a_ready = !(p->stages[s + 1].shifted && p->stages[s + 1].shifted[0]);
     }
   }

@@ -7,10 +7,6 @@
 
 namespace ivit {
 
-// A compile-time integer as a value (template arguments of the row routines picked by a generic lambda).
-template <int V>
-struct Int { static constexpr int value = V; };
-
 // Integer square root, floor(sqrt(n)) for n < 2^26, one result bit per step (no division): the value the
 // guarded iteration of Eq. (iterative) converges to.  Equality with the oracle's iteration is checked
 // exhaustively over the whole range by a test (ivit_isqrt_range).
@@ -95,10 +91,9 @@ __device__ __forceinline__ void ln_fold_consts(int nwords, int4* sm_s, int4* sm_
 // (rows past nrows are not touched), results to out with stride ldout.  The row sums are reduced together and the
 // per-row scalars (mean, sum of squared deviations, square root, reciprocal) are computed by R lanes in parallel.
 // CG: read the rows with L2 loads (rows written by other CTAs of the running kernel).
-// store(r, idx, word): receives word idx (four channels) of result row r.
-template <int WPL, int R, bool CG, class Store>
-__device__ __forceinline__ void layernorm_rows_to(const int8_t* in, int64_t ldin, int nrows, int C, int M_ln, unsigned mean_magic,
-                                                  const LnConsts& k, int lane, Store store) {
+template <int WPL, int R, bool CG>
+__device__ __forceinline__ void layernorm_rows(const int8_t* in, int64_t ldin, int nrows, int C, int M_ln, unsigned mean_magic,
+                                               const LnConsts& k, int8_t* out, int64_t ldout, int lane) {
   const int nwords = C >> 2;
   int w[R][WPL];
 #pragma unroll
@@ -165,28 +160,20 @@ __device__ __forceinline__ void layernorm_rows_to(const int8_t* in, int64_t ldin
           unsigned t, d;
           asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(t) : "r"(v[3]), "r"(v[2]), "r"(0));
           asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(v[1]), "r"(v[0]), "r"(t));
-          store(r, idx, d);
+          reinterpret_cast<int*>(out + (int64_t)r * ldout)[idx] = (int)d;
         }
       }
     }
   }
-}
-template <int WPL, int R, bool CG>
-__device__ __forceinline__ void layernorm_rows(const int8_t* in, int64_t ldin, int nrows, int C, int M_ln, unsigned mean_magic,
-                                               const LnConsts& k, int8_t* out, int64_t ldout, int lane) {
-  layernorm_rows_to<WPL, R, CG>(in, ldin, nrows, C, M_ln, mean_magic, k, lane, [&](int r, int idx, unsigned w) {
-    reinterpret_cast<unsigned*>(out + (int64_t)r * ldout)[idx] = w;
-  });
 }
 
 // ---- ShiftGELU --------------------------------------------------------------------------------------------
 // One warp, R rows of `cols` int8 values (cols % 16 == 0, cols <= 512 * WPL): row maximum, then one look-up per
 // value in row max(0, maximum) of the 128 x 256 table; `tab` is the warp's staging space for the R table rows
 // (R x 64 words of shared memory, 256-byte aligned).  in == out is allowed.
-// store(r, idx, int4): receives the idx-th 16 bytes of result row r.
-template <int WPL, int R, bool CG, class Store>
-__device__ __forceinline__ void shiftgelu_rows_to(const int8_t* in, int64_t ldin, int nrows, int cols, const int8_t* table,
-                                                  unsigned* tab, int lane, int fixed_max, Store store) {
+template <int WPL, int R, bool CG>
+__device__ __forceinline__ void shiftgelu_rows(const int8_t* in, int64_t ldin, int nrows, int cols, const int8_t* table,
+                                               unsigned* tab, int8_t* out, int64_t ldout, int lane, int fixed_max = -1) {
   const int nvec = cols >> 4;
   int4 w[R][WPL];
   int mx[R];
@@ -219,6 +206,7 @@ __device__ __forceinline__ void shiftgelu_rows_to(const int8_t* in, int64_t ldin
       // shared-memory address of entry 0 of this row's table: 256-byte aligned, so that one byte permute puts
       // the index x + 128 into its low byte
       const uint32_t t8 = (uint32_t)__cvta_generic_to_shared(tab + 64 * r);
+      int4* dst = reinterpret_cast<int4*>(out + (int64_t)r * ldout);
 #pragma unroll
       for (int i = 0; i < WPL; ++i) {
         const int idx = lane + 32 * i;
@@ -236,18 +224,11 @@ __device__ __forceinline__ void shiftgelu_rows_to(const int8_t* in, int64_t ldin
             }
             vout[q] = (int)__byte_perm(__byte_perm(e[0], e[1], 0x0040), __byte_perm(e[2], e[3], 0x0040), 0x5410);
           }
-          store(r, idx, make_int4(vout[0], vout[1], vout[2], vout[3]));
+          dst[idx] = make_int4(vout[0], vout[1], vout[2], vout[3]);
         }
       }
     }
   }
-}
-template <int WPL, int R, bool CG>
-__device__ __forceinline__ void shiftgelu_rows(const int8_t* in, int64_t ldin, int nrows, int cols, const int8_t* table,
-                                               unsigned* tab, int8_t* out, int64_t ldout, int lane, int fixed_max = -1) {
-  shiftgelu_rows_to<WPL, R, CG>(in, ldin, nrows, cols, table, tab, lane, fixed_max, [&](int r, int idx, int4 v) {
-    reinterpret_cast<int4*>(out + (int64_t)r * ldout)[idx] = v;
-  });
 }
 
 }  // namespace ivit

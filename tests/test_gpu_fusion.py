@@ -97,40 +97,3 @@ def test_linear_then_layernorm_tail_many_row_blocks_random_values():
     finally:
         c.set_row_fusion(False)
     assert c.poll_status() == 0
-
-
-@pytest.mark.parametrize("B,T,D,heads,H", [(1, 1, 16, 1, 16), (1, 33, 48, 1, 80), (1, 197, 192, 3, 768), (2, 257, 384, 6, 1536),
-                                           (9, 197, 384, 6, 1552), (2, 65, 768, 12, 3072), (1, 130, 1024, 16, 4096),
-                                           (24, 197, 384, 6, 1536), (60, 49, 768, 24, 3072), (1, 40, 1040, 5, 4112)])
-def test_row_operators_in_front_of_the_dense_layers(B, T, D, heads, H):
-    """Layers of few rows: LayerNorm (and, in model forwards, ShiftGELU) in front of the MMAs of the Dense layer that
-    reads it.  Contraction tails of 16, ragged row blocks and channel groups, one to four channel tiles per CTA, sizes
-    on both sides of what the kernel takes; the block as kernels of their own gives the same bytes."""
-    import gpu_util as g
-    c = g.binding.Context(0)
-    blk = make_block(_Ids(5000 + B + D), 2, B, T, D, heads, H)
-    X = make_block_input(B + D, B, T, D)
-    dblk = g.binding.DeviceBlock(blk, "cuda")
-    dX = torch.from_numpy(X).cuda()
-    want = O.block_forward(blk, X)
-    g.assert_equal(g.host(c.block_forward(dblk, dX)), want, "default")
-    c.set_row_fusion(False)
-    g.assert_equal(g.host(c.block_forward(dblk, dX)), want, "kernels of their own")
-    assert c.poll_status() == 0
-
-
-@pytest.mark.parametrize("batch,img,D,heads,H", [(1, 224, 192, 3, 768), (3, 160, 384, 6, 1536), (2, 64, 768, 12, 3072), (1, 32, 1024, 16, 4096)])
-def test_small_model_forwards_with_prologues(batch, img, D, heads, H):
-    """Two-block model forwards small enough for every Dense layer to take its row operator along."""
-    import gpu_util as g
-    from ivit_inputs.gen import make_image, make_vit
-    c = g.binding.Context(0)
-    model, image = make_vit(60 + batch, batch, img, D, heads, H, 2), make_image(61, batch, img)
-    dm = g.binding.DeviceVit(model, "cuda")
-    d_img = torch.from_numpy(image).cuda()
-    c.vit_forward(dm, d_img)           # builds the ShiftGELU tables
-    n0 = c.launch_count()
-    got = g.host(c.vit_forward(dm, d_img))
-    assert c.launch_count() - n0 == 3 + 5 * 2 + 1      # patches, embedding, class rows; five kernels per block; the head
-    g.assert_equal(got, O.vit_forward(model, image), "logits")
-    assert c.poll_status() == 0

@@ -503,3 +503,34 @@ def test_layernorm_square_root_routine_equals_the_iteration_exhaustively():
         assert np.array_equal(got, want), f"first mismatch at n = {n0 + int(np.argmax(got != want))}"
     with pytest.raises(g.binding.IvitError):
         c.isqrt_range((1 << 26) - 4, 8)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 4, 16), (32, 128, 128), (33, 132, 144), (128, 260, 2064), (1184, 512, 96), (1185, 512, 96),
+                                   (4736, 388, 80), (4737, 388, 80), (31, 1000, 6144), (31, 1000, 6160)])
+def test_linear_one_wave_of_small_tiles(M, N, K):
+    """The kernel for layers of one wave (32 to 128 rows per tile, resident input rows) and the sizes next to its limits:
+    tile and contraction remainders, ring wrap-around, residual shifts on both sides of 39 (from there on the residual
+    term rounds to 0), wrapped residual rows, grouped output rows, int32 output."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(M + 3 * N + 5 * K)
+    A, W = rand_i8(rng, (M, K)), rand_i8(rng, (N, K))
+    bias = rng.integers(-20000, 20000, N).astype(np.int32)
+    acc_std = np.sqrt(K) * 40 * 40
+    scale = scale_channels(rng.uniform(20, 60, N) / acc_std)
+    dA, dW, db, ds = g.dev(A), g.dev(W), torch.from_numpy(bias).cuda(), g.binding.DevScale(scale, "cuda")
+    for ratio, rows in ((0.99, M), (2.0 ** -7, M), (2.0 ** -8 * 0.999, max(1, M // 3))):
+        res, rs = rand_i8(rng, (rows, N), std=120), Scale(*dyadic(ratio))
+        got = c.linear(dA, dW, db, ds, res=g.dev(res), res_scale=g.binding.DevScale(rs, "cuda"), out=g.dev(np.zeros((M, N), np.int8)))
+        g.assert_equal(g.host(got), O.linear(A, W, bias, scale, res=res, res_scale=rs), f"residual {ratio}")
+    pt = Scale(*dyadic(3000.0 / acc_std))
+    got = c.linear(dA, dW, db, g.binding.DevScale(pt, "cuda"), out_dtype=g.binding.I32, out=g.dev(np.zeros((M, N), np.int32), 4))
+    g.assert_equal(g.host(got), O.linear(A, W, bias, pt, out_dtype=O.I32), "int32")
+    group = max(1, M // 2)
+    out = g.dev(np.full((M // group * (group + 3) + group, N), 77, np.int8))
+    c.linear(dA, dW, None, ds, out=out, out_group_rows=group, out_group_stride=group + 3)
+    want = np.full(out.shape, 77, np.int8)
+    r = np.arange(M)
+    want[r // group * (group + 3) + r % group] = O.linear(A, W, None, scale)
+    g.assert_equal(g.host(out), want, "grouped rows")
+    assert c.poll_status() == 0
