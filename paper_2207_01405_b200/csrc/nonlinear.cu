@@ -122,32 +122,149 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
   }
 }
 
-// Rows of up to 1024 channels: a warp takes R rows at a time (layernorm_rows); the per-channel constants are
-// prepared once per block in shared memory, before the wait for the previous kernel (they are parameters, not
-// results).
-template <int WPL, int R>
-__global__ void __launch_bounds__(128) layernorm_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
-                                                             const int32_t* __restrict__ beta, int M_ln,
-                                                             int8_t* __restrict__ out, int64_t ldout, int64_t rows, int C,
-                                                             unsigned mean_magic, int vec) {
-  extern __shared__ int4 ln_consts[];   // [3][C / 4]: multipliers, shifts, addends (or betas)
+// Rows of up to 1024 channels.  L lanes share a row (G = 32 / L rows side by side in a warp), a lane holds WPL words of four
+// channels of R such rows, and the constants of its channels in registers (fetched before the wait for the previous
+// kernel: they are parameters).  kExact: C = 4 L WPL, nothing to mask.  Rows past the end are read as the last row and not
+// stored: the body has no branch but the one on the form of the constants.  What bounds it is instruction issue: byte,
+// multiply-add, mad.hi, shift and half a pack per value, and about 130 instructions for the scalars of G R rows at once.
+// With a branch around every word and row, constants in shared memory and one row per 32 lanes, three of four
+// instructions were overhead.  Measured, back to back: 25216 x 768 16.3 -> 10.9 us, 18464 x 1024 17.5 -> 12.1, 12608 x 384
+// 6.2 -> 4.0, 200704 x 96 27.4 -> 12.1, 197 x 192 2.4 -> 1.5.
+// fast: every channel of the warp has s >= 33 and a small beta (see LnConsts): m, sh = s - 32 and add = 2^(sh-1) + beta 2^sh.
+template <int WPL>
+struct LnLane {
+  int m[WPL][4], s[WPL][4], b[WPL][4];
+  bool fast;
+  // words idx0, idx0 + L, ... of the row
+  __device__ __forceinline__ void fetch(const ScaleDev& gs, const int32_t* beta, int nwords, int vec, int idx0, int L) {
+    fast = true;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+      const int idx = idx0 + L * i;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) { m[i][k] = 1; s[i][k] = 33; b[i][k] = 0; }
+      if (idx < nwords) {
+        if (vec) {
+          const int4 m4 = __ldg(reinterpret_cast<const int4*>(gs.mult_c) + idx);
+          const uchar4 s4 = __ldg(reinterpret_cast<const uchar4*>(gs.shift_c) + idx);
+          m[i][0] = m4.x; m[i][1] = m4.y; m[i][2] = m4.z; m[i][3] = m4.w;
+          s[i][0] = s4.x; s[i][1] = s4.y; s[i][2] = s4.z; s[i][3] = s4.w;
+          if (beta) {
+            const int4 b4 = __ldg(reinterpret_cast<const int4*>(beta) + idx);
+            b[i][0] = b4.x; b[i][1] = b4.y; b[i][2] = b4.z; b[i][3] = b4.w;
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            m[i][k] = gs.m(idx * 4 + k);
+            s[i][k] = gs.s(idx * 4 + k);
+            if (beta) b[i][k] = __ldg(beta + idx * 4 + k);
+          }
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        s[i][k] = clamp_shift(s[i][k]);
+        const int sh = s[i][k] - 32;
+        fast = fast && sh >= 1 && b[i][k] > -(1 << (29 - sh)) && b[i][k] < (1 << (29 - sh));
+      }
+    }
+    fast = __all_sync(0xffffffffu, fast);
+    if (fast) {
+#pragma unroll
+      for (int i = 0; i < WPL; ++i)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          s[i][k] -= 32;
+          b[i][k] = (1 << (s[i][k] - 1)) + b[i][k] * (1 << s[i][k]);
+        }
+    }
+  }
+};
+
+template <int L, int WPL, int R, int PER_SM, bool kExact>
+__global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
+                                                                     const int32_t* __restrict__ beta, int M_ln,
+                                                                     int8_t* __restrict__ out, int64_t ldout, int rows, int C,
+                                                                     unsigned mean_magic, int vec) {
+  static_assert(R <= L, "a lane per row for the scalars");
+  constexpr int G = 32 / L;
   pdl_trigger();
-  const int nwords = C >> 2;
-  int4* sm_m = ln_consts;
-  int4* sm_s = ln_consts + nwords;
-  int4* sm_b = ln_consts + 2 * nwords;
-  bool fast = ln_stage_consts(gs, beta, nwords, vec, sm_m, sm_s, sm_b, threadIdx.x, blockDim.x);
-  fast = __syncthreads_and(fast) != 0;
-  if (fast) ln_fold_consts(nwords, sm_s, sm_b, threadIdx.x, blockDim.x);
-  __syncthreads();
-  const LnConsts k{sm_m, sm_s, sm_b, fast};
+  const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
+  const int nwords = kExact ? L * WPL : C >> 2;
+  LnLane<WPL> k;
+  k.fetch(gs, beta, nwords, vec, li, L);
   pdl_wait();
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t r0 = warp * R; r0 < rows; r0 += nwarps * R) {
-    const int nrows = (int)(rows - r0 < R ? rows - r0 : R);
-    layernorm_rows<WPL, R, false>(in + r0 * ldin, ldin, nrows, C, M_ln, mean_magic, k, out + r0 * ldout, ldout, lane);
+  const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int stride = (int)((gridDim.x * blockDim.x) >> 5) * (G * R);
+  for (int r0 = warp * (G * R) + grp; r0 - grp < rows; r0 += stride) {
+    int w[R][WPL];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int* src = reinterpret_cast<const int*>(in + (int64_t)min(r0 + r * G, rows - 1) * ldin) + li;
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) w[r][i] = kExact || li + L * i < nwords ? __ldg(src + L * i) : 0;
+    }
+    int my_s1 = 0, my_s2 = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      int s1 = 0, s2 = 0;
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) {
+        s1 = __dp4a(w[r][i], 0x01010101, s1);
+        s2 = __dp4a(w[r][i], w[r][i], s2);
+      }
+      if (L == 32) {
+        s1 = __reduce_add_sync(0xffffffffu, s1);
+        s2 = __reduce_add_sync(0xffffffffu, s2);
+      } else {
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) {
+          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+      }
+      my_s1 = li == r ? s1 : my_s1;
+      my_s2 = li == r ? s2 : my_s2;
+    }
+    // lane r < R of every group: the scalars of its r-th row (see layernorm_rows)
+    const int mu = (int)__umulhi((unsigned)(2 * my_s1 + 257 * C), mean_magic) - 128;
+    const unsigned V = (unsigned)(my_s2 - 2 * mu * my_s1 + C * mu * mu);
+    const unsigned sd = isqrt_bits26(V);
+    const int F = sd == 0 ? 0 : (int)((1u << M_ln) / sd);
+    const int muF = (int)((unsigned)mu * (unsigned)F);
+    auto rows_out = [&](auto fast) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int Fr = __shfl_sync(0xffffffffu, F, grp * L + r), muFr = __shfl_sync(0xffffffffu, muF, grp * L + r);
+        const int row = r0 + r * G;
+        int* dst = reinterpret_cast<int*>(out + (int64_t)row * ldout) + li;
+#pragma unroll
+        for (int i = 0; i < WPL; ++i) {
+          int v[4];
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            int xb;   // byte b, sign-extended
+            asm("prmt.b32 %0, %1, %1, %2;" : "=r"(xb) : "r"(w[r][i]), "r"(0x8880 + 0x1111 * b));
+            // (x - mu) * F modulo 2^32: the difference fits, |y F| <= 2^(M_ln + 1)
+            const int yF = (int)((unsigned)xb * (unsigned)Fr - (unsigned)muFr);
+            if (decltype(fast)::value) {
+              int h;
+              asm("mad.hi.s32 %0, %1, %2, %3;" : "=r"(h) : "r"(yF), "r"(k.m[i][b]), "r"(k.b[i][b]));
+              v[b] = h >> k.s[i][b];
+            } else {
+              // (the rare form: constants from global memory, so that they do not take registers from the other)
+              const int c = min((li + L * i) * 4 + b, C - 1);
+              v[b] = rq(yF, gs.m(c), gs.s(c)) + (beta ? __ldg(beta + c) : 0);
+            }
+          }
+          const int word = (int)pack_sat8_u(v[0], v[1], v[2], v[3]);
+          if (row < rows && (kExact || li + L * i < nwords)) dst[L * i] = word;
+        }
+      }
+    };
+    if (k.fast) rows_out(std::true_type{});
+    else rows_out(std::false_type{});
   }
 }
 
@@ -242,23 +359,32 @@ int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, 
   }
   const int8_t* x = (const int8_t*)in;
   const int wpl = (int)((C / 4 + 31) / 32);
-  if (wpl <= 8) {
-    // four rows per warp (eight for rows of at most 128 channels, two above 512): short per-warp work lets the blocks of this
-    // kernel slip into the tail of the kernel before it and out of the way of the one after it
-    const int rpw = wpl <= 1 ? 8 : (wpl <= 4 ? 4 : 2), tb = 128;
-    const int64_t warps = (rows + rpw - 1) / rpw;
-    const int64_t wantb = (warps + tb / 32 - 1) / (tb / 32);
-    const int gridb = (int)(wantb < (int64_t)ctx->sm_count * 12 ? wantb : (int64_t)ctx->sm_count * 12);
+  if (wpl <= 8 && rows < (1ll << 31) - (1 << 20)) {
     const unsigned magic = (unsigned)(0x100000000ull / (unsigned long long)(2 * C)) + 1u;
     const int vec = gs.mult_c && gs.shift_c && !(reinterpret_cast<uintptr_t>(gs.mult_c) & 15) && !(reinterpret_cast<uintptr_t>(gs.shift_c) & 3) &&
                     !(reinterpret_cast<uintptr_t>(beta) & 15);
-    const size_t cbytes = (size_t)(C / 4) * 3 * sizeof(int4);
-    if (wpl <= 1) launch_k(layernorm_rows_kernel<1, 8>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
-    else if (wpl <= 2) launch_k(layernorm_rows_kernel<2, 4>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
-    else if (wpl <= 3) launch_k(layernorm_rows_kernel<3, 4>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
-    else if (wpl <= 4) launch_k(layernorm_rows_kernel<4, 4>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
-    else if (wpl <= 6) launch_k(layernorm_rows_kernel<6, 2>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
-    else launch_k(layernorm_rows_kernel<8, 2>, dim3(gridb), dim3(tb), cbytes, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C, magic, vec);
+    // (rows: rows of a warp and pass)
+    auto run = [&](auto kernel, int rpw, int per_sm) {
+      const int64_t blocks = (rows + 4 * rpw - 1) / (4 * rpw), cap = (int64_t)ctx->sm_count * per_sm;
+      launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(128), 0, st, x, ldin, gs, beta, M_ln, out, ldout, (int)rows, (int)C, magic, vec);
+    };
+    // Blocks per SM: as many as the registers allow without spilling much (25216 x 768: 10.9 us at three, 12.7 at four,
+    // 16.2 at five; 12608 x 384: 4.0 at five, 4.3 at six).  Up to 1024 rows one row per group of lanes: with so few rows the
+    // chain of one warp counts (197 x 192: 1.45 against 1.8 us).
+    const bool few = rows <= 1024;
+    switch (C) {
+      case 96: few ? run(layernorm_rows_kernel<8, 3, 1, 5, true>, 4, 5) : run(layernorm_rows_kernel<8, 3, 4, 5, true>, 16, 5); break;
+      case 192: few ? run(layernorm_rows_kernel<16, 3, 1, 5, true>, 2, 5) : run(layernorm_rows_kernel<16, 3, 4, 5, true>, 8, 5); break;
+      case 384: few ? run(layernorm_rows_kernel<32, 3, 1, 5, true>, 1, 5) : run(layernorm_rows_kernel<32, 3, 4, 5, true>, 4, 5); break;
+      case 512: run(layernorm_rows_kernel<32, 4, 4, 4, true>, 4, 4); break;
+      case 768: few ? run(layernorm_rows_kernel<32, 6, 1, 4, true>, 1, 4) : run(layernorm_rows_kernel<32, 6, 4, 3, true>, 4, 3); break;
+      case 1024: few ? run(layernorm_rows_kernel<32, 8, 1, 3, true>, 1, 3) : run(layernorm_rows_kernel<32, 8, 4, 2, true>, 4, 2); break;
+      default:
+        if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);
+        else if (wpl <= 2) run(layernorm_rows_kernel<32, 2, 4, 8, false>, 4, 8);
+        else if (wpl <= 4) run(layernorm_rows_kernel<32, 4, 4, 5, false>, 4, 5);
+        else run(layernorm_rows_kernel<32, 8, 2, 3, false>, 2, 3);
+    }
     return ls.done();
   }
   if (wpl <= 12) launch_k(layernorm_i8_kernel<12>, dim3(grid), dim3(threads), 0, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C);

@@ -534,3 +534,23 @@ def test_linear_one_wave_of_small_tiles(M, N, K):
     want[r // group * (group + 3) + r % group] = O.linear(A, W, None, scale)
     g.assert_equal(g.host(out), want, "grouped rows")
     assert c.poll_status() == 0
+
+
+@pytest.mark.parametrize("C", [4, 96, 128, 132, 192, 384, 512, 600, 768, 1020, 1024])
+def test_layernorm_row_counts_and_forms(C):
+    """The row kernel packs several short rows into a warp and takes one row per lane group up to 1024 rows: row counts
+    around a warp's share and around that limit, constants of both forms (a shift of 32 leaves the high-word form),
+    per-tensor scale without beta."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(C)
+    for rows in (1, 3, 17, 1024, 1025, 1043):
+        x = rand_i8(rng, (rows, C), std=25)
+        x[rows // 2] = 7                                             # a constant row: F = 0
+        ratios = rng.uniform(20, 40, C) * np.sqrt(C) / 2.0 ** 20
+        beta = rng.integers(-20, 20, C).astype(np.int32)
+        for sc, b in ((scale_channels(ratios), beta), (scale_channels(np.where(np.arange(C) == C // 2, 0.3, ratios)), beta),
+                      (Scale(*dyadic(30.0 * np.sqrt(C) / 2.0 ** 20)), None)):
+            got = c.layernorm(g.dev(x), g.binding.DevScale(sc, "cuda"), None if b is None else torch.from_numpy(b).cuda(), 20)
+            g.assert_equal(g.host(got), O.layernorm(x, sc, b, 20), f"rows={rows} C={C}")
+    assert c.poll_status() == 0
