@@ -15,6 +15,7 @@
 // V is consumed as stored ([token, d] rows, MN-major B operand).  Every wait is bounded.
 // What bounds the passes: issue slots.  mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer
 // instructions two cycles of their pipe, a look-up one of the SM's shared-memory cycles.
+#include "shiftmax.cuh"
 #include "tc_ptx.cuh"
 #include <cstdlib>
 
@@ -30,51 +31,6 @@ __device__ __forceinline__ uint32_t prob_word(unsigned factor, int e0, int e1, i
   return pack_sat8(min((int)(__umulhi(factor, (unsigned)e0) >> osh), omax), min((int)(__umulhi(factor, (unsigned)e1) >> osh), omax),
                    min((int)(__umulhi(factor, (unsigned)e2) >> osh), omax), min((int)(__umulhi(factor, (unsigned)e3) >> osh), omax));
 }
-// The same for k_out = 8 with factor4 = 4 floor(2^45 / sum): the probability is byte 1 of the high product word.  The one
-// probability that can reach 128, and is clamped to 127, belongs to a row whose only non-zero exponential is a power of
-// two; prob_factor4 takes one off the reciprocal there, which gives 127.
-__device__ __forceinline__ uint32_t prob_word8(unsigned factor4, int e0, int e1, int e2, int e3) {
-  return __byte_perm(__byte_perm(__umulhi(factor4, (unsigned)e0), __umulhi(factor4, (unsigned)e1), 0x0051),
-                     __byte_perm(__umulhi(factor4, (unsigned)e2), __umulhi(factor4, (unsigned)e3), 0x0051), 0x5410);
-}
-
-// ShiftExp of one packed score x (int8): the table entry at t - 4 cp x, where `sel` holds -4 cp in the byte that holds x.
-// (Not volatile: the table does not change once the CTA's first barrier is behind, so look-ups may be moved freely.)
-__device__ __forceinline__ unsigned exp_entry(uint32_t w, uint32_t sel, uint32_t t) {
-  unsigned e;
-  asm("{\n\t.reg .u32 a;\n\tdp4a.s32.s32 a, %1, %2, %3;\n\tld.shared.u32 %0, [a];\n\t}" : "=r"(e) : "r"(w), "r"(sel), "r"(t));
-  return e;
-}
-
-// floor(2^45 / s) for 2^15 < s < 2^32.  With d = s 2^z, 2^31 <= d < 2^32, it is floor(2^63 / d) >> (18 - z) (nested floor
-// quotients).  v starts at 2^63 / (middle of the 2^24 values that share d's upper byte), relative error below 2^-8, from
-// a table of 128 entries; two Newton steps square that twice; the shift (by at least 2) leaves at most one unit, which
-// the exact remainder puts right.  (Checked on the CPU for every s of the range; a 64-bit division takes 700 cycles on
-// the row's critical path.)
-__device__ __forceinline__ unsigned recip_seed(int i) { return (unsigned)((1ull << 40) / (unsigned)(2 * (128 + i) + 1)); }
-__device__ __forceinline__ unsigned recip45(unsigned s, const unsigned* seeds) {
-  const int z = __clz(s);
-  const unsigned d = s << z;
-  unsigned v = seeds[(d >> 24) & 127u];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) {
-    const int e = (int)(0x80000000u - __umulhi(v, d));               // 2^31 - v d / 2^32
-    v += (unsigned)__mulhi((int)(v >> 1), e << 2);
-  }
-  if (d == 0x80000000u) v = 0xffffffffu;   // 2^32 itself does not fit
-  unsigned q = v >> (18 - z);
-  long long r = (long long)((1ull << 45) - (unsigned long long)q * s);
-  if (r < 0) { --q; r += s; }
-  if (r >= (long long)s) ++q;
-  return q;
-}
-// Four times the reciprocal for prob_word8; `top` = I0 2^N > 2^15, the largest exponential.
-__device__ __forceinline__ unsigned prob_factor4(unsigned sum, unsigned top, const unsigned* seeds) {
-  unsigned f = recip45(sum, seeds);
-  if (sum == top && (sum & (sum - 1u)) == 0u) --f;
-  return f << 2;
-}
-
 // Fields that both kernels use.
 struct AttnArgs {
   int T, d, heads;
@@ -121,14 +77,6 @@ struct __align__(16) AttnItem {
 __device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, const int (&pos)[3], int row, int h, int b) {
   tma_load_4d(dst, map, bar, 0, pos[0] == 1 ? row : (pos[1] == 1 ? h : b), pos[0] == 2 ? row : (pos[1] == 2 ? h : b),
               pos[0] == 3 ? row : (pos[1] == 3 ? h : b));
-}
-
-// The ShiftExp table: entry i, copy c at word i cp + c; consecutive lanes write different banks.  n threads.
-__device__ __forceinline__ void build_exp_table(const AttnArgs& a, uint8_t* tab, int st, int n) {
-  const unsigned e = shiftexp(-(st & 255), a.smax.I0, a.smax.N);
-  const int per = 32 / a.cp;                  // entries per 32 banks
-  for (int c = st >> 8; c < a.cp; c += n >> 8)
-    *reinterpret_cast<unsigned*>(tab + 4u * ((unsigned)(st & 255) * a.cp + ((c + (st & 31) / per) & (a.cp - 1)))) = e;
 }
 
 // Constants of the inner loops, held in registers (the compiler would fetch them again for every use).
@@ -351,7 +299,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
     const int qd = warp & 3;
     const int half = (warp - 1) >> 2;
     const int trow = qd * 32 + lane;              // row inside the tile
-    build_exp_table(a, gen + tab_off, st, 256);
+    build_exp_table(a.smax.I0, a.smax.N, a.cp, gen + tab_off, st, 256);
     // probabilities that no item writes are 0: columns past the last chunk, other windows' columns
     for (int c = (kPack ? 0 : a.chunks) + half; c < a.kpad / 16; c += 2)
       *reinterpret_cast<uint4*>(gen + p_off + (c >> 3) * (128 * 128) + trow * 128 + (((c & 7) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -749,7 +697,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
     const int qd = warp & 3;
     const int part = (warp - kRowsFirst) >> 2;    // 0..3
     const int trow = qd * 32 + lane;              // row inside the tile
-    build_exp_table(a, gen + tab_off, st, 512);
+    build_exp_table(a.smax.I0, a.smax.N, a.cp, gen + tab_off, st, 512);
     // probabilities of columns past the last chunk are never written again: zero (P V contracts over kpad columns)
     for (int c = a.chunks + part; c < a.kpad / 16; c += 4)
       for (int u = 0; u < 2; ++u)
@@ -973,7 +921,7 @@ static void fill_args(ivit_ctx* ctx, AttnArgs& a, const ivit_block_params* p, in
 static bool fit_table(AttnArgs& a, size_t fixed, size_t limit) {
   a.cp = 32;
   while (a.cp > 1 && fixed + 1024 * a.cp > limit) a.cp >>= 1;
-  for (int i = 0; i < 4; ++i) a.sel[i] = ((uint32_t)(-4 * a.cp) & 0xffu) << (8 * i);
+  for (int i = 0; i < 4; ++i) a.sel[i] = exp_sel(a.cp, i);
   return fixed + 1024 * a.cp <= limit;
 }
 // The arithmetic forms fixed at compile time: k_out = 8, both requantisation shifts >= 33, the largest exponential (and

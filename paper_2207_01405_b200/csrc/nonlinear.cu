@@ -2,6 +2,7 @@
 // One warp owns one row; rows are read once from HBM as coalesced 32-bit words and
 // kept in registers between the reduction and the output pass.
 #include "rowops.cuh"
+#include "shiftmax.cuh"
 #include <type_traits>
 
 namespace ivit {
@@ -419,11 +420,132 @@ struct RowLoader {
   }
 };
 
-// WPL words per lane in registers (d <= 128 * WPL); WPL == 0: re-read the row for each pass.
-// Bytes are handled as biased values u = x + 128 (x ^ 0x80), so that one byte permute yields the table index:
-// ShiftExp(x - max) = tab[max - x] = tab[(max + 128) - u].  Positions past d hold u = 0 (x = -128); they never
-// win the maximum and their table entries are taken out of the sum again.
-template <int WPL, int ROWS, bool FROM_I32>
+// Rows of up to 2048 values.  L lanes share a row (32 / L rows side by side in a warp); a lane holds WPL words of four
+// values, their exponentials stay in registers between the row sum and the output.  Look-ups, reciprocal and
+// probabilities as in the attention kernels (shiftmax.cuh).  Positions past d hold -128: they never win the maximum, their
+// exponentials are taken out of the sum again, and their probabilities are masked.
+// FAST: k_out = 8, I0 2^N > 2^15 and (int32 input) a shift >= 33 in front; otherwise the general arithmetic.
+// What bounds it: instruction issue (about nine instructions per value, two of them multiply-highs with int32 input).
+// Measured, back to back (before: a warp per row, one table, byte permutes, a 64-bit division per row): int32 18464 x 577
+// 17.8 -> 9.3 us (5.7 TB/s), 75648 x 197 33.4 -> 12.6, 200000 x 49 50.4 -> 14.3; int8 75648 x 197 17.5 -> 9.5.
+template <int L, int WPL, bool FROM_I32, bool FAST>
+__global__ void __launch_bounds__(512, WPL > 8 ? 1 : 2) shiftmax_rows_kernel(RowLoader<FROM_I32> ld, ivit_exp_params p, int cp,
+                                                               int8_t* __restrict__ out, int64_t ldout, int rows, int d) {
+  extern __shared__ __align__(128) uint8_t sm_tab[];   // [256 x cp][128 seeds of the reciprocal]
+  constexpr int G = 32 / L;
+  pdl_trigger();
+  build_exp_table(p.I0, p.N, cp, sm_tab, threadIdx.x, blockDim.x);
+  unsigned* seeds = reinterpret_cast<unsigned*>(sm_tab + 1024 * cp);
+  if (threadIdx.x < 128) seeds[threadIdx.x] = recip_seed(threadIdx.x);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
+  const int nwords = (d + 3) >> 2, nwords_out = ((d + 15) >> 4) << 2;
+  uint32_t mask[WPL];   // bytes of this lane's words that hold values
+#pragma unroll
+  for (int i = 0; i < WPL; ++i) {
+    const int left = d - 4 * (li + L * i);
+    mask[i] = left >= 4 ? 0xffffffffu : (left <= 0 ? 0u : 0xffffffffu >> (8 * (4 - left)));
+  }
+  uint32_t sel[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) sel[b] = exp_sel(cp, b);
+  const uint32_t tab_lane = (uint32_t)__cvta_generic_to_shared(sm_tab) + 4u * (unsigned)(lane & (cp - 1));
+  const unsigned top = (unsigned)p.I0 << p.N;
+  const int osh = 14 - p.k_out, omax = (1 << (p.k_out - 1)) - 1;
+  const int rnd = FROM_I32 && FAST ? 1 << (ld.pre_s - 33) : 0, sh = ld.pre_s - 32;
+  pdl_wait();
+  const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), stride = (int)((gridDim.x * blockDim.x) >> 5) * G;
+  for (int r0 = warp * G; r0 < rows; r0 += stride) {
+    const bool row_ok = r0 + grp < rows;
+    const int r = row_ok ? r0 + grp : rows - 1;   // (a row past the end repeats the last one, not stored)
+    uint32_t x[WPL];
+    if (FROM_I32) {
+      const int4* src = reinterpret_cast<const int4*>((const int32_t*)ld.in + (int64_t)r * ld.ldin) + li;
+      int4 a[WPL];
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) a[i] = li + L * i < nwords ? __ldg(src + L * i) : make_int4(0, 0, 0, 0);
+      if (ld.bias32) {
+        const int4* bs = reinterpret_cast<const int4*>(ld.bias32 + (int64_t)((unsigned)r % (unsigned)ld.bias_rows) * ld.ldbias) + li;
+#pragma unroll
+        for (int i = 0; i < WPL; ++i)
+          if (li + L * i < nwords) {
+            const int4 b = __ldg(bs + L * i);
+            a[i].x += b.x; a[i].y += b.y; a[i].z += b.z; a[i].w += b.w;
+          }
+      }
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) {
+        int v[4] = {a[i].x, a[i].y, a[i].z, a[i].w};
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          if (FAST) {
+            asm("mad.hi.s32 %0, %0, %1, %2;" : "+r"(v[b]) : "r"(ld.pre_m), "r"(rnd));
+            v[b] >>= sh;
+          } else {
+            v[b] = rq(v[b], ld.pre_m, ld.pre_s);
+          }
+        }
+        x[i] = pack_sat8_u(v[0], v[1], v[2], v[3]);
+      }
+    } else {
+      const uint32_t* src = reinterpret_cast<const uint32_t*>((const int8_t*)ld.in + (int64_t)r * ld.ldin) + li;
+#pragma unroll
+      for (int i = 0; i < WPL; ++i) x[i] = li + L * i < nwords ? __ldg(src + L * i) : 0u;
+    }
+    // row maximum: pairs of 16-bit values whose upper bytes are bytes 3 and 1, or 2 and 0 (the lower bytes only break ties)
+    unsigned m31 = 0x80808080u, m20 = 0x80808080u;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+      x[i] = (x[i] & mask[i]) | (0x80808080u & ~mask[i]);
+      m31 = __vmaxs2(m31, x[i]);
+      m20 = __vmaxs2(m20, x[i] << 8);
+    }
+    const unsigned m = __vmaxs2(m31, m20);
+    int mx = max((int)m >> 24, (int)(m << 16) >> 24);
+    if (L == 32) {
+      mx = __reduce_max_sync(0xffffffffu, mx);
+    } else {
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    // ShiftExp(I - I_max), row sum
+    const uint32_t tmx = tab_lane + (uint32_t)(4 * cp * mx);
+    unsigned e[WPL][4], sum = 0;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+#pragma unroll
+      for (int b = 0; b < 4; ++b) e[i][b] = exp_entry(x[i], sel[b], tmx);
+      sum += (e[i][0] + e[i][1]) + (e[i][2] + e[i][3]);
+    }
+    if (L == 32) {
+      sum = __reduce_add_sync(0xffffffffu, sum);
+    } else {
+#pragma unroll
+      for (int o = L / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    sum -= (unsigned)(4 * L * WPL - d) * exp_entry(0x80u, sel[0], tmx);
+    // Eq. (IntDiv) with M = 45
+    const unsigned factor = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)sum);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(out + (int64_t)r * ldout) + li;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) {
+      uint32_t o;
+      if (FAST) {
+        o = prob_word8(factor, (int)e[i][0], (int)e[i][1], (int)e[i][2], (int)e[i][3]);
+      } else {
+        int q[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) q[b] = min((int)(__umulhi(factor, e[i][b]) >> osh), omax);
+        o = pack_sat8_u(q[0], q[1], q[2], q[3]);
+      }
+      if (row_ok && li + L * i < nwords_out) dst[L * i] = o & mask[i];
+    }
+  }
+}
+
+// Any d: the row is read again for each pass.  Bytes are handled as biased values u = x + 128 (x ^ 0x80): one byte permute
+// yields the table index, ShiftExp(x - max) = tab[(max + 128) - u].  Positions past d hold u = 0 (x = -128).
+template <bool FROM_I32>
 __global__ void __launch_bounds__(256) shiftmax_kernel(RowLoader<FROM_I32> ld, ivit_exp_params p,
                                                        int8_t* __restrict__ out, int64_t ldout,
                                                        int64_t rows, int d) {
@@ -438,113 +560,97 @@ __global__ void __launch_bounds__(256) shiftmax_kernel(RowLoader<FROM_I32> ld, i
   const int nwords = (d + 3) >> 2;
   const int nwords_out = ((d + 15) >> 4) << 2;  // zero-fill up to the next multiple of 16
   const int npad = nwords * 4 - d;              // bytes past d in the last word
-  constexpr int W = WPL > 0 ? WPL : 1;
-  constexpr int R = WPL > 0 ? ROWS : 1;         // rows a warp works on together (their reciprocals in parallel lanes)
-  const int iters = WPL > 0 ? WPL : (nwords_out + 31) / 32;
-  // biased word idx of row r: bytes past d (and whole words past the row) read as 0
-  auto load_biased = [&](int64_t r, int idx) -> unsigned {
-    if (idx >= nwords) return 0u;
-    unsigned v = (unsigned)ld.load(r, idx) ^ 0x80808080u;
-    if (idx == nwords - 1 && npad) v &= 0xffffffffu >> (8 * npad);
-    return v;
-  };
-  for (int64_t r0 = warp * R; r0 < rows; r0 += nwarps * R) {
-    unsigned e[R][W][4];
-    unsigned my_sum = 1, my_mxu = 0;
-#pragma unroll
-    for (int q = 0; q < R; ++q) {
-      const int64_t r = r0 + q < rows ? r0 + q : rows - 1;   // a row past the end repeats the last one (not stored)
-      unsigned w[W];
-      // pass 1: row max
-      unsigned mxu = 0;
-#pragma unroll
-      for (int i = 0; i < iters; ++i) {
-        const unsigned v = load_biased(r, lane + 32 * i);
-        if (WPL > 0) w[i] = v;
-        mxu = max(max(mxu, __byte_perm(v, 0, 0x4440)), max(__byte_perm(v, 0, 0x4441), max(__byte_perm(v, 0, 0x4442), v >> 24)));
-      }
-      mxu = __reduce_max_sync(0xffffffffu, mxu);   // biased maximum = I_max + 128
-      // pass 2: sum of ShiftExp(I - I_max): entry (I_max + 128) - u
-      const uint8_t* tmx = reinterpret_cast<const uint8_t*>(exp_tab) + 4 * mxu;
-      unsigned sum = 0;
-#pragma unroll
-      for (int i = 0; i < iters; ++i) {
-        const unsigned v = WPL > 0 ? w[i] : load_biased(r, lane + 32 * i);
-        unsigned e0 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4440));
-        unsigned e1 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4441));
-        unsigned e2 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4442));
-        unsigned e3 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)(v >> 24));
-        if (WPL > 0) { e[q][i][0] = e0; e[q][i][1] = e1; e[q][i][2] = e2; e[q][i][3] = e3; }
-        sum += (e0 + e1) + (e2 + e3);
-      }
-      sum = __reduce_add_sync(0xffffffffu, sum);
-      // every position past d of the 32 * iters words counted exp_tab[I_max + 128]: take them out
-      sum -= (unsigned)(32 * iters * 4 - d) * exp_tab[mxu];
-      if (lane == q) { my_sum = sum; my_mxu = mxu; }
+  const int iters = (nwords_out + 31) / 32;
+  const int osh = 14 - p.k_out, omax = (1 << (p.k_out - 1)) - 1;
+  for (int64_t r = warp; r < rows; r += nwarps) {
+    // biased word idx of the row: bytes past d (and whole words past the row) read as 0
+    auto load_biased = [&](int idx) -> unsigned {
+      if (idx >= nwords) return 0u;
+      unsigned v = (unsigned)ld.load(r, idx) ^ 0x80808080u;
+      if (idx == nwords - 1 && npad) v &= 0xffffffffu >> (8 * npad);
+      return v;
+    };
+    unsigned mxu = 0;
+    for (int i = 0; i < iters; ++i) {
+      const unsigned v = load_biased(lane + 32 * i);
+      mxu = max(max(mxu, __byte_perm(v, 0, 0x4440)), max(__byte_perm(v, 0, 0x4441), max(__byte_perm(v, 0, 0x4442), v >> 24)));
     }
-    // Eq. (IntDiv): one reciprocal per row (lane q for row q), M = 45:
-    // (floor(2^45 / sum) * e) >> (45 - (k_out - 1)) == umulhi(factor, e) >> (14 - k_out) since factor <= 2^31.
-    const unsigned my_factor = (unsigned)((1ull << 45) / (unsigned long long)my_sum);
-    const int osh = 14 - p.k_out;
-    const int omax = (1 << (p.k_out - 1)) - 1;   // the one possible 2^(k_out-1) is clamped
+    mxu = __reduce_max_sync(0xffffffffu, mxu);   // biased maximum = I_max + 128
+    const uint8_t* tmx = reinterpret_cast<const uint8_t*>(exp_tab) + 4 * mxu;
+    auto entries = [&](unsigned v, unsigned (&e)[4]) {
 #pragma unroll
-    for (int q = 0; q < R; ++q) {
-      const unsigned factor = __shfl_sync(0xffffffffu, my_factor, q);
-      const unsigned mxu = __shfl_sync(0xffffffffu, my_mxu, q);
-      const int64_t r = r0 + q;
-      if (r >= rows) break;
-      const uint8_t* tmx = reinterpret_cast<const uint8_t*>(exp_tab) + 4 * mxu;
-      int* dst = reinterpret_cast<int*>(out + r * ldout);
-#pragma unroll
-      for (int i = 0; i < iters; ++i) {
-        const int idx = lane + 32 * i;
-        if (idx < nwords_out) {
-          unsigned e0, e1, e2, e3;
-          if (WPL > 0) {
-            e0 = e[q][i][0]; e1 = e[q][i][1]; e2 = e[q][i][2]; e3 = e[q][i][3];
-          } else {
-            const unsigned v = load_biased(r, idx);
-            e0 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4440));
-            e1 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4441));
-            e2 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4442));
-            e3 = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)(v >> 24));
-          }
-          unsigned packed = pack_sat8_u(min((int)(__umulhi(factor, e0) >> osh), omax), min((int)(__umulhi(factor, e1) >> osh), omax),
-                                        min((int)(__umulhi(factor, e2) >> osh), omax), min((int)(__umulhi(factor, e3) >> osh), omax));
-          // positions past d are written as zero
-          if (idx >= nwords) packed = 0;
-          else if (idx == nwords - 1 && npad) packed &= 0xffffffffu >> (8 * npad);
-          dst[idx] = (int)packed;
-        }
-      }
+      for (int b = 0; b < 4; ++b) e[b] = *reinterpret_cast<const unsigned*>(tmx - 4 * (int)__byte_perm(v, 0, 0x4440 + b));
+    };
+    unsigned sum = 0;
+    for (int i = 0; i < iters; ++i) {
+      unsigned e[4];
+      entries(load_biased(lane + 32 * i), e);
+      sum += (e[0] + e[1]) + (e[2] + e[3]);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    // every position past d of the 32 * iters words counted exp_tab[I_max + 128]: take them out
+    sum -= (unsigned)(32 * iters * 4 - d) * exp_tab[mxu];
+    // Eq. (IntDiv) with M = 45: (floor(2^45 / sum) * e) >> (45 - (k_out - 1)) == umulhi(factor, e) >> (14 - k_out)
+    const unsigned factor = (unsigned)((1ull << 45) / (unsigned long long)sum);
+    int* dst = reinterpret_cast<int*>(out + r * ldout);
+    for (int i = 0; i < iters; ++i) {
+      const int idx = lane + 32 * i;
+      if (idx >= nwords_out) break;
+      unsigned e[4];
+      entries(load_biased(idx), e);
+      unsigned packed = pack_sat8_u(min((int)(__umulhi(factor, e[0]) >> osh), omax), min((int)(__umulhi(factor, e[1]) >> osh), omax),
+                                    min((int)(__umulhi(factor, e[2]) >> osh), omax), min((int)(__umulhi(factor, e[3]) >> osh), omax));
+      if (idx >= nwords) packed = 0;
+      else if (idx == nwords - 1 && npad) packed &= 0xffffffffu >> (8 * npad);
+      dst[idx] = (int)packed;
     }
   }
 }
 
 template <bool FROM_I32>
-static void shiftmax_dispatch(RowLoader<FROM_I32> ld, ivit_exp_params p, int8_t* out, int64_t ldout,
-                              int64_t rows, int d, int grid, cudaStream_t st) {
-  const int wpl = (((d + 15) / 16) * 4 + 31) / 32;
-  if (wpl <= 2) launch_k(shiftmax_kernel<2, 4, FROM_I32>, dim3(grid), dim3(256), 0, st, ld, p, out, ldout, rows, d);
-  else if (wpl <= 5) launch_k(shiftmax_kernel<5, 2, FROM_I32>, dim3(grid), dim3(256), 0, st, ld, p, out, ldout, rows, d);
-  else if (wpl <= 8) launch_k(shiftmax_kernel<8, 1, FROM_I32>, dim3(grid), dim3(256), 0, st, ld, p, out, ldout, rows, d);
-  else if (wpl <= 16) launch_k(shiftmax_kernel<16, 1, FROM_I32>, dim3(grid), dim3(256), 0, st, ld, p, out, ldout, rows, d);
-  else launch_k(shiftmax_kernel<0, 1, FROM_I32>, dim3(grid), dim3(256), 0, st, ld, p, out, ldout, rows, d);
+static void shiftmax_dispatch(ivit_ctx* ctx, RowLoader<FROM_I32> ld, ivit_exp_params p, int8_t* out, int64_t ldout,
+                              int64_t rows, int d) {
+  const int words = (d + 15) / 16 * 4;
+  if (words > 512 || rows >= (1ll << 31) - (1 << 20) || (FROM_I32 && ld.bias_rows >= (1ll << 31))) {
+    const int64_t want = (rows + 7) / 8, cap = (int64_t)ctx->sm_count * 8;
+    launch_k(shiftmax_kernel<FROM_I32>, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, ctx->stream, ld, p, out, ldout, rows, d);
+    return;
+  }
+  const bool fast = p.k_out == 8 && ((int64_t)p.I0 << p.N) > (1 << 15) && (!FROM_I32 || ld.pre_s >= 33);
+  // G rows per warp.  Two blocks of sixteen warps per SM with a table copy per lane; few rows: small blocks on more SMs and
+  // fewer copies to build.
+  auto run = [&](auto kernel, int G) {
+    const bool few = rows <= (int64_t)ctx->sm_count * 16 * G;
+    const int threads = few ? 128 : 512, cp = few ? 8 : 32;
+    const int64_t per_block = (int64_t)(threads / 32) * G, want = (rows + per_block - 1) / per_block, cap = (int64_t)ctx->sm_count * (few ? 8 : (words > 256 ? 1 : 2));
+    launch_k(kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(threads), (size_t)(1024 * cp + 512), ctx->stream, ld, p, cp, out, ldout,
+             (int)rows, d);
+  };
+  auto pick = [&](auto f) {
+    constexpr bool F = decltype(f)::value;
+    if (words <= 16) run(shiftmax_rows_kernel<8, 2, FROM_I32, F>, 4);
+    else if (words <= 32) run(shiftmax_rows_kernel<8, 4, FROM_I32, F>, 4);
+    else if (words <= 56) run(shiftmax_rows_kernel<8, 7, FROM_I32, F>, 4);
+    else if (words <= 96) run(shiftmax_rows_kernel<16, 6, FROM_I32, F>, 2);
+    else if (words <= 160) run(shiftmax_rows_kernel<32, 5, FROM_I32, F>, 1);
+    else if (words <= 256) run(shiftmax_rows_kernel<32, 8, FROM_I32, F>, 1);
+    else run(shiftmax_rows_kernel<32, 16, FROM_I32, F>, 1);
+  };
+  if (fast) pick(std::true_type{});
+  else pick(std::false_type{});
 }
 
 int launch_shiftmax(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, const int32_t* bias32,
                     int64_t ldbias, int64_t bias_rows, ScaleDev pre, ivit_exp_params p, int8_t* out,
                     int64_t ldout, int64_t rows, int64_t d) {
   if (rows == 0) return IVIT_OK;
-  const int64_t want = (rows + 7) / 8;
-  const int grid = (int)(want < (int64_t)ctx->sm_count * 8 ? want : (int64_t)ctx->sm_count * 8);
   LaunchScope ls(ctx, KIND_SHIFTMAX, (double)rows * (double)d * (in_dtype == IVIT_I32 ? 5.0 : 2.0));
   if (in_dtype == IVIT_I8) {
     RowLoader<false> ld{in, ldin, nullptr, 0, 1, 0, 1};
-    shiftmax_dispatch<false>(ld, p, out, ldout, rows, (int)d, grid, ctx->stream);
+    shiftmax_dispatch<false>(ctx, ld, p, out, ldout, rows, (int)d);
   } else {
     RowLoader<true> ld{in, ldin, bias32, ldbias, bias_rows < 1 ? 1 : bias_rows, pre.mult, clamp_shift(pre.shift)};
-    shiftmax_dispatch<true>(ld, p, out, ldout, rows, (int)d, grid, ctx->stream);
+    shiftmax_dispatch<true>(ctx, ld, p, out, ldout, rows, (int)d);
   }
   return ls.done();
 }

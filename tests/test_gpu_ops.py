@@ -554,3 +554,27 @@ def test_layernorm_row_counts_and_forms(C):
             got = c.layernorm(g.dev(x), g.binding.DevScale(sc, "cuda"), None if b is None else torch.from_numpy(b).cuda(), 20)
             g.assert_equal(g.host(got), O.layernorm(x, sc, b, 20), f"rows={rows} C={C}")
     assert c.poll_status() == 0
+
+
+@pytest.mark.parametrize("d", [64, 65, 128, 129, 224, 225, 384, 385, 640, 641, 1024, 1025, 2048, 2049])
+def test_shiftmax_row_forms(d):
+    """Both sides of every row width at which the lanes are shared out differently; one row, an odd number, more than a
+    wave of blocks; int8 and int32 input, with and without bias, shifts below 33, k_out below 8, and I0 = 16 (the largest
+    exponential is a power of two) with rows whose maximum stands alone: probability 128, clamped to 127."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(d)
+    pre, low = Scale(*dyadic(30.0 / 8192.0)), Scale(*dyadic(0.3))
+    for rows, p in ((1, ExpParams(17, 15)), (77, ExpParams(16, 15)), (2501 if d > 700 else 10001, ExpParams(23, 15)), (33, ExpParams(13, 15, 45, 6))):
+        x = rand_i8(rng, (rows, d), std=30)
+        x[::3] = -100
+        x[::3, d // 2] = 100                     # a lone maximum
+        g.assert_equal(g.host(c.shiftmax(g.dev(x), p)), O.shiftmax(x, p), f"int8 rows={rows}")
+        x32 = np.rint(rng.standard_normal((rows, d)) * 8192).astype(np.int32)
+        x32[::3, 0] = 1 << 19
+        bias = np.rint(rng.standard_normal((5, d)) * 2000).astype(np.int32)
+        for sc, b in ((pre, None), (pre, bias), (low, None)):
+            y = x32 if sc is pre else x32 // 200
+            got = c.shiftmax(g.dev(y, 4), p, pre=g.binding.DevScale(sc, "cuda"), bias32=None if b is None else g.dev(b, 4))
+            g.assert_equal(g.host(got), O.shiftmax(y, p, pre=sc, bias32=b), f"int32 rows={rows} bias={b is not None}")
+    assert c.poll_status() == 0
