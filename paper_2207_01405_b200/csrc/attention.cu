@@ -73,9 +73,13 @@ struct __align__(16) AttnItem {
   }
 };
 
-// Tile load; pos: which coordinate of the map (1..3) carries the row, the head and the image or window.
+// Named barriers: id, number of threads that arrive or wait.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+// Tile load by a converged warp; pos: which coordinate of the map (1..3) carries the row, the head and the image or window.
 __device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, const int (&pos)[3], int row, int h, int b) {
-  tma_load_4d(dst, map, bar, 0, pos[0] == 1 ? row : (pos[1] == 1 ? h : b), pos[0] == 2 ? row : (pos[1] == 2 ? h : b),
+  tma_load_4d_w(dst, map, bar, 0, pos[0] == 1 ? row : (pos[1] == 1 ? h : b), pos[0] == 2 ? row : (pos[1] == 2 ? h : b),
               pos[0] == 3 ? row : (pos[1] == 3 ? h : b));
 }
 
@@ -179,18 +183,20 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
   const uint32_t bar_qk = base + bar_off, bar_v = bar_qk + 8, bar_s = bar_qk + 16, bar_p = bar_qk + 24,
                  bar_o = bar_qk + 32, bar_e = bar_qk + 40;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 48);
+  volatile uint32_t* dead = tmem_slot + 1;               // set when a wait of the control warp ran out
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     prefetch_tmap(&tmQ);
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
     mbar_init(bar_qk, 1);
     mbar_init(bar_v, 1);
-    mbar_init(bar_s, 2);      // the MMAs, and the control thread (the item is in the ring)
+    mbar_init(bar_s, 1);
     mbar_init(bar_p, 8);
     mbar_init(bar_o, 1);
     mbar_init(bar_e, 8);
+    *dead = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
@@ -198,7 +204,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   pdl_trigger();
   // items of this CTA: a snake over all of them, or (kPack) a contiguous range
   const uint32_t rounds = (uint32_t)a.items / gridDim.x, left = (uint32_t)a.items % gridDim.x;
@@ -208,7 +214,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
 
   if (warp == 0) {
     pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
-    if (lane == 0 && n_items > 0) {
+    if (n_items > 0) {
       auto item_at = [&](AttnItem& it, uint32_t n) {
         if (kPack) {
           const unsigned t = first + n, grp = t / imgs, img = t - grp * imgs;
@@ -221,7 +227,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
         }
       };
       auto load_qk = [&](const AttnItem& it) {
-        mbar_expect_tx(bar_qk, 128u * a.d + k_bytes);
+        mbar_expect_tx_w(bar_qk, 128u * a.d + k_bytes);
         if (kPack) {
           load_box(base, &tmQ, bar_qk, a.q_pos, 0, it.h, it.b);
         } else {
@@ -231,7 +237,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
         load_box(base + k_off, &tmK, bar_qk, a.k_pos, 0, it.h, it.b);
       };
       auto load_v = [&](const AttnItem& it) {
-        mbar_expect_tx(bar_v, v_bytes);
+        mbar_expect_tx_w(bar_v, v_bytes);
         load_box(base + v_off, &tmV, bar_v, a.v_pos, 0, it.h, it.b);
       };
       // descriptor words: rows of d bytes (Q, K, V: swizzled over their width) or 128 bytes (P)
@@ -251,46 +257,62 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
       load_qk(cur);
       load_v(cur);
       bool ok = true;
+      bool scores_out = false;
+      uint32_t done = 0;                // items whose output is there
       for (uint32_t n = 0; n < n_items; ++n) {
         const uint32_t par = n & 1u;
-        ok = mbar_wait(bar_qk, par, a.status);
+        ok = mbar_wait_warp(bar_qk, par, a.status);
         qk_flying = !ok;
         // the output of the previous item must have left tensor memory
-        if (ok && n > 0) ok = mbar_wait(bar_e, par ^ 1u, a.status);
+        if (ok && n > 0) ok = mbar_wait_warp(bar_e, par ^ 1u, a.status);
         if (!ok) break;
-        item_ring[par] = cur;
+        if (lane == 0) item_ring[par] = cur;
         tc_fence_after();
         for (int k = 0; k < ks; ++k)
-          umma_i8_lohi(tmem, q_lo + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
-        umma_commit(bar_s);
-        mbar_arrive(bar_s);   // releases the item written to the ring
+          umma_i8_lohi_w(tmem, q_lo + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
+        umma_commit_w(bar_s);
         const bool more = n + 1 < n_items;
         if (more) item_at(next, n + 1);
         // Q and K may be overwritten once the score MMAs have read them
-        ok = mbar_wait(bar_s, par, a.status);
+        ok = mbar_wait_warp(bar_s, par, a.status);
         if (!ok) break;
+        bar_arrive(6, kShortThreads);   // scores and item are there
+        scores_out = true;
         if (more) { load_qk(next); qk_flying = true; qk_par = par ^ 1u; }
         // O = P V once the probabilities are in shared memory and V has landed
-        ok = mbar_wait(bar_p, par, a.status);
-        if (ok) { ok = mbar_wait(bar_v, par, a.status); v_flying = !ok; }
+        ok = mbar_wait_warp(bar_p, par, a.status);
+        if (ok) { ok = mbar_wait_warp(bar_v, par, a.status); v_flying = !ok; }
         if (!ok) break;
         tc_fence_after();
         uint32_t p_lo = p_lo0, v_lo = v_lo0;
         int k = 0;
         for (; k + 4 <= ks2; k += 4, p_lo += (128 * 128) >> 4, v_lo += 4 * v_step)
-          umma_i8_x4(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
+          umma_i8_x4_w(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
         for (; k < ks2; ++k, p_lo += UK >> 4, v_lo += v_step)
-          umma_i8_lohi(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
-        umma_commit(bar_o);
+          umma_i8_lohi_w(tmem, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
+        umma_commit_w(bar_o);
         // V may be overwritten once these MMAs have read it
-        ok = mbar_wait(bar_o, par, a.status);
+        ok = mbar_wait_warp(bar_o, par, a.status);
         if (!ok) break;
+        bar_arrive(7, kShortThreads);   // the output is there
+        ++done;
+        scores_out = false;
         if (more) { load_v(next); v_flying = true; v_par = par ^ 1u; }
         cur = next;
       }
-      // nothing may be in flight at exit (after a wait that timed out)
-      if (qk_flying) mbar_wait(bar_qk, qk_par, a.status);
-      if (v_flying) mbar_wait(bar_v, v_par, a.status);
+      if (!ok) {
+        // A wait ran out: the Shiftmax threads, told by the flag, walk on through their barriers without work.  (`done`
+        // items have been released twice; of the one at which the wait ran out the scores may have been released.)
+        if (lane == 0) *dead = 1;
+        __syncwarp();
+        for (uint32_t n = done; n < n_items; ++n) {
+          if (n > done || !scores_out) bar_arrive(6, kShortThreads);
+          bar_arrive(7, kShortThreads);
+        }
+      }
+      // nothing may be in flight at exit
+      if (qk_flying) mbar_wait_warp(bar_qk, qk_par, a.status);
+      if (v_flying) mbar_wait_warp(bar_v, v_par, a.status);
     }
   } else {
     // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the two warps of a quarter take the even / odd
@@ -325,10 +347,13 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
     uint32_t img = kPack ? first % imgs : 0u;   // kPack: items with the present bias that are behind
     asm volatile("bar.sync 1, 256;" ::: "memory");   // the table is complete
 
-    bool alive = true;   // false after a wait that timed out: no more waits, no more work, only the barriers
+    bool alive = true;   // false after a wait of the control warp timed out: no more work, only the barriers
     for (uint32_t n = 0; n < n_items; ++n) {
       const uint32_t par = n & 1u;
-      alive = alive && mbar_wait(bar_s, par, a.status);
+      // The control warp alone polls the barriers of the MMAs; the others wait in hardware barriers (eight polling warps
+      // per CTA issued a third of the kernel's instructions).
+      bar_sync(6, kShortThreads);
+      alive = *dead == 0;
       const AttnItem item = item_ring[par];
       const int b = kPack ? item.b + slot : item.b;          // image / window of this row
       const int m0 = kPack ? qd * 32 - slot * sa.R : item.m0 + ((qd - item.rot) & 3) * 32;   // first row (token) of this lane quarter
@@ -474,7 +499,8 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);
       // ---- output, heads concatenated along the feature dimension ----
-      alive = alive && mbar_wait(bar_o, par, a.status);
+      bar_sync(7, kShortThreads);
+      alive = alive && *dead == 0;
       if (work && alive) {
         tc_fence_after();
         int8_t* orow = a.O + ((int64_t)b * a.T + r) * a.D + (int64_t)item.h * a.d;
@@ -551,7 +577,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
                  bar_p = bar_q + 64, bar_o = bar_q + 72;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen + bar_off + 80);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     prefetch_tmap(&tmQ);
     prefetch_tmap(&tmK);
@@ -572,7 +598,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t o_col = 2u * (uint32_t)ra.wb;
   pdl_trigger();
   const int nblk = ra.nblk;
@@ -581,14 +607,14 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
   if (warp < kRowsFirst) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     if (warp == 0) pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
-    if (warp == 0 && lane == 0 && n_items > 0) {
+    if (warp == 0 && n_items > 0) {
       auto load_q = [&](const AttnItem& it) {
-        mbar_expect_tx(bar_q, 128u * a.d);
+        mbar_expect_tx_w(bar_q, 128u * a.d);
         for (int g = 0; g < 4; ++g)
           load_box(base + (uint32_t)((g + it.rot) & 3) * 32u * a.d, &tmQ, bar_q, a.q_pos, it.m0 + 32 * g, it.h, it.b);
       };
       auto load_v = [&](const AttnItem& it) {
-        mbar_expect_tx(bar_v, v_bytes);
+        mbar_expect_tx_w(bar_v, v_bytes);
         for (int i = 0; i < ra.nv; ++i)
           load_box(base + v_off + (uint32_t)(i * ra.vbox) * a.d, &tmV, bar_v, a.v_pos, i * ra.vbox, it.h, it.b);
       };
@@ -607,9 +633,9 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
       auto load_k = [&](const AttnItem& it, int j) {
         const uint32_t buf = gk & 1u, ph = (gk >> 1) & 1u;
         // the MMAs of the block two before this one have read the buffer
-        if (gk >= 2) ok = mbar_wait(bar_s + 8 * buf, ph ^ 1u, a.status);
+        if (gk >= 2) ok = mbar_wait_warp(bar_s + 8 * buf, ph ^ 1u, a.status);
         if (!ok) return;
-        mbar_expect_tx(bar_k + 8 * buf, kbuf_bytes);
+        mbar_expect_tx_w(bar_k + 8 * buf, kbuf_bytes);
         load_box(base + k_off + buf * kbuf_bytes, &tmK, bar_k + 8 * buf, a.k_pos, j * (16 * kBlkChunks), it.h, it.b);
         k_fly[buf] = true;
         k_par[buf] = ph;
@@ -618,22 +644,23 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
       // S_buf = Q K_j^T for key block j of the n-th item of this CTA
       auto issue_block = [&](const AttnItem& it, int j, uint32_t n) {
         const uint32_t buf = g & 1u, ph = (g >> 1) & 1u;
-        ok = mbar_wait(bar_k + 8 * buf, ph, a.status);
+        ok = mbar_wait_warp(bar_k + 8 * buf, ph, a.status);
         k_fly[buf] = !ok;
-        if (ok && j == 0) { ok = mbar_wait(bar_q, n & 1u, a.status); q_fly = !ok; }
+        if (ok && j == 0) { ok = mbar_wait_warp(bar_q, n & 1u, a.status); q_fly = !ok; }
         // pass A of the block that used this score buffer two blocks ago has read it.  (With it every Shiftmax thread is
         // past item n - 2, whose place in the ring item n takes: nblk >= 2.)
-        if (ok && g >= 2) ok = mbar_wait(bar_f + 8 * buf, ph ^ 1u, a.status);
+        if (ok && g >= 2) ok = mbar_wait_warp(bar_f + 8 * buf, ph ^ 1u, a.status);
         if (!ok) return;
-        if (j == 0) item_ring[n & 1u] = it;
+        if (j == 0 && lane == 0) item_ring[n & 1u] = it;
         tc_fence_after();
         const int w = j == nblk - 1 ? 16 * a.chunks - j * 16 * kBlkChunks : 16 * kBlkChunks;
         const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(w >> 3) << 17) | (8u << 24);
         const uint32_t k_lo = k_lo0 + buf * (kbuf_bytes >> 4), d_tmem = tmem + buf * (uint32_t)ra.wb;
         for (int k = 0; k < ks; ++k)
-          umma_i8_lohi(d_tmem, q_lo0 + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
-        umma_commit(bar_s + 8 * buf);
-        mbar_arrive(bar_s + 8 * buf);   // releases the item written to the ring
+          umma_i8_lohi_w(d_tmem, q_lo0 + k * (UK >> 4), row_hi, k_lo + k * (UK >> 4), row_hi, idesc, k != 0);
+        umma_commit_w(bar_s + 8 * buf);
+        if (lane == 0) mbar_arrive(bar_s + 8 * buf);   // releases the item written to the ring
+        __syncwarp();
         ++g;
       };
 
@@ -657,7 +684,7 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
         if (!ok) break;
         if (more) {
           // Q may be overwritten once the score MMAs of the last block have read it
-          ok = mbar_wait(bar_s + 8 * ((g - 1) & 1u), ((g - 1) >> 1) & 1u, a.status);
+          ok = mbar_wait_warp(bar_s + 8 * ((g - 1) & 1u), ((g - 1) >> 1) & 1u, a.status);
           if (!ok) break;
           load_q(next); q_fly = true; q_par = (n + 1) & 1u;
           issue_block(next, 0, n + 1);
@@ -666,28 +693,28 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
         }
         // O = P V once the probabilities are in shared memory (every warp has then read the previous output too)
         // and V has landed
-        ok = mbar_wait(bar_p, n & 1u, a.status);
-        if (ok) { ok = mbar_wait(bar_v, n & 1u, a.status); v_fly = !ok; }
+        ok = mbar_wait_warp(bar_p, n & 1u, a.status);
+        if (ok) { ok = mbar_wait_warp(bar_v, n & 1u, a.status); v_fly = !ok; }
         if (!ok) break;
         tc_fence_after();
         uint32_t p_lo = p_lo0 + (n & 1u) * (ra.p_stride >> 4), v_lo = v_lo0;
         int k = 0;
         for (; k + 4 <= ks2; k += 4, p_lo += (128 * 128) >> 4, v_lo += 4 * v_step)
-          umma_i8_x4(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
+          umma_i8_x4_w(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0, UK >> 4, v_step);
         for (; k < ks2; ++k, p_lo += UK >> 4, v_lo += v_step)
-          umma_i8_lohi(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
-        umma_commit(bar_o);
+          umma_i8_lohi_w(tmem + o_col, p_lo, p_hi, v_lo, row_hi, idesc2, k != 0);
+        umma_commit_w(bar_o);
         // V may be overwritten once these MMAs have read it
-        ok = mbar_wait(bar_o, n & 1u, a.status);
+        ok = mbar_wait_warp(bar_o, n & 1u, a.status);
         if (!ok) break;
         if (more) { load_v(next); v_fly = true; v_par = (n + 1) & 1u; }
         cur = next;
       }
       // end of work (or a wait that timed out): nothing may be in flight at exit
-      if (q_fly) mbar_wait(bar_q, q_par, a.status);
-      if (v_fly) mbar_wait(bar_v, v_par, a.status);
+      if (q_fly) mbar_wait_warp(bar_q, q_par, a.status);
+      if (v_fly) mbar_wait_warp(bar_v, v_par, a.status);
       for (int i = 0; i < 2; ++i)
-        if (k_fly[i]) mbar_wait(bar_k + 8 * i, k_par[i], a.status);
+        if (k_fly[i]) mbar_wait_warp(bar_k + 8 * i, k_par[i], a.status);
     }
   } else {
     // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the four warps of a quarter share its 32 rows

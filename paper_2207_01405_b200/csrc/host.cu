@@ -401,16 +401,19 @@ int ivit_ctx_create(ivit_ctx** out, int device, void* cuda_stream) {
   *out = nullptr;
   int count = 0;
   if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) return IVIT_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return IVIT_ERR_CUDA;
-  if (prop.major != 10) return IVIT_ERR_CUDA;  // kernels are built for sm_100a only
+  // (single attributes: the whole property structure takes milliseconds to fill)
+  int major = 0, sms = 0;
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
+    return IVIT_ERR_CUDA;
+  if (major != 10) return IVIT_ERR_CUDA;  // kernels are built for sm_100a only
   if (cudaSetDevice(device) != cudaSuccess) return IVIT_ERR_CUDA;
   ivit_ctx* c = new (std::nothrow) ivit_ctx();
   if (!c) return IVIT_ERR_CUDA;
   std::memset(c, 0, sizeof(*c));
   c->device = device;
   c->stream = (cudaStream_t)cuda_stream;
-  c->sm_count = prop.multiProcessorCount;
+  c->sm_count = sms;
   if (cudaHostAlloc((void**)&c->status_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess) { delete c; return IVIT_ERR_CUDA; }
   *c->status_host = 0;
   if (cudaHostGetDevicePointer((void**)&c->status_dev, c->status_host, 0) != cudaSuccess ||
