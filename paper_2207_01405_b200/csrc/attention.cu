@@ -135,35 +135,43 @@ __device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Rows of up to 256 tokens: a CTA of eight Shiftmax warps, two threads per score row (they take alternate 16-column
-// chunks), two or three CTAs per SM.  The CTAs of an SM are at different points of their items, which covers the waits
-// that an item cannot avoid (score MMAs, row exchanges, P V) and mixes passes that need different pipes.
-//   kPack = false  128 rows of one image
+// Rows of up to 256 tokens.  Several CTAs per SM: they are at different points of their items, which covers the waits that
+// an item cannot avoid (score MMAs, row exchanges, P V) and mixes passes that need different pipes.  Only the control
+// warp polls; the others wait in hardware barriers that it releases.
+//   kPack = false  128 rows of one image; two CTAs (tensor memory holds two score tiles of 256 columns), two threads per
+//                  score row, which take alternate 16-column chunks
 //   kPack = true   G windows of up to R = 128 / G tokens share the 128 rows (window attention): the score tile is
 //                  block-diagonal and the probabilities outside a row's own window stay 0.  The int32 score bias of
 //                  the tile's windows is kept in shared memory (rows padded to an odd number of words, so that the 32
 //                  rows of a warp fall into different banks) and only fetched when it differs from the last item's;
 //                  items are ordered so that it rarely does (per head and window position, images innermost).  Read
-//                  straight from global memory, one row per lane, it took most of the kernel's time.
+//                  straight from global memory, one row per lane, it took most of the kernel's time.  Four CTAs with a
+//                  thread per score row: no row exchange (4096 windows of 49 tokens, 6 heads of 32, bias: 113 us; two
+//                  CTAs with two threads per row 146, three 158).
 // Everything of an item stays in tensor memory: the score columns hold the packed int8 scores after pass A, the
 // exponentials after pass B, and O = P V at the end.
-// Measured, back to back (before: one table, items drawn from a counter, bias read from global memory):
-//   64 x 197 tokens, 6 heads of 64      29.0 -> 22.3 us        128 x 197, 12 heads of 64   89.1 -> 69.4 us
-//   4096 windows of 49, 3 heads, bias    125 -> 87.7 us        1 x 197, 3 heads            10.1 ->  7.2 us
-constexpr int kShortThreads = 288;   // warp 0: TMA + MMA issue + TMEM owner; warps 1..8: two threads per score row
+// Measured, back to back (before: one table, items drawn from a counter, bias read from global memory, every warp polling):
+// 64 x 197 tokens, 6 heads of 64 29.0 -> 19.5 us; 128 x 197, 12 heads 89.1 -> 61.7; 1 x 197, 3 heads 10.1 -> 5.9.
+// Threads per score row (TPR) and CTAs per SM.  Warp 0: TMA + MMA issue + TMEM owner; TPR warps per lane quarter.
+template <bool kPack>
+struct ShortShape {
+  static constexpr int TPR = kPack ? 1 : 2, kCtas = kPack ? 4 : 2, kWorkers = 128 * TPR, kThreads = 32 + kWorkers;
+};
 
 struct ShortArgs {
   AttnArgs a;
   int G, R, Btot;                   // kPack: windows per tile, rows per window slot, windows in the tensor
+  unsigned t_magic;                 // floor(2^32 / T) + 1
   int units, npos;                  // kPack: tiles per head; window-position groups with a bias of their own per head
   int tmem_cols;
 };
 
 template <bool kPack, bool FAST, bool BIAS>
-__global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_kernel(const __grid_constant__ CUtensorMap tmQ,
+__global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>::kCtas) attention_short_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                                        const __grid_constant__ CUtensorMap tmK,
                                                                                        const __grid_constant__ CUtensorMap tmV,
                                                                                        ShortArgs sa) {
+  constexpr int TPR = ShortShape<kPack>::TPR, kShortThreads = ShortShape<kPack>::kThreads, kWorkers = ShortShape<kPack>::kWorkers;
   const AttnArgs& a = sa.a;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -193,9 +201,9 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
     mbar_init(bar_qk, 1);
     mbar_init(bar_v, 1);
     mbar_init(bar_s, 1);
-    mbar_init(bar_p, 8);
+    mbar_init(bar_p, 4 * TPR);
     mbar_init(bar_o, 1);
-    mbar_init(bar_e, 8);
+    mbar_init(bar_e, 4 * TPR);
     *dead = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
@@ -321,9 +329,9 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
     const int qd = warp & 3;
     const int half = (warp - 1) >> 2;
     const int trow = qd * 32 + lane;              // row inside the tile
-    build_exp_table(a.smax.I0, a.smax.N, a.cp, gen + tab_off, st, 256);
+    build_exp_table(a.smax.I0, a.smax.N, a.cp, gen + tab_off, st, kWorkers);
     // probabilities that no item writes are 0: columns past the last chunk, other windows' columns
-    for (int c = (kPack ? 0 : a.chunks) + half; c < a.kpad / 16; c += 2)
+    for (int c = (kPack ? 0 : a.chunks) + half; c < a.kpad / 16; c += TPR)
       *reinterpret_cast<uint4*>(gen + p_off + (c >> 3) * (128 * 128) + trow * 128 + (((c & 7) ^ (trow & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
     unsigned* seeds = reinterpret_cast<unsigned*>(gen + seed_off);
     if (st < 128) seeds[st] = recip_seed(st);
@@ -340,12 +348,12 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
     // second thread (whose share is never the larger one) takes as a piece of eight or sixteen columns
     const int slot = kPack ? trow / sa.R : 0;
     const int c_lo = kPack ? slot * (sa.R >> 4) : 0, c_full = c_lo + (a.T >> 4);
-    const int rem = half == 1 ? a.T & 15 : 0;
+    const int rem = half == TPR - 1 ? a.T & 15 : 0;
     uint8_t* const p_row = gen + p_off + trow * 128;
     auto p_addr = [&](int c) { return reinterpret_cast<uint4*>(p_row + (c >> 3) * (128 * 128) + (((c & 7) ^ (trow & 7)) << 4)); };
     const int bias_ld = a.T | 1;
     uint32_t img = kPack ? first % imgs : 0u;   // kPack: items with the present bias that are behind
-    asm volatile("bar.sync 1, 256;" ::: "memory");   // the table is complete
+    bar_sync(1, kWorkers);   // the table is complete
 
     bool alive = true;   // false after a wait of the control warp timed out: no more work, only the barriers
     for (uint32_t n = 0; n < n_items; ++n) {
@@ -365,18 +373,23 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
         // (decided on the item's number alone: every thread takes the same branch)
         if (n == 0 || img == imgs) {
           if (img == imgs) img = 0;
-          asm volatile("bar.sync 1, 256;" ::: "memory");     // pass A of the last item is behind
+          bar_sync(1, kWorkers);     // pass A of the last item is behind
           for (int s = 0; alive && s < sa.G; ++s) {
             const int32_t* src = a.bias + (int64_t)((unsigned)((item.b + s) * a.heads + item.h) % (unsigned)a.bias_batches) * a.T * a.T;
             int* dst = reinterpret_cast<int*>(gen + bias_off) + s * a.T * bias_ld;
-            int rr = st / a.T, cc = st - rr * a.T;
-            for (int i = st; i < a.T * a.T; i += 256) {
-              dst[rr * bias_ld + cc] = __ldg(src + i);
-              cc += 256;
-              while (cc >= a.T) { cc -= a.T; ++rr; }
+            const int tt = a.T * a.T;
+            for (int i0 = st; i0 < tt; i0 += kWorkers * 8) {   // eight loads in flight
+              int v[8];
+#pragma unroll
+              for (int u = 0; u < 8; ++u) v[u] = i0 + kWorkers * u < tt ? __ldg(src + i0 + kWorkers * u) : 0;
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const unsigned i = (unsigned)(i0 + kWorkers * u), rr = __umulhi(i, sa.t_magic);   // i / T
+                if (i < (unsigned)tt) dst[rr * bias_ld + (i - rr * a.T)] = v[u];
+              }
             }
           }
-          asm volatile("bar.sync 1, 256;" ::: "memory");
+          bar_sync(1, kWorkers);
         }
         ++img;
         brow = reinterpret_cast<const int*>(gen + bias_off) + (slot * a.T + (row_ok ? r : 0)) * bias_ld - 16 * c_lo;
@@ -393,14 +406,14 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
 
       // pass A; four packed scores to a word in the first columns of the chunk's own
       if (alive) tc_fence_after();
+      int mx = -128;
       if (work) {
-        int mx = -128;
 #pragma unroll 1
-        for (int c = c_lo + half; c < c_full; c += 4) {
+        for (int c = c_lo + half; c < c_full; c += 2 * TPR) {
           int v[2][16];
-          const bool second = c + 2 < c_full;
+          const bool second = c + TPR < c_full;
           tmem_ld16_issue(t_row + 16 * c, v[0]);
-          if (second) tmem_ld16_issue(t_row + 16 * c + 32, v[1]);
+          if (second) tmem_ld16_issue(t_row + 16 * (c + TPR), v[1]);
           uint32_t x[4];
           tmem_ld_wait16(v[0]);
           add_bias(v[0], 16 * c, 16);
@@ -408,9 +421,9 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
           tmem_st4(t_row + 16 * c, x);
           if (second) {
             tmem_ld_wait16(v[1]);
-            add_bias(v[1], 16 * c + 32, 16);
+            add_bias(v[1], 16 * (c + TPR), 16);
             score_piece<FAST, false>(a, kc, v[1], 16, mx, x);
-            tmem_st4(t_row + 16 * c + 32, x);
+            tmem_st4(t_row + 16 * (c + TPR), x);
           }
         }
         if (rem > 8) {
@@ -429,16 +442,20 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
           tmem_st2(t_row + 16 * c_full, x);
         }
         tmem_st_wait();
-        part_max[half * 128 + trow] = max(-128, min(127, mx));
+        mx = max(-128, min(127, mx));
+        if (TPR > 1) part_max[half * 128 + trow] = mx;
       }
-      // only the two warps that share these 32 rows exchange partial results: a barrier of their own
-      asm volatile("bar.sync %0, 64;" ::"r"(2 + qd) : "memory");
+      // the threads of a row exchange their partial results: a barrier of the warps that share its 32 rows
+      if (TPR > 1) {
+        bar_sync(2 + qd, 32 * TPR);
+        mx = max(part_max[trow], part_max[128 + trow]);
+      }
+      unsigned sum = 0;
       if (work) {
         // pass B: entry (I_max - I) of this lane's table copy stands at tab_lane + 4 cp (I_max - I)
-        const uint32_t tmx = tab_lane + (uint32_t)(4 * a.cp * max(part_max[trow], part_max[128 + trow]));
-        unsigned sum = 0;
+        const uint32_t tmx = tab_lane + (uint32_t)(4 * a.cp * mx);
 #pragma unroll 2
-        for (int c = c_lo + half; c < c_full; c += 2) {
+        for (int c = c_lo + half; c < c_full; c += TPR) {
           uint32_t x[4];
           tmem_ld4(t_row + 16 * c, x);
           int e[16];
@@ -460,12 +477,14 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
           tmem_st16(t_row + 16 * c_full, e);
         }
         tmem_st_wait();
-        part_sum[half * 128 + trow] = sum;
+        if (TPR > 1) part_sum[half * 128 + trow] = sum;
       }
-      asm volatile("bar.sync %0, 64;" ::"r"(2 + qd) : "memory");
+      if (TPR > 1) {
+        bar_sync(2 + qd, 32 * TPR);
+        sum = part_sum[trow] + part_sum[128 + trow];
+      }
       if (work) {
         // pass C: Eq. (IntDiv) with M = 45
-        const unsigned sum = part_sum[trow] + part_sum[128 + trow];
         const unsigned factor = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
         auto words = [&](const int (&e)[16]) {
           uint32_t o[4];
@@ -476,16 +495,16 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
           return make_uint4(o[0], o[1], o[2], o[3]);
         };
 #pragma unroll 1
-        for (int c = c_lo + half; c < c_full; c += 4) {
+        for (int c = c_lo + half; c < c_full; c += 2 * TPR) {
           int e[2][16];
-          const bool second = c + 2 < c_full;
+          const bool second = c + TPR < c_full;
           tmem_ld16_issue(t_row + 16 * c, e[0]);
-          if (second) tmem_ld16_issue(t_row + 16 * c + 32, e[1]);
+          if (second) tmem_ld16_issue(t_row + 16 * (c + TPR), e[1]);
           tmem_ld_wait16(e[0]);
           *p_addr(c) = words(e[0]);
           if (second) {
             tmem_ld_wait16(e[1]);
-            *p_addr(c + 2) = words(e[1]);
+            *p_addr(c + TPR) = words(e[1]);
           }
         }
         if (rem) {
@@ -505,7 +524,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
         tc_fence_after();
         int8_t* orow = a.O + ((int64_t)b * a.T + r) * a.D + (int64_t)item.h * a.d;
 #pragma unroll 1
-        for (int c = half; c < a.d / 16; c += 2) {
+        for (int c = half; c < a.d / 16; c += TPR) {
           int v[16];
           tmem_ld16(t_row + 16 * c, v);
           const uint4 w = output_piece<FAST>(a, v);
@@ -535,7 +554,7 @@ __global__ void __launch_bounds__(kShortThreads, kPack ? 3 : 2) attention_short_
 //           stand;
 //   output  O = P V has tensor-memory columns of its own and is read beside the reciprocals of the NEXT item's rows.
 // The chunk loops are rolled: straight-line code for all chunks waited for instructions more than for anything else.
-// Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 190 us (before: one table, remainders dealt to all threads, a wait
+// Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 178 us (before: one table, remainders dealt to all threads, a wait
 // for P V in every item).  On rows of up to 256 tokens the two CTAs per SM of the kernel above win: 22.3 against 29.6 us
 // at 64 x 197, 6 heads.
 // Warps 0..3: warp 0 loads, issues MMAs and owns tensor memory (the others of its warpgroup only lend their registers);
@@ -1025,12 +1044,13 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
     else if (per > 0 && per % sa.G == 0 && B % per == 0) sa.npos = (int)(per / sa.G);
     else sa.npos = sa.units;
     if (a.bias) bias_bytes = (size_t)sa.G * T * (T | 1) * 4;
+    sa.t_magic = (unsigned)(0x100000000ull / (unsigned long long)T) + 1u;
   }
   sa.tmem_cols = pack || a.chunks <= 8 ? 128 : 256;
   const uint32_t p_off = (128u * a.d + (pack ? 128u : (uint32_t)a.kbox) * a.d + (uint32_t)a.kpad * a.d + 1023u) & ~1023u;
   const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + 4 * 128 * 4 + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
   // CTAs per SM: as many as leave room for four copies of the table
-  int per_sm = pack ? 3 : 2;
+  int per_sm = pack ? ShortShape<true>::kCtas : ShortShape<false>::kCtas;
   auto budget = [](int n) { return n == 1 ? (size_t)(227 * 1024) : (size_t)(228 * 1024 / n - 1024); };
   while (per_sm > 1 && fixed + 4 * 1024 > budget(per_sm)) --per_sm;
   if (!fit_table(a, fixed, budget(per_sm))) return IVIT_ERR_UNSUPPORTED;
@@ -1043,7 +1063,7 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
       !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, pack ? sa.R : a.kpad, swizzle_of(d), a.v_pos, sa.G))
     return IVIT_ERR_UNSUPPORTED;
   const int64_t slots = (int64_t)per_sm * ctx->sm_count;
-  const dim3 grid((unsigned)(a.items < slots ? a.items : slots)), block(kShortThreads);
+  const dim3 grid((unsigned)(a.items < slots ? a.items : slots)), block(pack ? ShortShape<true>::kThreads : ShortShape<false>::kThreads);
   LaunchScope ls(ctx, KIND_ATTENTION, 4.0 * (double)(B * h) * (double)T * (double)T * (double)d);
   auto run = [&](auto kernel) { launch_k(kernel, grid, block, smem, ctx->stream, tmQ, tmK, tmV, sa); };
   switch ((pack ? 4 : 0) | (fast_form(a) ? 2 : 0) | (a.bias ? 1 : 0)) {
