@@ -465,14 +465,20 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
 #pragma unroll
           for (int i = 0; i < 16; i += 4) sum += ((unsigned)e[i] + (unsigned)e[i + 1]) + ((unsigned)e[i + 2] + (unsigned)e[i + 3]);
         }
-        if (rem) {
+        if (rem) {   // word by word: a class token leaves one or five columns
           uint32_t x[4];
           tmem_ld4(t_row + 16 * c_full, x);
           int e[16];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            e[i] = i < rem ? (int)exp_entry(x[i >> 2], kc.sel[i & 3], tmx) : 0;
-            sum += (unsigned)e[i];
+          for (int q = 0; q < 4; ++q) {
+            e[4 * q] = e[4 * q + 1] = e[4 * q + 2] = e[4 * q + 3] = 0;
+            if (4 * q < rem) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                e[4 * q + i] = 4 * q + i < rem ? (int)exp_entry(x[q], kc.sel[i], tmx) : 0;
+                sum += (unsigned)e[4 * q + i];
+              }
+            }
           }
           tmem_st16(t_row + 16 * c_full, e);
         }
@@ -486,13 +492,12 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       if (work) {
         // pass C: Eq. (IntDiv) with M = 45
         const unsigned factor = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
+        auto word = [&](int e0, int e1, int e2, int e3) {
+          return FAST ? prob_word8(factor, e0, e1, e2, e3) : prob_word(factor, e0, e1, e2, e3, osh, omax);
+        };
         auto words = [&](const int (&e)[16]) {
-          uint32_t o[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            o[q] = FAST ? prob_word8(factor, e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3])
-                        : prob_word(factor, e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3], osh, omax);
-          return make_uint4(o[0], o[1], o[2], o[3]);
+          return make_uint4(word(e[0], e[1], e[2], e[3]), word(e[4], e[5], e[6], e[7]), word(e[8], e[9], e[10], e[11]),
+                            word(e[12], e[13], e[14], e[15]));
         };
 #pragma unroll 1
         for (int c = c_lo + half; c < c_full; c += 2 * TPR) {
@@ -510,7 +515,11 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
         if (rem) {
           int e[16];
           tmem_ld16(t_row + 16 * c_full, e);
-          *p_addr(c_full) = words(e);
+          uint32_t o[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (4 * q < rem) o[q] = word(e[4 * q], e[4 * q + 1], e[4 * q + 2], e[4 * q + 3]);
+          *p_addr(c_full) = make_uint4(o[0], o[1], o[2], o[3]);
         }
         fence_async_smem();
       }
@@ -756,7 +765,6 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
     const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16);
     int* part_max = reinterpret_cast<int*>(gen + part_off);
     unsigned* part_sum = reinterpret_cast<unsigned*>(gen + part_off + 4 * 128 * 4);
-    unsigned* recips = reinterpret_cast<unsigned*>(gen + part_off + 8 * 128 * 4);
     const uint32_t tab_lane = base + tab_off + 4u * (unsigned)(lane & (a.cp - 1));
     const unsigned top = (unsigned)a.smax.I0 << a.smax.N;    // the largest exponential
     const int osh = 14 - a.smax.k_out, omax = (1 << (a.smax.k_out - 1)) - 1;
@@ -884,15 +892,11 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
         part_sum[part * 128 + trow] = sum;
       }
       asm volatile("bar.sync %0, 128;" ::"r"(2 + qd) : "memory");
-      // one reciprocal per row (Eq. (IntDiv) with M = 45), and the output of the previous item
-      if (part == 3 && work) {
-        const unsigned sum = (part_sum[trow] + part_sum[128 + trow]) + (part_sum[256 + trow] + part_sum[384 + trow]);
-        recips[trow] = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
-      }
+      // the output of the previous item; the reciprocal (Eq. (IntDiv) with M = 45), by every thread for its row
       if (n > 0) store_output(n - 1);
-      asm volatile("bar.sync %0, 128;" ::"r"(2 + qd) : "memory");
       if (work) {
-        const unsigned factor = recips[trow];
+        const unsigned sum = (part_sum[trow] + part_sum[128 + trow]) + (part_sum[256 + trow] + part_sum[384 + trow]);
+        const unsigned factor = FAST ? prob_factor4(sum, top, seeds) : (unsigned)((1ull << 45) / (unsigned long long)(sum ? sum : 1u));
         auto words = [&](const uint4& w) {
           const uint32_t x[4] = {w.x, w.y, w.z, w.w};
           uint32_t o[4];
