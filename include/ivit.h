@@ -94,7 +94,8 @@ typedef struct {
 /* Dense layers with a long contraction (K >= 1024, output channels a multiple of 256, enough rows to give every pair of
  * SMs a tile of 256 x 256, int8 output in one of the staged forms) run on pairs of CTAs: two SMs share a tile of 256 channels x 256 rows (tcgen05
  * cta_group::2; a CUDA implementation choice, the paper has no counterpart), each loading its own 128 weight rows and
- * half of the activation rows.  On by default; results are identical in both modes.  enable: 0 = off, non-zero = on.
+ * half of the activation rows.  Results are identical in both modes.  enable: 0 = off, 2 = where the size makes it
+ * the faster form (the default), any other value = wherever the form exists.
  * Host graphs kept by the context are dropped.  Returns IVIT_OK, or IVIT_ERR_INVALID_ARG for a null context. */
 int ivit_ctx_set_gemm_pairs(ivit_ctx* ctx, int enable);
 

@@ -249,9 +249,10 @@ class Context:
     def set_gemm_engine(self, engine: int):
         _chk(self.lib.ivit_ctx_set_gemm_engine(self.h, engine), "ivit_ctx_set_gemm_engine")
 
-    def set_gemm_pairs(self, enable: bool):
-        """CTA pairs (cta_group::2) for Dense layers with K >= 1536 and N % 256 == 0."""
-        _chk(self.lib.ivit_ctx_set_gemm_pairs(self.h, 1 if enable else 0), "ivit_ctx_set_gemm_pairs")
+    def set_gemm_pairs(self, enable: Optional[bool]):
+        """CTA pairs (cta_group::2) for Dense layers with K >= 1024 and N % 256 == 0: everywhere (True), nowhere (False) or
+        where the size makes them the faster form (None, the state of a new context)."""
+        _chk(self.lib.ivit_ctx_set_gemm_pairs(self.h, 2 if enable is None else (1 if enable else 0)), "ivit_ctx_set_gemm_pairs")
 
     def set_row_fusion(self, enable: bool):
         """ivit_ctx_set_row_fusion: LayerNorm / ShiftGELU in the tail of the producing Dense kernel (default) or alone."""

@@ -46,7 +46,7 @@ struct ivit_ctx {
   int gemm_engine;
   int sm_count;
   void* tmap_encode;  // cuTensorMapEncodeTiled, resolved at context creation
-  int gemm_pairs;     // CTA pairs (cta_group::2) for Dense layers with a long contraction (ivit_ctx_set_gemm_pairs)
+  int gemm_pairs;     // CTA pairs (cta_group::2) for Dense layers: 0 never, 1 wherever possible, 2 by size (ivit_ctx_set_gemm_pairs)
   void* tmap_cache;   // encoded tensor maps by (address, extents, strides, box, swizzle); see make_tensor_map
   // ivit_vit_forward_host: input copies run on their own stream into two staging buffers (created on first use)
   cudaStream_t copy_stream;

@@ -134,9 +134,9 @@ struct TcArgs {
   int64_t sCo, sCi;
   int batches_inner;
   int total_tiles;
-  int tiles_each, tiles_extra;   // every CTA walks tiles_each tiles, tiles_extra CTAs one more: the first ones, or
-  int long_last;                 // (long_last) the last ones, when the short tiles of a ragged last row block, which
-                                 // end the tile order, can make up for the extra tile
+  int tiles_each, tiles_extra;   // every CTA walks tiles_each tiles, the first tiles_extra CTAs one more ...
+  int short_tiles;               // ... of all tiles (0), or of the full ones only: then the tiles of the ragged last row
+                                 // block (this many) are dealt out after them, see TileRange
   int tiles_p, tiles_q;
   int BN;            // columns of the tile (multiple of 32, <= 256)
   int stages;
@@ -145,6 +145,8 @@ struct TcArgs {
   int q_mn;          // 1: the Q operand tile is MN-major ([k, n] rows of q_row_bytes)
   int q_row_bytes;
   int q_stage_bytes;
+  int q_last_bytes;  // the same for a tile of the last block: a Dense layer fetches only the chunks of 32 rows that exist
+                     // there (tmL: rows past the end, which a wider box fills with zeros, take as long to arrive as others)
   int p_pos[3], q_pos[3];  // tensor-map dimension (1..3) that holds the row / inner-batch / outer-batch coordinate
   int tma_out;       // Dense orientation, int8: the output tile is staged in shared memory and stored by TMA
   int tma_res;       // ... and the residual tile of the same shape is fetched by TMA into shared memory
@@ -176,19 +178,60 @@ __device__ __forceinline__ TileCoord tile_coord(const TcArgs& a, int t) {
   return c;
 }
 
-// Walks a contiguous range of tiles without divisions: p-block fastest, then q-block, then batch.
+// The tiles of one worker (a CTA, or a pair of them): a contiguous range and, when the tiles of a ragged last row block
+// are dealt out by themselves, up to two of those.  They cost a fraction of a whole tile, so the workers that have one
+// whole tile less take them first (one each, then a second one), then the others take one each.  Without that a ragged
+// block can add a whole round: 12608 rows are 49 blocks of 256 and one of 64, and three channel tiles of 50 blocks on 148
+// workers are 150 tiles, two rounds, instead of 147 tiles and three short ones, one round and a quarter.
+// Measured: 12608 x 384 x 1536 10.9 -> 10.4 us, 4728 x 1024 x 1024 9.7 -> 8.6, 12608 x 768 x 3072 24.8 -> 23.5 (all on
+// single CTAs).
+// (DEAL: a kernel that can do so; the others keep the shorter walk, which is worth 2 % where a tile is one or two k-blocks.)
+template <bool DEAL>
+struct TileRange {
+  int begin, end;         // tile numbers; the short tiles are counted behind the whole ones
+  int jump, jump_p;       // after this many tiles the walk goes on at channel block jump_p of the last row block
+  __device__ __forceinline__ TileRange(const TcArgs& a, int worker, int workers) {
+    const int lng = worker < a.tiles_extra ? 1 : 0, whole = a.tiles_each + lng;
+    begin = worker * a.tiles_each + min(worker, a.tiles_extra);
+    int n_short = 0;
+    jump_p = 0;
+    if (DEAL && a.short_tiles) {
+      const int n_brief = workers - a.tiles_extra;                // workers with one whole tile less
+      const int to_brief = min(a.short_tiles, 2 * n_brief), two = max(to_brief - n_brief, 0);
+      if (lng) {
+        n_short = worker < a.short_tiles - to_brief ? 1 : 0;
+        jump_p = to_brief + worker;
+      } else {
+        const int i = worker - a.tiles_extra;
+        n_short = (i < to_brief ? 1 : 0) + (i < two ? 1 : 0);
+        jump_p = i + min(i, two);
+      }
+      if (whole == 0) begin = a.tiles_p * (a.tiles_q - 1) + jump_p;
+    }
+    end = begin + whole + n_short;
+    jump = whole > 0 && n_short > 0 ? whole : 0x7fffffff;
+  }
+};
+
+// Walks the tiles of a range without divisions: p-block fastest, then q-block, then batch.
+template <bool DEAL>
 struct TileIter {
+  int left, jump_p;       // tiles before the jump, see TileRange
   int p, q, bi, bo;       // block indices
   int batch;
   int pstep, poff;        // lanes between consecutive p-blocks (two tiles when a CTA pair shares them) and this CTA's offset
-  __device__ __forceinline__ void init(const TcArgs& a, int t, int poff_ = 0) {
-    const TileCoord c = tile_coord(a, t);
+  __device__ __forceinline__ void init(const TcArgs& a, const TileRange<DEAL>& range, int poff_ = 0) {
+    const TileCoord c = tile_coord(a, range.begin);
+    if (DEAL) { left = range.jump; jump_p = range.jump_p; }
     p = c.p0 / BM; q = c.q0 / a.BN; bi = c.bi; bo = c.bo; batch = c.batch;
     pstep = a.pair ? 2 * BM : BM;
     poff = poff_;
   }
   __device__ __forceinline__ void next(const TcArgs& a) {
-    if (++p == a.tiles_p) {
+    if (DEAL && --left == 0) {
+      p = jump_p;
+      q = a.tiles_q - 1;
+    } else if (++p == a.tiles_p) {
       p = 0;
       if (++q == a.tiles_q) {
         q = 0;
@@ -199,6 +242,9 @@ struct TileIter {
   }
   __device__ __forceinline__ int p0() const { return p * pstep + poff; }
   __device__ __forceinline__ int q0(const TcArgs& a) const { return q * a.BN; }
+  __device__ __forceinline__ bool last(const TcArgs& a) const { return DEAL && q == a.tiles_q - 1; }
+  // columns of the tile that the MMAs compute (DEAL: a ragged last tile is cut to whole chunks of 32)
+  __device__ __forceinline__ int cols(const TcArgs& a) const { return DEAL ? min(a.BN, (a.Q - q * a.BN + 31) & ~31) : a.BN; }
 };
 
 // MODE fixes the run-time choices of the epilogue at compile time for the shapes of an encoder block, so that
@@ -214,9 +260,11 @@ struct TileIter {
 // row routine each) that are dealt to all epilogue warps of the grid in a fixed order; a warp works on its slices
 // after its CTA's last tile, straight out of L2, waiting (bounded) only for the ready flag of the slice's block.
 // The last CTA to finish leaves counters and flags at zero for the next launch.
-template <int MODE, int ROP, bool PAIR = false>
+// DEAL: the tiles of a ragged last block of rows are dealt out by themselves (TileRange).
+template <int MODE, int ROP, bool PAIR = false, bool DEAL = PAIR>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmP,
                                                               const __grid_constant__ CUtensorMap tmQ,
+                                                              const __grid_constant__ CUtensorMap tmL,
                                                               const __grid_constant__ CUtensorMap tmO,
                                                               const __grid_constant__ CUtensorMap tmR, TcArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -242,15 +290,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
 
   // (read from lane 0, so that the compiler knows it to be the same in all lanes)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-  // this CTA's (with PAIR: this CTA pair's) contiguous range of tiles
+  // this CTA's (with PAIR: this CTA pair's) tiles
   const uint32_t rank = PAIR ? cluster_ctarank() : 0u;      // PAIR: 0 = the CTA that issues the MMAs of the pair
   const int poff = (int)rank * BM;                          // this CTA's 128 channels inside the pair's 256
   const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
   const int workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  const int first_long = a.long_last ? workers - a.tiles_extra : 0;   // first worker with one tile more
-  const int n_long = worker - first_long;                              // long workers before this one
-  const int t_begin = worker * a.tiles_each + min(max(n_long, 0), a.tiles_extra);
-  const int t_end = t_begin + a.tiles_each + ((n_long >= 0 && n_long < a.tiles_extra) ? 1 : 0);
+  const TileRange<DEAL> range(a, worker, workers);
+  const int t_begin = range.begin, t_end = range.end;
 
   // set-up, spread over the epilogue threads: one barrier (or descriptor prefetch) each
   {
@@ -277,6 +323,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       if (a.tma_out) prefetch_tmap(&tmO);
     } else if (i == 2 * kMaxStages + 8 + 2 * kEpiWarps) {
       if (a.tma_res) prefetch_tmap(&tmR);
+    } else if (i == 2 * kMaxStages + 9 + 2 * kEpiWarps) {
+      if (a.q_last_bytes != a.q_stage_bytes) prefetch_tmap(&tmL);
     }
     if (i >= 0 && i < 2 * kMaxStages + 5 + 2 * kEpiWarps) {
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -316,8 +364,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       int s = 0, wrap = 0;       // ring slot of the next k-block and how often the ring has wrapped
       bool ok = true;
       int pit = 0, qi = 0, cur_q = -1;
-      TileIter ti;
-      ti.init(a, t_begin, poff);
+      TileIter<DEAL> ti;
+      ti.init(a, range, poff);
       // which tensor-map coordinate (1..3) carries the row / inner batch / outer batch index
       const int pr = a.p_pos[0], pbi = a.p_pos[1], qr = a.q_pos[0], qbi = a.q_pos[1];
       // PAIR: both CTAs load (their 128 weight rows, their half of the activation rows); the bytes of both are
@@ -337,16 +385,18 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       if (a.lanes_are_channels && t_begin < t_end) {
         pre = kblocks < a.stages ? kblocks : a.stages;
         for (int kb = 0; kb < pre; ++kb) {
-          arm(full0 + 8 * kb, BM * BK + a.q_stage_bytes);
+          arm(full0 + 8 * kb, BM * BK + (ti.last(a) ? a.q_last_bytes : a.q_stage_bytes));
           load(base + kb * stage_bytes, &tmP, full0 + 8 * kb, kb * BK, pr == 1 ? ti.p0() : 0, pr == 2 ? ti.p0() : 0,
                pr == 3 ? ti.p0() : 0);
         }
       }
       pdl_wait();
       for (int t = t_begin; ok && t < t_end; ++t, ++pit, ti.next(a)) {
-        const int p0 = ti.p0(), q0 = ti.q0(a) + (PAIR ? (int)rank * (a.BN >> 1) : 0);   // PAIR: this CTA's half of the rows
+        const int p0 = ti.p0(), q0 = ti.q0(a) + (PAIR ? (int)rank * (ti.cols(a) >> 1) : 0);   // PAIR: this CTA's half of the rows
         const int pc1 = pr == 1 ? p0 : (pbi == 1 ? ti.bi : ti.bo), pc2 = pr == 2 ? p0 : (pbi == 2 ? ti.bi : ti.bo),
                   pc3 = pr == 3 ? p0 : (pbi == 3 ? ti.bi : ti.bo);
+        const CUtensorMap* const map_q = ti.last(a) ? &tmL : &tmQ;
+        const uint32_t q_bytes = ti.last(a) ? a.q_last_bytes : a.q_stage_bytes;
         bool bring_q = false;
         if (a.q_resident && q0 != cur_q) {
           // new activation row block: its k-blocks come in beside this tile's weight k-blocks, once every MMA
@@ -360,15 +410,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (wrap > 0 && !mbar_wait_warp(empty0 + 8 * s, (wrap & 1) ^ 1, a.status)) { ok = false; break; }
           const uint32_t sp = base + s * stage_bytes, sq = sp + BM * BK;
           const bool early = t == t_begin && kb < pre;   // barrier armed and weights requested before the wait
-          if (!early) arm(full0 + 8 * s, stage_bytes + (bring_q ? a.q_stage_bytes : 0));
+          if (!early) arm(full0 + 8 * s, BM * BK + (bring_q || !a.q_resident ? q_bytes : 0));
           if (bring_q)
-            load(qres + kb * a.q_stage_bytes, &tmQ, full0 + 8 * s, kb * BK, qr == 1 ? q0 : 0, qr == 2 ? q0 : 0,
+            load(qres + kb * a.q_stage_bytes, map_q, full0 + 8 * s, kb * BK, qr == 1 ? q0 : 0, qr == 2 ? q0 : 0,
                  qr == 3 ? q0 : 0);
           if (!early) load(sp, &tmP, full0 + 8 * s, kb * BK, pc1, pc2, pc3);
           if (!a.q_resident) {
             const int qrow = a.q_mn ? kb * BK : q0;     // MN-major: rows of the map are k, the inner index is n
             const int qc0 = a.q_mn ? q0 : kb * BK;
-            load(sq, &tmQ, full0 + 8 * s, qc0, qr == 1 ? qrow : (qbi == 1 ? ti.bi : ti.bo),
+            load(sq, map_q, full0 + 8 * s, qc0, qr == 1 ? qrow : (qbi == 1 ? ti.bi : ti.bo),
                  qr == 2 ? qrow : (qbi == 2 ? ti.bi : ti.bo), qr == 3 ? qrow : (qbi == 3 ? ti.bi : ti.bo));
           }
           *issued_slot = ++issued;
@@ -379,10 +429,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     if (rank == 0) {   // PAIR: CTA rank 0 issues for both CTAs
-      // instruction descriptor: D = S32, A = B = signed 8 bit, A K-major, M = 128 (PAIR: 256 over both CTAs), N = BN,
-      // no saturation
-      const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a.q_mn << 16) |
-                             ((uint32_t)(a.BN >> 3) << 17) | ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
+      // instruction descriptor: D = S32, A = B = signed 8 bit, A K-major, M = 128 (PAIR: 256 over both CTAs), no
+      // saturation; N = the tile's columns is added for each tile
+      const uint32_t idesc0 = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a.q_mn << 16) |
+                              ((uint32_t)((PAIR ? 2 * BM : BM) >> 4) << 24);
       // P descriptors: K-major rows of 128 bytes (128B swizzle, 1024 bytes per 8 rows).  Q: the same,
       // or MN-major rows of q_row_bytes (swizzle = row width, 8 rows per group).  Along K a descriptor
       // advances by 32 bytes (K-major) or 32 rows (MN-major): an add on the low word.
@@ -398,16 +448,17 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       int consumed = 0, s = 0, wrap = 0, it = 0;
       bool ok = true;
       int cur_q = -1;
-      TileIter ti;
-      ti.init(a, t_begin, poff);
+      TileIter<DEAL> ti;
+      ti.init(a, range, poff);
       for (int t = t_begin; ok && t < t_end; ++t, ++it) {
         const int buf = it & 1;
+        const uint32_t idesc = idesc0 | ((uint32_t)(ti.cols(a) >> 3) << 17);
         bool last_of_q = false;
-        if (a.q_resident) {
-          // a new activation row block arrives k-block by k-block on the stage barriers of this tile
+        if (DEAL || a.q_resident) {
+          // q_resident: a new activation row block arrives k-block by k-block on the stage barriers of this tile
           cur_q = ti.q0(a);
           ti.next(a);
-          last_of_q = t + 1 >= t_end || ti.q0(a) != cur_q;
+          last_of_q = a.q_resident && (t + 1 >= t_end || ti.q0(a) != cur_q);
         }
         // the epilogue must have drained this buffer (its use two tiles ago)
         if (it >= 2 && !mbar_wait_warp(acce0 + 8 * buf, ((it >> 1) & 1) ^ 1, a.status)) { ok = false; break; }
@@ -441,7 +492,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (PAIR) umma_commit_pair_w(accf0 + 8 * buf);
           else umma_commit_w(accf0 + 8 * buf);
         }
-        if (ok && last_of_q) umma_commit_w(qrese);   // the resident tile may be replaced once these MMAs are done
+        if (ok && last_of_q) {   // the resident tile may be replaced once these MMAs are done (PAIR: in both CTAs)
+          if (PAIR) umma_commit_pair_w(qrese);
+          else umma_commit_w(qrese);
+        }
       }
       if (!ok) {
         // drain: copies that were issued but never consumed (only after a timeout)
@@ -491,8 +545,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       }
     };
     // the first tile's coordinates, computed once (they cost integer divisions)
-    TileIter ti_first;
-    ti_first.init(a, t_begin, poff);
+    TileIter<DEAL> ti_first;
+    ti_first.init(a, range, poff);
     if (dense && t_begin < t_end) fetch_channel(ti_first.p0());
     // MatMul orientation: one per-tensor constant set
     const int um = e.scale.mult, us = clamp_shift(e.scale.shift);
@@ -511,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     // rot = chunks of this CTA's earlier tiles), so that a tile whose chunk count is no multiple of kParts
     // does not leave the same part idle every time.
     // The warp's chunk sequence two chunks ahead (residual fetches):
-    TileIter pf_ti;
+    TileIter<DEAL> pf_ti;
     int pf_t = t_begin;
     int pf_ck = part;
     int pf_rot = 0;
@@ -552,7 +606,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     int it = 0;
     int rot = 0;          // chunks of this CTA's earlier tiles, modulo kParts
     int tiles_in_q = 0;   // ROP: tiles of the current block of output rows that this CTA has finished
-    TileIter ti = ti_first;
+    TileIter<DEAL> ti = ti_first;
     for (int t = t_begin; t < t_end; ++t, ++it) {
       TileCoord tc;
       tc.batch = ti.batch; tc.bo = ti.bo; tc.bi = ti.bi; tc.p0 = ti.p0(); tc.q0 = ti.q0(a);
@@ -947,36 +1001,64 @@ int pow2_at_least(int v) {
 }
 
 constexpr size_t kSmemBudget = 227 * 1024;
-constexpr int64_t kPairMinK = 1024;   // contraction length from which a CTA pair per tile pays (measured)
+constexpr int64_t kPairMinK = 1024;   // contraction length from which the form with a CTA pair per tile is offered
 // alignment slack + one KB of barriers, tensor-memory slot, flags and the two 256-entry tables of the residual /
 // activation port; a row operator's shared memory follows it
 constexpr size_t kSmemFixed = 1024 + 1024;
 static_assert(8 * (2 * kMaxStages + 5 + 2 * kEpiWarps) + 32 + 512 <= 1024, "barrier block");
 
 
-// Tile width along the TMEM columns: the candidate with the least (rounds of tiles per CTA) x (time of a tile).
-// Model of a tile's time: the larger of its operand traffic, (128 + bn) x K bytes at about 60 bytes per clock into
-// an SM's shared memory, and its epilogue, which grows with the tile's width now that chunks are dealt to the
-// epilogue parts across tiles, plus a fixed cost per tile.  The constants are fitted to measured launch times of the
-// DeiT-S / ViT-B / ViT-L layer shapes at widths 128 ... 256 (the pick is within 4 % of the best width on each).
-int pick_bn(int64_t extent, int64_t tiles_other, int64_t K, int sm_count, bool single_batch) {
+// Clocks that the busiest of `workers` spends when `extent` columns are cut into tiles of bn and each block of columns has
+// tiles_other tiles.  A tile costs its operand traffic, (128 + columns) x K bytes (a worker that is a CTA pair: half of
+// the columns' bytes per SM) at about 60 bytes per clock into an SM's shared memory, and 900 clocks; the epilogue of all
+// but the last one runs beside the next tile.  *dealt: the tiles of a ragged last block are dealt out after the whole ones
+// (TileRange), which a kernel that can (deal) does where there is a whole block and it is the shorter way.
+// The constants are fitted to 120 measured launch times of Dense layers (4728 ... 50176 rows, 192 ... 4096 channels in and
+// out): the width picked with them is 0.7 % slower than the best of the five on average.
+double busiest_clocks(int64_t extent, int64_t bn, int64_t tiles_other, int64_t K, int64_t workers, bool pair,
+                      bool deal, bool* dealt) {
+  auto tile = [&](int64_t cols) { return (double)K * (128.0 + (double)cols * (pair ? 0.5 : 1.0)) / 60.0 + 900.0; };
+  auto last = [](int64_t cols) { return 4.0 * (double)cols; };
+  const int64_t tiles = tiles_other * ((extent + bn - 1) / bn);
+  if (workers > tiles) workers = tiles;
+  const double plain = (double)((tiles + workers - 1) / workers) * tile(bn) + last(bn);
+  *dealt = false;
+  const int64_t ragged = extent % bn;
+  if (!deal || ragged == 0 || extent < bn) return plain;
+  const int64_t whole = tiles - tiles_other, each = whole / workers, lng = whole % workers, brief = workers - lng;
+  if (tiles_other > 2 * brief + lng) return plain;
+  const double of_long = lng == 0 ? 0.0 : (double)(each + 1) * tile(bn) + (tiles_other > 2 * brief ? tile(ragged) + last(ragged) : last(bn));
+  const double of_brief = (double)each * tile(bn) + (tiles_other > brief ? 2.0 : 1.0) * tile(ragged) + last(ragged);
+  const double clocks = (of_long > of_brief ? of_long : of_brief) + 190.0 * (double)(each + 2);   // (the longer walk)
+  if (clocks >= plain) return plain;
+  *dealt = true;
+  return clocks;
+}
+
+// Where CTA pairs are faster than single CTAs.  A single CTA fetches (128 + 256) x K bytes per tile, a CTA of a pair
+// (128 + 128) x K, but a pair starts later (cluster launch, two barriers across it) and has half as many workers to
+// spread the tiles over.  From 1536 on the difference shows once the activations no longer stay in the near L2, at about
+// 38 MB of them, and only with enough work per launch (us, pairs / single CTAs): 18464 x 1024 x 4096 55 / 73,
+// 25216 x 768 x 3072 48 / 58, 15760 x 1536 x 2048 39.7 / 40.9, but 9232 x 1024 x 3072 24.8 / 22.9,
+// 4728 x 4096 x 3072 55 / 44 and 25216 x 512 x 1536 20.8 / 19.3.  Below 1536 the pair's gain is the resident activation
+// tile, which with a residual port does not fit: 18464 x 4096 x 1024 59 / 61, 18464 x 3072 x 1024 44.3 / 45.1, but
+// 12608 x 3072 x 1024 34.5 / 30.4 and, with the port, 18464 x 1024 x 1024 23.1 / 19.3.
+bool pair_pays(int64_t M, int64_t N, int64_t K, bool res) {
+  const double macs = (double)M * (double)N * (double)K;
+  if (K < 1536) return !res && macs >= 52e9;
+  return (double)M * (double)K >= 38e6 && macs >= (K < 3072 ? 36e9 : 29e9);
+}
+
+// Tile width along the TMEM columns: the candidate that keeps the busiest CTA the shortest time.
+int pick_bn(int64_t extent, int64_t tiles_other, int64_t K, int sm_count, bool deal) {
   if (extent <= 256) return (int)((extent + 31) / 32 * 32);
   int best = 0;
-  double best_cost = 0;
+  double best_clocks = 0;
   for (int bn : {256, 224, 192, 160, 128}) {
-    const int64_t tiles = tiles_other * ((extent + bn - 1) / bn);
-    double rounds = (double)((tiles + sm_count - 1) / sm_count);
-    // a ragged last block of at most half a tile: if every CTA that needs an extra tile gets one of its short tiles
-    // (long_last in the launcher), the extra tile costs about half a round
-    const int64_t ragged = extent % bn, extra = tiles % sm_count, each = tiles / sm_count;
-    // (only from two full rounds on: measured inside an encoder block, a launch of one round and a half
-    // of wide tiles loses to two rounds of narrow ones although it wins when timed alone)
-    if (single_batch && each >= 2 && ragged != 0 && ragged <= bn / 2 && extra != 0 && (extra - 1) * (each + 1) < tiles_other) rounds -= 0.5;
-    const double feed = (double)K * (128.0 + bn) / 60.0;
-    const double epilogue = 8.0 * bn;
+    bool dealt;
+    const double clocks = busiest_clocks(extent, bn, tiles_other, K, sm_count, false, deal, &dealt);
     // ties go to the narrower tile (its MMAs, loads and stores are shorter): the loop runs from wide to narrow
-    const double cost = rounds * ((feed > epilogue ? feed : epilogue) + 900.0);
-    if (!best || cost <= best_cost) { best = bn; best_cost = cost; }
+    if (!best || clocks <= best_clocks) { best = bn; best_clocks = clocks; }
   }
   return best;
 }
@@ -992,6 +1074,8 @@ int gemm_tc_prepare_device() {
       cudaFuncSetAttribute(gemm_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<1, 0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<2, 0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<1, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<2, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess)
     return IVIT_ERR_CUDA;
@@ -1012,27 +1096,28 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
   a.status = ctx->status_dev;
   CUtensorMap tmP, tmQ;
   const bool dense = g.transB && batches == 1 && !e.bias32;
+  bool deal = false;   // short tiles may be dealt out by themselves
   if (dense) {
     if (g.N % 4 || e.ldo % 4 || (reinterpret_cast<uintptr_t>(e.out) & 3)) return IVIT_ERR_UNSUPPORTED;
     // Dense orientation: lanes = output channels (rows of W), columns = output rows (rows of A)
     a.lanes_are_channels = 1;
     a.P = (int)g.N; a.Q = (int)g.M;
     a.tiles_p = (int)((a.P + BM - 1) / BM);
-    // Long contractions are bound by the operand feed from L2 and by the issuing thread's loop: a pair of CTAs per
-    // tile of 256 channels (cta_group::2) halves the activation bytes per SM and the MMAs issued per SM.  Taken
-    // when the layer has whole pairs of channel tiles and the epilogue is one of the specialised forms.
-    a.pair = (ctx->gemm_pairs && g.K >= kPairMinK && g.N % (2 * BM) == 0 && ctx->sm_count % 2 == 0 &&
-              (g.N / (2 * BM)) * ((g.M + 255) / 256) >= ctx->sm_count / 2 &&   // a pair-tile for every pair of SMs
-             
-              e.out_dtype == IVIT_I8 && e.group_rows <= 0 && !(reinterpret_cast<uintptr_t>(e.out) & 15) && e.ldo % 16 == 0 &&
-              (!e.res || (e.res_rows >= g.M && !(reinterpret_cast<uintptr_t>(e.res) & 15) && e.ldres % 16 == 0)) &&
-              !e.act_table && !(e.rop.kind && ctx->row_fusion)) ? 1 : 0;
+    // A pair of CTAs per tile of 256 channels (cta_group::2) halves the activation bytes per SM and the MMAs issued per
+    // SM.  Possible when the layer has whole pairs of channel tiles, a tile for every pair of SMs, and one of the
+    // specialised epilogues; pair_pays() says where it is the faster form.
+    deal = e.out_dtype == IVIT_I8 && e.group_rows <= 0 && !(reinterpret_cast<uintptr_t>(e.out) & 15) && e.ldo % 16 == 0 &&
+           (!e.res || (e.res_rows >= g.M && !(reinterpret_cast<uintptr_t>(e.res) & 15) && e.ldres % 16 == 0)) &&
+           !e.act_table && !(e.rop.kind && ctx->row_fusion);   // one of the specialised epilogues (mode 1 or 2 below)
+    a.pair = (deal && ctx->gemm_pairs && g.K >= kPairMinK && g.N % (2 * BM) == 0 && ctx->sm_count % 2 == 0 &&
+              (g.N / (2 * BM)) * ((g.M + 255) / 256) >= ctx->sm_count / 2 &&
+              (ctx->gemm_pairs == 1 || pair_pays(g.M, g.N, g.K, e.res != nullptr))) ? 1 : 0;
     if (a.pair) {
       a.tiles_p = (int)(g.N / (2 * BM));   // pairs of channel tiles
       a.BN = 256;
       a.q_stage_bytes = (a.BN / 2) * BK;   // every CTA of a pair loads half of the activation rows
     } else {
-      a.BN = pick_bn(a.Q, a.tiles_p, g.K, ctx->sm_count, batches == 1);
+      a.BN = pick_bn(a.Q, a.tiles_p, g.K, ctx->sm_count, deal);
       a.q_stage_bytes = a.BN * BK;
     }
     if (!make_tensor_map(ctx, &tmP, g.B, g.K, g.N, 1, 1, g.ldb, 0, 0, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B, a.p_pos) ||
@@ -1068,6 +1153,15 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
         return IVIT_ERR_UNSUPPORTED;
     }
   }
+  CUtensorMap tmL = tmQ;
+  a.q_last_bytes = a.q_stage_bytes;
+  if (deal && a.Q % a.BN != 0) {
+    const int rows = ((a.Q % a.BN + 31) & ~31) / (a.pair ? 2 : 1);
+    int lpos[3];
+    if (!make_tensor_map(ctx, &tmL, g.A, g.K, g.M, 1, 1, g.lda, 0, 0, BK, rows, CU_TENSOR_MAP_SWIZZLE_128B, lpos))
+      return IVIT_ERR_UNSUPPORTED;
+    a.q_last_bytes = rows * BK;
+  }
   CUtensorMap tmO = tmP;
   if (dense && e.out_dtype == IVIT_I8 && e.group_rows <= 0 && !(reinterpret_cast<uintptr_t>(e.out) & 15) && e.ldo % 16 == 0) {
     int opos[3];
@@ -1099,7 +1193,7 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
   // short K: keep the activation tile resident if that still leaves four weight stages
   const size_t kblocks = (size_t)((g.K + BK - 1) / BK);
   const size_t qres_bytes = kblocks * a.q_stage_bytes;
-  a.q_resident = (dense && !a.pair && kSmemFixed + rop_bytes + out_stage + qres_bytes + 4 * (size_t)BM * BK <= kSmemBudget) ? 1 : 0;
+  a.q_resident = (dense && kSmemFixed + rop_bytes + out_stage + qres_bytes + 4 * (size_t)BM * BK <= kSmemBudget) ? 1 : 0;
   const size_t stage = (size_t)BM * BK + (a.q_resident ? 0 : a.q_stage_bytes);
   const size_t fixed = out_stage + (a.q_resident ? qres_bytes : 0);
   int stages = (int)((kSmemBudget - kSmemFixed - rop_bytes - fixed) / stage);
@@ -1115,26 +1209,29 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
   const int workers_max = a.pair ? ctx->sm_count / 2 : ctx->sm_count;   // CTAs, or CTA pairs
   const int workers = a.total_tiles < workers_max ? a.total_tiles : workers_max;
   const unsigned grid = (unsigned)(a.pair ? 2 * workers : workers);
-  a.tiles_each = a.total_tiles / workers;
-  a.tiles_extra = a.total_tiles % workers;
-  // ... which needs a short tile in the range of every long CTA
-  a.long_last = (a.Q % a.BN != 0 && a.Q % a.BN <= a.BN / 2 && batches == 1 && a.tiles_extra > 0 &&
-                 (int64_t)(a.tiles_extra - 1) * (a.tiles_each + 1) < a.tiles_p) ? 1 : 0;
-  LaunchScope ls(ctx, KIND_GEMM_TC, 2.0 * (double)batches * (double)g.M * (double)g.N * (double)g.K);
   // the encoder block's Dense layers take the specialised instantiations
   int mode = (a.lanes_are_channels && a.tma_out && (!e.res || a.tma_res)) ? (a.tma_res ? 2 : 1) : 0;
   if (e.act_table) mode = mode == 1 ? 3 : 0;
+  bool dealt;
+  busiest_clocks(a.Q, a.BN, a.tiles_p, g.K, workers_max, a.pair != 0, deal && (mode == 1 || mode == 2) && rop == 0, &dealt);
+  a.short_tiles = dealt ? a.tiles_p : 0;
+  const int dealt_evenly = a.total_tiles - a.short_tiles;   // all tiles, or the whole ones
+  a.tiles_each = dealt_evenly / workers;
+  a.tiles_extra = dealt_evenly % workers;
+  LaunchScope ls(ctx, KIND_GEMM_TC, 2.0 * (double)batches * (double)g.M * (double)g.N * (double)g.K);
   if (a.pair && (mode != 1 && mode != 2)) return IVIT_ERR_UNSUPPORTED;   // (the conditions above imply mode 1 or 2)
   if (a.pair) ++ctx->pair_launches;
-  if (a.pair && mode == 2) launch_k_pair(gemm_tc_kernel<2, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (a.pair) launch_k_pair(gemm_tc_kernel<1, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (rop == 1 && mode == 2) launch_k(gemm_tc_kernel<2, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (rop == 1 && mode == 1) launch_k(gemm_tc_kernel<1, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (rop == 2 && mode == 1) launch_k(gemm_tc_kernel<1, 2>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (mode == 3) launch_k(gemm_tc_kernel<3, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (mode == 2) launch_k(gemm_tc_kernel<2, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else if (mode == 1) launch_k(gemm_tc_kernel<1, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
-  else launch_k(gemm_tc_kernel<0, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a);
+  if (a.pair && mode == 2) launch_k_pair(gemm_tc_kernel<2, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (a.pair) launch_k_pair(gemm_tc_kernel<1, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (rop == 1 && mode == 2) launch_k(gemm_tc_kernel<2, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (rop == 1 && mode == 1) launch_k(gemm_tc_kernel<1, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (rop == 2 && mode == 1) launch_k(gemm_tc_kernel<1, 2>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (dealt && mode == 2) launch_k(gemm_tc_kernel<2, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (dealt && mode == 1) launch_k(gemm_tc_kernel<1, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (mode == 3) launch_k(gemm_tc_kernel<3, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (mode == 2) launch_k(gemm_tc_kernel<2, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else if (mode == 1) launch_k(gemm_tc_kernel<1, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  else launch_k(gemm_tc_kernel<0, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
   ctx->rowop_fused = (rop != 0 && (mode == 1 || mode == 2)) ? 1 : 0;
   return ls.done();
 }

@@ -438,7 +438,7 @@ int ivit_ctx_create(ivit_ctx** out, int device, void* cuda_stream) {
   }
   c->rowblk_dev = reinterpret_cast<unsigned*>(c->gelu_tables + (size_t)kGeluTableSlots * kGeluTableBytes);
   c->row_fusion = 0;
-  c->gemm_pairs = 1;
+  c->gemm_pairs = 2;
   *out = c;
   return IVIT_OK;
 }
@@ -512,7 +512,7 @@ int ivit_ctx_set_row_fusion(ivit_ctx* ctx, int enable) {
 
 int ivit_ctx_set_gemm_pairs(ivit_ctx* ctx, int enable) {
   if (!ctx) return IVIT_ERR_INVALID_ARG;
-  ctx->gemm_pairs = enable ? 1 : 0;
+  ctx->gemm_pairs = enable == 0 || enable == 2 ? enable : 1;
   for (int i = 0; i < 2; ++i) host_graph_drop(ctx, i);
   return IVIT_OK;
 }

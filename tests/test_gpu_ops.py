@@ -130,6 +130,33 @@ def test_linear_cta_pairs(M, N, K, with_res):
         c.set_gemm_pairs(True)
 
 
+@pytest.mark.parametrize("M,N,K,with_res", [(12545, 384, 1536, True), (12608, 384, 1536, False), (9505, 512, 512, False),
+                                            (37889, 120, 400, False), (6177, 768, 1024, True), (6177, 768, 1024, False)])
+def test_linear_short_tiles_dealt_out(M, N, K, with_res):
+    """A ragged last block of rows (1 ... 64 of 256) whose tiles are dealt out after the whole ones: to the workers with a
+    tile less (one or two each), or to others too; single CTAs and, where the layer has that form, CTA pairs."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(M + N * 3 + K)
+    A, W = rand_i8(rng, (M, K)), rand_i8(rng, (N, K))
+    bias = rng.integers(-20000, 20000, N).astype(np.int32)
+    scale = scale_channels(rng.uniform(20, 60, N) / (np.sqrt(K) * 40 * 40))
+    res = rand_i8(rng, (M, N)) if with_res else None
+    rs = Scale(*dyadic(0.9))
+    want = O.linear(A, W, bias, scale, res=res, res_scale=rs if with_res else None)
+    try:
+        for pairs in (False, True):
+            c.set_gemm_pairs(pairs)
+            got = c.linear(g.dev(A), g.dev(W), torch.from_numpy(bias).cuda(), g.binding.DevScale(scale, "cuda"),
+                           res=None if res is None else g.dev(res),
+                           res_scale=g.binding.DevScale(rs, "cuda") if with_res else None,
+                           out=g.dev(np.full((M, N), 77, np.int8)))
+            g.assert_equal(g.host(got), want, f"linear pairs={pairs}")
+            assert c.poll_status() == 0
+    finally:
+        c.set_gemm_pairs(None)
+
+
 @pytest.mark.parametrize("M,N,K", [(130, 200, 16), (260, 128, 32)])
 def test_linear_low_shifts(M, N, K):
     """Per-channel shifts of 31 and 32 next to larger ones: the requantisation leaves its high-word form."""
