@@ -267,7 +267,8 @@ int launch_shiftgelu_static(ivit_ctx* ctx, const int8_t* in, int64_t ldin, ivit_
 int launch_shiftgelu(ivit_ctx* ctx, const int8_t* in, int64_t ldin, ivit_exp_params p, ivit_scale post,
                      int8_t* out, int64_t ldout, int64_t rows, int64_t cols);
 int launch_patchify(ivit_ctx* ctx, const int8_t* img, int64_t B, int64_t C, int64_t Hi, int64_t Wi,
-                    int64_t P, int64_t window, int8_t* out, int64_t ldout);
+                    int64_t P, int64_t window, int8_t* out, int64_t ldout, const int8_t* fill_src = nullptr, int64_t fill_width = 0,
+                    int8_t* fill_dst = nullptr, int64_t fill_stride = 0);   // fill_src: also this row to every image's fill_dst
 int launch_gather_rows(ivit_ctx* ctx, const int8_t* src, int64_t ldsrc, const int32_t* index,
                        int64_t n_rows, int64_t width, int8_t* dst, int64_t lddst);
 int launch_fill_rows(ivit_ctx* ctx, const int8_t* src_row, int64_t width, int8_t* dst,

@@ -131,6 +131,7 @@ constexpr int kThreads = 32 * kFirstEpiWarp + kEpiThreads;
 struct TcArgs {
   GemmEpilogue epi;
   int P, Q, K;       // extents along TMEM lanes / TMEM columns / contraction (32-bit: the launcher checks the sizes)
+  int res_rows, group_rows;   // of the epilogue, cut to 32 bits (there are fewer output rows than that)
   int64_t sCo, sCi;
   int batches_inner;
   int total_tiles;
@@ -247,11 +248,25 @@ struct TileIter {
   __device__ __forceinline__ int cols(const TcArgs& a) const { return DEAL ? min(a.BN, (a.Q - q * a.BN + 31) & ~31) : a.BN; }
 };
 
+// The map of the last block's activation rows: only the kernels that use it carry it in their parameters.
+template <bool DEAL>
+struct LastMap {
+  CUtensorMap map;
+  __device__ __forceinline__ const CUtensorMap* get(const CUtensorMap*) const { return &map; }
+};
+template <>
+struct LastMap<false> {
+  __device__ __forceinline__ const CUtensorMap* get(const CUtensorMap* other) const { return other; }
+};
+
 // MODE fixes the run-time choices of the epilogue at compile time for the shapes of an encoder block, so that
 // the per-chunk code carries no branches on kernel arguments: 0 = everything decided at run time (any
 // orientation, output type and residual port), 1 = Dense orientation, int8 output staged for TMA stores, no
 // residual, 2 = the same with the residual tile fetched by TMA, 3 = as 1 with an activation table applied to the
-// saturated value (the element-wise ShiftGELU variant inside FC1).
+// saturated value (the element-wise ShiftGELU variant inside FC1), 4 = as 2 for output rows in groups with a gap between
+// them and a residual that repeats (the patch embedding with its class rows and position table): the slots are filled and
+// emptied by the warp itself, residual words one chunk ahead.  (As MODE 0, with byte loads of the residual and 4-byte
+// stores, the embedding took as long as two such layers: 25088 x 768 x 768 39.1 us, plain 18.0.)
 // ROP != 0 (MODE 1 or 2 only): a row operator on the output, run by this same kernel: 1 = I-LayerNorm into a second
 // tensor (the input of the next Dense layer), 2 = ShiftGELU in place (Algorithm 2 with its row maximum).  Both need
 // whole output rows, i.e. every channel tile of a block of rows, and those tiles may belong to several CTAs.  So
@@ -264,9 +279,9 @@ struct TileIter {
 template <int MODE, int ROP, bool PAIR = false, bool DEAL = PAIR>
 __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ CUtensorMap tmP,
                                                               const __grid_constant__ CUtensorMap tmQ,
-                                                              const __grid_constant__ CUtensorMap tmL,
                                                               const __grid_constant__ CUtensorMap tmO,
-                                                              const __grid_constant__ CUtensorMap tmR, TcArgs a) {
+                                                              const __grid_constant__ CUtensorMap tmR, TcArgs a,
+                                                              const __grid_constant__ LastMap<DEAL> tmL) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // carve: [stages x (P tile | Q tile)] [barriers] [tmem address, issued count]
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -324,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     } else if (i == 2 * kMaxStages + 8 + 2 * kEpiWarps) {
       if (a.tma_res) prefetch_tmap(&tmR);
     } else if (i == 2 * kMaxStages + 9 + 2 * kEpiWarps) {
-      if (a.q_last_bytes != a.q_stage_bytes) prefetch_tmap(&tmL);
+      if (DEAL && a.q_last_bytes != a.q_stage_bytes) prefetch_tmap(tmL.get(&tmQ));
     }
     if (i >= 0 && i < 2 * kMaxStages + 5 + 2 * kEpiWarps) {
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -395,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         const int p0 = ti.p0(), q0 = ti.q0(a) + (PAIR ? (int)rank * (ti.cols(a) >> 1) : 0);   // PAIR: this CTA's half of the rows
         const int pc1 = pr == 1 ? p0 : (pbi == 1 ? ti.bi : ti.bo), pc2 = pr == 2 ? p0 : (pbi == 2 ? ti.bi : ti.bo),
                   pc3 = pr == 3 ? p0 : (pbi == 3 ? ti.bi : ti.bo);
-        const CUtensorMap* const map_q = ti.last(a) ? &tmL : &tmQ;
+        const CUtensorMap* const map_q = ti.last(a) ? tmL.get(&tmQ) : &tmQ;
         const uint32_t q_bytes = ti.last(a) ? a.q_last_bytes : a.q_stage_bytes;
         bool bring_q = false;
         if (a.q_resident && q0 != cur_q) {
@@ -520,6 +535,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     const bool dense = MODE ? true : a.lanes_are_channels != 0;
     const bool tma_out = MODE ? true : a.tma_out != 0;
     const bool tma_res = MODE ? MODE == 2 : a.tma_res != 0;   // MODE 3 = MODE 1 + activation table
+    constexpr bool kGroup = MODE == 4;
+    const bool smem_res = kGroup || tma_res;
     const bool ldg_res = MODE ? false : (e.res != nullptr && !a.tma_res);
     const bool out_i32 = MODE ? false : e.out_dtype == IVIT_I32;
     const int8_t* res_tab0 = res_tab + 128;   // entry of residual byte 0
@@ -602,6 +619,26 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
       pf_fetch();
       pf_fetch();
     }
+    // MODE 4: a lane's eight words of the next chunk's residual rows (lane >> 3) + 4 k, fetched one chunk ahead
+    uint32_t rw[8];
+    auto group_fetch = [&]() {
+      if (pf_t >= t_end) return;
+      const int c = pf_ti.p0() + c_first + 4 * (lane & 7);
+      int rr = (int)((uint32_t)(pf_ti.q0(a) + 32 * pf_ck) % (uint32_t)a.res_rows) + (lane >> 3);   // (res_rows >= 32)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (rr >= a.res_rows) rr -= a.res_rows;
+        rw[k] = c < a.P ? __ldg(reinterpret_cast<const uint32_t*>(e.res + (int64_t)rr * e.ldres + c)) : 0u;
+        rr += 4;
+      }
+      pf_ck += kParts;
+      pf_settle();
+    };
+    if (kGroup && t_begin < t_end) {
+      pf_ti = ti_first;
+      pf_settle();
+      group_fetch();
+    }
 
     int it = 0;
     int rot = 0;          // chunks of this CTA's earlier tiles, modulo kParts
@@ -673,20 +710,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             }
           }
           // residual port
-          if (tma_res) {
+          if (smem_res) {
             // residual bytes of this chunk in shared memory: [row][32 channels]
             const uint8_t* rt = gen_base + (my_res - base) + (g & 1u) * 1024 + h * 512 + lane;
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] += (int)res_tab0[(int)*reinterpret_cast<const int8_t*>(rt + j * 32)];
           } else if (ldg_res) {
-            int64_t rr = (int64_t)((uint64_t)r0 % (uint64_t)e.res_rows);
+            int rr = (int)((uint32_t)r0 % (uint32_t)a.res_rows);   // (the same in all lanes)
+            const int8_t* rp = e.res + (int64_t)rr * e.ldres + c;
 #pragma unroll
             for (int g = 0; g < 16; g += 8) {
               int xr[8];
 #pragma unroll
               for (int j = 0; j < 8; ++j) {
-                xr[j] = (c_ok && g + j < nrow) ? (int)__ldg(e.res + rr * e.ldres + c) : 0;
-                if (++rr == e.res_rows) rr = 0;
+                xr[j] = (c_ok && g + j < nrow) ? (int)__ldg(rp) : 0;
+                rp += e.ldres;
+                if (++rr == a.res_rows) { rr = 0; rp = e.res + c; }
               }
 #pragma unroll
               for (int j = 0; j < 8; ++j) v[g + j] += (int)res_tab0[xr[j]];
@@ -722,10 +761,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             for (int k = 0; k < 4; ++k) *reinterpret_cast<uint32_t*>(pe + 512 * h + 128 * k) = w[k];
           } else {
             // direct stores (grouped output rows): this lane's first word is row r0 + li, then + 4 per word
-            int64_t row = (int64_t)r0 + li, ro = row, grem = 0;
+            int64_t ro = (int64_t)r0 + li;
+            int grem = 0;
             if (e.group_rows > 0) {
-              grem = (int64_t)((uint64_t)row % (uint64_t)e.group_rows);
-              ro = (int64_t)((uint64_t)row / (uint64_t)e.group_rows) * e.group_stride + grem;
+              const uint32_t g0 = (uint32_t)r0 / (uint32_t)a.group_rows;   // (the same in all lanes)
+              grem = r0 - (int)g0 * a.group_rows + li;
+              ro = (int64_t)g0 * e.group_stride + grem;
+              while (grem >= a.group_rows) { grem -= a.group_rows; ro += e.group_stride - a.group_rows; }
             }
             const int cbase = tc.p0 + qd * 32 + (lane & ~3);
             const bool cg_ok = cbase < a.P;   // P % 4 == 0: a group of four channels is valid as a whole
@@ -736,7 +778,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
               ro += 4;
               if (e.group_rows > 0) {
                 grem += 4;
-                while (grem >= e.group_rows) { grem -= e.group_rows; ro += e.group_stride - e.group_rows; }
+                while (grem >= a.group_rows) { grem -= a.group_rows; ro += e.group_stride - a.group_rows; }
               }
             }
           }
@@ -748,7 +790,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
           if (tma_out) {
             const uint32_t sl = g & 1u;
             // the store that used this slot two chunks ago must have read it; the residual bytes must be here
-            tma_store_wait_read1();   // (every lane: only the one that issued the stores has any to wait for)
+            if (!kGroup) tma_store_wait_read1();   // (every lane: only the one that issued the stores has any to wait for)
+            if (kGroup) {
+              uint32_t* rs = reinterpret_cast<uint32_t*>(gen_base + (my_res - base) + sl * 1024) + lane;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) rs[32 * k] = rw[k];
+              group_fetch();
+            }
             if (tma_res && c_any) {
               if (ok) ok = mbar_wait_warp(my_resf + 8u * sl, (rpar >> sl) & 1u, a.status);
               if (ok) { rpar ^= 1u << sl; rpend &= ~(1u << sl); }
@@ -816,7 +864,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             tmem_ld16(t_row + (uint32_t)(32 * ck + 16), v);
             half(v, ck, 1, pe);
           }
-          if (tma_out) {
+          if (kGroup) {
+            // the staged rows leave as 16-byte stores, each to its place in its group
+            __syncwarp();
+            const int r0 = tc.q0 + 32 * ck, c = tc.p0 + c_first + 16 * (lane & 1);
+            const uint32_t g0 = (uint32_t)r0 / (uint32_t)a.group_rows;
+            const uint4* so = reinterpret_cast<const uint4*>(gen_base + (my_out - base) + 1024u * (g & 1u)) + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int row = 16 * h + (lane >> 1);
+              const int in_group = r0 - (int)g0 * a.group_rows + row;
+              int64_t ro = (int64_t)g0 * e.group_stride + in_group;
+              if (in_group >= a.group_rows) ro += e.group_stride - a.group_rows;   // (group_rows >= 32)
+              if (r0 + row < a.Q && c < a.P) *reinterpret_cast<uint4*>(reinterpret_cast<int8_t*>(e.out) + ro * e.ldo + c) = so[32 * h];
+            }
+            ++g;
+          } else if (tma_out) {
             fence_async_smem();
             __syncwarp();
             if (c_any) tma_store_4d_w(&tmO, my_out + 1024u * (g & 1u), tc.p0 + c_first, tc.q0 + 32 * ck, 0, 0);
@@ -962,7 +1025,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         }
       }
     }
-    if (tma_out) tma_store_wait_all();
+    if (tma_out && !kGroup) tma_store_wait_all();
     // only after a timeout: residual bytes fetched for chunks that were never worked on may be in flight
     if (tma_res && !ok && lane == 0)
       for (uint32_t sl = 0; sl < 2; ++sl)
@@ -1071,6 +1134,7 @@ int gemm_tc_prepare_device() {
       cudaFuncSetAttribute(gemm_tc_kernel<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<2, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<3, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
+      cudaFuncSetAttribute(gemm_tc_kernel<4, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<2, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
       cudaFuncSetAttribute(gemm_tc_kernel<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess ||
@@ -1092,6 +1156,8 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
 
   TcArgs a{};
   a.epi = e;
+  a.res_rows = e.res_rows > 2147483647LL ? 2147483647 : (int)e.res_rows;
+  a.group_rows = e.group_rows > 2147483647LL ? 2147483647 : (int)e.group_rows;
   a.K = (int)g.K; a.sCo = g.sCo; a.sCi = g.sCi; a.batches_inner = (int)g.batches_inner;
   a.status = ctx->status_dev;
   CUtensorMap tmP, tmQ;
@@ -1174,10 +1240,14 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
     a.tma_res = make_tensor_map(ctx, &tmR, e.res, g.N, g.M, 1, 1, e.ldres, 0, 0, 32, 32, CU_TENSOR_MAP_SWIZZLE_NONE,
                                 rpos) ? 1 : 0;
   }
+  // grouped output rows: the warps fill and empty the staging slots themselves (MODE 4)
+  const bool grouped = dense && e.out_dtype == IVIT_I8 && e.group_rows >= 32 && g.N % 16 == 0 && !(reinterpret_cast<uintptr_t>(e.out) & 15) &&
+                       e.ldo % 16 == 0 && e.res && e.res_rows >= 32 && !(reinterpret_cast<uintptr_t>(e.res) & 3) && e.ldres % 4 == 0 && !e.act_table;
+  if (grouped) a.tma_out = a.tma_res = 1;   // (the slots exist)
   // The row operator runs in this kernel when the epilogue is one of the specialised forms (staged int8 output,
   // residual absent or fetched by TMA), the rows fit the tail routines and there is a counter per row block.
   int rop = 0;
-  if (e.rop.kind && a.lanes_are_channels && a.tma_out && (!e.res || a.tma_res) && !e.act_table && ctx->row_fusion) {
+  if (e.rop.kind && !grouped && a.lanes_are_channels && a.tma_out && (!e.res || a.tma_res) && !e.act_table && ctx->row_fusion) {
     const int64_t blocks_q = (a.Q + a.BN - 1) / a.BN;
     if (blocks_q <= kRowCounters && e.rop.kind == 1 && g.N <= 1024 && (ctx->row_fusion & 1)) rop = 1;
     if (blocks_q <= kRowCounters && e.rop.kind == 2 && g.N % 16 == 0 && g.N <= 4096 && !e.res && (ctx->row_fusion & 2)) rop = 2;
@@ -1212,26 +1282,29 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
   // the encoder block's Dense layers take the specialised instantiations
   int mode = (a.lanes_are_channels && a.tma_out && (!e.res || a.tma_res)) ? (a.tma_res ? 2 : 1) : 0;
   if (e.act_table) mode = mode == 1 ? 3 : 0;
+  if (grouped) mode = 4;
   bool dealt;
   busiest_clocks(a.Q, a.BN, a.tiles_p, g.K, workers_max, a.pair != 0, deal && (mode == 1 || mode == 2) && rop == 0, &dealt);
   a.short_tiles = dealt ? a.tiles_p : 0;
   const int dealt_evenly = a.total_tiles - a.short_tiles;   // all tiles, or the whole ones
   a.tiles_each = dealt_evenly / workers;
   a.tiles_extra = dealt_evenly % workers;
+  const LastMap<true> last_map{tmL};
   LaunchScope ls(ctx, KIND_GEMM_TC, 2.0 * (double)batches * (double)g.M * (double)g.N * (double)g.K);
   if (a.pair && (mode != 1 && mode != 2)) return IVIT_ERR_UNSUPPORTED;   // (the conditions above imply mode 1 or 2)
   if (a.pair) ++ctx->pair_launches;
-  if (a.pair && mode == 2) launch_k_pair(gemm_tc_kernel<2, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (a.pair) launch_k_pair(gemm_tc_kernel<1, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (rop == 1 && mode == 2) launch_k(gemm_tc_kernel<2, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (rop == 1 && mode == 1) launch_k(gemm_tc_kernel<1, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (rop == 2 && mode == 1) launch_k(gemm_tc_kernel<1, 2>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (dealt && mode == 2) launch_k(gemm_tc_kernel<2, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (dealt && mode == 1) launch_k(gemm_tc_kernel<1, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (mode == 3) launch_k(gemm_tc_kernel<3, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (mode == 2) launch_k(gemm_tc_kernel<2, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else if (mode == 1) launch_k(gemm_tc_kernel<1, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
-  else launch_k(gemm_tc_kernel<0, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmL, tmO, tmR, a);
+  if (a.pair && mode == 2) launch_k_pair(gemm_tc_kernel<2, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, last_map);
+  else if (a.pair) launch_k_pair(gemm_tc_kernel<1, 0, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, last_map);
+  else if (rop == 1 && mode == 2) launch_k(gemm_tc_kernel<2, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (rop == 1 && mode == 1) launch_k(gemm_tc_kernel<1, 1>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (rop == 2 && mode == 1) launch_k(gemm_tc_kernel<1, 2>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (dealt && mode == 2) launch_k(gemm_tc_kernel<2, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, last_map);
+  else if (dealt && mode == 1) launch_k(gemm_tc_kernel<1, 0, false, true>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, last_map);
+  else if (mode == 4) launch_k(gemm_tc_kernel<4, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (mode == 3) launch_k(gemm_tc_kernel<3, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (mode == 2) launch_k(gemm_tc_kernel<2, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else if (mode == 1) launch_k(gemm_tc_kernel<1, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
+  else launch_k(gemm_tc_kernel<0, 0>, dim3(grid), dim3(kThreads), smem, ctx->stream, tmP, tmQ, tmO, tmR, a, LastMap<false>{});
   ctx->rowop_fused = (rop != 0 && (mode == 1 || mode == 2)) ? 1 : 0;
   return ls.done();
 }

@@ -757,12 +757,12 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
   int8_t* Y = reinterpret_cast<int8_t*>(ws + w.Y);
   int8_t* Z = reinterpret_cast<int8_t*>(ws + w.Z);
   const ivit_scale none{nullptr, nullptr, 1, 1};
-  if ((rc = launch_patchify(ctx, image, B, 3, p->img, p->img, p->patch, 0, patches, Kpe))) return rc;
+  // the patches, and the class token in front of every image's tokens
+  if ((rc = launch_patchify(ctx, image, B, 3, p->img, p->img, p->patch, 0, patches, Kpe, p->cls, D, X, T * D))) return rc;
   // patch embedding as a Dense layer; the position embedding enters through the residual port;
   // patch q of image b lands in token row b*T + 1 + q
   if ((rc = launch_gemm(ctx, linear_problem(patches, Kpe, p->Wpe, Kpe, p->bpe, p->pe_scale, p->pos, D, np,
                                             p->pos_scale, X + D, D, IVIT_I8, np, T, B * np, D, Kpe)))) return rc;
-  if ((rc = launch_fill_rows(ctx, p->cls, D, X, T * D, B))) return rc;
   bool a_ready = false;   // LayerNorm 1 of the next block already produced by the previous block's last Dense layer
   for (int64_t l = 0; l < p->depth; ++l) {
     const ivit_block_params* next = l + 1 < p->depth ? &p->blocks[l + 1] : nullptr;

@@ -179,6 +179,29 @@ def test_linear_low_shifts(M, N, K):
     assert c.poll_status() == 0
 
 
+@pytest.mark.parametrize("M,grp,stride,period,N,K", [(13720, 196, 197, 196, 144, 64), (19000, 33, 40, 32, 400, 96),
+                                                     (9900, 32, 32, 50, 784, 48), (20011, 577, 600, 1000, 128, 768)])
+def test_linear_row_groups_and_repeated_residual(M, grp, stride, period, N, K):
+    """Grouped output rows with a residual that repeats, in the form that stages both in shared memory: groups and periods
+    down to the 32 rows of a chunk, channels that end inside a warp's 32, a last group that is not full."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(M + grp + N)
+    A, W, pos = rand_i8(rng, (M, K)), rand_i8(rng, (N, K)), rand_i8(rng, (period, N))
+    bias = rng.integers(-20000, 20000, N).astype(np.int32)
+    scale = scale_channels(rng.uniform(20, 60, N) / (np.sqrt(K) * 40 * 40))
+    ps = Scale(*dyadic(0.7))
+    rows = (M + grp - 1) // grp * stride + 1
+    buf = g.dev(np.full((rows, N), 77, np.int8))
+    c.linear(g.dev(A), g.dev(W), torch.from_numpy(bias).cuda(), g.binding.DevScale(scale, "cuda"), res=g.dev(pos),
+             res_scale=g.binding.DevScale(ps, "cuda"), res_rows=period, out=buf[1:], out_group_rows=grp, out_group_stride=stride)
+    want = np.full((rows, N), 77, np.int8)
+    r = np.arange(M)
+    want[1 + r // grp * stride + r % grp] = O.linear(A, W, bias, scale, res=pos[r % period], res_scale=ps)
+    g.assert_equal(g.host(buf), want, "grouped rows")
+    assert c.poll_status() == 0
+
+
 @pytest.mark.parametrize("engine", [1, 0])
 def test_linear_output_row_groups(engine):
     g = _g()
@@ -475,6 +498,32 @@ def test_helpers_parity():
     want = np.zeros((20, 32), np.int8)
     want[::5] = row
     g.assert_equal(g.host(dst), want, "fill rows")
+
+
+@pytest.mark.parametrize("B,C,Hi,Wi,P,window", [(1, 3, 4, 4, 4, 0), (3, 1, 28, 56, 4, 7), (5, 4, 60, 20, 4, 5), (2, 3, 48, 32, 16, 0),
+                                                (7, 3, 96, 64, 32, 1), (3, 3, 48, 96, 16, 3), (2, 3, 24, 40, 8, 0)])
+def test_patchify_forms(B, C, Hi, Wi, P, window):
+    """Patch extraction by patches of four, by 16-byte pieces and by words; images that are not square, windows."""
+    g = _g()
+    rng = np.random.default_rng(B * 100 + Hi + P)
+    img = rng.integers(-128, 128, (B, C, Hi, Wi)).astype(np.int8)
+    got = g.ctx().patchify(torch.from_numpy(img).cuda(), P, window=window)
+    g.assert_equal(g.host(got), O.patchify(img, P, window=window), "patchify")
+
+
+@pytest.mark.parametrize("rows,width,T", [(1, 16, 1), (37, 48, 37), (196, 144, 49), (2000, 16, 8), (333, 1536, 9), (21, 112, 3)])
+def test_gather_and_token_mean_forms(rows, width, T):
+    """Row gathers with an odd number of pieces; token means over the row counts around the eight warps of a block, for
+    widths that are a multiple of four and others."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(rows + width)
+    x, idx = rand_i8(rng, (rows, width)), rng.integers(0, rows, rows).astype(np.int32)
+    g.assert_equal(g.host(c.gather_rows(g.dev(x), torch.from_numpy(idx).cuda())), O.gather_rows(x, idx), "gather")
+    sc = Scale(*dyadic(0.9 / T))
+    for C in (width, width - 4, width - 3):
+        xc = np.ascontiguousarray(x[:rows // T * T, :C])
+        g.assert_equal(g.host(c.token_mean(g.dev(xc), T, g.binding.DevScale(sc, "cuda"))), O.token_mean(xc, T, sc), f"mean {C}")
 
 
 def test_argument_validation_is_synchronous():
