@@ -846,6 +846,62 @@ __global__ void shiftgelu_table_kernel(ivit_exp_params p, int post_m, int post_s
   table[m * 256 + threadIdx.x] = (int8_t)out;
 }
 
+// Rows of NV vectors of 16 values with NV R = 32 W: R rows fill the lanes of W loads (rows of 24 or 48 vectors would
+// leave a quarter of them idle).  A lane's i-th vector belongs to row (lane + 32 i) / NV.
+// What bounds it: instruction issue, about five instructions per four values and a look-up each.  Measured, back to back,
+// against a warp per row: 200704 x 384 33.7 -> 31.6 us, 50176 x 768 15.8 -> 13.0, 197 x 768 2.4 -> 2.1.  (All 128 table
+// rows in shared memory, one block of 1024 per SM, instead of a row staged per row: 31.9 and 15.1 us.)
+template <int NV, int R>
+__global__ void __launch_bounds__(256) shiftgelu_side_kernel(const int8_t* __restrict__ in, int64_t ldin,
+                                                             const int8_t* __restrict__ table, int8_t* __restrict__ out,
+                                                             int64_t ldout, int64_t rows, int fixed_max) {
+  constexpr int W = NV * R / 32;
+  static_assert(W * 32 == NV * R && NV >= 16, "whole loads, at most three rows in each");
+  __shared__ __align__(256) unsigned tab[8][R * 64];
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const unsigned k256 = gelu_k256();
+  int row[W], off[W];
+  uint32_t t8[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    row[i] = (lane + 32 * i) / NV;
+    off[i] = (lane + 32 * i - row[i] * NV) * 16;
+    t8[i] = (uint32_t)__cvta_generic_to_shared(tab[wib] + 64 * row[i]);
+  }
+  pdl_wait();
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t r0 = warp * R; r0 < rows; r0 += nwarps * R) {
+    int4 w[W];
+    int m[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) w[i] = __ldg(reinterpret_cast<const int4*>(in + min(r0 + row[i], rows - 1) * ldin + off[i]));
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+      ByteMax b;
+      b.add(w[i]);
+      m[i] = b.value();
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      int mx = fixed_max;   // >= 0: the static-maximum variant
+      if (fixed_max < 0) {
+        mx = 0;
+#pragma unroll
+        for (int i = r * NV / 32; i <= (r * NV + NV - 1) / 32; ++i) mx = max(mx, row[i] == r ? m[i] : 0);
+        mx = __reduce_max_sync(0xffffffffu, mx);
+      }
+      gelu_stage_row(table + mx * 256, tab[wib] + 64 * r, lane);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+      if (r0 + row[i] < rows) *reinterpret_cast<int4*>(out + (r0 + row[i]) * ldout + off[i]) = gelu_vec(w[i], t8[i], k256);
+  }
+}
+
 // WPL > 0: rows of up to 512 * WPL values, R rows per warp at a time, kept in registers between the maximum and
 // the look-ups (shiftgelu_rows).  WPL == 0: any width; the row is read twice.
 template <int WPL, int R>
@@ -958,7 +1014,9 @@ static int shiftgelu_rows(ivit_ctx* ctx, const int8_t* in, int64_t ldin, ivit_ex
   const int grid = (int)(want < (int64_t)ctx->sm_count * 12 ? want : (int64_t)ctx->sm_count * 12);
   cudaStream_t st = ctx->stream;
   LaunchScope ls(ctx, KIND_SHIFTGELU, 2.0 * (double)rows * (double)cols);
-  if (wpl <= 1) launch_k(shiftgelu_kernel<1, 4>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, (int)cols, fixed_max);
+  if (cols == 384) launch_k(shiftgelu_side_kernel<24, 4>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, fixed_max);
+  else if (cols == 768) launch_k(shiftgelu_side_kernel<48, 2>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, fixed_max);
+  else if (wpl <= 1) launch_k(shiftgelu_kernel<1, 4>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, (int)cols, fixed_max);
   else if (wpl <= 2) launch_k(shiftgelu_kernel<2, 2>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, (int)cols, fixed_max);
   else if (wpl <= 3) launch_k(shiftgelu_kernel<3, 1>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, (int)cols, fixed_max);
   else if (wpl <= 4) launch_k(shiftgelu_kernel<4, 2>, dim3(grid), dim3(256), 0, st, in, ldin, table, out, ldout, rows, (int)cols, fixed_max);

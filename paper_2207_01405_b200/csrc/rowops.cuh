@@ -168,6 +168,54 @@ __device__ __forceinline__ void layernorm_rows(const int8_t* in, int64_t ldin, i
 }
 
 // ---- ShiftGELU --------------------------------------------------------------------------------------------
+// Maximum of int8 values, four to a word: as pairs of 16-bit values whose upper bytes are bytes 3 and 1, or 2 and 0 (the
+// lower bytes only break ties; the four-byte maximum is no single instruction).
+struct ByteMax {
+  unsigned m31 = 0x80808080u, m20 = 0x80808080u;
+  __device__ __forceinline__ void add(unsigned w) {
+    m31 = __vmaxs2(m31, w);
+    m20 = __vmaxs2(m20, w << 8);
+  }
+  __device__ __forceinline__ void add(const int4& v) { add((unsigned)v.x); add((unsigned)v.y); add((unsigned)v.z); add((unsigned)v.w); }
+  __device__ __forceinline__ int value() const {
+    const unsigned m = __vmaxs2(m31, m20);
+    return max((int)m >> 24, (int)(m << 16) >> 24);
+  }
+};
+
+// A table row (256 bytes, 256-byte aligned) staged so that the byte of x, taken as unsigned, is its place: the halves of
+// the row, which is ordered by x + 128, change places.  `tab` is this warp's copy.
+__device__ __forceinline__ void gelu_stage_row(const int8_t* row, unsigned* tab, int lane) {
+  const unsigned* trow = reinterpret_cast<const unsigned*>(row);
+  tab[lane + 32] = __ldg(trow + lane);
+  tab[lane] = __ldg(trow + lane + 32);
+}
+
+// Look-up of the four bytes of w in the row at shared-memory address t8: one byte permute makes an address; the results
+// are put together by multiply-adds (k = 256, in a register), which run beside the permutes.
+__device__ __forceinline__ int gelu_word(unsigned w, uint32_t t8, unsigned k) {
+  unsigned e[4];
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {
+    const unsigned a = __byte_perm(w, t8, 0x7650 + b);
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(e[b]) : "r"(a));
+  }
+  unsigned lo, hi;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(lo) : "r"(e[1]), "r"(k), "r"(e[0]));
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(hi) : "r"(e[3]), "r"(k), "r"(e[2]));
+  return (int)__byte_perm(lo, hi, 0x5410);
+}
+__device__ __forceinline__ int4 gelu_vec(const int4& v, uint32_t t8, unsigned k) {
+  return make_int4(gelu_word((unsigned)v.x, t8, k), gelu_word((unsigned)v.y, t8, k), gelu_word((unsigned)v.z, t8, k),
+                   gelu_word((unsigned)v.w, t8, k));
+}
+// 256, hidden from the compiler so that the multiply-adds stay such
+__device__ __forceinline__ unsigned gelu_k256() {
+  unsigned k;
+  asm volatile("mov.u32 %0, 256;" : "=r"(k));
+  return k;
+}
+
 // One warp, R rows of `cols` int8 values (cols % 16 == 0, cols <= 512 * WPL): row maximum, then one look-up per
 // value in row max(0, maximum) of the 128 x 256 table; `tab` is the warp's staging space for the R table rows
 // (R x 64 words of shared memory, 256-byte aligned).  in == out is allowed.
@@ -175,57 +223,43 @@ template <int WPL, int R, bool CG>
 __device__ __forceinline__ void shiftgelu_rows(const int8_t* in, int64_t ldin, int nrows, int cols, const int8_t* table,
                                                unsigned* tab, int8_t* out, int64_t ldout, int lane, int fixed_max = -1) {
   const int nvec = cols >> 4;
+  const unsigned k256 = gelu_k256();
   int4 w[R][WPL];
   int mx[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int4* src = reinterpret_cast<const int4*>(in + (int64_t)r * ldin);
-    int m4 = (int)0x80808080;
 #pragma unroll
     for (int i = 0; i < WPL; ++i) {
       const int idx = lane + 32 * i;
       int4 v = make_int4((int)0x80808080, (int)0x80808080, (int)0x80808080, (int)0x80808080);
       if (r < nrows && idx < nvec) v = CG ? __ldcg(src + idx) : __ldg(src + idx);
       w[r][i] = v;
-      m4 = (int)__vmaxs4(__vmaxs4((unsigned)v.x, (unsigned)v.y), __vmaxs4(__vmaxs4((unsigned)v.z, (unsigned)v.w), (unsigned)m4));
     }
-    mx[r] = max(max((int)(int8_t)m4, (int)(int8_t)(m4 >> 8)), max((int)(int8_t)(m4 >> 16), (int)(int8_t)(m4 >> 24)));
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    ByteMax m;
+#pragma unroll
+    for (int i = 0; i < WPL; ++i) m.add(w[r][i]);
+    mx[r] = m.value();
   }
   __syncwarp();
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     mx[r] = fixed_max >= 0 ? fixed_max : max(0, __reduce_max_sync(0xffffffffu, mx[r]));   // fixed_max: the static-maximum variant
-    const unsigned* trow = reinterpret_cast<const unsigned*>(table + mx[r] * 256);
-    tab[64 * r + lane] = __ldg(trow + lane);
-    tab[64 * r + lane + 32] = __ldg(trow + lane + 32);
+    gelu_stage_row(table + mx[r] * 256, tab + 64 * r, lane);
   }
   __syncwarp();
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     if (r < nrows) {
-      // shared-memory address of entry 0 of this row's table: 256-byte aligned, so that one byte permute puts
-      // the index x + 128 into its low byte
       const uint32_t t8 = (uint32_t)__cvta_generic_to_shared(tab + 64 * r);
       int4* dst = reinterpret_cast<int4*>(out + (int64_t)r * ldout);
 #pragma unroll
       for (int i = 0; i < WPL; ++i) {
         const int idx = lane + 32 * i;
-        if (idx < nvec) {
-          const int vin[4] = {w[r][i].x, w[r][i].y, w[r][i].z, w[r][i].w};
-          int vout[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const unsigned u = (unsigned)vin[q] ^ 0x80808080u;   // x + 128 per byte
-            unsigned e[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-              const unsigned a = __byte_perm(u, t8, 0x7650 + b);
-              asm volatile("ld.shared.u8 %0, [%1];" : "=r"(e[b]) : "r"(a));
-            }
-            vout[q] = (int)__byte_perm(__byte_perm(e[0], e[1], 0x0040), __byte_perm(e[2], e[3], 0x0040), 0x5410);
-          }
-          dst[idx] = make_int4(vout[0], vout[1], vout[2], vout[3]);
-        }
+        if (idx < nvec) dst[idx] = gelu_vec(w[r][i], t8, k256);
       }
     }
   }

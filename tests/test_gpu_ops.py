@@ -375,6 +375,26 @@ def test_shiftexp_and_gelu_exhaustive_domain():
         g.assert_equal(g.host(got), O.shiftmax(x, p), f"shiftmax domain I0={I0}")
 
 
+@pytest.mark.parametrize("rows", [1, 2, 3, 5, 8, 4099])
+def test_shiftgelu_rows_side_by_side(rows):
+    """Widths of 384 and 768 share a warp's loads between four or two rows: row counts around those, rows whose maximum is
+    at either end of the row, negative or 127, and a row pitch wider than the row."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(rows)
+    post = Scale(*dyadic(1.0 / (128 * 0.9)))
+    for cols in (384, 768):
+        x = rand_i8(rng, (rows, cols + 16))
+        x[1::5] = -np.abs(x[1::5] // 2) - 1
+        x[::3, 0], x[::4, cols - 1], x[:, cols:] = 127, 126, 127
+        p = ExpParams(33, 23)
+        want = O.shiftgelu(np.ascontiguousarray(x[:, :cols]), p, post)
+        got = c.shiftgelu(torch.from_numpy(x).cuda()[:, :cols], p, g.binding.DevScale(post, "cuda"),
+                          out=torch.empty((rows, cols), dtype=torch.int8, device="cuda"))
+        g.assert_equal(g.host(got), want, f"shiftgelu {rows} x {cols}")
+    assert c.poll_status() == 0
+
+
 @pytest.mark.parametrize("rows,cols,I0", [(1, 16, 29), (200, 768, 31), (300, 1536, 33), (64, 3072, 35), (40, 4096, 37),
                                           (7, 8192, 29), (5, 12288, 30)])
 def test_shiftgelu_parity(rows, cols, I0):
