@@ -253,6 +253,12 @@ int launch_attention_fused(ivit_ctx* ctx, const ivit_block_params* p, const int8
 
 int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, ScaleDev gs,
                      const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C);
+// I-LayerNorm of gathered rows: row r is row index[r] (inner: inner[index[r]]) of the input, also copied to `copy`; or
+// (quarters) put together from the rows index[4 r + k], a quarter as wide.  For the widths that layernorm_gathers names.
+bool layernorm_gathers(int64_t rows, int64_t C, bool quarters);
+int launch_layernorm_gather(ivit_ctx* ctx, const int8_t* in, int64_t ldin, const int32_t* index, const int32_t* inner, bool quarters,
+                            ScaleDev gs, const int32_t* beta, int M_ln, int8_t* copy, int64_t ldcopy, int8_t* out, int64_t ldout,
+                            int64_t rows, int64_t C);
 int launch_shiftmax(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, const int32_t* bias32,
                     int64_t ldbias, int64_t bias_rows, ScaleDev pre, ivit_exp_params p, int8_t* out,
                     int64_t ldout, int64_t rows, int64_t d);

@@ -885,33 +885,55 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
   ivit_block_params fin{};
   fin.ln1_gamma = p->lnf_gamma; fin.ln1_beta = p->lnf_beta; fin.M_ln = p->M_ln;
   bool a_ready = false;   // the LayerNorm output that the next block (or the pooling) reads sits in the block workspace
+  // Row permutations between blocks are read through their index by the LayerNorm that follows, which also leaves the
+  // permuted rows in `third` for the residual.  order: token row q is row order[q] of cur (nullptr: row q).
+  const int32_t* order = nullptr;
   for (int64_t s = 0; s < p->n_stages; ++s) {
     const ivit_swin_stage* st = &p->stages[s];
     const int64_t C = st->C;
+    const bool gathers = layernorm_gathers(rows, C, false);
     for (int64_t l = 0; l < st->depth; ++l) {
       const bool sh = st->shifted && st->shifted[l];
       const bool sh_next = l + 1 < st->depth && st->shifted && st->shifted[l + 1];
+      const ivit_block_params* blk = &st->blocks[l];
       // LayerNorm 1 of the next block comes out of this block's last Dense layer when the next block reads this
       // block's output rows as they are (no row permutation in between)
       const ivit_block_params* next = (l + 1 < st->depth && !sh && !sh_next) ? &st->blocks[l + 1] : nullptr;
       if (l + 1 == st->depth && s + 1 == p->n_stages && !sh) next = &fin;
-      if (sh) {
+      if (gathers && (sh || order)) {
+        if ((rc = launch_layernorm_gather(ctx, cur, C, sh ? st->shift_index : order, sh ? order : nullptr, false, to_dev(blk->ln1_gamma),
+                                          blk->ln1_beta, blk->M_ln, third, C, reinterpret_cast<int8_t*>(wsb), C, rows, C))) return rc;
+        if ((rc = block_impl(ctx, blk, third, other, wsb, true, sh ? nullptr : next, &a_ready))) return rc;
+        int8_t* t = cur; cur = other; other = t;
+        order = sh ? st->unshift_index : nullptr;
+      } else if (sh) {
         if ((rc = launch_gather_rows(ctx, cur, C, st->shift_index, rows, C, third, C))) return rc;
-        if ((rc = block_impl(ctx, &st->blocks[l], third, other, wsb, false, nullptr, nullptr))) return rc;
+        if ((rc = block_impl(ctx, blk, third, other, wsb, false, nullptr, nullptr))) return rc;
         if ((rc = launch_gather_rows(ctx, other, C, st->unshift_index, rows, C, cur, C))) return rc;
         a_ready = false;
       } else {
-        if ((rc = block_impl(ctx, &st->blocks[l], cur, other, wsb, a_ready, next, &a_ready))) return rc;
+        if ((rc = block_impl(ctx, blk, cur, other, wsb, a_ready, next, &a_ready))) return rc;
         int8_t* t = cur; cur = other; other = t;
       }
     }
     if (st->merge_index) {
       // 2x2 patch merging: four C-wide slices per output row, LayerNorm over 4C, Dense to 2C
-      if ((rc = launch_gather_rows(ctx, cur, C, st->merge_index, rows, C, other, C))) return rc;
-      rows /= 4;
+      const int64_t merged = rows / 4;
+      if (layernorm_gathers(merged, 4 * C, true)) {
+        if ((rc = launch_layernorm_gather(ctx, cur, C, st->merge_index, order, true, to_dev(st->merge_ln_gamma), st->merge_ln_beta, p->M_ln,
+                                          nullptr, 0, third, 4 * C, merged, 4 * C))) return rc;
+      } else {
+        if (order) {
+          if ((rc = launch_gather_rows(ctx, cur, C, order, rows, C, third, C))) return rc;
+          int8_t* t = cur; cur = third; third = t;
+        }
+        if ((rc = launch_gather_rows(ctx, cur, C, st->merge_index, rows, C, other, C))) return rc;
+        if ((rc = launch_layernorm(ctx, other, IVIT_I8, 4 * C, to_dev(st->merge_ln_gamma), st->merge_ln_beta, p->M_ln, third,
+                                   4 * C, merged, 4 * C))) return rc;
+      }
+      order = nullptr;
+      rows = merged;
       res /= 2;
-      if ((rc = launch_layernorm(ctx, other, IVIT_I8, 4 * C, to_dev(st->merge_ln_gamma), st->merge_ln_beta, p->M_ln, third,
-                                 4 * C, rows, 4 * C))) return rc;
       // ... followed by LayerNorm 1 of the next stage's first block (into the block workspace, where it expects it)
       const ivit_block_params* nb = &p->stages[s + 1].blocks[0];
       if ((rc = dense_then_layernorm(ctx, linear_problem(third, 4 * C, st->Wmerge, 4 * C, nullptr, st->merge_scale, nullptr, 0, 1,
@@ -921,6 +943,10 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
     }
   }
   const int64_t Cl = p->stages[p->n_stages - 1].C;
+  if (order) {   // the last block was a shifted one
+    if ((rc = launch_gather_rows(ctx, cur, Cl, order, rows, Cl, third, Cl))) return rc;
+    cur = third;
+  }
   if (tokens && cudaMemcpyAsync(tokens, cur, (size_t)(rows * Cl), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
     return IVIT_ERR_CUDA;
   const int8_t* normed = reinterpret_cast<const int8_t*>(wsb);

@@ -183,11 +183,29 @@ struct LnLane {
   }
 };
 
-template <int L, int WPL, int R, int PER_SM, bool kExact>
+// GA = 1: row r is row index[r] of the input (inner: inner[index[r]]), and is also copied to row r of `copy`: a window
+// shift or its inverse without a pass of its own.  GA = 2: quarter k of row r is row index[4 r + k] of the input, a quarter
+// as wide: the gather of a 2 x 2 patch merging.  Measured, back to back, against a gather kernel in front: a Swin-T forward of 64 images,
+// 15 launches fewer, 1492 -> 1452 us.
+template <int GA>
+struct LnSource {
+  const int32_t *index, *inner;
+  int8_t* copy;
+  int64_t ldcopy;
+  __device__ __forceinline__ int row(int r) const {
+    const int q = __ldg(index + r);
+    return inner ? __ldg(inner + q) : q;
+  }
+};
+template <>
+struct LnSource<0> {};
+
+template <int L, int WPL, int R, int PER_SM, bool kExact, int GA = 0>
 __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
                                                                      const int32_t* __restrict__ beta, int M_ln,
                                                                      int8_t* __restrict__ out, int64_t ldout, int rows, int C,
-                                                                     unsigned mean_magic, int vec) {
+                                                                     unsigned mean_magic, int vec, LnSource<GA> source) {
+  static_assert(GA == 0 || kExact, "whole rows");
   static_assert(R <= L, "a lane per row for the scalars");
   constexpr int G = 32 / L;
   pdl_trigger();
@@ -202,9 +220,28 @@ __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_
     int w[R][WPL];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const int* src = reinterpret_cast<const int*>(in + (int64_t)min(r0 + r * G, rows - 1) * ldin) + li;
+      const int row = min(r0 + r * G, rows - 1);
+      if constexpr (GA == 2) {
+        constexpr int Q = L * WPL / 4;   // words of a quarter
+        int q[WPL];
 #pragma unroll
-      for (int i = 0; i < WPL; ++i) w[r][i] = kExact || li + L * i < nwords ? __ldg(src + L * i) : 0;
+        for (int i = 0; i < WPL; ++i) q[i] = source.row(4 * row + (li + L * i) / Q);
+#pragma unroll
+        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(reinterpret_cast<const int*>(in + (int64_t)q[i] * ldin) + (li + L * i) % Q);
+      } else {
+        int64_t from = row;
+        if constexpr (GA == 1) from = source.row(row);
+        const int* src = reinterpret_cast<const int*>(in + from * ldin) + li;
+#pragma unroll
+        for (int i = 0; i < WPL; ++i) w[r][i] = kExact || li + L * i < nwords ? __ldg(src + L * i) : 0;
+      }
+    }
+    if constexpr (GA == 1) {
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int i = 0; i < WPL; ++i)
+          if (r0 + r * G < rows) reinterpret_cast<int*>(source.copy + (int64_t)(r0 + r * G) * source.ldcopy)[li + L * i] = w[r][i];
     }
     int my_s1 = 0, my_s2 = 0;
 #pragma unroll
@@ -346,6 +383,51 @@ __global__ void __launch_bounds__(256) layernorm_i32_kernel(const int32_t* __res
   }
 }
 
+// layernorm_rows_kernel for int8 rows of C channels; false: no form for that width.
+template <int GA>
+static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDev gs, const int32_t* beta, int M_ln, int8_t* out,
+                           int64_t ldout, int64_t rows, int64_t C, LnSource<GA> source) {
+  if (rows >= (1ll << 31) / (GA == 2 ? 4 : 1) - (1 << 20)) return false;
+  const int wpl = (int)((C / 4 + 31) / 32);
+  const unsigned magic = (unsigned)(0x100000000ull / (unsigned long long)(2 * C)) + 1u;
+  const int vec = gs.mult_c && gs.shift_c && !(reinterpret_cast<uintptr_t>(gs.mult_c) & 15) && !(reinterpret_cast<uintptr_t>(gs.shift_c) & 3) &&
+                  !(reinterpret_cast<uintptr_t>(beta) & 15);
+  // (rpw: rows of a warp and pass)
+  auto run = [&](auto kernel, int rpw, int per_sm) {
+    const int64_t blocks = (rows + 4 * rpw - 1) / (4 * rpw), cap = (int64_t)ctx->sm_count * per_sm;
+    launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(128), 0, ctx->stream, x, ldin, gs, beta, M_ln, out, ldout, (int)rows,
+             (int)C, magic, vec, source);
+  };
+  // Blocks per SM: as many as the registers allow without spilling much (25216 x 768: 10.9 us at three, 12.7 at four,
+  // 16.2 at five; 12608 x 384: 4.0 at five, 4.3 at six).  Up to 1024 rows one row per group of lanes: with so few rows the
+  // chain of one warp counts (197 x 192: 1.45 against 1.8 us).
+  const bool few = rows <= 1024;
+  switch (C) {
+    case 96:
+      if (GA == 2) return false;
+      if constexpr (GA != 2) few ? run(layernorm_rows_kernel<8, 3, 1, 5, true, GA>, 4, 5) : run(layernorm_rows_kernel<8, 3, 4, 5, true, GA>, 16, 5);
+      return true;
+    case 192:
+      if (GA == 2) return false;
+      if constexpr (GA != 2) few ? run(layernorm_rows_kernel<16, 3, 1, 5, true, GA>, 2, 5) : run(layernorm_rows_kernel<16, 3, 4, 5, true, GA>, 8, 5);
+      return true;
+    case 384: few ? run(layernorm_rows_kernel<32, 3, 1, 5, true, GA>, 1, 5) : run(layernorm_rows_kernel<32, 3, 4, 5, true, GA>, 4, 5); return true;
+    case 512: run(layernorm_rows_kernel<32, 4, 4, 4, true, GA>, 4, 4); return true;
+    case 768: few ? run(layernorm_rows_kernel<32, 6, 1, 4, true, GA>, 1, 4) : run(layernorm_rows_kernel<32, 6, 4, 3, true, GA>, 4, 3); return true;
+    case 1024: few ? run(layernorm_rows_kernel<32, 8, 1, 3, true, GA>, 1, 3) : run(layernorm_rows_kernel<32, 8, 4, 2, true, GA>, 4, 2); return true;
+    case 1536: run(layernorm_rows_kernel<32, 12, 1, 2, true, GA>, 1, 2); return true;
+  }
+  if constexpr (GA == 0) {
+    if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);
+    else if (wpl <= 2) run(layernorm_rows_kernel<32, 2, 4, 8, false>, 4, 8);
+    else if (wpl <= 4) run(layernorm_rows_kernel<32, 4, 4, 5, false>, 4, 5);
+    else if (wpl <= 8) run(layernorm_rows_kernel<32, 8, 2, 3, false>, 2, 3);
+    else return false;
+    return true;
+  }
+  return false;
+}
+
 int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, ScaleDev gs,
                      const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C) {
   if (rows == 0) return IVIT_OK;
@@ -360,37 +442,25 @@ int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, 
   }
   const int8_t* x = (const int8_t*)in;
   const int wpl = (int)((C / 4 + 31) / 32);
-  if (wpl <= 8 && rows < (1ll << 31) - (1 << 20)) {
-    const unsigned magic = (unsigned)(0x100000000ull / (unsigned long long)(2 * C)) + 1u;
-    const int vec = gs.mult_c && gs.shift_c && !(reinterpret_cast<uintptr_t>(gs.mult_c) & 15) && !(reinterpret_cast<uintptr_t>(gs.shift_c) & 3) &&
-                    !(reinterpret_cast<uintptr_t>(beta) & 15);
-    // (rows: rows of a warp and pass)
-    auto run = [&](auto kernel, int rpw, int per_sm) {
-      const int64_t blocks = (rows + 4 * rpw - 1) / (4 * rpw), cap = (int64_t)ctx->sm_count * per_sm;
-      launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(128), 0, st, x, ldin, gs, beta, M_ln, out, ldout, (int)rows, (int)C, magic, vec);
-    };
-    // Blocks per SM: as many as the registers allow without spilling much (25216 x 768: 10.9 us at three, 12.7 at four,
-    // 16.2 at five; 12608 x 384: 4.0 at five, 4.3 at six).  Up to 1024 rows one row per group of lanes: with so few rows the
-    // chain of one warp counts (197 x 192: 1.45 against 1.8 us).
-    const bool few = rows <= 1024;
-    switch (C) {
-      case 96: few ? run(layernorm_rows_kernel<8, 3, 1, 5, true>, 4, 5) : run(layernorm_rows_kernel<8, 3, 4, 5, true>, 16, 5); break;
-      case 192: few ? run(layernorm_rows_kernel<16, 3, 1, 5, true>, 2, 5) : run(layernorm_rows_kernel<16, 3, 4, 5, true>, 8, 5); break;
-      case 384: few ? run(layernorm_rows_kernel<32, 3, 1, 5, true>, 1, 5) : run(layernorm_rows_kernel<32, 3, 4, 5, true>, 4, 5); break;
-      case 512: run(layernorm_rows_kernel<32, 4, 4, 4, true>, 4, 4); break;
-      case 768: few ? run(layernorm_rows_kernel<32, 6, 1, 4, true>, 1, 4) : run(layernorm_rows_kernel<32, 6, 4, 3, true>, 4, 3); break;
-      case 1024: few ? run(layernorm_rows_kernel<32, 8, 1, 3, true>, 1, 3) : run(layernorm_rows_kernel<32, 8, 4, 2, true>, 4, 2); break;
-      default:
-        if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);
-        else if (wpl <= 2) run(layernorm_rows_kernel<32, 2, 4, 8, false>, 4, 8);
-        else if (wpl <= 4) run(layernorm_rows_kernel<32, 4, 4, 5, false>, 4, 5);
-        else run(layernorm_rows_kernel<32, 8, 2, 3, false>, 2, 3);
-    }
-    return ls.done();
-  }
+  if (layernorm_rows<0>(ctx, x, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<0>{})) return ls.done();
   if (wpl <= 12) launch_k(layernorm_i8_kernel<12>, dim3(grid), dim3(threads), 0, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C);
   else launch_k(layernorm_i8_long_kernel, dim3(grid), dim3(threads), 0, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C);
   return ls.done();
+}
+
+int launch_layernorm_gather(ivit_ctx* ctx, const int8_t* in, int64_t ldin, const int32_t* index, const int32_t* inner, bool quarters,
+                            ScaleDev gs, const int32_t* beta, int M_ln, int8_t* copy, int64_t ldcopy, int8_t* out, int64_t ldout,
+                            int64_t rows, int64_t C) {
+  if (rows == 0) return IVIT_OK;
+  LaunchScope ls(ctx, KIND_LAYERNORM, (double)rows * (double)C * (quarters ? 2.0 : 3.0));
+  const bool done = quarters ? layernorm_rows<2>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<2>{index, inner, nullptr, 0})
+                             : layernorm_rows<1>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<1>{index, inner, copy, ldcopy});
+  return done ? ls.done() : IVIT_ERR_UNSUPPORTED;
+}
+
+bool layernorm_gathers(int64_t rows, int64_t C, bool quarters) {
+  return rows < (1ll << 31) / 4 - (1 << 20) &&
+         (C == 384 || C == 512 || C == 768 || C == 1024 || C == 1536 || (!quarters && (C == 96 || C == 192)));
 }
 
 // ------------------------------------------------------------------ Shiftmax
