@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
 // stored: the body has no branch but the one on the form of the constants.  What bounds it is instruction issue: byte,
 // multiply-add, mad.hi, shift and half a pack per value, and about 130 instructions for the scalars of G R rows at once.
 // With a branch around every word and row and one row per 32 lanes, three of four instructions were overhead.  Measured, back
-// to back: 200704 x 96 27.4 -> 12.1 us, 197 x 192 2.4 -> 1.5.  (More than 1024 rows of a multiple of 128 channels: the next kernel.)
+// to back: 197 x 192 2.4 -> 1.5 us.  (More than 1024 rows of 96, 192 or a multiple of 128 channels: the next kernel.)
 // fast: every channel of the warp has s >= 33 and a small beta (see LnConsts): m, sh = s - 32 and add = 2^(sh-1) + beta 2^sh.
 template <int WPL>
 struct LnLane {
@@ -305,43 +305,45 @@ __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_
   }
 }
 
-// The same for C = 128 WPL with the constants in shared memory, fetched once per word and R rows: the registers go to rows,
+// The same for C = 4 L WPL with the constants in shared memory, fetched once per word and R rows: the registers go to rows,
 // so that most launches are one or two passes, and twice the warps are in flight.  Bound by issue and by the chain of the
 // scalars of a pass.  Measured, back to back, against constants in registers: 18464 x 1024 12.4 -> 9.5 us, 9232 x 1024 8.4 ->
-// 5.4, 25216 x 768 11.3 -> 10.6, 12608 x 768 7.1 -> 5.8, 12608 x 384 4.2 -> 3.7, 3136 x 1536 9.0 -> 4.2.
-template <int WPL, int R, int GA = 0>
+// 5.4, 25216 x 768 11.3 -> 10.6, 12608 x 768 7.1 -> 5.8, 12608 x 384 4.2 -> 3.7, 3136 x 1536 9.0 -> 4.2, 12544 x 192
+// 3.65 -> 3.1, 200704 x 96 12.4 -> 11.9.
+template <int L, int WPL, int R, int GA = 0>
 __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
                                                                             const int32_t* __restrict__ beta, int M_ln,
                                                                             int8_t* __restrict__ out, int64_t ldout, int rows, int C,
                                                                             unsigned mean_magic, int vec, LnSource<GA> source) {
-  static_assert(R <= 32, "a lane per row for the scalars");
-  __shared__ int4 sm_m[32 * WPL], sm_s[32 * WPL], sm_b[32 * WPL];
+  static_assert(R <= L, "a lane per row for the scalars");
+  constexpr int G = 32 / L, kWords = L * WPL;
+  __shared__ int4 sm_m[kWords], sm_s[kWords], sm_b[kWords];
   pdl_trigger();
-  const int lane = threadIdx.x & 31;
-  const bool fast = __syncthreads_and(ln_stage_consts(gs, beta, 32 * WPL, vec, sm_m, sm_s, sm_b, threadIdx.x, 256)) != 0;
-  if (fast) ln_fold_consts(32 * WPL, sm_s, sm_b, threadIdx.x, 256);
+  const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
+  const bool fast = __syncthreads_and(ln_stage_consts(gs, beta, kWords, vec, sm_m, sm_s, sm_b, threadIdx.x, 256)) != 0;
+  if (fast) ln_fold_consts(kWords, sm_s, sm_b, threadIdx.x, 256);
   __syncthreads();
   pdl_wait();
   const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int stride = (int)((gridDim.x * blockDim.x) >> 5) * R;
-  for (int r0 = warp * R; r0 < rows; r0 += stride) {
+  const int stride = (int)((gridDim.x * blockDim.x) >> 5) * (G * R);
+  for (int r0 = warp * (G * R) + grp; r0 - grp < rows; r0 += stride) {
     int w[R][WPL];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const int row = min(r0 + r, rows - 1);
+      const int row = min(r0 + r * G, rows - 1);
       if constexpr (GA == 2) {
-        constexpr int Q = 8 * WPL;   // words of a quarter
+        constexpr int Q = kWords / 4;   // words of a quarter
         int q[WPL];
 #pragma unroll
-        for (int i = 0; i < WPL; ++i) q[i] = source.row(4 * row + (lane + 32 * i) / Q);
+        for (int i = 0; i < WPL; ++i) q[i] = source.row(4 * row + (li + L * i) / Q);
 #pragma unroll
-        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(reinterpret_cast<const int*>(in + (int64_t)q[i] * ldin) + (lane + 32 * i) % Q);
+        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(reinterpret_cast<const int*>(in + (int64_t)q[i] * ldin) + (li + L * i) % Q);
       } else {
         int64_t from = row;
         if constexpr (GA == 1) from = source.row(row);
-        const int* src = reinterpret_cast<const int*>(in + from * ldin) + lane;
+        const int* src = reinterpret_cast<const int*>(in + from * ldin) + li;
 #pragma unroll
-        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(src + 32 * i);
+        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(src + L * i);
       }
     }
     if constexpr (GA == 1) {
@@ -349,7 +351,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
       for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int i = 0; i < WPL; ++i)
-          if (r0 + r < rows) reinterpret_cast<int*>(source.copy + (int64_t)(r0 + r) * source.ldcopy)[lane + 32 * i] = w[r][i];
+          if (r0 + r * G < rows) reinterpret_cast<int*>(source.copy + (int64_t)(r0 + r * G) * source.ldcopy)[li + L * i] = w[r][i];
     }
     int my_s1 = 0, my_s2 = 0;
 #pragma unroll
@@ -360,10 +362,18 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
         s1 = __dp4a(w[r][i], 0x01010101, s1);
         s2 = __dp4a(w[r][i], w[r][i], s2);
       }
-      s1 = __reduce_add_sync(0xffffffffu, s1);
-      s2 = __reduce_add_sync(0xffffffffu, s2);
-      my_s1 = lane == r ? s1 : my_s1;
-      my_s2 = lane == r ? s2 : my_s2;
+      if (L == 32) {
+        s1 = __reduce_add_sync(0xffffffffu, s1);
+        s2 = __reduce_add_sync(0xffffffffu, s2);
+      } else {
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) {
+          s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+          s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+      }
+      my_s1 = li == r ? s1 : my_s1;
+      my_s2 = li == r ? s2 : my_s2;
     }
     const int mu = (int)__umulhi((unsigned)(2 * my_s1 + 257 * C), mean_magic) - 128;
     const unsigned V = (unsigned)(my_s2 - 2 * mu * my_s1 + C * mu * mu);
@@ -373,14 +383,14 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
     int Fr[R], muFr[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      Fr[r] = __shfl_sync(0xffffffffu, F, r);
-      muFr[r] = __shfl_sync(0xffffffffu, muF, r);
+      Fr[r] = __shfl_sync(0xffffffffu, F, grp * L + r);
+      muFr[r] = __shfl_sync(0xffffffffu, muF, grp * L + r);
     }
-    int* dst = reinterpret_cast<int*>(out + (int64_t)r0 * ldout) + lane;
+    int* dst = reinterpret_cast<int*>(out + (int64_t)r0 * ldout) + li;
     auto rows_out = [&](auto is_fast) {
 #pragma unroll
       for (int i = 0; i < WPL; ++i) {
-        const int4 m4 = sm_m[lane + 32 * i], s4 = sm_s[lane + 32 * i], b4 = sm_b[lane + 32 * i];
+        const int4 m4 = sm_m[li + L * i], s4 = sm_s[li + L * i], b4 = sm_b[li + L * i];
         const int m[4] = {m4.x, m4.y, m4.z, m4.w}, sh[4] = {s4.x, s4.y, s4.z, s4.w}, be[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -399,7 +409,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
             }
           }
           const int word = (int)pack_sat8_u(v[0], v[1], v[2], v[3]);
-          if (r0 + r < rows) reinterpret_cast<int*>(reinterpret_cast<int8_t*>(dst) + (int64_t)r * ldout)[32 * i] = word;
+          if (r0 + r * G < rows) reinterpret_cast<int*>(reinterpret_cast<int8_t*>(dst) + (int64_t)(r * G) * ldout)[L * i] = word;
         }
       }
     };
@@ -503,15 +513,15 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
   // Up to 1024 rows one row per group of lanes, constants in registers: with so few rows the chain of one warp counts
   // (788 x 384: 1.9 us, shared constants 2.6; 197 x 192: 1.45, four rows 1.8).
   const bool few = rows <= 1024;
-  // Beyond, for whole multiples of 128 channels: constants in shared memory, two blocks per SM, and as many rows per warp
+  // Beyond: constants in shared memory, two blocks per SM, and as many rows per warp
   // as make passes x (1 + rows) least, a pass costing about that (12608 x 384, 5.3 rows per warp: six rows 3.7 us, four 4.9,
   // eight 4.6; 4590 x 384, 1.9 rows per warp: two rows 2.8, six 3.3; 18464 x 1024, 7.8: four rows 9.5, six 10.9).
   const int64_t warps = (int64_t)ctx->sm_count * 16;
-  auto pick = [&](std::initializer_list<int> offered) {
+  auto pick = [&](std::initializer_list<int> offered, int64_t side = 1) {   // side: rows side by side in a warp
     int best = 0;
     int64_t best_cost = 0;
     for (int r : offered) {
-      const int64_t cost = (rows + r * warps - 1) / (r * warps) * (1 + r);
+      const int64_t cost = (rows + r * side * warps - 1) / (r * side * warps) * (1 + r);
       if (!best || cost < best_cost) { best = r; best_cost = cost; }
     }
     return best;
@@ -521,39 +531,45 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
     launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0, ctx->stream, x, ldin, gs, beta, M_ln, out, ldout, (int)rows,
              (int)C, magic, vec, source);
   };
-  auto up_to_six = [&](auto two, auto four, auto six) {
-    const int r = pick({6, 4, 2});
-    if (r == 6) shared(six, 6);
-    else if (r == 4) shared(four, 4);
-    else shared(two, 2);
+  auto up_to_six = [&](auto two, auto four, auto six, int side = 1) {
+    const int r = pick({6, 4, 2}, side);
+    if (r == 6) shared(six, 6 * side);
+    else if (r == 4) shared(four, 4 * side);
+    else shared(two, 2 * side);
   };
   switch (C) {
     case 96:
       if (GA == 2) return false;
-      if constexpr (GA != 2) few ? run(layernorm_rows_kernel<8, 3, 1, 5, true, GA>, 4, 5) : run(layernorm_rows_kernel<8, 3, 4, 5, true, GA>, 16, 5);
+      if constexpr (GA != 2) {
+        if (few) run(layernorm_rows_kernel<8, 3, 1, 5, true, GA>, 4, 5);
+        else up_to_six(layernorm_shared_rows_kernel<8, 3, 2, GA>, layernorm_shared_rows_kernel<8, 3, 4, GA>, layernorm_shared_rows_kernel<8, 3, 6, GA>, 4);
+      }
       return true;
     case 192:
       if (GA == 2) return false;
-      if constexpr (GA != 2) few ? run(layernorm_rows_kernel<16, 3, 1, 5, true, GA>, 2, 5) : run(layernorm_rows_kernel<16, 3, 4, 5, true, GA>, 8, 5);
+      if constexpr (GA != 2) {
+        if (few) run(layernorm_rows_kernel<16, 3, 1, 5, true, GA>, 2, 5);
+        else up_to_six(layernorm_shared_rows_kernel<16, 3, 2, GA>, layernorm_shared_rows_kernel<16, 3, 4, GA>, layernorm_shared_rows_kernel<16, 3, 6, GA>, 2);
+      }
       return true;
     case 384:
       if (few) run(layernorm_rows_kernel<32, 3, 1, 5, true, GA>, 1, 5);
-      else up_to_six(layernorm_shared_rows_kernel<3, 2, GA>, layernorm_shared_rows_kernel<3, 4, GA>, layernorm_shared_rows_kernel<3, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 3, 2, GA>, layernorm_shared_rows_kernel<32, 3, 4, GA>, layernorm_shared_rows_kernel<32, 3, 6, GA>);
       return true;
     case 512:
       if (few) run(layernorm_rows_kernel<32, 4, 1, 4, true, GA>, 1, 4);
-      else up_to_six(layernorm_shared_rows_kernel<4, 2, GA>, layernorm_shared_rows_kernel<4, 4, GA>, layernorm_shared_rows_kernel<4, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 4, 2, GA>, layernorm_shared_rows_kernel<32, 4, 4, GA>, layernorm_shared_rows_kernel<32, 4, 6, GA>);
       return true;
     case 768:
       if (few) run(layernorm_rows_kernel<32, 6, 1, 4, true, GA>, 1, 4);
-      else up_to_six(layernorm_shared_rows_kernel<6, 2, GA>, layernorm_shared_rows_kernel<6, 4, GA>, layernorm_shared_rows_kernel<6, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 6, 2, GA>, layernorm_shared_rows_kernel<32, 6, 4, GA>, layernorm_shared_rows_kernel<32, 6, 6, GA>);
       return true;
     case 1024:
       if (few) run(layernorm_rows_kernel<32, 8, 1, 3, true, GA>, 1, 3);
-      else if (pick({4, 2}) == 4) shared(layernorm_shared_rows_kernel<8, 4, GA>, 4);
-      else shared(layernorm_shared_rows_kernel<8, 2, GA>, 2);
+      else if (pick({4, 2}) == 4) shared(layernorm_shared_rows_kernel<32, 8, 4, GA>, 4);
+      else shared(layernorm_shared_rows_kernel<32, 8, 2, GA>, 2);
       return true;
-    case 1536: shared(layernorm_shared_rows_kernel<12, 2, GA>, 2); return true;
+    case 1536: shared(layernorm_shared_rows_kernel<32, 12, 2, GA>, 2); return true;
   }
   if constexpr (GA == 0) {
     if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);

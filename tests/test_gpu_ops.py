@@ -652,19 +652,20 @@ def test_layernorm_row_counts_and_forms(C):
     assert c.poll_status() == 0
 
 
-@pytest.mark.parametrize("C", [384, 512, 768, 1024, 1536])
+@pytest.mark.parametrize("C", [96, 192, 384, 512, 768, 1024, 1536])
 def test_layernorm_rows_per_warp(C):
     """Beyond 1024 rows a warp takes two, four or six rows at a time, by the number of rows: each of them, in one pass and
     in several, with a last share that is not full; both forms of the constants."""
     g = _g()
     c = g.ctx()
     rng = np.random.default_rng(C + 1)
-    x = rand_i8(rng, (29001, C), std=25)
+    most = 60001 if C < 384 else 29001
+    x = rand_i8(rng, (most, C), std=25)
     ratios = rng.uniform(20, 40, C) * np.sqrt(C) / 2.0 ** 20
     beta = torch.from_numpy(rng.integers(-20, 20, C).astype(np.int32))
     for sc in (scale_channels(ratios), scale_channels(np.where(np.arange(C) == C // 2, 0.3, ratios))):
         want = O.layernorm(x, sc, beta.numpy(), 20)
-        for rows in (1025, 4735, 4738, 9471, 14203, 18945, 29001):
+        for rows in (1025, 4735, 4738, 9471, 14203, 18945, 29001, most):
             got = c.layernorm(g.dev(x[:rows]), g.binding.DevScale(sc, "cuda"), beta.cuda(), 20)
             g.assert_equal(g.host(got), want[:rows], f"rows={rows} C={C}")
     assert c.poll_status() == 0
