@@ -24,6 +24,9 @@
  *    points do not synchronise (ivit_ctx_profile_stop and ivit_ctx_destroy
  *    do).  Device-side failures (a bounded wait that ran out) are
  *    reported by ivit_ctx_poll_status after the stream has been synchronised.
+ *  - Calls on one context take effect in the order in which they are made: any
+ *    operand or parameter array of a call may be written by work that was
+ *    enqueued on the stream before it, an earlier library call included.
  *  - A context belongs to one device; the caller keeps that device current
  *    (cudaSetDevice) while calling into the library with that context.
  *    Kernel attributes are set per device by ivit_ctx_create, so several

@@ -151,6 +151,12 @@ struct LaunchScope {
 // of the stream may be scheduled (and run its set-up) while this one drains.  A kernel therefore
 // calls pdl_wait() before it reads or writes anything another kernel may touch, and pdl_trigger()
 // to let its successor be scheduled early.
+// Only the kernels of one block or model forward read ahead of that wait, and only what the caller's description
+// of the model points to (weights, biases, scales, LayerNorm constants), which no kernel of the forward writes.  The
+// first kernel of a forward triggers after its own wait: whatever was enqueued before the forward, and may have
+// written those parameters, has finished before the forward's second kernel can start.  An operator call
+// (ivit_linear, ivit_matmul, ivit_layernorm, ...) takes any operand from the call before it: it reads nothing
+// ahead of its wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -234,6 +240,8 @@ struct GemmProblem {
   int64_t sCo, sCi;        // batch offsets of out (elements)
   int64_t batches_outer, batches_inner;
   int64_t M, N, K;
+  int b_is_param;          // B, bias and scale belong to the model whose forward this launch is part of: read before the
+                           // wait for the previous kernel.  0: an earlier kernel may still be writing them
   GemmEpilogue epi;
 };
 
@@ -251,8 +259,10 @@ int attention_prepare_device();
 // Fused Q K^T -> requant -> Shiftmax -> P V -> requant; IVIT_ERR_UNSUPPORTED when the shape does not qualify.
 int launch_attention_fused(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O);
 
+// params: gs and beta belong to the model whose forward this launch is part of, and it is not the forward's first
+// (read before the wait for the previous kernel); false: an earlier kernel may still be writing them.
 int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, ScaleDev gs,
-                     const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C);
+                     const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C, bool params);
 // I-LayerNorm of gathered rows: row r is row index[r] (inner: inner[index[r]]) of the input, also copied to `copy`; or
 // (quarters) put together from the rows index[4 r + k], a quarter as wide.  For the widths that layernorm_gathers names.
 bool layernorm_gathers(int64_t rows, int64_t C, bool quarters);

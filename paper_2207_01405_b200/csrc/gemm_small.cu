@@ -4,8 +4,8 @@
 // Such a layer is a chain of latencies: launch, first loads, MMAs, epilogue.  Against the persistent kernel (gemm_tc.cu) the
 // tiles are narrower, so that more SMs share the work and the MMAs and the epilogue of a tile are shorter; there is no
 // tile loop; the output leaves with direct stores instead of staged TMA stores.
-//   warp 0      requests the weight k-blocks (TMA ring), the first ones before the wait for the previous kernel, and the
-//               input rows, which stay resident;
+//   warp 0      requests the weight k-blocks (TMA ring), the first ones of a model's layer before the wait for the previous
+//               kernel, and the input rows, which stay resident;
 //   warp 1      issues the MMAs;
 //   warps 2..17 epilogue: a lane owns one channel, 4x4 byte transposes, direct 4-byte stores.  The residual words are
 //               requested before the MMAs are awaited.
@@ -31,6 +31,7 @@ struct SmallArgs {
   int stages;
   int tmem_cols;
   int p_pos[3], q_pos[3];
+  int b_is_param;                   // see GemmProblem
   int* status;
 };
 
@@ -80,7 +81,8 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
       tma_load_4d_w(base + q_off + kb * q_block, &tmQ, full0 + 8 * s, kb * SM_BK, a.q_pos[0] == 1 ? q0 : 0,
                     a.q_pos[0] == 2 ? q0 : 0, a.q_pos[0] == 3 ? q0 : 0);
     };
-    for (int kb = 0; kb < pre; ++kb) request(kb, kb);   // weights are parameters: before the wait for the previous kernel
+    if (!a.b_is_param) pdl_wait();
+    for (int kb = 0; kb < pre; ++kb) request(kb, kb);   // weights of a model: before the wait for the previous kernel
     pdl_wait();
     for (int kb = 0; kb < pre; ++kb) request_q(kb, kb);
     int s = 0;
@@ -119,7 +121,8 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
   } else {
     // ---------------- epilogue ----------------
     const GemmEpilogue& e = a.epi;
-    // constants of this thread's channel (parameters: before the wait)
+    // constants of this thread's channel (parameters of a model: before the wait)
+    if (!a.b_is_param) pdl_wait();
     const int qd = warp & 3;            // TMEM lane quarter
     const int c = p0 + qd * 32 + lane, cbase = c & ~3;
     const bool cg_ok = cbase < a.P;     // P % 4 == 0: a group of four channels is valid as a whole
@@ -257,6 +260,7 @@ int launch_gemm_small(ivit_ctx* ctx, const GemmProblem& g) {
   if (a.stages > kblocks) a.stages = kblocks;
   a.epi = e;
   a.P = (int)g.N; a.Q = (int)g.M; a.K = (int)g.K;
+  a.b_is_param = g.b_is_param;
   a.status = ctx->status_dev;
   a.tmem_cols = 32;
   while (a.tmem_cols < a.BN) a.tmem_cols <<= 1;

@@ -155,6 +155,7 @@ struct TcArgs {
                      // weight rows and half of the activation rows; tiles_p then counts channel PAIRS of tiles
   int q_resident;    // Dense orientation, short K: all k-blocks of the Q (activation row) tile stay in shared
                      // memory while the CTA walks the channel blocks; only weight tiles stream through the ring
+  int b_is_param;    // see GemmProblem
   RowOpArgs rop;     // row operator on finished blocks of output rows (Dense orientation, staged int8 output)
   int* status;
 };
@@ -393,11 +394,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         if (PAIR) tma_load_4d_pair_w(dst, map, mapa_rank0(bar), c0, c1, c2, c3);
         else tma_load_4d_w(dst, map, bar, c0, c1, c2, c3);
       };
-      // Dense orientation: the P operand is the weight matrix, which no kernel writes.  The weight k-blocks of the
-      // first tile are requested before the wait for the previous kernel (whose last CTAs may still be running
-      // elsewhere); the activation k-blocks that complete the same stage barriers follow after the wait.
+      // Dense layer of a model: the P operand is the weight matrix, which no kernel of the forward writes.  The weight
+      // k-blocks of the first tile are requested before the wait for the previous kernel (whose last CTAs may still be
+      // running elsewhere); the activation k-blocks that complete the same stage barriers follow after the wait.
       int pre = 0;
-      if (a.lanes_are_channels && t_begin < t_end) {
+      if (a.b_is_param && a.lanes_are_channels && t_begin < t_end) {
         pre = kblocks < a.stages ? kblocks : a.stages;
         for (int kb = 0; kb < pre; ++kb) {
           arm(full0 + 8 * kb, BM * BK + (ti.last(a) ? a.q_last_bytes : a.q_stage_bytes));
@@ -1159,6 +1160,7 @@ int launch_gemm_tc(ivit_ctx* ctx, const GemmProblem& g) {
   a.res_rows = e.res_rows > 2147483647LL ? 2147483647 : (int)e.res_rows;
   a.group_rows = e.group_rows > 2147483647LL ? 2147483647 : (int)e.group_rows;
   a.K = (int)g.K; a.sCo = g.sCo; a.sCi = g.sCi; a.batches_inner = (int)g.batches_inner;
+  a.b_is_param = g.b_is_param;
   a.status = ctx->status_dev;
   CUtensorMap tmP, tmQ;
   const bool dense = g.transB && batches == 1 && !e.bias32;

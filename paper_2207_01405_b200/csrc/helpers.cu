@@ -55,8 +55,8 @@ struct FillRows {
 // One thread per 4 output bytes (px .. px+3 of one patch row); P % 4 == 0.
 __global__ void patchify_kernel(const int8_t* __restrict__ img, int64_t B, int C, int Hi, int Wi, int P,
                                 int window, int8_t* __restrict__ out, int64_t ldout, int64_t total_words) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: the first kernel of a forward)
   const int gh = Hi / P, gw = Wi / P;
   const int kw = C * P * P / 4;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total_words;
@@ -84,8 +84,8 @@ __global__ void patchify_kernel(const int8_t* __restrict__ img, int64_t B, int C
 __global__ void patchify_vec_kernel(const int8_t* __restrict__ img, FastDiv per_row, FastDiv Hi, FastDiv C, FastDiv segs, FastDiv P,
                                     PatchOrder order, unsigned patches, int8_t* __restrict__ out, int64_t ldout,
                                     unsigned total_vecs, FillRows fill) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: the first kernel of a forward)
   const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
   for (unsigned t = t0; t < total_vecs; t += stride) {
     // t enumerates the image in memory order: consecutive threads read consecutive 16-byte pieces
@@ -103,8 +103,8 @@ __global__ void patchify_vec_kernel(const int8_t* __restrict__ img, FastDiv per_
 // 16 bytes per channel.  64 images of 224 x 224 x 3, back to back: 26.5 -> 4.9 us (one word per thread, 64-bit divisions).
 __global__ void patchify4_kernel(const int8_t* __restrict__ img, int C, int Hi, int Wi, FastDiv gw, FastDiv gh, PatchOrder order,
                                  int8_t* __restrict__ out, int64_t ldout, unsigned total_patches) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: the first kernel of a forward)
   const unsigned patches = gw.d * gh.d;
   for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < total_patches; t += gridDim.x * blockDim.x) {
     unsigned gx, gy;
@@ -139,8 +139,8 @@ __global__ void gather_rows_kernel(const int8_t* __restrict__ src, int64_t ldsrc
 }
 
 __global__ void fill_rows_kernel(FillRows fill) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: the first kernel of a forward)
   fill.run(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 

@@ -67,6 +67,7 @@ int check_block(const ivit_block_params* p) {
   return check_exp(p->gelu, p->H, true);
 }
 
+// A Dense layer of a model: W, bias and scale are the model's (b_is_param).
 GemmProblem linear_problem(const int8_t* A, int64_t lda, const int8_t* W, int64_t ldw, const int32_t* bias,
                            ivit_scale scale, const int8_t* res, int64_t ldres, int64_t res_rows,
                            ivit_scale res_scale, void* out, int64_t ldo, int out_dtype, int64_t group_rows,
@@ -75,6 +76,7 @@ GemmProblem linear_problem(const int8_t* A, int64_t lda, const int8_t* W, int64_
   g.A = A; g.lda = lda; g.B = W; g.ldb = ldw; g.transB = 1;
   g.batches_outer = g.batches_inner = 1;
   g.M = M; g.N = N; g.K = K;
+  g.b_is_param = 1;
   g.epi.bias = bias;
   g.epi.bias32 = nullptr; g.epi.ldbias = 0; g.epi.bias_batches = 1;
   g.epi.scale = to_dev(scale);
@@ -132,7 +134,8 @@ void want_layernorm(GemmProblem& g, const ivit_scale& gamma, const int32_t* beta
 // layer produced it); next: the block that follows on Y with the same shape, or nullptr - its LayerNorm 1 is then
 // run in the tail of this block's last Dense layer, where that is possible.  *a_next_ready tells the caller whether
 // it was.  Row operators that a Dense kernel cannot take on run as kernels of their own, with the same result.
-int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_t* Y, char* ws, bool a_ready = false,
+// first: the block is a forward of its own, whose first kernel reads no parameter ahead of its wait.
+int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_t* Y, char* ws, bool first, bool a_ready = false,
                const ivit_block_params* next = nullptr, bool* a_next_ready = nullptr) {
   const BlockWs w = block_ws(p);
   const int64_t M = p->B * p->T, D = p->D, H = p->H;
@@ -145,7 +148,7 @@ int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_
   int rc;
   if (a_next_ready) *a_next_ready = false;
   // X^ = MSA(LayerNorm(X)) + X
-  if (!a_ready && (rc = launch_layernorm(ctx, X, IVIT_I8, D, to_dev(p->ln1_gamma), p->ln1_beta, p->M_ln, A, D, M, D))) return rc;
+  if (!a_ready && (rc = launch_layernorm(ctx, X, IVIT_I8, D, to_dev(p->ln1_gamma), p->ln1_beta, p->M_ln, A, D, M, D, !first))) return rc;
   if ((rc = launch_gemm(ctx, linear_problem(A, D, p->Wqkv, D, p->bqkv, p->qkv_scale, nullptr, 0, 1, none, QKV, 3 * D,
                                             IVIT_I8, 0, 0, M, 3 * D, D)))) return rc;
   if ((rc = attention_impl(ctx, p, QKV, O, ws, w))) return rc;
@@ -156,7 +159,7 @@ int block_impl(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* X, int8_
   if ((rc = launch_gemm(ctx, proj))) return rc;
   // Y = MLP(LayerNorm(X^)) + X^
   if (!ctx->rowop_fused &&
-      (rc = launch_layernorm(ctx, Xh, IVIT_I8, D, to_dev(p->ln2_gamma), p->ln2_beta, p->M_ln, A, D, M, D))) return rc;
+      (rc = launch_layernorm(ctx, Xh, IVIT_I8, D, to_dev(p->ln2_gamma), p->ln2_beta, p->M_ln, A, D, M, D, true))) return rc;
   GemmProblem fc1 = linear_problem(A, D, p->W1, D, p->b1, p->fc1_scale, nullptr, 0, 1, none, G, H, IVIT_I8, 0, 0, M, H, D);
   if (p->gelu_static_max) {
     // static-maximum ShiftGELU variant: element-wise, applied to the requantised value inside the FC1 epilogue
@@ -542,8 +545,10 @@ int ivit_linear(ivit_ctx* ctx, const int8_t* A, int64_t lda, const int8_t* W, in
     if (!aligned16(res) || ldres % 16) return IVIT_ERR_ALIGNMENT;
   }
   if (out_group_rows > 0 && out_group_stride < out_group_rows) return IVIT_ERR_INVALID_ARG;
-  return launch_gemm(ctx, linear_problem(A, lda, W, ldw, bias, scale, res, ldres, res_rows, res_scale, out, ldo,
-                                         out_dtype, out_group_rows, out_group_stride, M, N, K));
+  GemmProblem g = linear_problem(A, lda, W, ldw, bias, scale, res, ldres, res_rows, res_scale, out, ldo, out_dtype,
+                                 out_group_rows, out_group_stride, M, N, K);
+  g.b_is_param = 0;   // W, bias and scale may come from the call before this one
+  return launch_gemm(ctx, g);
 }
 
 int ivit_matmul(ivit_ctx* ctx, const int8_t* A, int64_t lda, int64_t sAo, int64_t sAi,
@@ -637,7 +642,7 @@ int ivit_layernorm(ivit_ctx* ctx, const void* in, int32_t in_dtype, int64_t ldin
   if (ldin < C || ldout < C) return IVIT_ERR_INVALID_ARG;
   if (!aligned16(in) || !aligned16(out) || ldout % 16 || ldin % (in_dtype == IVIT_I8 ? 16 : 4)) return IVIT_ERR_ALIGNMENT;
   if (!scale_ok(gamma_scale)) return IVIT_ERR_RANGE;
-  return launch_layernorm(ctx, in, in_dtype, ldin, to_dev(gamma_scale), beta, M_ln, out, ldout, rows, C);
+  return launch_layernorm(ctx, in, in_dtype, ldin, to_dev(gamma_scale), beta, M_ln, out, ldout, rows, C, false);
 }
 
 size_t ivit_block_workspace_bytes(const ivit_block_params* p) {
@@ -653,7 +658,7 @@ int ivit_block_forward(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* 
   if (!aligned16(X) || !aligned16(Y)) return IVIT_ERR_ALIGNMENT;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < block_ws(p).total)
     return IVIT_ERR_WORKSPACE;
-  return block_impl(ctx, p, X, Y, static_cast<char*>(workspace));
+  return block_impl(ctx, p, X, Y, static_cast<char*>(workspace), true);
 }
 
 // Scratch of ivit_block_forward_static: part of the library image, present on every GPU that loads it.
@@ -681,7 +686,7 @@ int ivit_block_forward_static(ivit_ctx* ctx, const ivit_block_params* p, const i
     if (err != cudaSuccess || !ptr) return IVIT_ERR_CUDA;
     scratch_of_device[ctx->device] = ptr;
   }
-  return block_impl(ctx, p, X, Y, static_cast<char*>(scratch_of_device[ctx->device]));
+  return block_impl(ctx, p, X, Y, static_cast<char*>(scratch_of_device[ctx->device]), true);
 }
 
 int ivit_attention(ivit_ctx* ctx, const ivit_block_params* p, const int8_t* QKV, int8_t* O,
@@ -766,13 +771,13 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
   bool a_ready = false;   // LayerNorm 1 of the next block already produced by the previous block's last Dense layer
   for (int64_t l = 0; l < p->depth; ++l) {
     const ivit_block_params* next = l + 1 < p->depth ? &p->blocks[l + 1] : nullptr;
-    if ((rc = block_impl(ctx, &p->blocks[l], X, Y, ws + w.block, a_ready, next, &a_ready))) return rc;
+    if ((rc = block_impl(ctx, &p->blocks[l], X, Y, ws + w.block, false, a_ready, next, &a_ready))) return rc;
     int8_t* t = X; X = Y; Y = t;
   }
   if (tokens && cudaMemcpyAsync(tokens, X, (size_t)(B * T * D), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
     return IVIT_ERR_CUDA;
   // final LayerNorm on the class-token rows, then the classifier (int32 logits, not saturated)
-  if ((rc = launch_layernorm(ctx, X, IVIT_I8, T * D, to_dev(p->lnf_gamma), p->lnf_beta, p->blocks[0].M_ln, Z, D, B, D))) return rc;
+  if ((rc = launch_layernorm(ctx, X, IVIT_I8, T * D, to_dev(p->lnf_gamma), p->lnf_beta, p->blocks[0].M_ln, Z, D, B, D, true))) return rc;
   return launch_gemm(ctx, linear_problem(Z, D, p->Whead, D, p->bhead, p->head_scale, nullptr, 0, 1, none, logits,
                                          p->classes, IVIT_I32, 0, 0, B, p->classes, D));
 }
@@ -855,7 +860,7 @@ static int dense_then_layernorm(ivit_ctx* ctx, GemmProblem g, const ivit_scale& 
   int rc = launch_gemm(ctx, g);
   if (rc) return rc;
   if (ctx->rowop_fused) return IVIT_OK;
-  return launch_layernorm(ctx, g.epi.out, IVIT_I8, g.epi.ldo, to_dev(gamma), beta, M_ln, ln_out, N, M, N);
+  return launch_layernorm(ctx, g.epi.out, IVIT_I8, g.epi.ldo, to_dev(gamma), beta, M_ln, ln_out, N, M, N, true);
 }
 
 int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* image, int32_t* logits,
@@ -903,16 +908,16 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
       if (gathers && (sh || order)) {
         if ((rc = launch_layernorm_gather(ctx, cur, C, sh ? st->shift_index : order, sh ? order : nullptr, false, to_dev(blk->ln1_gamma),
                                           blk->ln1_beta, blk->M_ln, third, C, reinterpret_cast<int8_t*>(wsb), C, rows, C))) return rc;
-        if ((rc = block_impl(ctx, blk, third, other, wsb, true, sh ? nullptr : next, &a_ready))) return rc;
+        if ((rc = block_impl(ctx, blk, third, other, wsb, false, true, sh ? nullptr : next, &a_ready))) return rc;
         int8_t* t = cur; cur = other; other = t;
         order = sh ? st->unshift_index : nullptr;
       } else if (sh) {
         if ((rc = launch_gather_rows(ctx, cur, C, st->shift_index, rows, C, third, C))) return rc;
-        if ((rc = block_impl(ctx, blk, third, other, wsb, false, nullptr, nullptr))) return rc;
+        if ((rc = block_impl(ctx, blk, third, other, wsb, false, false, nullptr, nullptr))) return rc;
         if ((rc = launch_gather_rows(ctx, other, C, st->unshift_index, rows, C, cur, C))) return rc;
         a_ready = false;
       } else {
-        if ((rc = block_impl(ctx, blk, cur, other, wsb, a_ready, next, &a_ready))) return rc;
+        if ((rc = block_impl(ctx, blk, cur, other, wsb, false, a_ready, next, &a_ready))) return rc;
         int8_t* t = cur; cur = other; other = t;
       }
     }
@@ -929,7 +934,7 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
         }
         if ((rc = launch_gather_rows(ctx, cur, C, st->merge_index, rows, C, other, C))) return rc;
         if ((rc = launch_layernorm(ctx, other, IVIT_I8, 4 * C, to_dev(st->merge_ln_gamma), st->merge_ln_beta, p->M_ln, third,
-                                   4 * C, merged, 4 * C))) return rc;
+                                   4 * C, merged, 4 * C, true))) return rc;
       }
       order = nullptr;
       rows = merged;
@@ -951,7 +956,7 @@ int ivit_swin_forward(ivit_ctx* ctx, const ivit_swin_params* p, const int8_t* im
     return IVIT_ERR_CUDA;
   const int8_t* normed = reinterpret_cast<const int8_t*>(wsb);
   if (!a_ready) {
-    if ((rc = launch_layernorm(ctx, cur, IVIT_I8, Cl, to_dev(p->lnf_gamma), p->lnf_beta, p->M_ln, other, Cl, rows, Cl))) return rc;
+    if ((rc = launch_layernorm(ctx, cur, IVIT_I8, Cl, to_dev(p->lnf_gamma), p->lnf_beta, p->M_ln, other, Cl, rows, Cl, true))) return rc;
     normed = other;
   }
   if ((rc = launch_token_mean(ctx, normed, Cl, B, rows / (B > 0 ? B : 1), Cl, to_dev(p->pool_scale), Z, Cl))) return rc;

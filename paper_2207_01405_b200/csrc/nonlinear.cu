@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
                                                            ScaleDev gs, const int32_t* __restrict__ beta,
                                                            int M_ln, int8_t* __restrict__ out, int64_t ldout,
                                                            int64_t rows, int C) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: it may be the first kernel of a forward)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
 }
 
 // Rows of up to 1024 channels.  L lanes share a row (G = 32 / L rows side by side in a warp), a lane holds WPL words of four
-// channels of R such rows, and the constants of its channels in registers (fetched before the wait for the previous
-// kernel: they are parameters).  kExact: C = 4 L WPL, nothing to mask.  Rows past the end are read as the last row and not
+// channels of R such rows, and the constants of its channels in registers (inside a forward fetched before the wait for
+// the previous kernel).  kExact: C = 4 L WPL, nothing to mask.  Rows past the end are read as the last row and not
 // stored: the body has no branch but the one on the form of the constants.  What bounds it is instruction issue: byte,
 // multiply-add, mad.hi, shift and half a pack per value, and about 130 instructions for the scalars of G R rows at once.
 // With a branch around every word and row and one row per 32 lanes, three of four instructions were overhead.  Measured, back
@@ -203,10 +203,11 @@ template <int L, int WPL, int R, int PER_SM, bool kExact, int GA = 0>
 __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
                                                                      const int32_t* __restrict__ beta, int M_ln,
                                                                      int8_t* __restrict__ out, int64_t ldout, int rows, int C,
-                                                                     unsigned mean_magic, int vec, LnSource<GA> source) {
+                                                                     unsigned mean_magic, int vec, int params, LnSource<GA> source) {
   static_assert(GA == 0 || kExact, "whole rows");
   static_assert(R <= L, "a lane per row for the scalars");
   constexpr int G = 32 / L;
+  if (!params) pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
   const int nwords = kExact ? L * WPL : C >> 2;
@@ -309,15 +310,18 @@ __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_
 // so that most launches are one or two passes, and twice the warps are in flight.  Bound by issue and by the chain of the
 // scalars of a pass.  Measured, back to back, against constants in registers: 18464 x 1024 12.4 -> 9.5 us, 9232 x 1024 8.4 ->
 // 5.4, 25216 x 768 11.3 -> 10.6, 12608 x 768 7.1 -> 5.8, 12608 x 384 4.2 -> 3.7, 3136 x 1536 9.0 -> 4.2, 12544 x 192
-// 3.65 -> 3.1, 200704 x 96 12.4 -> 11.9.
+// 3.65 -> 3.1, 200704 x 96 12.4 -> 11.9.  These are
+// launches inside a forward; an operator call, whose constants are fetched behind the wait, takes about 0.9 us longer
+// (25216 x 768 12.4 us; the first rows requested ahead of the constants: 12.5).
 template <int L, int WPL, int R, int GA = 0>
 __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
                                                                             const int32_t* __restrict__ beta, int M_ln,
                                                                             int8_t* __restrict__ out, int64_t ldout, int rows, int C,
-                                                                            unsigned mean_magic, int vec, LnSource<GA> source) {
+                                                                            unsigned mean_magic, int vec, int params, LnSource<GA> source) {
   static_assert(R <= L, "a lane per row for the scalars");
   constexpr int G = 32 / L, kWords = L * WPL;
   __shared__ int4 sm_m[kWords], sm_s[kWords], sm_b[kWords];
+  if (!params) pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
   const bool fast = __syncthreads_and(ln_stage_consts(gs, beta, kWords, vec, sm_m, sm_s, sm_b, threadIdx.x, 256)) != 0;
@@ -423,8 +427,8 @@ __global__ void __launch_bounds__(256) layernorm_i8_long_kernel(const int8_t* __
                                                                 ScaleDev gs, const int32_t* __restrict__ beta,
                                                                 int M_ln, int8_t* __restrict__ out,
                                                                 int64_t ldout, int64_t rows, int C) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: it may be the first kernel of a forward)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -465,8 +469,8 @@ __global__ void __launch_bounds__(256) layernorm_i32_kernel(const int32_t* __res
                                                             ScaleDev gs, const int32_t* __restrict__ beta,
                                                             int M_ln, int8_t* __restrict__ out, int64_t ldout,
                                                             int64_t rows, int C) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();   // (after the wait: it may be the first kernel of a forward)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -498,7 +502,7 @@ __global__ void __launch_bounds__(256) layernorm_i32_kernel(const int32_t* __res
 // layernorm_rows_kernel for int8 rows of C channels; false: no form for that width.
 template <int GA>
 static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDev gs, const int32_t* beta, int M_ln, int8_t* out,
-                           int64_t ldout, int64_t rows, int64_t C, LnSource<GA> source) {
+                           int64_t ldout, int64_t rows, int64_t C, bool params, LnSource<GA> source) {
   if (rows >= (1ll << 31) / (GA == 2 ? 4 : 1) - (1 << 20)) return false;
   const int wpl = (int)((C / 4 + 31) / 32);
   const unsigned magic = (unsigned)(0x100000000ull / (unsigned long long)(2 * C)) + 1u;
@@ -508,7 +512,7 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
   auto run = [&](auto kernel, int rpw, int per_sm) {
     const int64_t blocks = (rows + 4 * rpw - 1) / (4 * rpw), cap = (int64_t)ctx->sm_count * per_sm;
     launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(128), 0, ctx->stream, x, ldin, gs, beta, M_ln, out, ldout, (int)rows,
-             (int)C, magic, vec, source);
+             (int)C, magic, vec, (int)params, source);
   };
   // Up to 1024 rows one row per group of lanes, constants in registers: with so few rows the chain of one warp counts
   // (788 x 384: 1.9 us, shared constants 2.6; 197 x 192: 1.45, four rows 1.8).
@@ -529,7 +533,7 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
   auto shared = [&](auto kernel, int rpw) {
     const int64_t blocks = (rows + 8 * rpw - 1) / (8 * rpw), cap = (int64_t)ctx->sm_count * 2;
     launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(256), 0, ctx->stream, x, ldin, gs, beta, M_ln, out, ldout, (int)rows,
-             (int)C, magic, vec, source);
+             (int)C, magic, vec, (int)params, source);
   };
   auto up_to_six = [&](auto two, auto four, auto six, int side = 1) {
     const int r = pick({6, 4, 2}, side);
@@ -583,7 +587,7 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
 }
 
 int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, ScaleDev gs,
-                     const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C) {
+                     const int32_t* beta, int M_ln, int8_t* out, int64_t ldout, int64_t rows, int64_t C, bool params) {
   if (rows == 0) return IVIT_OK;
   const int threads = 256, wpb = threads / 32;
   const int64_t want = (rows + wpb - 1) / wpb;
@@ -596,7 +600,7 @@ int launch_layernorm(ivit_ctx* ctx, const void* in, int in_dtype, int64_t ldin, 
   }
   const int8_t* x = (const int8_t*)in;
   const int wpl = (int)((C / 4 + 31) / 32);
-  if (layernorm_rows<0>(ctx, x, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<0>{})) return ls.done();
+  if (layernorm_rows<0>(ctx, x, ldin, gs, beta, M_ln, out, ldout, rows, C, params, LnSource<0>{})) return ls.done();
   if (wpl <= 12) launch_k(layernorm_i8_kernel<12>, dim3(grid), dim3(threads), 0, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C);
   else launch_k(layernorm_i8_long_kernel, dim3(grid), dim3(threads), 0, st, x, ldin, gs, beta, M_ln, out, ldout, rows, (int)C);
   return ls.done();
@@ -607,8 +611,8 @@ int launch_layernorm_gather(ivit_ctx* ctx, const int8_t* in, int64_t ldin, const
                             int64_t rows, int64_t C) {
   if (rows == 0) return IVIT_OK;
   LaunchScope ls(ctx, KIND_LAYERNORM, (double)rows * (double)C * (quarters ? 2.0 : 3.0));
-  const bool done = quarters ? layernorm_rows<2>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<2>{index, inner, nullptr, 0})
-                             : layernorm_rows<1>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, LnSource<1>{index, inner, copy, ldcopy});
+  const bool done = quarters ? layernorm_rows<2>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, true, LnSource<2>{index, inner, nullptr, 0})
+                             : layernorm_rows<1>(ctx, in, ldin, gs, beta, M_ln, out, ldout, rows, C, true, LnSource<1>{index, inner, copy, ldcopy});
   return done ? ls.done() : IVIT_ERR_UNSUPPORTED;
 }
 
