@@ -15,6 +15,7 @@
 // V is consumed as stored ([token, d] rows, MN-major B operand).  Every wait is bounded.
 // What bounds the passes: issue slots.  mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer
 // instructions two cycles of their pipe, a look-up one of the SM's shared-memory cycles.
+#include "handover.cuh"
 #include "shiftmax.cuh"
 #include "tc_ptx.cuh"
 #include <cstdlib>
@@ -76,6 +77,10 @@ struct __align__(16) AttnItem {
 // Named barriers: id, number of threads that arrive or wait.
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+template <int kThreads>
+struct BlockBarriers {
+  __device__ __forceinline__ void sync(int id) const { bar_sync(id, kThreads); }
+};
 
 // Tile load by a converged warp; pos: which coordinate of the map (1..3) carries the row, the head and the image or window.
 __device__ __forceinline__ void load_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, const int (&pos)[3], int row, int h, int b) {
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
         // Q and K may be overwritten once the score MMAs have read them
         ok = mbar_wait_warp(bar_s, par, a.status);
         if (!ok) break;
-        bar_arrive(6, kShortThreads);   // scores and item are there
+        bar_arrive(kBarScores, kShortThreads);
         scores_out = true;
         if (more) { load_qk(next); qk_flying = true; qk_par = par ^ 1u; }
         // O = P V once the probabilities are in shared memory and V has landed
@@ -302,21 +307,17 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
         // V may be overwritten once these MMAs have read it
         ok = mbar_wait_warp(bar_o, par, a.status);
         if (!ok) break;
-        bar_arrive(7, kShortThreads);   // the output is there
+        bar_arrive(kBarOutput, kShortThreads);
         ++done;
         scores_out = false;
         if (more) { load_v(next); v_flying = true; v_par = par ^ 1u; }
         cur = next;
       }
       if (!ok) {
-        // A wait ran out: the Shiftmax threads, told by the flag, walk on through their barriers without work.  (`done`
-        // items have been released twice; of the one at which the wait ran out the scores may have been released.)
+        // a wait ran out: see walk_out
         if (lane == 0) *dead = 1;
         __syncwarp();
-        for (uint32_t n = done; n < n_items; ++n) {
-          if (n > done || !scores_out) bar_arrive(6, kShortThreads);
-          bar_arrive(7, kShortThreads);
-        }
+        walk_out(BlockBarriers<kShortThreads>{}, done, n_items, scores_out);
       }
       // nothing may be in flight at exit
       if (qk_flying) mbar_wait_warp(bar_qk, qk_par, a.status);
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       const uint32_t par = n & 1u;
       // The control warp alone polls the barriers of the MMAs; the others wait in hardware barriers (eight polling warps
       // per CTA issued a third of the kernel's instructions).
-      bar_sync(6, kShortThreads);
+      bar_sync(kBarScores, kShortThreads);
       alive = *dead == 0;
       const AttnItem item = item_ring[par];
       const int b = kPack ? item.b + slot : item.b;          // image / window of this row
@@ -527,7 +528,7 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);
       // ---- output, heads concatenated along the feature dimension ----
-      bar_sync(7, kShortThreads);
+      bar_sync(kBarOutput, kShortThreads);
       alive = alive && *dead == 0;
       if (work && alive) {
         tc_fence_after();
