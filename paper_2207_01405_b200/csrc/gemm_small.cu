@@ -13,6 +13,7 @@
 // 7.6 -> 4.6, 197 x 768 x 3072 10.7 -> 6.2, 1576 x 384 x 1536 5.6 -> 5.0.  LayerNorm and ShiftGELU computed here, in front
 // of the MMAs, instead of in kernels of their own were slower on every batch size (four DeiT-T blocks of one image 154
 // against 130 us): the row kernels' launches overlap their neighbours', the prologue does not.
+#include "ring.cuh"
 #include "tc_ptx.cuh"
 
 namespace ivit {
@@ -85,14 +86,16 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
     for (int kb = 0; kb < pre; ++kb) request(kb, kb);   // weights of a model: before the wait for the previous kernel
     pdl_wait();
     for (int kb = 0; kb < pre; ++kb) request_q(kb, kb);
-    int s = 0;
+    int s = 0, requested = pre;
     uint32_t par = 0;
-    for (int kb = pre; kb < kblocks; ++kb) {
+    for (; requested < kblocks; ++requested) {
       if (!mbar_wait_warp(empty0 + 8 * s, par, a.status)) break;
-      request(s, kb);
-      request_q(s, kb);
+      request(s, requested);
+      request_q(s, requested);
       if (++s == a.stages) { s = 0; par ^= 1u; }
     }
+    // nothing that was requested may be in flight at exit, also when the MMA warp gave up before it was through
+    drain_ring(requested, a.stages, [&](int stage, uint32_t parity) { mbar_wait_warp(full0 + 8 * stage, parity, a.status); });
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.BN >> 3) << 17) | ((uint32_t)(SM_BM >> 4) << 24);
@@ -114,10 +117,6 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
       if (++s == a.stages) { s = 0; par ^= 1u; }
     }
     umma_commit_w(accf);
-    if (!ok) {
-      // after a timeout: nothing that was requested may be in flight at exit (waits that run out end the drain)
-      for (int i = 0; i < a.stages; ++i) mbar_wait_warp(full0 + 8 * i, 0, a.status);
-    }
   } else {
     // ---------------- epilogue ----------------
     const GemmEpilogue& e = a.epi;
