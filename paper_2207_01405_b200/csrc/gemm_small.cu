@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
     drain_ring(requested, a.stages, [&](int stage, uint32_t parity) { mbar_wait_warp(full0 + 8 * stage, parity, a.status); });
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
+    pdl_wait();   // the previous kernel's time does not count against the limit of the polls below
     const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.BN >> 3) << 17) | ((uint32_t)(SM_BM >> 4) << 24);
     const uint32_t hi = desc_hi(1024, 2), p_lo0 = desc_lo(base, 16), q_lo0 = desc_lo(base + q_off, 16);
     const int tail_steps = (a.K - (kblocks - 1) * SM_BK + 31) / 32;

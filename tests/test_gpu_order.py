@@ -166,3 +166,28 @@ def test_forwards_see_parameters_written_by_the_call_before():
         logits = c.vit_forward(dm, dimg, workspace=ws)
         g.assert_equal(g.host(logits), want_m, f"model {k}")
     assert c.poll_status() == 0
+
+
+def test_small_dense_layer_behind_a_long_kernel():
+    """The limit of a kernel's own waits does not run while the kernel in front of it does: a CUDA-core product of some
+    tenths of a second, then a layer of one wave that reads its output."""
+    g = _g()
+    c = g.ctx()
+    n, K = 8192, 65536
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    A, W = (torch.randint(-128, 128, (n, K), dtype=torch.int8, device="cuda", generator=gen) for _ in range(2))
+    ds = g.binding.DevScale(Scale(*dyadic(30.0 / (np.sqrt(K) * 74.0 ** 2))), "cuda")
+    rng = np.random.default_rng(4)
+    W2 = rand_i8(rng, (128, n))
+    s2 = Scale(*dyadic(30.0 / (np.sqrt(n) * 900)))
+    dW2, ds2 = g.dev(W2), g.binding.DevScale(s2, "cuda")
+    long_out = torch.zeros((n, n), dtype=torch.int8, device="cuda")
+    torch.cuda.synchronize()
+    c.set_gemm_engine(1)
+    c.linear(A, W, None, ds, out=long_out)
+    c.set_gemm_engine(0)
+    got = g.host(c.linear(long_out[:64], dW2, None, ds2))
+    assert c.poll_status() == 0
+    x = g.host(long_out[:64])
+    assert len(np.unique(x)) > 100
+    g.assert_equal(got, O.linear(x, W2, None, s2), "layer behind a long kernel")
