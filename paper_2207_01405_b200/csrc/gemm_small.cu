@@ -259,6 +259,7 @@ int launch_gemm_small(ivit_ctx* ctx, const GemmProblem& g) {
   if (a.stages > kSmallStages) a.stages = kSmallStages;
   if (a.stages > kblocks) a.stages = kblocks;
   a.epi = e;
+  if (e.group_rows > g.M) a.epi.group_rows = g.M;   // one group (the kernel divides 32-bit row numbers)
   a.P = (int)g.N; a.Q = (int)g.M; a.K = (int)g.K;
   a.b_is_param = g.b_is_param;
   a.status = ctx->status_dev;

@@ -99,6 +99,22 @@ def test_linear_residual_full_rows(M, N, K):
     assert c.poll_status() == 0
 
 
+@pytest.mark.parametrize("M,N,K", [(70, 64, 48), (9500, 512, 64)])
+@pytest.mark.parametrize("group", [1 << 32, (1 << 32) + 20, (1 << 40) + 33, 1 << 31])
+def test_linear_group_larger_than_the_rows(M, N, K, group):
+    """Groups of more rows than there are (more than 32 bits count, too) are one group: the rows stay where they are."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(M + N + K)
+    A, W = rand_i8(rng, (M, K)), rand_i8(rng, (N, K))
+    scale = scale_channels(rng.uniform(20, 60, N) / (np.sqrt(K) * 40 * 40))
+    res, rs = rand_i8(rng, (M, N)), Scale(*dyadic(0.9))
+    ds, drs = g.binding.DevScale(scale, "cuda"), g.binding.DevScale(rs, "cuda")
+    got = c.linear(g.dev(A), g.dev(W), None, ds, res=g.dev(res), res_scale=drs, out_group_rows=group, out_group_stride=group + 5)
+    g.assert_equal(g.host(got), O.linear(A, W, None, scale, res=res, res_scale=rs), "one group")
+    assert c.poll_status() == 0
+
+
 @pytest.mark.parametrize("M,N,K,with_res", [(9500, 512, 1024, False), (19000, 256, 1536, True), (9477, 512, 1600, True),
                                             (6400, 768, 1024, False), (4800, 1024, 3072, True)])
 def test_linear_cta_pairs(M, N, K, with_res):
