@@ -29,6 +29,7 @@
 #include "tc_ptx.cuh"
 #include <cstring>
 #include <new>
+#include "residual_rows.cuh"
 #include "rowops.cuh"
 
 namespace ivit {
@@ -625,12 +626,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     auto group_fetch = [&]() {
       if (pf_t >= t_end) return;
       const int c = pf_ti.p0() + c_first + 4 * (lane & 7);
-      int rr = (int)((uint32_t)(pf_ti.q0(a) + 32 * pf_ck) % (uint32_t)a.res_rows) + (lane >> 3);   // (res_rows >= 32)
+      const int row0 = pf_ti.q0(a) + 32 * pf_ck, first = (int)((uint32_t)row0 % (uint32_t)a.res_rows);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        if (rr >= a.res_rows) rr -= a.res_rows;
-        rw[k] = c < a.P ? __ldg(reinterpret_cast<const uint32_t*>(e.res + (int64_t)rr * e.ldres + c)) : 0u;
-        rr += 4;
+        const int rr = residual_row(row0, first, (lane >> 3) + 4 * k, a.Q, a.res_rows);
+        rw[k] = c < a.P && rr >= 0 ? __ldg(reinterpret_cast<const uint32_t*>(e.res + (int64_t)rr * e.ldres + c)) : 0u;
       }
       pf_ck += kParts;
       pf_settle();
