@@ -229,6 +229,7 @@ int launch_patchify(ivit_ctx* ctx, const int8_t* img, int64_t B, int64_t C, int6
 int launch_gather_rows(ivit_ctx* ctx, const int8_t* src, int64_t ldsrc, const int32_t* index,
                        int64_t n_rows, int64_t width, int8_t* dst, int64_t lddst) {
   const int64_t per_row = width / 16, slice = kMaxPieces / per_row;
+  if (slice == 0) return IVIT_ERR_UNSUPPORTED;   // a row of 2^35 bytes
   for (int64_t r = 0; r < n_rows; r += slice) {
     const int64_t total = (n_rows - r < slice ? n_rows - r : slice) * per_row;
     LaunchScope ls(ctx, KIND_MOVE, 32.0 * (double)total);
@@ -243,6 +244,7 @@ int launch_gather_rows(ivit_ctx* ctx, const int8_t* src, int64_t ldsrc, const in
 int launch_fill_rows(ivit_ctx* ctx, const int8_t* src_row, int64_t width, int8_t* dst,
                      int64_t group_stride, int64_t groups) {
   const int64_t per_row = width / 16, slice = kMaxPieces / per_row;
+  if (slice == 0) return IVIT_ERR_UNSUPPORTED;   // a row of 2^35 bytes
   for (int64_t g = 0; g < groups; g += slice) {
     const int64_t total = (groups - g < slice ? groups - g : slice) * per_row;
     LaunchScope ls(ctx, KIND_MOVE, 16.0 * (double)total);

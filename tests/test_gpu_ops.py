@@ -583,6 +583,19 @@ def test_argument_validation_is_synchronous():
     assert c.poll_status() == 0
 
 
+def test_row_movers_refuse_rows_wider_than_they_count():
+    """Rows of 2^35 bytes and more: an error, and nothing enqueued."""
+    g = _g()
+    c = g.ctx()
+    x = torch.zeros(64, dtype=torch.int8, device="cuda")
+    index = torch.zeros(1, dtype=torch.int32, device="cuda")
+    n0 = c.launch_count()
+    for width in (1 << 35, 1 << 36, (1 << 40) + 16):
+        assert c.lib.ivit_gather_rows(c.h, x.data_ptr(), width, index.data_ptr(), 1, width, x.data_ptr(), width) == -4
+        assert c.lib.ivit_fill_rows(c.h, x.data_ptr(), width, x.data_ptr(), width, 1) == -4
+    assert c.launch_count() == n0
+
+
 def test_tensor_core_engine_takes_the_model_shapes():
     """The tcgen05 kernel (not the CUDA-core one) serves the Dense and attention shapes of the workloads."""
     g = _g()
