@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from ivit_inputs import make_config
+from ivit_inputs.gen import make_image, make_swin, shift_indices, shift_mask
 from oracle import api as O
 
 pytestmark = pytest.mark.gpu
@@ -54,6 +55,40 @@ def test_swin_shifted_windows_bit_exact():
     # the shift changes the result
     plain, _ = make_config(3, batch=2)
     assert not np.array_equal(want, O.swin_forward(plain, image))
+    assert c.poll_status() == 0
+
+
+def _shift(model, flags):
+    """The model with the blocks that `flags` names (stage by stage) shifted: indices, and the mask folded into the bias."""
+    T = model.window ** 2
+    for st, fl in zip(model.stages, flags):
+        st.shifted = list(fl)
+        st.shift_index, st.unshift_index = shift_indices(model.B, st.res, model.window)
+        m = shift_mask(st.res, model.window)
+        for blk, sh in zip(st.blocks, fl):
+            if sh:
+                blk.attn_bias = (blk.attn_bias[None] + m[:, None]).reshape(-1, T, T)
+    return model
+
+
+@pytest.mark.parametrize("dims,heads,img", [((32, 64), (1, 2), 56), ((128, 256), (4, 8), 56), ((96, 192), (3, 6), 112),
+                                            ((512, 1024), (16, 32), 56)])
+@pytest.mark.parametrize("flags", [((False, True, True), (True, False, True)), ((True, True, False, True), (False, True, True)),
+                                   ((True,), (True, True)), ((True, False), (False, False))])
+def test_swin_shift_sequences_bit_exact(dims, heads, img, flags):
+    """Shifted blocks first, last, two in a row and next to a merge, on widths that read every permutation, none, or only
+    those of blocks or only those of merges through the LayerNorm that follows: tokens and logits."""
+    g = _g()
+    c = g.ctx()
+    p = make_swin(seed=31, B=2, img=img, dims=dims, heads=heads, depths=tuple(len(f) for f in flags), classes=12)
+    p = _shift(p, flags)
+    image = make_image(31, 2, img)
+    want, want_tokens = O.swin_forward(p, image, return_tokens=True)
+    dm = g.binding.DeviceSwin(p, "cuda")
+    logits, tokens = g.binding.swin_forward(c, dm, torch.from_numpy(image).cuda(), return_tokens=True)
+    g.assert_equal(g.host(tokens), want_tokens, "tokens")
+    g.assert_equal(g.host(logits), want, "logits")
+    assert len(np.unique(want_tokens)) > 50
     assert c.poll_status() == 0
 
 

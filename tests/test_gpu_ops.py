@@ -143,7 +143,7 @@ def test_linear_cta_pairs(M, N, K, with_res):
             assert c.pair_launch_count() - p0 == (1 if pairs else 0)   # the pair form really ran (needs >= 74 pair tiles)
             assert c.poll_status() == 0
     finally:
-        c.set_gemm_pairs(True)
+        c.set_gemm_pairs(None)
 
 
 @pytest.mark.parametrize("M,N,K,with_res", [(12545, 384, 1536, True), (12608, 384, 1536, False), (9505, 512, 512, False),
