@@ -13,12 +13,13 @@
 //   pass C  one reciprocal per row (Eq. (IntDiv)), then exp * reciprocal >> shift per value; the int8 probabilities are
 //           written to shared memory in the K-major 128B-swizzled layout that P V consumes as its A operand.
 // V is consumed as stored ([token, d] rows, MN-major B operand).  Every wait is bounded.
-// What bounds the passes: issue slots.  mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer
-// instructions two cycles of their pipe, a look-up one of the SM's shared-memory cycles.
+// What bounds the kernels: the chain of an item (scores, pass A, exchange, pass B, exchange, pass C, P V, output), of which
+// an SM has two in flight, or parts of two: on short rows issue slots are busy in 43 % of the cycles and no pipe in more than
+// 28 %.  Inside a pass mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer instructions two
+// cycles of their pipe, a look-up one of the SM's shared-memory cycles.
 #include "handover.cuh"
 #include "shiftmax.cuh"
 #include "tc_ptx.cuh"
-#include <cstdlib>
 
 namespace ivit {
 
@@ -565,7 +566,7 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
 //   output  O = P V has tensor-memory columns of its own and is read beside the reciprocals of the NEXT item's rows.
 // The chunk loops are rolled: straight-line code for all chunks waited for instructions more than for anything else.
 // Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 178 us (before: one table, remainders dealt to all threads, a wait
-// for P V in every item).  On rows of up to 256 tokens the two CTAs per SM of the kernel above win: 22.3 against 29.6 us
+// for P V in every item).  On rows of up to 256 tokens the two CTAs per SM of the kernel above win: 19.5 against 29.6 us
 // at 64 x 197, 6 heads.
 // Warps 0..3: warp 0 loads, issues MMAs and owns tensor memory (the others of its warpgroup only lend their registers);
 // warps 4..19: the Shiftmax threads.  The launch gives every warp 96 registers (640 threads); the first warpgroup hands

@@ -82,11 +82,6 @@ __device__ __forceinline__ int rq(int a, int m, int s) {
   return (int)(p >> s);
 }
 
-// Same value, for a shift known to be >= 32 (the product's low word only feeds the carry).
-__device__ __forceinline__ int rq_hi(int a, int m, int s) {
-  long long p = (long long)a * (long long)m + (1ll << (s - 1));
-  return (int)(p >> 32) >> (s - 32);
-}
 
 // Shifts are bounded to [31, 62]: with 0 < mult < 2^31 and |a| < 2^31 the requantised value then fits 32 bits.
 __host__ __device__ __forceinline__ int clamp_shift(int s) { return s < 31 ? 31 : (s > 62 ? 62 : s); }

@@ -810,7 +810,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             // fragment form: 16 channels x 32 rows per step; the packed words are the fragment that one stmatrix
             // stores transposed, i.e. as rows of 16 consecutive channels, into the [32 rows][32 channels] slot
             const uint32_t out_slot = my_out + 1024u * (g & 1u) + (uint32_t)lane * 32u;
-            const uint8_t* res_slot = gen_base + (my_res - base) + (g & 1u) * 1024 + (2 * (lane & 3)) * 32 + (lane >> 2);
             // both halves are requested before the arithmetic on the first begins
             int vv[32];
             tmem_ld_frag16_issue<0>(t_row + (uint32_t)(32 * ck), vv);
@@ -836,17 +835,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     v[4 * i + 2 * u] = (int)(mad_wide(v[4 * i + 2 * u], m, c64) >> sft);
                     v[4 * i + 2 * u + 1] = (int)(mad_wide(v[4 * i + 2 * u + 1], m, c64) >> sft);
                   }
-                }
-              }
-              if (tma_res) {
-                // residual bytes [row][32 channels]: rows 8 i + 2 (l & 3) + {0, 1}, channels 16 h + (l >> 2) + {0, 8}
-                const uint8_t* rt = res_slot + 16 * h;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  v[4 * i] += (int)res_tab0[(int)*reinterpret_cast<const int8_t*>(rt + i * 256)];
-                  v[4 * i + 1] += (int)res_tab0[(int)*reinterpret_cast<const int8_t*>(rt + i * 256 + 32)];
-                  v[4 * i + 2] += (int)res_tab0[(int)*reinterpret_cast<const int8_t*>(rt + i * 256 + 8)];
-                  v[4 * i + 3] += (int)res_tab0[(int)*reinterpret_cast<const int8_t*>(rt + i * 256 + 40)];
                 }
               }
               if (act) {

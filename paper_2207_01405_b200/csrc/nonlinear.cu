@@ -1,6 +1,6 @@
 // I-LayerNorm (Sec. 3.5), Shiftmax (Algorithm 1) and ShiftGELU (Algorithm 2) kernels, sm_100a.
-// One warp owns one row; rows are read once from HBM as coalesced 32-bit words and
-// kept in registers between the reduction and the output pass.
+// Warps own whole rows, one or several at a time, short ones side by side; a row is read once, as coalesced words, and
+// kept in registers between the reductions and the output pass (longer rows than the registers hold are read again).
 #include "rowops.cuh"
 #include "shiftmax.cuh"
 #include <type_traits>
@@ -8,11 +8,6 @@
 namespace ivit {
 
 __device__ __forceinline__ int warp_sum(int v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ unsigned warp_sum_u(unsigned v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -129,7 +124,8 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
 // stored: the body has no branch but the one on the form of the constants.  What bounds it is instruction issue: byte,
 // multiply-add, mad.hi, shift and half a pack per value, and about 130 instructions for the scalars of G R rows at once.
 // With a branch around every word and row and one row per 32 lanes, three of four instructions were overhead.  Measured, back
-// to back: 197 x 192 2.4 -> 1.5 us.  (More than 1024 rows of 96, 192 or a multiple of 128 channels: the next kernel.)
+// to back: 197 x 192 2.4 -> 1.5 us.  (More than 1024 rows of 96, 192, 384, 512, 768 or
+// 1024 channels, and 1536 channels at any number of rows: the next kernel.)
 // fast: every channel of the warp has s >= 33 and a small beta (see LnConsts): m, sh = s - 32 and add = 2^(sh-1) + beta 2^sh.
 template <int WPL>
 struct LnLane {

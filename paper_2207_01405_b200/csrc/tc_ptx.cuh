@@ -25,9 +25,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
 // One poll: the thread may be suspended by the hardware while the phase is incomplete and resumes when it completes.
 // (Without a suspend-time hint: with one of 2 us the wait became poll + NANOSLEEP and every hand-over between warps took
 // longer, 1.7 us over the six of an attention item.)
@@ -36,16 +33,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// One non-blocking test of the phase.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t}"
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
@@ -59,35 +46,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* st
   return false;
 }
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
-
-// Tile store shared -> global (4-D map); completion is tracked by bulk async-groups.
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
-  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-               ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// Blocks until the shared-memory source of every committed store has been read.
-__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// ... of every committed store but the latest.
+// Blocks until the shared-memory source of every committed store but the latest has been read.
 __device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-// ... of every committed store of this thread, or of all but the one committed last.
-__device__ __forceinline__ void tma_store_wait_read1_or_all(bool keep_last) {
-  if (keep_last) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-  else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// Adds to a 32-bit word in shared memory and returns the old value; releases this thread's earlier writes.
-// A thread that acts on the additions of others it has observed follows up with fence_acquire_cta().
-__device__ __forceinline__ uint32_t smem_add_release(uint32_t addr, uint32_t v) {
-  uint32_t old;
-  asm volatile("atom.release.cta.shared::cta.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(addr), "r"(v) : "memory");
-  return old;
-}
-__device__ __forceinline__ void fence_acquire_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
@@ -100,13 +60,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
 // Same, with the two descriptors given as (low, high) words: the issuing thread then advances a
 // descriptor along K with one 32-bit add on the low word (the start-address field).
 __device__ __forceinline__ void umma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
@@ -118,37 +71,6 @@ __device__ __forceinline__ void umma_i8_lohi(uint32_t d_tmem, uint32_t a_lo, uin
       "setp.ne.b32 p, %6, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, p;\n\t}"
       ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Four MMAs of one 128-byte k-block in one go: the descriptors advance along K by a_step / b_step (units of 16
-// bytes, added to the low words); the first MMA accumulates only if `accumulate`, the others always.  The issuing
-// thread shares its scheduler with busy epilogue warps, so every instruction it saves shortens the time until the
-// tensor core has its work.
-__device__ __forceinline__ void umma_i8_x4(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                           uint32_t idesc, uint32_t accumulate, uint32_t a_step, uint32_t b_step) {
-  asm volatile(
-      "{\n\t.reg .pred p, pt;\n\t.reg .b64 da, db;\n\t.reg .b32 al, bl;\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "setp.eq.b32 pt, 0, 0;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, p;\n\t"
-      "add.u32 al, %1, %7;\n\t"
-      "add.u32 bl, %3, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, pt;\n\t"
-      "add.u32 al, al, %7;\n\t"
-      "add.u32 bl, bl, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, pt;\n\t"
-      "add.u32 al, al, %7;\n\t"
-      "add.u32 bl, bl, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, pt;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(a_step), "r"(b_step)
-      : "memory");
 }
 // ---- a pair of CTAs on one tile (cta_group::2): both CTAs of a two-CTA cluster hold half of the accumulator rows,
 // each loads its own A rows and half of the B rows, and CTA rank 0 issues every MMA for both ----
@@ -173,63 +95,13 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t cols
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
-// Tile load into this CTA's shared memory whose bytes are counted by a barrier of CTA rank 0 (`bar0` = mapa_rank0 of
-// the barrier).  No multicast: every CTA fetches its own tile.
-__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar0, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(map), "r"(bar0), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
-}
-// Four M256 x N x K32 MMAs of one k-block over both CTAs (issued by CTA rank 0), descriptors as in umma_i8_x4.
-__device__ __forceinline__ void umma_i8_x4_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                                uint32_t idesc, uint32_t accumulate, uint32_t a_step, uint32_t b_step) {
-  asm volatile(
-      "{\n\t.reg .pred p, pt;\n\t.reg .b64 da, db;\n\t.reg .b32 al, bl;\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "setp.eq.b32 pt, 0, 0;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %5, p;\n\t"
-      "add.u32 al, %1, %7;\n\t"
-      "add.u32 bl, %3, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %5, pt;\n\t"
-      "add.u32 al, al, %7;\n\t"
-      "add.u32 bl, bl, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %5, pt;\n\t"
-      "add.u32 al, al, %7;\n\t"
-      "add.u32 bl, bl, %8;\n\t"
-      "mov.b64 da, {al, %2};\n\t"
-      "mov.b64 db, {bl, %4};\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %5, pt;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(a_step), "r"(b_step)
-      : "memory");
-}
-__device__ __forceinline__ void umma_i8_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                             uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "tcgen05.mma.cta_group::2.kind::i8 [%0], da, db, %5, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
-}
-// Arrives, once every MMA issued so far by this thread has completed, on the barrier at this shared-memory offset in
-// BOTH CTAs of the pair.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"((unsigned short)3) : "memory");
-}
 // Arrive on a barrier of another CTA of the cluster (`bar` a shared::cluster address, e.g. from mapa_rank0).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
-// Low / high words of a shared-memory matrix descriptor (see smem_desc).
+// Low / high words of a shared-memory matrix descriptor (sm_100 format): start address, leading / stride byte offsets
+// in 16-byte units, descriptor version 1, swizzle mode in the top three bits.
 __device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo_bytes) {
   return ((addr >> 4) & 0x3FFF) | (((lbo_bytes >> 4) & 0x3FFF) << 16);
 }
@@ -253,11 +125,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, in
   __threadfence_system();
   return false;
 }
-__device__ __forceinline__ bool elect_one() {
-  uint32_t e;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
-  return e != 0;
-}
 __device__ __forceinline__ void mbar_expect_tx_w(uint32_t bar, uint32_t bytes) {
   asm volatile("{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "@pe mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes) : "memory");
@@ -268,18 +135,23 @@ __device__ __forceinline__ void tma_load_4d_w(uint32_t dst, const CUtensorMap* m
       "@pe cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];\n\t}"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
+// Tile load into this CTA's shared memory whose bytes are counted by a barrier of CTA rank 0 (`bar0` = mapa_rank0 of
+// the barrier).  No multicast: every CTA fetches its own tile.
 __device__ __forceinline__ void tma_load_4d_pair_w(uint32_t dst, const CUtensorMap* map, uint32_t bar0, int c0, int c1, int c2, int c3) {
   asm volatile(
       "{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "@pe cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];\n\t}"
       ::"r"(dst), "l"(map), "r"(bar0), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
+// Tile store shared -> global (4-D map); completion is tracked by bulk async-groups.
 __device__ __forceinline__ void tma_store_4d_w(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2, int c3) {
   asm volatile("{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "@pe cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n\t"
       "@pe cp.async.bulk.commit_group;\n\t}"
                ::"l"(map), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
 }
+// The two descriptors come as (low, high) words: a descriptor advances along K with one 32-bit add on the low word (the
+// start-address field).
 __device__ __forceinline__ void umma_i8_lohi_w(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                              uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -291,6 +163,10 @@ __device__ __forceinline__ void umma_i8_lohi_w(uint32_t d_tmem, uint32_t a_lo, u
       "@pe tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %5, p;\n\t}"
       ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
+// Four MMAs of one 128-byte k-block in one go: the descriptors advance along K by a_step / b_step (units of 16
+// bytes, added to the low words); the first MMA accumulates only if `accumulate`, the others always.  The issuing
+// warp shares its scheduler with busy epilogue warps, so every instruction it saves shortens the time until the
+// tensor core has its work.
 __device__ __forceinline__ void umma_i8_x4_w(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                            uint32_t idesc, uint32_t accumulate, uint32_t a_step, uint32_t b_step) {
   asm volatile(
@@ -319,6 +195,7 @@ __device__ __forceinline__ void umma_i8_x4_w(uint32_t d_tmem, uint32_t a_lo, uin
       ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(a_step), "r"(b_step)
       : "memory");
 }
+// Four M256 x N x K32 MMAs of one k-block over both CTAs of a pair (issued by CTA rank 0).
 __device__ __forceinline__ void umma_i8_x4_pair_w(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
                                                 uint32_t idesc, uint32_t accumulate, uint32_t a_step, uint32_t b_step) {
   asm volatile(
@@ -362,6 +239,8 @@ __device__ __forceinline__ void umma_commit_w(uint32_t bar) {
   asm volatile("{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
+// Arrives, once every MMA issued so far by the elected lane has completed, on the barrier at this shared-memory offset in
+// BOTH CTAs of the pair.
 __device__ __forceinline__ void umma_commit_pair_w(uint32_t bar) {
   asm volatile("{\n\t.reg .pred pe;\n\telect.sync _|pe, 0xffffffff;\n\t"
       "@pe tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
@@ -429,18 +308,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, int (&v)[32]) {
   tmem_ld32_issue(taddr, v);
   tmem_ld_wait(v);
 }
-// Stores 32 registers to 32 consecutive columns of this thread's row in tensor memory.
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const int (&v)[32]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-      :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-         "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
-         "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
-         "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]),
-         "r"(taddr) : "memory");
-}
 // Stores 16 / 4 registers to consecutive columns of this thread's row in tensor memory; loads 4.
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const int (&v)[16]) {
   asm volatile(
@@ -449,21 +316,11 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const int (&v)[16]) {
       :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr) : "memory");
 }
-// Accumulator-fragment load: 16 TMEM lanes x 32 columns per warp.  Thread l receives, for i = 0..3,
-//   v[4i], v[4i+1] = lane (l >> 2),     columns 8i + 2 (l & 3), + 1
-//   v[4i+2], v[4i+3] = lane (l >> 2) + 8, the same two columns
-// (lanes counted from the lane field of taddr, which may be the warp's quarter or its upper half).  Packed four to
-// a word this is the fragment that stmatrix_x4_trans_b8 stores transposed.
-__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, int (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr) : "memory");
-}
-// The same load without the wait: into v[O .. O + 15]; valid after tmem_ld_wait(v).
+// Accumulator-fragment load: 16 TMEM lanes x 32 columns per warp, into u = v + O.  Thread l receives, for i = 0..3,
+//   u[4i], u[4i+1] = lane (l >> 2),     columns 8i + 2 (l & 3), + 1
+//   u[4i+2], u[4i+3] = lane (l >> 2) + 8, the same two columns
+// (lanes counted from the lane field of taddr, which may be the warp's quarter or its upper half), valid after
+// tmem_ld_wait(v).  Packed four to a word this is the fragment that stmatrix_x4_trans_b8 stores transposed.
 template <int O>
 __device__ __forceinline__ void tmem_ld_frag16_issue(uint32_t taddr, int (&v)[32]) {
   asm volatile(
@@ -480,22 +337,12 @@ __device__ __forceinline__ void stmatrix_x4_trans_b8(uint32_t row_addr, uint32_t
   asm volatile("stmatrix.sync.aligned.m16n8.x4.trans.shared.b8 [%0], {%1, %2, %3, %4};"
                ::"r"(row_addr), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
 }
-// 8 and 2 consecutive columns of this thread's lane.
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, int (&v)[8]) {
   tmem_ld8_issue(taddr, v);
   tmem_ld_wait8(v);
 }
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const int (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-               :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(taddr) : "memory");
-}
 __device__ __forceinline__ void tmem_st2(uint32_t taddr, const uint32_t (&v)[2]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%2], {%0, %1};" :: "r"(v[0]), "r"(v[1]), "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, uint32_t (&v)[2]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];\n\t"
-               "tcgen05.wait::ld.sync.aligned;"
-               : "=r"(v[0]), "=r"(v[1]) : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&v)[4]) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%4], {%0, %1, %2, %3};"
@@ -505,28 +352,6 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\n\t"
                "tcgen05.wait::ld.sync.aligned;"
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
-}
-// Split forms (issue, then wait) for loads that stay in flight while other registers are worked on.
-__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, uint32_t (&v)[4]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait4(uint32_t (&v)[4]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]) :: "memory");
-}
-__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t v0, uint32_t v1) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%2], {%0, %1};" :: "r"(v0), "r"(v1), "r"(taddr) : "memory");
-}
-// Stores 8 registers to 8 consecutive columns of this thread's row in tensor memory.
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-               :: "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
-               "tcgen05.wait::ld.sync.aligned;"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
@@ -539,18 +364,6 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
 // Makes generic-proxy writes to shared memory visible to the async proxy (TMA, tcgen05.mma).
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// Shared-memory matrix descriptor (sm_100 format): start address, leading / stride byte offsets
-// in 16-byte units, descriptor version 1, swizzle mode in the top three bits.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes, uint32_t layout_type) {
-  uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32;
-  d |= 1ull << 46;
-  d |= (uint64_t)layout_type << 61;
-  return d;
-}
-
-// saturating pack of four int32 into int8x4 (x0 in the lowest byte)
 // High word of a * m + c: one multiply-add with a 64-bit addend.
 __device__ __forceinline__ int mad_wide_hi(int a, int m, long long c) {
   int hi;
@@ -571,26 +384,12 @@ __device__ __forceinline__ long long mad_wide(int a, int m, long long c) {
   return t;
 }
 
+// saturating pack of four int32 into int8x4 (x0 in the lowest byte)
 __device__ __forceinline__ uint32_t pack_sat8(int x0, int x1, int x2, int x3) {
   uint32_t t, d;
   asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(t) : "r"(x3), "r"(x2), "r"(0));
   asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(x1), "r"(x0), "r"(t));
   return d;
 }
-
-// Per output channel, prepared once per tile: v = (acc * m + c) >> s with c = bias * m + 2^(s-1).
-// sh holds s - 32 when every channel of the tile has s >= 32 (fast form: the high word of the
-// 64-bit multiply-add shifted by s - 32), else s itself (general form, s in [31, 62]).
-struct __align__(16) ChanParam {
-  int c_lo, c_hi, m, sh;
-};
-
-__device__ __forceinline__ long long chan_mad(int acc, const int4& p) {
-  return (long long)acc * (long long)p.z + (((long long)p.y << 32) | (unsigned)p.x);
-}
-// every shift of the tile >= 32
-__device__ __forceinline__ int requant_hi(int acc, const int4& p) { return (int)(chan_mad(acc, p) >> 32) >> p.w; }
-// any shift in [31, 62]
-__device__ __forceinline__ int requant_any(int acc, const int4& p) { return (int)(chan_mad(acc, p) >> p.w); }
 
 }  // namespace ivit
