@@ -124,8 +124,8 @@ __global__ void __launch_bounds__(256) layernorm_i8_kernel(const int8_t* __restr
 // stored: the body has no branch but the one on the form of the constants.  What bounds it is instruction issue: byte,
 // multiply-add, mad.hi, shift and half a pack per value, and about 130 instructions for the scalars of G R rows at once.
 // With a branch around every word and row and one row per 32 lanes, three of four instructions were overhead.  Measured, back
-// to back: 197 x 192 2.4 -> 1.5 us.  (More than 1024 rows of 96, 192, 384, 512, 768 or
-// 1024 channels, and 1536 channels at any number of rows: the next kernel.)
+// to back: 197 x 192 2.4 -> 1.5 us.  (More than 1024 rows, operator
+// calls, and rows of 1536 channels: the next kernel.)
 // fast: every channel of the warp has s >= 33 and a small beta (see LnConsts): m, sh = s - 32 and add = 2^(sh-1) + beta 2^sh.
 template <int WPL>
 struct LnLane {
@@ -302,26 +302,27 @@ __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_
   }
 }
 
-// The same for C = 4 L WPL with the constants in shared memory, fetched once per word and R rows: the registers go to rows,
+// The same with the constants in shared memory, fetched once per word and R rows: the registers go to rows,
 // so that most launches are one or two passes, and twice the warps are in flight.  Bound by issue and by the chain of the
 // scalars of a pass.  Measured, back to back, against constants in registers: 18464 x 1024 12.4 -> 9.5 us, 9232 x 1024 8.4 ->
 // 5.4, 25216 x 768 11.3 -> 10.6, 12608 x 768 7.1 -> 5.8, 12608 x 384 4.2 -> 3.7, 3136 x 1536 9.0 -> 4.2, 12544 x 192
-// 3.65 -> 3.1, 200704 x 96 12.4 -> 11.9.  These are
-// launches inside a forward; an operator call, whose constants are fetched behind the wait, takes about 0.9 us longer
-// (25216 x 768 12.4 us; the first rows requested ahead of the constants: 12.5).
-template <int L, int WPL, int R, int GA = 0>
+// 3.65 -> 3.1, 200704 x 96 12.4 -> 11.9; with words masked 25216 x 640 17.4 -> 9.8, 25216 x 304 9.4 -> 7.0.  (As operator
+// calls, whose constants are fetched behind the wait, about 0.6 us more: 25216 x 768 10.8, 2500 x 768 2.7 -> 3.3.)
+template <int L, int WPL, int R, bool kExact, int GA = 0>
 __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int8_t* __restrict__ in, int64_t ldin, ScaleDev gs,
                                                                             const int32_t* __restrict__ beta, int M_ln,
                                                                             int8_t* __restrict__ out, int64_t ldout, int rows, int C,
                                                                             unsigned mean_magic, int vec, int params, LnSource<GA> source) {
+  static_assert(GA == 0 || kExact, "whole rows");
   static_assert(R <= L, "a lane per row for the scalars");
   constexpr int G = 32 / L, kWords = L * WPL;
+  const int nwords = kExact ? kWords : C >> 2;
   __shared__ int4 sm_m[kWords], sm_s[kWords], sm_b[kWords];
   if (!params) pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31, li = lane & (L - 1), grp = lane / L;
-  const bool fast = __syncthreads_and(ln_stage_consts(gs, beta, kWords, vec, sm_m, sm_s, sm_b, threadIdx.x, 256)) != 0;
-  if (fast) ln_fold_consts(kWords, sm_s, sm_b, threadIdx.x, 256);
+  const bool fast = __syncthreads_and(ln_stage_consts(gs, beta, nwords, vec, sm_m, sm_s, sm_b, threadIdx.x, 256)) != 0;
+  if (fast) ln_fold_consts(nwords, sm_s, sm_b, threadIdx.x, 256);
   __syncthreads();
   pdl_wait();
   const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
         if constexpr (GA == 1) from = source.row(row);
         const int* src = reinterpret_cast<const int*>(in + from * ldin) + li;
 #pragma unroll
-        for (int i = 0; i < WPL; ++i) w[r][i] = __ldg(src + L * i);
+        for (int i = 0; i < WPL; ++i) w[r][i] = kExact || li + L * i < nwords ? __ldg(src + L * i) : 0;
       }
     }
     if constexpr (GA == 1) {
@@ -390,6 +391,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
     auto rows_out = [&](auto is_fast) {
 #pragma unroll
       for (int i = 0; i < WPL; ++i) {
+        if (!kExact && li + L * i >= nwords) break;
         const int4 m4 = sm_m[li + L * i], s4 = sm_s[li + L * i], b4 = sm_b[li + L * i];
         const int m[4] = {m4.x, m4.y, m4.z, m4.w}, sh[4] = {s4.x, s4.y, s4.z, s4.w}, be[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
@@ -510,9 +512,10 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
     launch_k(kernel, dim3((unsigned)(blocks < cap ? blocks : cap)), dim3(128), 0, ctx->stream, x, ldin, gs, beta, M_ln, out, ldout, (int)rows,
              (int)C, magic, vec, (int)params, source);
   };
-  // Up to 1024 rows one row per group of lanes, constants in registers: with so few rows the chain of one warp counts
-  // (788 x 384: 1.9 us, shared constants 2.6; 197 x 192: 1.45, four rows 1.8).
-  const bool few = rows <= 1024;
+  // Up to 1024 rows of a forward one row per group of lanes, constants in registers: with so few rows the chain of one warp
+  // counts (788 x 384: 1.9 us, shared constants 2.6; 197 x 192: 1.45, four rows 1.8).  Not where the constants are
+  // fetched behind the wait: every warp would wait for copies of its own (400 x 768 as an operator call 4.5 us, shared 2.6).
+  const bool few = rows <= 1024 && params;
   // Beyond: constants in shared memory, two blocks per SM, and as many rows per warp
   // as make passes x (1 + rows) least, a pass costing about that (12608 x 384, 5.3 rows per warp: six rows 3.7 us, four 4.9,
   // eight 4.6; 4590 x 384, 1.9 rows per warp: two rows 2.8, six 3.3; 18464 x 1024, 7.8: four rows 9.5, six 10.9).
@@ -542,42 +545,64 @@ static bool layernorm_rows(ivit_ctx* ctx, const int8_t* x, int64_t ldin, ScaleDe
       if (GA == 2) return false;
       if constexpr (GA != 2) {
         if (few) run(layernorm_rows_kernel<8, 3, 1, 5, true, GA>, 4, 5);
-        else up_to_six(layernorm_shared_rows_kernel<8, 3, 2, GA>, layernorm_shared_rows_kernel<8, 3, 4, GA>, layernorm_shared_rows_kernel<8, 3, 6, GA>, 4);
+        else up_to_six(layernorm_shared_rows_kernel<8, 3, 2, true, GA>, layernorm_shared_rows_kernel<8, 3, 4, true, GA>, layernorm_shared_rows_kernel<8, 3, 6, true, GA>, 4);
       }
       return true;
     case 192:
       if (GA == 2) return false;
       if constexpr (GA != 2) {
         if (few) run(layernorm_rows_kernel<16, 3, 1, 5, true, GA>, 2, 5);
-        else up_to_six(layernorm_shared_rows_kernel<16, 3, 2, GA>, layernorm_shared_rows_kernel<16, 3, 4, GA>, layernorm_shared_rows_kernel<16, 3, 6, GA>, 2);
+        else up_to_six(layernorm_shared_rows_kernel<16, 3, 2, true, GA>, layernorm_shared_rows_kernel<16, 3, 4, true, GA>, layernorm_shared_rows_kernel<16, 3, 6, true, GA>, 2);
       }
       return true;
     case 384:
       if (few) run(layernorm_rows_kernel<32, 3, 1, 5, true, GA>, 1, 5);
-      else up_to_six(layernorm_shared_rows_kernel<32, 3, 2, GA>, layernorm_shared_rows_kernel<32, 3, 4, GA>, layernorm_shared_rows_kernel<32, 3, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 3, 2, true, GA>, layernorm_shared_rows_kernel<32, 3, 4, true, GA>, layernorm_shared_rows_kernel<32, 3, 6, true, GA>);
       return true;
     case 512:
       if (few) run(layernorm_rows_kernel<32, 4, 1, 4, true, GA>, 1, 4);
-      else up_to_six(layernorm_shared_rows_kernel<32, 4, 2, GA>, layernorm_shared_rows_kernel<32, 4, 4, GA>, layernorm_shared_rows_kernel<32, 4, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 4, 2, true, GA>, layernorm_shared_rows_kernel<32, 4, 4, true, GA>, layernorm_shared_rows_kernel<32, 4, 6, true, GA>);
       return true;
     case 768:
       if (few) run(layernorm_rows_kernel<32, 6, 1, 4, true, GA>, 1, 4);
-      else up_to_six(layernorm_shared_rows_kernel<32, 6, 2, GA>, layernorm_shared_rows_kernel<32, 6, 4, GA>, layernorm_shared_rows_kernel<32, 6, 6, GA>);
+      else up_to_six(layernorm_shared_rows_kernel<32, 6, 2, true, GA>, layernorm_shared_rows_kernel<32, 6, 4, true, GA>, layernorm_shared_rows_kernel<32, 6, 6, true, GA>);
       return true;
     case 1024:
       if (few) run(layernorm_rows_kernel<32, 8, 1, 3, true, GA>, 1, 3);
-      else if (pick({4, 2}) == 4) shared(layernorm_shared_rows_kernel<32, 8, 4, GA>, 4);
-      else shared(layernorm_shared_rows_kernel<32, 8, 2, GA>, 2);
+      else if (pick({4, 2}) == 4) shared(layernorm_shared_rows_kernel<32, 8, 4, true, GA>, 4);
+      else shared(layernorm_shared_rows_kernel<32, 8, 2, true, GA>, 2);
       return true;
-    case 1536: shared(layernorm_shared_rows_kernel<32, 12, 2, GA>, 2); return true;
+    case 1536: shared(layernorm_shared_rows_kernel<32, 12, 2, true, GA>, 2); return true;
   }
-  if constexpr (GA == 0) {
-    if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);
-    else if (wpl <= 2) run(layernorm_rows_kernel<32, 2, 4, 8, false>, 4, 8);
-    else if (wpl <= 4) run(layernorm_rows_kernel<32, 4, 4, 5, false>, 4, 5);
-    else if (wpl <= 8) run(layernorm_rows_kernel<32, 8, 2, 3, false>, 2, 3);
-    else return false;
-    return true;
+  if constexpr (GA == 0) {   // other widths: the words past the row masked
+    if (few) {
+      if (wpl <= 1) run(layernorm_rows_kernel<32, 1, 8, 10, false>, 8, 10);
+      else if (wpl <= 2) run(layernorm_rows_kernel<32, 2, 4, 8, false>, 4, 8);
+      else if (wpl <= 4) run(layernorm_rows_kernel<32, 4, 4, 5, false>, 4, 5);
+      else if (wpl <= 8) run(layernorm_rows_kernel<32, 8, 2, 3, false>, 2, 3);
+      else return false;
+      return true;
+    }
+    auto masked = [&](auto w) {
+      constexpr int W = decltype(w)::value;
+      if constexpr (W <= 6) {
+        up_to_six(layernorm_shared_rows_kernel<32, W, 2, false>, layernorm_shared_rows_kernel<32, W, 4, false>, layernorm_shared_rows_kernel<32, W, 6, false>);
+      } else {
+        if (pick({4, 2}) == 4) shared(layernorm_shared_rows_kernel<32, W, 4, false>, 4);
+        else shared(layernorm_shared_rows_kernel<32, W, 2, false>, 2);
+      }
+      return true;
+    };
+    switch (wpl) {
+      case 1: return masked(std::integral_constant<int, 1>{});
+      case 2: return masked(std::integral_constant<int, 2>{});
+      case 3: return masked(std::integral_constant<int, 3>{});
+      case 4: return masked(std::integral_constant<int, 4>{});
+      case 5: return masked(std::integral_constant<int, 5>{});
+      case 6: return masked(std::integral_constant<int, 6>{});
+      case 7: return masked(std::integral_constant<int, 7>{});
+      case 8: return masked(std::integral_constant<int, 8>{});
+    }
   }
   return false;
 }

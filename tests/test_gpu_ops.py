@@ -681,7 +681,7 @@ def test_layernorm_row_counts_and_forms(C):
     assert c.poll_status() == 0
 
 
-@pytest.mark.parametrize("C", [96, 192, 384, 512, 768, 1024, 1536])
+@pytest.mark.parametrize("C", [96, 192, 384, 512, 768, 1024, 1536, 4, 128, 132, 300, 516, 640, 764, 772, 896, 900, 1020])
 def test_layernorm_rows_per_warp(C):
     """Beyond 1024 rows a warp takes two, four or six rows at a time, by the number of rows: each of them, in one pass and
     in several, with a last share that is not full; both forms of the constants."""
