@@ -248,3 +248,23 @@ def test_attention_score_bias_layouts(B, T, heads, d, batches):
     got = g.host(c.attention(dblk, torch.from_numpy(QKV).cuda()))
     g.assert_equal(got, O.attention(blk, QKV), f"B={B} T={T} heads={heads} d={d} bias matrices={batches}")
     assert c.poll_status() == 0
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+@pytest.mark.parametrize("T", [80, 97, 130, 255, 256, 272, 321, 398])
+def test_attention_bias_rows_at_any_boundary(T, shift):
+    """A score bias read from global memory: rows that start at every place inside 16 bytes (by the row length, or because the
+    whole bias does), short and long rows, the last matrix ending with its buffer."""
+    g = _g()
+    c = g.ctx()
+    heads, d, B = 2, 32, 2
+    blk = make_block(_Ids(4500 + T), 1, B, T, heads * d, heads, 2 * heads * d, attn_bias_batches=B * heads)
+    dblk = g.binding.DeviceBlock(blk, "cuda")
+    flat = torch.zeros(blk.attn_bias.size + shift, dtype=torch.int32, device="cuda")
+    flat[shift:] = torch.from_numpy(np.ascontiguousarray(blk.attn_bias).reshape(-1)).cuda()
+    dblk.c.attn_bias = flat[shift:].data_ptr()
+    rng = np.random.default_rng(T + shift)
+    QKV = np.clip(np.rint(rng.standard_normal((B * T, 3 * heads * d)) * 32), -128, 127).astype(np.int8)
+    got = g.host(c.attention(dblk, torch.from_numpy(QKV).cuda()))
+    g.assert_equal(got, O.attention(blk, QKV), f"T={T} shift={shift}")
+    assert c.poll_status() == 0
