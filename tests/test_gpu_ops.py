@@ -722,3 +722,20 @@ def test_shiftmax_row_forms(d):
             got = c.shiftmax(g.dev(y, 4), p, pre=g.binding.DevScale(sc, "cuda"), bias32=None if b is None else g.dev(b, 4))
             g.assert_equal(g.host(got), O.shiftmax(y, p, pre=sc, bias32=b), f"int32 rows={rows} bias={b is not None}")
     assert c.poll_status() == 0
+
+
+@pytest.mark.parametrize("C", [4, 96, 384, 772])
+def test_token_mean_groups_on_both_sides_of_the_rule(C):
+    """Few and many groups of few and many rows: the rows of a group dealt to warps, or a thread per channel."""
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(C)
+    sc = Scale(*dyadic(0.05))
+    nb = (C // 4 + 31) // 32
+    for T in (1, 3, 15, 16, 49, 127, 128, 130):
+        for groups in {1, 444 // nb, 444 // nb + 1, 1184 // nb, 1184 // nb + 1, 1300}:
+            if groups * T * C > 3e7:
+                continue
+            x = rand_i8(rng, (groups * T, C))
+            g.assert_equal(g.host(c.token_mean(g.dev(x), T, g.binding.DevScale(sc, "cuda"))), O.token_mean(x, T, sc), f"{groups} x {T}")
+    assert c.poll_status() == 0
