@@ -402,7 +402,7 @@ int ivit_probe_int8_mma(ivit_ctx* ctx, int32_t iters, float* ms, double* ops);
 
 /* Verification aid for Sec. 3.5: out[i] = the integer square root that the I-LayerNorm kernels compute for the
  * radicand n0 + i, i < count (device uint16 array; n0 + count <= 2^26, more than the largest sum of squared deviations
- * of an int8 row of 1536 channels).  The kernels take the root bit by bit instead of running Eq. (iterative); a test
+ * of an int8 row of 1536 channels).  The kernels take it from the single-precision root instead of running Eq. (iterative); a test
  * compares this routine with the iteration over the whole range. */
 int ivit_isqrt_range(ivit_ctx* ctx, uint32_t n0, uint32_t count, uint16_t* out);
 

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(128, PER_SM) layernorm_rows_kernel(const int8_
     // lane r < R of every group: the scalars of its r-th row (see layernorm_rows)
     const int mu = (int)__umulhi((unsigned)(2 * my_s1 + 257 * C), mean_magic) - 128;
     const unsigned V = (unsigned)(my_s2 - 2 * mu * my_s1 + C * mu * mu);
-    const unsigned sd = isqrt_bits26(V);
+    const unsigned sd = isqrt26(V);
     const int F = sd == 0 ? 0 : (int)((1u << M_ln) / sd);
     const int muF = (int)((unsigned)mu * (unsigned)F);
     auto rows_out = [&](auto fast) {
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_shared_rows_kernel(const int
     }
     const int mu = (int)__umulhi((unsigned)(2 * my_s1 + 257 * C), mean_magic) - 128;
     const unsigned V = (unsigned)(my_s2 - 2 * mu * my_s1 + C * mu * mu);
-    const unsigned sd = isqrt_bits26(V);
+    const unsigned sd = isqrt26(V);
     const int F = sd == 0 ? 0 : (int)((1u << M_ln) / sd);
     const int muF = (int)((unsigned)mu * (unsigned)F);
     int Fr[R], muFr[R];
@@ -1291,7 +1291,7 @@ int launch_shiftgelu_static(ivit_ctx* ctx, const int8_t* in, int64_t ldin, ivit_
 namespace ivit {
 __global__ void isqrt_range_kernel(unsigned n0, unsigned count, uint16_t* __restrict__ out) {
   for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-    out[i] = (uint16_t)isqrt_bits26(n0 + i);
+    out[i] = (uint16_t)isqrt26(n0 + i);
 }
 }  // namespace ivit
 
