@@ -7,12 +7,14 @@
 //   warp 0      requests the weight k-blocks (TMA ring), the first ones of a model's layer before the wait for the previous
 //               kernel, and the input rows, which stay resident;
 //   warp 1      issues the MMAs;
-//   warps 2..17 epilogue: a lane owns one channel, 4x4 byte transposes, direct 4-byte stores.  The residual words are
-//               requested before the MMAs are awaited.
+//   warps 2..17 epilogue: a lane owns one channel and takes 8 rows at a time; 4x4 byte transposes, direct 4-byte stores.  The
+//               residual words are requested before the MMAs are awaited.
 // Measured, back to back (persistent kernel -> this one): 197 x 192 x 192 with residual 4.8 -> 3.3 us, 197 x 384 x 1536
 // 7.6 -> 4.6, 197 x 768 x 3072 10.7 -> 6.2, 1576 x 384 x 1536 5.6 -> 5.0.  LayerNorm and ShiftGELU computed here, in front
 // of the MMAs, instead of in kernels of their own were slower on every batch size (four DeiT-T blocks of one image 154
-// against 130 us): the row kernels' launches overlap their neighbours', the prologue does not.
+// against 130 us): the row kernels' launches overlap their neighbours', the prologue does not.  Behind the
+// MMAs, by a cluster of the CTAs of a row (totals by reductions into distributed shared memory), they were no faster either:
+// DeiT-T block of one image 25.3 against 24.7 us, ViT-B 33.9 against 31.2.
 #include "ring.cuh"
 #include "tc_ptx.cuh"
 
@@ -22,7 +24,8 @@ namespace {
 constexpr int SM_BM = 128;          // channels of a tile (TMEM lanes)
 constexpr int SM_BK = 128;          // bytes of K per stage
 constexpr int kSmallStages = 8;
-constexpr int NW = 16;              // epilogue warps (eight are as fast up to 64 rows and up to 1.4 times slower above)
+constexpr int NW = 16;              // epilogue warps
+constexpr int kMaxPieces = 4;       // 8-row pieces of a warp
 
 struct SmallArgs {
   GemmEpilogue epi;
@@ -135,90 +138,83 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
     const bool hi_only = __all_sync(0xffffffffu, s >= 33 && nb > -(1 << 30) && nb < (1 << 30));
     pdl_wait();
 
-    // one chunk of 32 rows x this warp's 32 channels per warp
-    static_assert(32 * NW / 4 >= 128, "a chunk for every warp");
-    const int ck = (warp - 2) >> 2;
+    // Pieces of 8 rows x this warp's 32 channels, in a loop.  The code of a launch this short runs cold, so its length counts: a
+    // piece is what the shortest tile gives each of the sixteen warps, and longer tiles run the same instructions again
+    // (with 32 rows to a warp, unrolled, this part took 2500 to 4400 clocks of a launch of 6000; per block of one image DeiT-T
+    // 28.1 -> 24.9 us, DeiT-S 30.0 -> 26.0, ViT-L 40.7 -> 37.2, DeiT-S of eight images 39.3 -> 37.7, of 27 50.1 -> 49.4).
+    const int npieces = (nrows + 7) >> 3, part = (warp - 2) >> 2;
+    static_assert(NW / 4 * 8 * kMaxPieces >= 128, "all rows");
     const int li = lane & 3;
     const uint32_t sel1 = (li & 1) ? 0x3715u : 0x6240u, sel2 = (li & 2) ? 0x3276u : 0x5410u;
     // 4 x 4 byte transpose inside every group of four lanes (its own inverse)
-    auto transpose4 = [&](uint32_t (&w)[4]) {
-      uint32_t o[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) o[k] = __shfl_xor_sync(0xffffffffu, w[k], 1);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = __byte_perm(w[k], o[k], sel1);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) o[k] = __shfl_xor_sync(0xffffffffu, w[k], 2);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) w[k] = __byte_perm(w[k], o[k], sel2);
+    auto transpose4 = [&](uint32_t w) {
+      w = __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 1), sel1);
+      return __byte_perm(w, __shfl_xor_sync(0xffffffffu, w, 2), sel2);
     };
     // rq(x; m, s) of an int8 x whose byte stands on top of a word: high word of (x 2^24) m + 2^(s+23), shifted by s - 8.
     // From s = 39 on |x m| < 2^(s-1): the result is 0.
     const int rs = clamp_shift(e.res_scale.shift);
     const int res_m = rs >= 39 ? 0 : e.res_scale.mult, res_sh = rs >= 39 ? 31 : rs - 8, res_rnd = rs >= 39 ? 0 : 1 << (rs - 9);
     const int8_t* res = e.res;
-    if (32 * ck < nrows) {
-      const int r0 = q0 + 32 * ck;
-      // residual words of the chunk, in flight while the MMAs finish: row li + 4 k of each half, four channels
-      uint32_t rw[2][4];
+    // residual words of this warp's pieces, in flight while the MMAs finish: row li + 4 k of each, four channels
+    uint32_t rw[kMaxPieces][2];
+    if (res) {
+#pragma unroll
+      for (int i = 0; i < kMaxPieces; ++i)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int row = q0 + 8 * (part + NW / 4 * i) + 4 * k + li;
+          rw[i][k] = 0;
+          if (part + NW / 4 * i < npieces && cg_ok && row < a.Q) {
+            const int64_t rr = row < e.res_rows ? row : (int64_t)((uint64_t)row % (uint64_t)e.res_rows);
+            rw[i][k] = *reinterpret_cast<const uint32_t*>(res + rr * e.ldres + cbase);
+          }
+        }
+    }
+    mbar_wait_warp(accf, 0, a.status);   // (after a timeout the results are meaningless and the status word says so)
+    tc_fence_after();
+    const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16);
+#pragma unroll 1
+    for (int piece = part; piece < npieces; piece += NW / 4) {
+      const int r0 = q0 + 8 * piece;
+      int v[8];
+      tmem_ld8(t_row + (uint32_t)(8 * piece), v);
+      if (hi_only) {
+        const int rnd = 1 << (s - 33), sh = s - 32;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = mad_hi(v[j] + nb, m, rnd) >> sh;
+      } else {
+        const long long c64 = (long long)nb * m + (1ll << (s - 1));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = (int)(mad_wide(v[j], m, c64) >> s);
+      }
       if (res) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t w = transpose4(rw[0][k]);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int row = r0 + 16 * h + 4 * k + li;
-            rw[h][k] = 0;
-            if (cg_ok && row < a.Q) {
-              const int64_t rr = row < e.res_rows ? row : (int64_t)((uint64_t)row % (uint64_t)e.res_rows);
-              rw[h][k] = *reinterpret_cast<const uint32_t*>(res + rr * e.ldres + cbase);
-            }
-          }
+          for (int b = 0; b < 4; ++b) v[4 * k + b] += mad_hi((int)__byte_perm(w, 0, (b << 12) | 0x444), res_m, res_rnd) >> res_sh;
+#pragma unroll
+          for (int i = 1; i < kMaxPieces; ++i) rw[i - 1][k] = rw[i][k];
+        }
       }
-      mbar_wait_warp(accf, 0, a.status);   // (after a timeout the results are meaningless and the status word says so)
-      tc_fence_after();
-      int vv[32];
-      tmem_ld32(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(32 * ck), vv);
+      if (e.out_dtype == IVIT_I32) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        int (&v)[16] = *reinterpret_cast<int (*)[16]>(&vv[16 * h]);
-        if (hi_only) {
-          const int rnd = 1 << (s - 33), sh = s - 32;
+        for (int j = 0; j < 8; ++j)
+          if (c < a.P && r0 + j < a.Q) reinterpret_cast<int32_t*>(e.out)[(int64_t)(r0 + j) * e.ldo + c] = v[j];
+        continue;
+      }
+      if (e.act_table) {   // element-wise activation of the saturated value (the static-maximum ShiftGELU variant)
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = mad_hi(v[j] + nb, m, rnd) >> sh;
-        } else {
-          const long long c64 = (long long)nb * m + (1ll << (s - 1));
+        for (int j = 0; j < 8; ++j) v[j] = (int)e.act_table[sat8(v[j]) + 128];
+      }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = (int)(mad_wide(v[j], m, c64) >> s);
-        }
-        if (res) {
-          transpose4(rw[h]);
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-              v[4 * k + b] += mad_hi((int)__byte_perm(rw[h][k], 0, (b << 12) | 0x444), res_m, res_rnd) >> res_sh;
-        }
-        if (e.out_dtype == IVIT_I32) {
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            if (c < a.P && r0 + 16 * h + j < a.Q) reinterpret_cast<int32_t*>(e.out)[(int64_t)(r0 + 16 * h + j) * e.ldo + c] = v[j];
-          continue;
-        }
-        if (e.act_table) {   // element-wise activation of the saturated value (the static-maximum ShiftGELU variant)
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] = (int)e.act_table[sat8(v[j]) + 128];
-        }
-        uint32_t w[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) w[k] = pack_sat8(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
-        transpose4(w);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int row = r0 + 16 * h + 4 * k + li;
-          int64_t ro = row;
-          if (e.group_rows > 0) ro = (int64_t)((unsigned)row / (unsigned)e.group_rows) * e.group_stride + (unsigned)row % (unsigned)e.group_rows;
-          if (cg_ok && row < a.Q) *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(e.out) + ro * e.ldo + cbase) = w[k];
-        }
+      for (int k = 0; k < 2; ++k) {
+        const uint32_t w = transpose4(pack_sat8(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]));
+        const int row = r0 + 4 * k + li;
+        int64_t ro = row;
+        if (e.group_rows > 0) ro = (int64_t)((unsigned)row / (unsigned)e.group_rows) * e.group_stride + (unsigned)row % (unsigned)e.group_rows;
+        if (cg_ok && row < a.Q) *reinterpret_cast<uint32_t*>(reinterpret_cast<int8_t*>(e.out) + ro * e.ldo + cbase) = w;
       }
     }
   }

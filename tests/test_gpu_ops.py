@@ -661,6 +661,27 @@ def test_linear_one_wave_of_small_tiles(M, N, K):
     assert c.poll_status() == 0
 
 
+# tiles of 32, 64, 96 and 128 rows by the number of channel tiles; rows on both sides of a piece of eight and of a warp's turn
+@pytest.mark.parametrize("M,N", [(7, 36), (9, 128), (25, 260), (41, 18900), (57, 9400), (72, 9400), (89, 9400), (105, 9400), (121, 9400), (127, 18900)])
+def test_linear_pieces_of_a_small_tile(M, N):
+    g = _g()
+    c = g.ctx()
+    rng = np.random.default_rng(M + N)
+    K = 80
+    A, W = rand_i8(rng, (M, K)), rand_i8(rng, (N, K))
+    bias = rng.integers(-20000, 20000, N).astype(np.int32)
+    acc_std = np.sqrt(K) * 40 * 40
+    scale = scale_channels(rng.uniform(20, 60, N) / acc_std)
+    dA, dW, db, ds = g.dev(A), g.dev(W), torch.from_numpy(bias).cuda(), g.binding.DevScale(scale, "cuda")
+    res, rs = rand_i8(rng, (M, N)), Scale(*dyadic(0.9))
+    out = g.dev(np.full((M + 9, N), 77, np.int8))
+    c.linear(dA, dW, db, ds, res=g.dev(res), res_scale=g.binding.DevScale(rs, "cuda"), out=out[:M])
+    want = np.full((M + 9, N), 77, np.int8)
+    want[:M] = O.linear(A, W, bias, scale, res=res, res_scale=rs)
+    g.assert_equal(g.host(out), want, "rows, and nothing behind them")
+    assert c.poll_status() == 0
+
+
 @pytest.mark.parametrize("C", [4, 96, 128, 132, 192, 384, 512, 600, 768, 1020, 1024])
 def test_layernorm_row_counts_and_forms(C):
     """The row kernel packs several short rows into a warp and takes one row per lane group up to 1024 rows: row counts
