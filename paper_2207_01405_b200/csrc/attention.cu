@@ -171,9 +171,10 @@ __device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
 // Rows of up to 256 tokens.  Several CTAs per SM: they are at different points of their items, which covers the waits that
 // an item cannot avoid (score MMAs, row exchanges, P V) and mixes passes that need different pipes.  Only the control
 // warp polls; the others wait in hardware barriers that it releases.
-//   kPack = false  128 rows of one image; two CTAs (tensor memory holds two score tiles of 256 columns), two threads per
+//   TPR = 2        128 rows of one image; two CTAs (tensor memory holds two score tiles of 256 columns), two threads per
 //                  score row, which take alternate 16-column chunks
-//   kPack = true   G windows of up to R = 128 / G tokens share the 128 rows (window attention): the score tile is
+//   TPR = 4        the same with one CTA and four threads per score row, for launches of at most one item per SM
+//   TPR = 1 (kPack)  G windows of up to R = 128 / G tokens share the 128 rows (window attention): the score tile is
 //                  block-diagonal and the probabilities outside a row's own window stay 0.  The int32 score bias of
 //                  the tile's windows is kept in shared memory (rows padded to an odd number of words, so that the 32
 //                  rows of a warp fall into different banks) and only fetched when it differs from the last item's;
@@ -186,9 +187,10 @@ __device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
 // Measured, back to back (before: one table, items drawn from a counter, bias read from global memory, every warp polling):
 // 64 x 197 tokens, 6 heads of 64 29.0 -> 19.5 us; 128 x 197, 12 heads 89.1 -> 61.7; 1 x 197, 3 heads 10.1 -> 5.9.
 // Threads per score row (TPR) and CTAs per SM.  Warp 0: TMA + MMA issue + TMEM owner; TPR warps per lane quarter.
-template <bool kPack>
+template <int TPR>
 struct ShortShape {
-  static constexpr int TPR = kPack ? 1 : 2, kCtas = kPack ? 4 : 2, kWorkers = 128 * TPR, kThreads = 32 + kWorkers;
+  static constexpr int kCtas = 4 / TPR, kWorkers = 128 * TPR, kThreads = 32 + kWorkers;
+  static constexpr int kPartials = (TPR > 1 ? 2 * TPR : 4) * 128 * 4;   // bytes
 };
 
 struct ShortArgs {
@@ -199,12 +201,13 @@ struct ShortArgs {
   int tmem_cols;
 };
 
-template <bool kPack, bool FAST, bool BIAS>
-__global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>::kCtas) attention_short_kernel(const __grid_constant__ CUtensorMap tmQ,
+template <int TPR, bool FAST, bool BIAS>
+__global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kCtas) attention_short_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                                        const __grid_constant__ CUtensorMap tmK,
                                                                                        const __grid_constant__ CUtensorMap tmV,
                                                                                        ShortArgs sa) {
-  constexpr int TPR = ShortShape<kPack>::TPR, kShortThreads = ShortShape<kPack>::kThreads, kWorkers = ShortShape<kPack>::kWorkers;
+  constexpr bool kPack = TPR == 1;
+  constexpr int kShortThreads = ShortShape<TPR>::kThreads, kWorkers = ShortShape<TPR>::kWorkers;
   const AttnArgs& a = sa.a;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -214,8 +217,8 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
   const uint32_t k_off = 128u * a.d, v_off = k_off + k_bytes;
   const uint32_t p_off = (v_off + v_bytes + 1023u) & ~1023u;
   const uint32_t tab_off = p_off + (uint32_t)((a.kpad + 127) / 128) * 128 * 128;
-  const uint32_t part_off = tab_off + 1024u * a.cp;      // [2 halves][128 rows] partial max, then partial sum
-  const uint32_t seed_off = part_off + 4 * 128 * 4;      // [128] seeds of the reciprocal
+  const uint32_t part_off = tab_off + 1024u * a.cp;      // [TPR][128 rows] partial max, then partial sum
+  const uint32_t seed_off = part_off + ShortShape<TPR>::kPartials;      // [128] seeds of the reciprocal
   const uint32_t item_off = seed_off + 128 * 4;          // [2] work item of even / odd iterations, written before its scores
   const uint32_t bar_off = item_off + 2 * sizeof(AttnItem);
   const uint32_t bias_off = bar_off + 64;                // kPack && BIAS: [G][T][T | 1]
@@ -352,9 +355,9 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       if (v_flying) mbar_wait_warp(bar_v, v_par, a.status);
     }
   } else {
-    // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the two warps of a quarter take the even / odd
-    //      chunks of the same 32 rows ----
-    const int st = threadIdx.x - 32;              // 0..255
+    // ---- Shiftmax / epilogue threads: TMEM lane quarter = warp % 4; the TPR warps of a quarter take every TPR-th chunk
+    //      of the same 32 rows ----
+    const int st = threadIdx.x - 32;
     const int qd = warp & 3;
     const int half = (warp - 1) >> 2;
     const int trow = qd * 32 + lane;              // row inside the tile
@@ -369,15 +372,15 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
     kc.init(a);
     const uint32_t t_row = tmem + ((uint32_t)(qd * 32) << 16);
     int* part_max = reinterpret_cast<int*>(gen + part_off);
-    unsigned* part_sum = reinterpret_cast<unsigned*>(gen + part_off + 2 * 128 * 4);
+    unsigned* part_sum = reinterpret_cast<unsigned*>(gen + part_off + TPR * 128 * 4);
     const uint32_t tab_lane = base + tab_off + 4u * (unsigned)(lane & (a.cp - 1));
     const unsigned top = (unsigned)a.smax.I0 << a.smax.N;    // the largest exponential
     const int osh = 14 - a.smax.k_out, omax = (1 << (a.smax.k_out - 1)) - 1;
-    // this row's whole chunks: c_lo .. c_full - 1, this thread takes every second one; rem columns remain, which the
-    // second thread (whose share is never the larger one) takes as a piece of eight or sixteen columns
+    // this row's whole chunks: c_lo .. c_full - 1, this thread takes every TPR-th one; rem columns remain, which the
+    // thread whose turn it is takes as a piece of eight or sixteen columns
     const int slot = kPack ? trow / sa.R : 0;
     const int c_lo = kPack ? slot * (sa.R >> 4) : 0, c_full = c_lo + (a.T >> 4);
-    const int rem = half == TPR - 1 ? a.T & 15 : 0;
+    const int rem = half == (c_full - c_lo) % TPR ? a.T & 15 : 0;
     uint8_t* const p_row = gen + p_off + trow * 128;
     auto p_addr = [&](int c) { return reinterpret_cast<uint4*>(p_row + (c >> 3) * (128 * 128) + (((c & 7) ^ (trow & 7)) << 4)); };
     const int bias_ld = a.T | 1;
@@ -481,7 +484,8 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       // the threads of a row exchange their partial results: a barrier of the warps that share its 32 rows
       if (TPR > 1) {
         bar_sync(2 + qd, 32 * TPR);
-        mx = max(part_max[trow], part_max[128 + trow]);
+#pragma unroll
+        for (int i = 0; i < TPR; ++i) mx = max(mx, part_max[i * 128 + trow]);
       }
       unsigned sum = 0;
       if (work) {
@@ -520,7 +524,9 @@ __global__ void __launch_bounds__(ShortShape<kPack>::kThreads, ShortShape<kPack>
       }
       if (TPR > 1) {
         bar_sync(2 + qd, 32 * TPR);
-        sum = part_sum[trow] + part_sum[128 + trow];
+        sum = 0;
+#pragma unroll
+        for (int i = 0; i < TPR; ++i) sum += part_sum[i * 128 + trow];
       }
       if (work) {
         // pass C: Eq. (IntDiv) with M = 45
@@ -974,10 +980,12 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
 
 // The shared-memory limit of a kernel is a per-device attribute: set for the current device at context creation.
 int attention_prepare_device() {
-  const void* kernels[] = {(const void*)attention_short_kernel<false, false, false>, (const void*)attention_short_kernel<false, false, true>,
-                           (const void*)attention_short_kernel<false, true, false>, (const void*)attention_short_kernel<false, true, true>,
-                           (const void*)attention_short_kernel<true, false, false>, (const void*)attention_short_kernel<true, false, true>,
-                           (const void*)attention_short_kernel<true, true, false>, (const void*)attention_short_kernel<true, true, true>,
+  const void* kernels[] = {(const void*)attention_short_kernel<1, false, false>, (const void*)attention_short_kernel<1, false, true>,
+                           (const void*)attention_short_kernel<1, true, false>, (const void*)attention_short_kernel<1, true, true>,
+                           (const void*)attention_short_kernel<2, false, false>, (const void*)attention_short_kernel<2, false, true>,
+                           (const void*)attention_short_kernel<2, true, false>, (const void*)attention_short_kernel<2, true, true>,
+                           (const void*)attention_short_kernel<4, false, false>, (const void*)attention_short_kernel<4, false, true>,
+                           (const void*)attention_short_kernel<4, true, false>, (const void*)attention_short_kernel<4, true, true>,
                            (const void*)attention_rows_kernel<true, false>, (const void*)attention_rows_kernel<true, true>,
                            (const void*)attention_rows_kernel<false, false>, (const void*)attention_rows_kernel<false, true>};
   for (const void* k : kernels)
@@ -1089,9 +1097,13 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
   }
   sa.tmem_cols = pack || a.chunks <= 8 ? 128 : 256;
   const uint32_t p_off = (128u * a.d + (pack ? 128u : (uint32_t)a.kbox) * a.d + (uint32_t)a.kpad * a.d + 1023u) & ~1023u;
-  const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + 4 * 128 * 4 + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
+  // Threads per score row: four where an SM has at most one item anyway (us per block, two -> four threads, 197 tokens: 8
+  // images of DeiT-T 29.3 -> 27.9, 8 of DeiT-S 37.9 -> 37.1, 20 of DeiT-T 37.9 -> 36.4; one image 24.9 -> 24.7).
+  const int tpr = pack ? 1 : (a.items <= ctx->sm_count ? 4 : 2);
+  const size_t partials = tpr == 4 ? ShortShape<4>::kPartials : ShortShape<2>::kPartials;
+  const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + partials + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
   // CTAs per SM: as many as leave room for four copies of the table
-  int per_sm = pack ? ShortShape<true>::kCtas : ShortShape<false>::kCtas;
+  int per_sm = pack ? ShortShape<1>::kCtas : ShortShape<2>::kCtas;
   auto budget = [](int n) { return n == 1 ? (size_t)(227 * 1024) : (size_t)(228 * 1024 / n - 1024); };
   while (per_sm > 1 && fixed + 4 * 1024 > budget(per_sm)) --per_sm;
   if (!fit_table(a, fixed, budget(per_sm))) return IVIT_ERR_UNSUPPORTED;
@@ -1104,19 +1116,16 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
       !make_tensor_map(ctx, &tmV, QKV + 2 * D, d, T, h, B, ldq, d, T * ldq, (int)d, pack ? sa.R : a.kpad, swizzle_of(d), a.v_pos, sa.G))
     return IVIT_ERR_UNSUPPORTED;
   const int64_t slots = (int64_t)per_sm * ctx->sm_count;
-  const dim3 grid((unsigned)(a.items < slots ? a.items : slots)), block(pack ? ShortShape<true>::kThreads : ShortShape<false>::kThreads);
+  const dim3 grid((unsigned)(a.items < slots ? a.items : slots)), block((unsigned)(32 + 128 * tpr));
   LaunchScope ls(ctx, KIND_ATTENTION, 4.0 * (double)(B * h) * (double)T * (double)T * (double)d);
   auto run = [&](auto kernel) { launch_k(kernel, grid, block, smem, ctx->stream, tmQ, tmK, tmV, sa); };
-  switch ((pack ? 4 : 0) | (fast_form(a) ? 2 : 0) | (a.bias ? 1 : 0)) {
-    case 0: run(attention_short_kernel<false, false, false>); break;
-    case 1: run(attention_short_kernel<false, false, true>); break;
-    case 2: run(attention_short_kernel<false, true, false>); break;
-    case 3: run(attention_short_kernel<false, true, true>); break;
-    case 4: run(attention_short_kernel<true, false, false>); break;
-    case 5: run(attention_short_kernel<true, false, true>); break;
-    case 6: run(attention_short_kernel<true, true, false>); break;
-    default: run(attention_short_kernel<true, true, true>); break;
-  }
+#define IVIT_SHORT(TPR) \
+  (fast_form(a) ? (a.bias ? run(attention_short_kernel<TPR, true, true>) : run(attention_short_kernel<TPR, true, false>)) \
+                : (a.bias ? run(attention_short_kernel<TPR, false, true>) : run(attention_short_kernel<TPR, false, false>)))
+  if (tpr == 1) IVIT_SHORT(1);
+  else if (tpr == 2) IVIT_SHORT(2);
+  else IVIT_SHORT(4);
+#undef IVIT_SHORT
   return ls.done();
 }
 

@@ -98,6 +98,23 @@ def test_fused_attention_kernel_serves_short_rows():
     assert c.poll_status() == 0
 
 
+# two tiles per head: at most 148 items take four threads per score row, more take two; remainders of 0, 1, 8, 9 columns for
+# each of the threads
+@pytest.mark.parametrize("B,T,D,heads,bias", [(1, 129, 64, 1, False), (2, 144, 128, 2, True), (3, 168, 64, 2, False), (1, 185, 64, 1, True),
+                                              (1, 201, 64, 2, False), (2, 217, 192, 3, True), (1, 233, 64, 1, False), (1, 249, 128, 1, True),
+                                              (74, 197, 64, 1, False), (75, 197, 64, 1, True), (1, 9, 64, 1, True), (148, 70, 64, 1, False),
+                                              (149, 70, 64, 1, False), (1, 256, 128, 2, True)])
+def test_attention_threads_per_row(B, T, D, heads, bias):
+    g = _g()
+    c = g.ctx()
+    blk = make_block(_Ids(40 + T), 2, B, T, D, heads, D, attn_bias_batches=heads if bias else 0)
+    rng = np.random.default_rng(B + T)
+    QKV = np.clip(np.rint(rng.standard_normal((B * T, 3 * D)) * 32), -128, 127).astype(np.int8)
+    got = c.attention(g.binding.DeviceBlock(blk, "cuda"), torch.from_numpy(QKV).cuda())
+    g.assert_equal(g.host(got), O.attention(blk, QKV), "attention")
+    assert c.poll_status() == 0
+
+
 @pytest.mark.parametrize("engine", [0, 1])
 @pytest.mark.parametrize("B,T,D,heads,H", [(3, 197, 384, 6, 1536), (2, 50, 192, 3, 200 * 4), (1, 9, 64, 1, 64)])
 def test_block_static_gelu_variant_bit_exact(engine, B, T, D, heads, H):
