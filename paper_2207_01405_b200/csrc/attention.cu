@@ -79,6 +79,7 @@ struct __align__(16) AttnItem {
 // Named barriers: id, number of threads that arrive or wait.
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+constexpr int kBarSetup = 8, kBarTmem = 9;   // (6 and 7: handover.cuh)
 template <int kThreads>
 struct BlockBarriers {
   __device__ __forceinline__ void sync(int id) const { bar_sync(id, kThreads); }
@@ -186,7 +187,7 @@ __device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
 // exponentials after pass B, and O = P V at the end.
 // Measured, back to back (before: one table, items drawn from a counter, bias read from global memory, every warp polling):
 // 64 x 197 tokens, 6 heads of 64 29.0 -> 19.5 us; 128 x 197, 12 heads 89.1 -> 61.7; 1 x 197, 3 heads 10.1 -> 5.9.
-// Threads per score row (TPR) and CTAs per SM.  Warp 0: TMA + MMA issue + TMEM owner; TPR warps per lane quarter.
+// Threads per score row (TPR) and CTAs per SM.  Warp 0: TMA + MMA issue; TPR warps per lane quarter, the first of which owns tensor memory.
 template <int TPR>
 struct ShortShape {
   static constexpr int kCtas = 4 / TPR, kWorkers = 128 * TPR, kThreads = 32 + kWorkers;
@@ -230,10 +231,9 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
   volatile uint32_t* dead = tmem_slot + 1;               // set when a wait of the control warp ran out
 
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  // Set-up.  The control warp initialises the barriers and goes on to its first loads; the warp behind it owns tensor memory,
+  // whose address the control warp takes at a barrier of the two in front of its first MMA.
   if (threadIdx.x == 0) {
-    prefetch_tmap(&tmQ);
-    prefetch_tmap(&tmK);
-    prefetch_tmap(&tmV);
     mbar_init(bar_qk, 1);
     mbar_init(bar_v, 1);
     mbar_init(bar_s, 1);
@@ -244,11 +244,25 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
   }
-  if (warp == 0) tmem_alloc(smem_u32(tmem_slot), (uint32_t)sa.tmem_cols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  uint32_t tmem = 0;
+  if (warp == 0) {
+    __syncwarp();
+    bar_arrive(kBarSetup, kShortThreads);
+    if (lane == 0) {
+      prefetch_tmap(&tmQ);
+      prefetch_tmap(&tmK);
+      prefetch_tmap(&tmV);
+    }
+  } else {
+    if (warp == 1) {
+      tmem_alloc(smem_u32(tmem_slot), (uint32_t)sa.tmem_cols);
+      tc_fence_before();
+      bar_arrive(kBarTmem, 64);
+    }
+    bar_sync(kBarSetup, kShortThreads);
+    tc_fence_after();
+    tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  }
   pdl_trigger();
   // items of this CTA: a snake over all of them, or (kPack) a contiguous range
   const uint32_t rounds = (uint32_t)a.items / gridDim.x, left = (uint32_t)a.items % gridDim.x;
@@ -257,7 +271,6 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
   const uint32_t imgs = kPack ? (uint32_t)sa.units / (uint32_t)sa.npos : 1u;   // kPack: items in a row with the same bias
 
   if (warp == 0) {
-    pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
     if (n_items > 0) {
       auto item_at = [&](AttnItem& it, uint32_t n) {
         if (kPack) {
@@ -298,8 +311,12 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
       item_at(cur, 0);
       bool qk_flying = true, v_flying = true;   // loads issued and not yet waited for (their barrier phase = item count)
       uint32_t qk_par = 0, v_par = 0;
+      pdl_wait();   // the QKV tensor comes from the previous kernel; the other warps build their table first
       load_qk(cur);
       load_v(cur);
+      bar_sync(kBarTmem, 64);
+      tc_fence_after();
+      tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
       bool ok = true;
       bool scores_out = false;
       uint32_t done = 0;                // items whose output is there
@@ -587,7 +604,7 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, (uint32_t)sa.tmem_cols);
   }
