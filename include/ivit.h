@@ -313,8 +313,10 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
  * of the context's own into one of two staging buffers used alternately, so the copy of one call
  * overlaps the compute of the call before it when calls are enqueued back to back (pinned host
  * memory is needed for that overlap; pageable memory works but copies synchronously).  The first
- * call on a context creates that stream and its events.  All calls on one context must use the
- * same workspace.  workspace must hold ivit_vit_host_workspace_bytes(p). */
+ * call on a context creates that stream and its events.  image_host must be complete when the call
+ * is made (the copy does not wait for work on the context's stream that might still fill it).  All calls on
+ * one context must use the same workspace; a call with another model or batch, or behind other work of
+ * the context, copies its image when that work is done.  workspace must hold ivit_vit_host_workspace_bytes(p). */
 size_t ivit_vit_host_workspace_bytes(const ivit_vit_params* p);
 int ivit_vit_forward_host(ivit_ctx* ctx, const ivit_vit_params* p, const int8_t* image_host,
                           int32_t* logits_host, void* workspace, size_t workspace_bytes);

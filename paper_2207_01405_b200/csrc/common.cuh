@@ -52,6 +52,9 @@ struct ivit_ctx {
   cudaStream_t copy_stream;
   cudaEvent_t img_ready[2], img_free[2];
   uint64_t host_calls;
+  const void* host_ws;      // workspace, offset and size of the staging buffers of the last host-buffer forward, and the
+  size_t host_off, host_img;   // launch count behind it: work enqueued since may use the memory that the next copy writes
+  int64_t host_launches;
   // ivit_ctx_set_host_graph: the forward of ivit_vit_forward_host replayed as an instantiated CUDA graph, one per
   // staging buffer, captured at the third call that repeats the same arguments
   int host_graph;

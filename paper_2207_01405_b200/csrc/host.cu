@@ -353,13 +353,22 @@ int host_forward(ivit_ctx* ctx, const int8_t* image_host, int32_t* logits_host, 
   const int slot = (int)(ctx->host_calls & 1);
   char* ws = static_cast<char*>(workspace);
   char* img_dev = ws + img_off + (size_t)slot * img_slot;
-  if (ctx->host_calls >= 2 && cudaStreamWaitEvent(ctx->copy_stream, ctx->img_free[slot], 0) != cudaSuccess) return IVIT_ERR_CUDA;
+  // Another layout of the workspace, or other work of this context since the last call: the buffer may be memory that work
+  // still running reads or writes, so the copy waits for all of it.
+  const bool repeated = ctx->host_calls > 0 && ctx->host_ws == workspace && ctx->host_off == img_off && ctx->host_img == img_slot &&
+                        ctx->host_launches == ctx->launches;
+  if (!repeated && cudaEventRecord(ctx->img_free[slot], ctx->stream) != cudaSuccess) return IVIT_ERR_CUDA;
+  if ((!repeated || ctx->host_calls >= 2) && cudaStreamWaitEvent(ctx->copy_stream, ctx->img_free[slot], 0) != cudaSuccess) return IVIT_ERR_CUDA;
+  ctx->host_ws = workspace;
+  ctx->host_off = img_off;
+  ctx->host_img = img_slot;
   if (cudaMemcpyAsync(img_dev, image_host, img_bytes, cudaMemcpyHostToDevice, ctx->copy_stream) != cudaSuccess ||
       cudaEventRecord(ctx->img_ready[slot], ctx->copy_stream) != cudaSuccess ||
       cudaStreamWaitEvent(ctx->stream, ctx->img_ready[slot], 0) != cudaSuccess)
     return IVIT_ERR_CUDA;
   ++ctx->host_calls;
   const int rc = run(reinterpret_cast<const int8_t*>(img_dev), reinterpret_cast<int32_t*>(ws + lg_off), slot);
+  ctx->host_launches = ctx->launches;
   // recorded even after an error: a later copy into this buffer waits for it
   if (cudaEventRecord(ctx->img_free[slot], ctx->stream) != cudaSuccess) return IVIT_ERR_CUDA;
   if (rc) return rc;

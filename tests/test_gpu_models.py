@@ -150,6 +150,32 @@ def test_host_forward_back_to_back_calls():
     assert c.poll_status() == 0
 
 
+def test_host_forward_layouts_in_turn_through_one_workspace():
+    """A batch of 64 and one of 8 by turns, then a device forward in between, all in one workspace and without a
+    synchronisation: the staging buffers of one layout are activations of the other."""
+    import gpu_util as g
+    c = g.ctx()
+    models = [make_config(1, batch=b, depth=2) for b in (64, 8)]
+    dms = [g.binding.DeviceVit(m, "cuda") for m, _ in models]
+    ws = dms[0].host_workspace()
+    want = [O.vit_forward(m, image[-2:]) for m, image in models]
+    h_img = [torch.from_numpy(image).pin_memory() for _, image in models]
+    d_img = torch.from_numpy(models[0][1]).cuda()
+    d_out = torch.zeros((64, models[0][0].classes), dtype=torch.int32, device="cuda")
+    order = [0, 1, 0, 1, 1, 0, 0, 1]
+    h_out = [torch.zeros((models[k][0].B, models[k][0].classes), dtype=torch.int32).pin_memory() for k in order]
+    torch.cuda.synchronize()
+    for n, (k, y) in enumerate(zip(order, h_out)):
+        if n == 4:
+            c.vit_forward(dms[0], d_img, logits=d_out, workspace=ws)
+        g.binding.vit_forward_host(c, dms[k], h_img[k], y, ws)
+    torch.cuda.synchronize()
+    for n, (k, y) in enumerate(zip(order, h_out)):
+        g.assert_equal(y.numpy()[-2:], want[k], f"call {n}")
+    g.assert_equal(g.host(d_out)[-2:], want[0], "device forward in between")
+    assert c.poll_status() == 0
+
+
 def test_host_forward_graph_replay_mode():
     """ivit_ctx_set_host_graph: the host-buffer forward replays a captured graph from the third repeat of the same
     arguments on (one graph per staging buffer).  Every call, before and after the capture, with changing images,
