@@ -780,11 +780,12 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
   bool a_ready = false;   // LayerNorm 1 of the next block already produced by the previous block's last Dense layer
   for (int64_t l = 0; l < p->depth; ++l) {
     const ivit_block_params* next = l + 1 < p->depth ? &p->blocks[l + 1] : nullptr;
-    if ((rc = block_impl(ctx, &p->blocks[l], X, Y, ws + w.block, false, a_ready, next, &a_ready))) return rc;
-    int8_t* t = X; X = Y; Y = t;
+    // (the caller's tensor, where the tokens are wanted, takes the last block's output: a copy behind it was 4 us)
+    int8_t* const to = tokens && !next ? tokens : Y;
+    if ((rc = block_impl(ctx, &p->blocks[l], X, to, ws + w.block, false, a_ready, next, &a_ready))) return rc;
+    Y = X;
+    X = to;
   }
-  if (tokens && cudaMemcpyAsync(tokens, X, (size_t)(B * T * D), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
-    return IVIT_ERR_CUDA;
   // final LayerNorm on the class-token rows, then the classifier (int32 logits, not saturated)
   if ((rc = launch_layernorm(ctx, X, IVIT_I8, T * D, to_dev(p->lnf_gamma), p->lnf_beta, p->blocks[0].M_ln, Z, D, B, D, true))) return rc;
   return launch_gemm(ctx, linear_problem(Z, D, p->Whead, D, p->bhead, p->head_scale, nullptr, 0, 1, none, logits,
