@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
 //           stand;
 //   output  O = P V has tensor-memory columns of its own and is read beside the reciprocals of the NEXT item's rows.
 // The chunk loops are rolled: straight-line code for all chunks waited for instructions more than for anything else.
-// Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 176 us (before: one table, remainders dealt to all threads, a wait
+// Measured: 32 x 577 tokens, 16 heads of 64: 282 -> 178 us (before: one table, remainders dealt to all threads, a wait
 // for P V in every item).  On rows of up to 256 tokens the two CTAs per SM of the kernel above win: 19.5 against 29.6 us
 // at 64 x 197, 6 heads.
 // Warps 0..3: warp 0 loads, issues MMAs and owns tensor memory (the others of its warpgroup only lend their registers);
@@ -872,45 +872,16 @@ __global__ void __launch_bounds__(kRowsThreads, 1) attention_rows_kernel(const _
         if constexpr (BIAS) { if (a.bias_vec) add_bias_row<true>(v, brow + col); else add_bias_row<false>(v, brow + col); }
       };
       p_row = gen + p_off + (n & 1u) * ra.p_stride + trow * 128;
+      // with one probability buffer the parked scores overwrite what the previous item's P V reads
+      if (ra.p_stride == 0 && n > 0) alive = alive && mbar_wait(bar_o, (n - 1) & 1u, a.status);
+
       // pass A, score block by score block, two chunks at a time
       int mx = -128;
       for (int j = 0; j < nblk; ++j, ++g) {
         if (j) alive = alive && mbar_wait(bar_s + 8 * (g & 1u), (g >> 1) & 1u, a.status);
         if (alive) tc_fence_after();
-        const uint32_t t_buf = t_row + (g & 1u) * (uint32_t)ra.wb - (uint32_t)j * (16 * kBlkChunks);
-        if (j == 0) {
-          // The first block (three whole chunks per thread: T > 256).  With one probability buffer the parked scores
-          // overwrite what the previous item's P V reads: they wait for it in registers, behind their arithmetic
-          // instead of in front of it (with the shorter last block, below, ViT-L at 384 x 384, 32 images, 12 blocks
-          // 5017 -> 4995 us under the power cap).
-          static_assert(kBlkChunks == 12, "three chunks per thread");
-          uint32_t x[3][4];
-          if (alive && warp_ok) {
-            int v[2][16];
-            tmem_ld16_issue(t_buf + 16 * part, v[0]);
-            tmem_ld16_issue(t_buf + 16 * part + 64, v[1]);
-            tmem_ld_wait16(v[0]);
-            tmem_ld_wait16(v[1]);
-            add_bias16(v[0], 16 * part);
-            score_piece<FAST, false>(a, kc, v[0], 16, mx, x[0]);
-            tmem_ld16_issue(t_buf + 16 * part + 128, v[0]);
-            add_bias16(v[1], 16 * part + 64);
-            score_piece<FAST, false>(a, kc, v[1], 16, mx, x[1]);
-            tmem_ld_wait16(v[0]);
-            add_bias16(v[0], 16 * part + 128);
-            score_piece<FAST, false>(a, kc, v[0], 16, mx, x[2]);
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_f + 8 * (g & 1u));
-          if (ra.p_stride == 0 && n > 0) alive = alive && mbar_wait(bar_o, (n - 1) & 1u, a.status);
-          if (alive && warp_ok) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) *p_addr(part + 4 * i) = make_uint4(x[i][0], x[i][1], x[i][2], x[i][3]);
-          }
-          continue;
-        }
         if (alive && warp_ok) {
+          const uint32_t t_buf = t_row + (g & 1u) * (uint32_t)ra.wb - (uint32_t)j * (16 * kBlkChunks);
           const int c_end = j == nblk - 1 ? c_full : (j + 1) * kBlkChunks;
 #pragma unroll 1
           for (int c = j * kBlkChunks + part; c < c_end; c += 8) {
@@ -1080,10 +1051,9 @@ static int launch_attention_rows(ivit_ctx* ctx, const ivit_block_params* p, cons
   AttnArgs& a = ra.a;
   fill_args(ctx, a, p, O);
   // two score buffers and the output share the 512 columns of tensor memory
-  // A last block of one chunk (a class token behind 192 k others) joins the block before it where the columns allow.
-  const int wide = a.chunks % kBlkChunks == 1 && d <= 64 ? 1 : 0;
-  ra.wb = a.kbox = 16 * (kBlkChunks + wide);
-  ra.nblk = (a.chunks - wide + kBlkChunks - 1) / kBlkChunks;
+  ra.wb = 16 * kBlkChunks;
+  ra.nblk = (a.chunks + kBlkChunks - 1) / kBlkChunks;
+  a.kbox = 16 * kBlkChunks;
   ra.nv = (a.kpad + 255) / 256;
   ra.vbox = ((a.kpad + ra.nv - 1) / ra.nv + 7) / 8 * 8;
   const uint32_t v_off = 128u * a.d + 2u * a.kbox * a.d;

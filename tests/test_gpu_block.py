@@ -98,22 +98,6 @@ def test_fused_attention_kernel_serves_short_rows():
     assert c.poll_status() == 0
 
 
-# last blocks of one chunk, which join the block before them (a single column, a full chunk), and their neighbours; several
-# items per CTA
-@pytest.mark.parametrize("B,T,D,heads,bias", [(1, 384, 64, 1, False), (1, 385, 64, 2, True), (2, 400, 128, 2, False), (1, 401, 64, 1, False),
-                                              (40, 577, 128, 2, False), (2, 577, 64, 2, True), (1, 592, 128, 2, True), (3, 769, 64, 1, False),
-                                              (1, 784, 128, 2, False), (2, 385, 256, 2, False), (1, 961, 32, 1, False)])
-def test_attention_last_block_of_one_chunk(B, T, D, heads, bias):
-    g = _g()
-    c = g.ctx()
-    blk = make_block(_Ids(60 + T), 2, B, T, D, heads, D, attn_bias_batches=heads if bias else 0)
-    rng = np.random.default_rng(B + T)
-    QKV = np.clip(np.rint(rng.standard_normal((B * T, 3 * D)) * 32), -128, 127).astype(np.int8)
-    got = c.attention(g.binding.DeviceBlock(blk, "cuda"), torch.from_numpy(QKV).cuda())
-    g.assert_equal(g.host(got), O.attention(blk, QKV), "attention")
-    assert c.poll_status() == 0
-
-
 # two tiles per head: at most 148 items take four threads per score row, more take two; remainders of 0, 1, 8, 9 columns for
 # each of the threads
 @pytest.mark.parametrize("B,T,D,heads,bias", [(1, 129, 64, 1, False), (2, 144, 128, 2, True), (3, 168, 64, 2, False), (1, 185, 64, 1, True),
