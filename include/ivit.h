@@ -299,8 +299,9 @@ size_t ivit_vit_workspace_bytes(const ivit_vit_params* p);
 int ivit_vit_forward(ivit_ctx* ctx, const ivit_vit_params* p, const int8_t* image, int32_t* logits,
                      void* workspace, size_t workspace_bytes);
 
-/* The same forward, additionally copying the output of the last encoder block, [B*T, D] int8 (ld = D), to
- * `tokens` (device, 16-byte aligned; NULL: no copy).  The class rows of that tensor are what the final LayerNorm
+/* The same forward, additionally leaving the output of the last encoder block, [B*T, D] int8 (ld = D), in
+ * `tokens` (device, 16-byte aligned; NULL: not wanted).  The last block writes that tensor itself (one that lies in the
+ * workspace is filled by a copy behind the block).  The class rows of that tensor are what the final LayerNorm
  * and the classifier read; the other rows reach no logit, so this is the call that lets a caller (or a parity
  * test) see every byte the encoder produced. */
 int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_t* image, int32_t* logits,

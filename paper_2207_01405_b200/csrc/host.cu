@@ -777,15 +777,19 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
   // patch q of image b lands in token row b*T + 1 + q
   if ((rc = launch_gemm(ctx, linear_problem(patches, Kpe, p->Wpe, Kpe, p->bpe, p->pe_scale, p->pos, D, np,
                                             p->pos_scale, X + D, D, IVIT_I8, np, T, B * np, D, Kpe)))) return rc;
+  // The last block writes the caller's tensor itself where the tokens are wanted (a copy behind it was 4 us), unless that lies in
+  // the workspace: the block still reads activations there while it writes, so the copy follows it.
+  const bool in_ws = tokens && tokens < reinterpret_cast<int8_t*>(ws + w.total) && tokens + B * T * D > reinterpret_cast<int8_t*>(ws);
   bool a_ready = false;   // LayerNorm 1 of the next block already produced by the previous block's last Dense layer
   for (int64_t l = 0; l < p->depth; ++l) {
     const ivit_block_params* next = l + 1 < p->depth ? &p->blocks[l + 1] : nullptr;
-    // (the caller's tensor, where the tokens are wanted, takes the last block's output: a copy behind it was 4 us)
-    int8_t* const to = tokens && !next ? tokens : Y;
+    int8_t* const to = tokens && !in_ws && !next ? tokens : Y;
     if ((rc = block_impl(ctx, &p->blocks[l], X, to, ws + w.block, false, a_ready, next, &a_ready))) return rc;
     Y = X;
     X = to;
   }
+  if (in_ws && cudaMemcpyAsync(tokens, X, (size_t)(B * T * D), cudaMemcpyDeviceToDevice, ctx->stream) != cudaSuccess)
+    return IVIT_ERR_CUDA;
   // final LayerNorm on the class-token rows, then the classifier (int32 logits, not saturated)
   if ((rc = launch_layernorm(ctx, X, IVIT_I8, T * D, to_dev(p->lnf_gamma), p->lnf_beta, p->blocks[0].M_ln, Z, D, B, D, true))) return rc;
   return launch_gemm(ctx, linear_problem(Z, D, p->Whead, D, p->bhead, p->head_scale, nullptr, 0, 1, none, logits,

@@ -129,6 +129,23 @@ def test_deit_small_b64_full_size_graph_replay_sampled():
     assert c.poll_status() == 0
 
 
+def test_tokens_inside_the_workspace():
+    """ivit_vit_forward_tokens with a token tensor that lies in the workspace, over activations that the last block still
+    reads while it writes its output: filled behind the block, all of it, and the logits are right."""
+    g = _g()
+    c = g.ctx()
+    model, image = make_config(1, batch=5, depth=2)
+    dm = g.binding.DeviceVit(model, "cuda")
+    ws = dm.workspace()
+    n = 5 * model.T * model.D
+    tokens = ws[ws.numel() - (n + 255) // 256 * 256:][:n].view(torch.int8).view(-1, model.D)
+    logits = c.vit_forward(dm, torch.from_numpy(image).cuda(), workspace=ws, tokens=tokens)
+    want_logits, want_tokens = O.vit_forward(model, image, return_tokens=True)
+    g.assert_equal(g.host(tokens), want_tokens, "tokens")
+    g.assert_equal(g.host(logits), want_logits, "logits")
+    assert c.poll_status() == 0
+
+
 def test_host_forward_back_to_back_calls():
     """ivit_vit_forward_host enqueued four times without a synchronisation in between: the input copy of a call
     overlaps the compute of the call before it (two staging buffers), and every call must still see its own image."""
