@@ -18,6 +18,7 @@
 // 28 %.  Inside a pass mad.hi / mul.hi take four cycles of a scheduler (measured), the other integer instructions two
 // cycles of their pipe, a look-up one of the SM's shared-memory cycles.
 #include "handover.cuh"
+#include "setup.cuh"
 #include "shiftmax.cuh"
 #include "tc_ptx.cuh"
 
@@ -80,6 +81,12 @@ struct __align__(16) AttnItem {
 __device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 constexpr int kBarSetup = 8, kBarTmem = 9;   // (6 and 7: handover.cuh)
+template <int kThreads>
+struct ShortSetup {
+  __device__ __forceinline__ void arrive() const { bar_arrive(kBarSetup, kThreads); }
+  __device__ __forceinline__ void sync() const { bar_sync(kBarSetup, kThreads); }
+  __device__ __forceinline__ void trigger() const { pdl_trigger(); }
+};
 template <int kThreads>
 struct BlockBarriers {
   __device__ __forceinline__ void sync(int id) const { bar_sync(id, kThreads); }
@@ -247,7 +254,7 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
   uint32_t tmem = 0;
   if (warp == 0) {
     __syncwarp();
-    bar_arrive(kBarSetup, kShortThreads);
+    end_of_setup(ShortSetup<kShortThreads>{}, true);
     if (lane == 0) {
       prefetch_tmap(&tmQ);
       prefetch_tmap(&tmK);
@@ -259,11 +266,10 @@ __global__ void __launch_bounds__(ShortShape<TPR>::kThreads, ShortShape<TPR>::kC
       tc_fence_before();
       bar_arrive(kBarTmem, 64);
     }
-    bar_sync(kBarSetup, kShortThreads);
+    end_of_setup(ShortSetup<kShortThreads>{}, false);
     tc_fence_after();
     tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   }
-  pdl_trigger();
   // items of this CTA: a snake over all of them, or (kPack) a contiguous range
   const uint32_t rounds = (uint32_t)a.items / gridDim.x, left = (uint32_t)a.items % gridDim.x;
   const uint32_t n_items = kPack ? rounds + (blockIdx.x < left ? 1u : 0u) : AttnItem::count(a);

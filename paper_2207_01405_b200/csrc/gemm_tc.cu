@@ -31,6 +31,7 @@
 #include <new>
 #include "residual_rows.cuh"
 #include "rowops.cuh"
+#include "setup.cuh"
 
 namespace ivit {
 
@@ -255,6 +256,18 @@ struct LastMap<false> {
   __device__ __forceinline__ const CUtensorMap* get(const CUtensorMap* other) const { return other; }
 };
 
+// The set-up barrier of a CTA.  (A barrier of its own: the warp that goes ahead may be through with its loads, and at the barrier
+// at the end, before the others are here.)  PAIR: also the other CTA's barriers are initialised behind it.
+template <bool PAIR>
+struct DenseSetup {
+  __device__ __forceinline__ void arrive() const { asm volatile("bar.arrive 3, %0;" ::"n"(kThreads) : "memory"); }
+  __device__ __forceinline__ void sync() const {
+    asm volatile("bar.sync 3, %0;" ::"n"(kThreads) : "memory");
+    if (PAIR) cluster_sync_all();
+  }
+  __device__ __forceinline__ void trigger() const { pdl_trigger(); }
+};
+
 // MODE fixes the run-time choices of the epilogue at compile time for the shapes of an encoder block, so that
 // the per-chunk code carries no branches on kernel arguments: 0 = everything decided at run time (any
 // orientation, output type and residual port), 1 = Dense orientation, int8 output staged for TMA stores, no
@@ -344,15 +357,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     else tmem_alloc(smem_u32(tmem_slot), (uint32_t)a.tmem_cols);
   }
   tc_fence_before();
-  // (a barrier of its own: warp 0 may be through with its loads, and at the barrier at the end, before the others are here)
-  if (!PAIR && warp == 0) asm volatile("bar.arrive 3, %0;" ::"n"(kThreads) : "memory");
-  else asm volatile("bar.sync 3, %0;" ::"n"(kThreads) : "memory");
-  if (PAIR) cluster_sync_all();   // the other CTA's barriers are initialised before anything arrives on them
+  // Barriers, tensor memory and tables are there for the warps behind this: they let the next kernel be scheduled, then wait
+  // for the previous kernel's results before touching global memory.
+  end_of_setup(DenseSetup<PAIR>{}, !PAIR && warp == 0);
   tc_fence_after();
   const uint32_t tmem_base = warp == 0 ? 0u : __shfl_sync(0xffffffffu, *tmem_slot, 0);   // (warp 0 has no use for it)
-  // set-up done (barriers, tensor memory, descriptor prefetch): let the next kernel be scheduled, then wait
-  // for the previous kernel's results before touching global memory
-  pdl_trigger();
   if (ROP == 1 && warp >= kFirstEpiWarp) {
     // I-LayerNorm constants of all channels into shared memory: parameters, read before the wait for the previous
     // kernel.  The form (fast / general, see LnConsts) is agreed on by all epilogue threads.
