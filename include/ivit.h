@@ -316,8 +316,10 @@ int ivit_vit_forward_tokens(ivit_ctx* ctx, const ivit_vit_params* p, const int8_
  * memory is needed for that overlap; pageable memory works but copies synchronously).  The first
  * call on a context creates that stream and its events.  image_host must be complete when the call
  * is made (the copy does not wait for work on the context's stream that might still fill it).  All calls on
- * one context must use the same workspace; a call with another model or batch, or behind other work of
- * the context, copies its image when that work is done.  workspace must hold ivit_vit_host_workspace_bytes(p). */
+ * one context must use the same workspace; a call with another model or batch, or behind other work that calls on
+ * the context enqueued, copies its image when that work is done.  (A CUDA graph that the caller captured around library calls is
+ * not seen when it is replayed: synchronise between such a replay and a host-buffer call that share a workspace.)
+ * IVIT_ERR_CUDA while the context's stream is being captured.  workspace must hold ivit_vit_host_workspace_bytes(p). */
 size_t ivit_vit_host_workspace_bytes(const ivit_vit_params* p);
 int ivit_vit_forward_host(ivit_ctx* ctx, const ivit_vit_params* p, const int8_t* image_host,
                           int32_t* logits_host, void* workspace, size_t workspace_bytes);

@@ -339,6 +339,13 @@ int host_forward(ivit_ctx* ctx, const int8_t* image_host, int32_t* logits_host, 
   const size_t img_off = inner, lg_off = inner + 2 * img_slot;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < lg_off + align_up(lg_bytes, 256))
     return IVIT_ERR_WORKSPACE;
+  // Refused while the compute stream is being captured: the copy stream would join the caller's graph and leave behind events
+  // that no later call can wait for.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return IVIT_ERR_CUDA;
+  }
   if (!ctx->copy_stream) {
     // first use: a stream of its own for the input copies, and the events that order it with the compute stream
     if (cudaSetDevice(ctx->device) != cudaSuccess ||

@@ -167,6 +167,44 @@ def test_host_forward_back_to_back_calls():
     assert c.poll_status() == 0
 
 
+@pytest.mark.parametrize("calls_before", [0, 1, 3])
+def test_host_forward_is_refused_under_capture(calls_before):
+    """A host-buffer forward on a stream that is being captured is refused, also as the context's first call and behind other
+    work of the context; neither the capture nor any later call suffers."""
+    import gpu_util as g
+    side = torch.cuda.Stream()
+    c = g.binding.Context(0, side)
+    model, image = make_config(1, batch=2, depth=1)
+    dm = g.binding.DeviceVit(model, "cuda")
+    ws = dm.host_workspace()
+    want = O.vit_forward(model, image)
+    d_img, h_img = torch.from_numpy(image).cuda(), torch.from_numpy(image).pin_memory()
+    d_out, h_out = (torch.zeros((2, model.classes), dtype=torch.int32) for _ in range(2))
+    d_out, h_out = d_out.cuda(), h_out.pin_memory()
+    torch.cuda.synchronize()
+    for _ in range(calls_before):
+        g.binding.vit_forward_host(c, dm, h_img, h_out, ws)
+    c.vit_forward(dm, d_img, logits=d_out, workspace=ws)
+    side.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        with pytest.raises(g.binding.IvitError) as e:
+            g.binding.vit_forward_host(c, dm, h_img, h_out, ws)
+        assert e.value.code == -6
+        c.vit_forward(dm, d_img, logits=d_out, workspace=ws)
+    for n in range(4):
+        h_out.zero_()
+        g.binding.vit_forward_host(c, dm, h_img, h_out, ws)
+        side.synchronize()
+        g.assert_equal(h_out.numpy(), want, f"call {n} behind the capture")
+    with torch.cuda.stream(side):
+        d_out.zero_()
+        graph.replay()
+    side.synchronize()
+    g.assert_equal(g.host(d_out), want, "the captured forward")
+    assert c.poll_status() == 0
+
+
 def test_host_forward_layouts_in_turn_through_one_workspace():
     """A batch of 64 and one of 8 by turns, then a device forward in between, all in one workspace and without a
     synchronisation: the staging buffers of one layout are activations of the other."""
