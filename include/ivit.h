@@ -209,7 +209,7 @@ int ivit_shiftgelu_static(ivit_ctx* ctx, const int8_t* in, int64_t ldin, ivit_ex
 /* ---- Sec. 3.5: I-LayerNorm over each row ----
  *   mu = floor((2*sum x + C) / (2C)); y = x - mu; V = sum y^2;
  *   sd = integer sqrt of V: the value of Eq. (iterative) with 10 guarded iterations, floor(sqrt(V)) (int8 rows
- *        of up to 1024 or of 1536 channels take it bit by bit without divisions, see ivit_isqrt_range);
+ *        of up to 1024 or of 1536 channels take it from a polynomial, see ivit_isqrt_range);
  *   F = sd ? floor(2^M_ln / sd) : 0;
  *   out[c] = sat8( rq(y[c] * F; gamma_scale[c]) + beta[c] )
  * gamma_scale per-channel or per-tensor; beta int32 [C] or NULL.
@@ -407,8 +407,8 @@ int ivit_probe_int8_mma(ivit_ctx* ctx, int32_t iters, float* ms, double* ops);
 
 /* Verification aid for Sec. 3.5: out[i] = the integer square root that the I-LayerNorm kernels compute for the
  * radicand n0 + i, i < count (device uint16 array; n0 + count <= 2^26, more than the largest sum of squared deviations
- * of an int8 row of 1536 channels).  The kernels take it from the single-precision root instead of running Eq. (iterative); a test
- * compares this routine with the iteration over the whole range. */
+ * of an int8 row of 1536 channels).  The kernels take it from a cubic in 32-bit integers, corrected by its square,
+ * instead of running Eq. (iterative); a test compares this routine with the iteration over the whole range. */
 int ivit_isqrt_range(ivit_ctx* ctx, uint32_t n0, uint32_t count, uint16_t* out);
 
 /* ---- data movement helpers (not in the paper; needed by the full models) ---- */

@@ -4,20 +4,9 @@
 #pragma once
 
 #include "common.cuh"
+#include "isqrt.cuh"
 
 namespace ivit {
-
-// Integer square root, floor(sqrt(n)) for n < 2^26, the value the guarded iteration of Eq. (iterative) converges to.  The
-// single-precision root (of n rounded to 24 bits) is off by less than 0.01, its integer part by at most one, which the
-// square tells.  A row's scalars are a chain between its loads and its stores: bit by bit, without a division, the root took 13
-// dependent steps (a LayerNorm call on 25216 x 768 12.5 -> 11.9 us, a Swin-T forward of 64 images 1410 -> 1399).
-// Equality with the oracle's iteration is checked exhaustively over the whole range by a test (ivit_isqrt_range).
-__device__ __forceinline__ unsigned isqrt26(unsigned n) {
-  float f;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(f) : "f"((float)n));
-  const int r = (int)f, left = (int)n - r * r;
-  return (unsigned)(r + (left > 2 * r ? 1 : 0) - (left < 0 ? 1 : 0));
-}
 
 // ---- I-LayerNorm ------------------------------------------------------------------------------------------
 // out[c] = sat8( rq((x[c] - mu) * F; m_c, s_c) + beta_c ),  mu = mean rounded half up,

@@ -616,7 +616,7 @@ def test_tensor_core_engine_takes_the_model_shapes():
 
 
 def test_layernorm_square_root_routine_equals_the_iteration_exhaustively():
-    """The I-LayerNorm kernels take floor(sqrt(V)) bit by bit; Sec. 3.5 prescribes Eq. (iterative).  Both are run
+    """The I-LayerNorm kernels take floor(sqrt(V)) from a polynomial; Sec. 3.5 prescribes Eq. (iterative).  Both are run
     over EVERY radicand an int8 row of up to 1024 channels can produce (V < 2^26) and compared with the oracle's
     iteration (which is pinned against floor(sqrt) on CPU)."""
     g = _g()
