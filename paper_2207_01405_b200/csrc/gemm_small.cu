@@ -199,9 +199,10 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
         }
       }
       if (e.out_dtype == IVIT_I32) {
+        int32_t* o = reinterpret_cast<int32_t*>(e.out) + (int64_t)r0 * e.ldo + c;
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (c < a.P && r0 + j < a.Q) reinterpret_cast<int32_t*>(e.out)[(int64_t)(r0 + j) * e.ldo + c] = v[j];
+        for (int j = 0; j < 8; ++j, o += e.ldo)
+          if (c < a.P && r0 + j < a.Q) *o = v[j];
         continue;
       }
       if (e.act_table) {   // element-wise activation of the saturated value (the static-maximum ShiftGELU variant)
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(64 + 32 * NW, 1) gemm_small_kernel(const __gri
 }
 
 constexpr size_t kSmallSmem = 227 * 1024;
+constexpr size_t kSmallSmemAlone = 116 * 1024;   // more than half of an SM's
 
 }  // namespace
 
@@ -265,8 +267,13 @@ int launch_gemm_small(ivit_ctx* ctx, const GemmProblem& g) {
   if (!make_tensor_map(ctx, &tmP, g.B, g.K, g.N, 1, 1, g.ldb, 0, 0, SM_BK, SM_BM, CU_TENSOR_MAP_SWIZZLE_128B, a.p_pos) ||
       !make_tensor_map(ctx, &tmQ, g.A, g.K, g.M, 1, 1, g.lda, 0, 0, SM_BK, a.BN, CU_TENSOR_MAP_SWIZZLE_128B, a.q_pos))
     return IVIT_ERR_UNSUPPORTED;
-  const size_t smem = fixed + (size_t)kblocks * a.BN * SM_BK + (size_t)a.stages * SM_BM * SM_BK;
   const dim3 grid((unsigned)(a.tiles_p * ((g.M + a.BN - 1) / a.BN))), block(64 + 32 * NW);
+  // A launch of more than half of the SMs takes one CTA per SM, by its shared memory.  Two would fit otherwise (56 registers), and
+  // a launch that starts while the one before it still runs then puts two of its CTAs on the SMs that are free first and leaves
+  // others idle (alone, two -> one: 1576 x 1152 x 384 5.4 -> 4.2 us, with residual 6.7 -> 5.0, 394 x 1536 x 384 with residual
+  // 4.5 -> 3.5; 1024 x 1152 x 384, whose 144 tiles leave no SM idle, 3.3 -> 3.5; a block of eight DeiT-S images 34.3 -> 32.6).
+  size_t smem = fixed + (size_t)kblocks * a.BN * SM_BK + (size_t)a.stages * SM_BM * SM_BK;
+  if (2 * grid.x > (unsigned)ctx->sm_count && smem < kSmallSmemAlone) smem = kSmallSmemAlone;
   LaunchScope ls(ctx, KIND_GEMM_TC, 2.0 * (double)g.M * (double)g.N * (double)g.K);
   launch_k(gemm_small_kernel, grid, block, smem, ctx->stream, tmP, tmQ, a);
   return ls.done();
