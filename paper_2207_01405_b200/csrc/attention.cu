@@ -181,7 +181,8 @@ __device__ __forceinline__ uint4 output_piece(const AttnArgs& a, int (&v)[16]) {
 // warp polls; the others wait in hardware barriers that it releases.
 //   TPR = 2        128 rows of one image; two CTAs (tensor memory holds two score tiles of 256 columns), two threads per
 //                  score row, which take alternate 16-column chunks
-//   TPR = 4        the same with one CTA and four threads per score row, for launches of at most one item per SM
+//   TPR = 4        the same with one CTA and four threads per score row, for launches of at most one item per SM whose rows are
+//                  long enough
 //   TPR = 1 (kPack)  G windows of up to R = 128 / G tokens share the 128 rows (window attention): the score tile is
 //                  block-diagonal and the probabilities outside a row's own window stay 0.  The int32 score bias of
 //                  the tile's windows is kept in shared memory (rows padded to an odd number of words, so that the 32
@@ -1120,9 +1121,13 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
   }
   sa.tmem_cols = pack || a.chunks <= 8 ? 128 : 256;
   const uint32_t p_off = (128u * a.d + (pack ? 128u : (uint32_t)a.kbox) * a.d + (uint32_t)a.kpad * a.d + 1023u) & ~1023u;
-  // Threads per score row: four where an SM has at most one item anyway (us per block, two -> four threads, 197 tokens: 8
-  // images of DeiT-T 29.3 -> 27.9, 8 of DeiT-S 37.9 -> 37.1, 20 of DeiT-T 37.9 -> 36.4; one image 24.9 -> 24.7).
-  const int tpr = pack ? 1 : (a.items <= ctx->sm_count ? 4 : 2);
+  // Threads per score row: four where an SM has at most one item anyway and the rows are long enough to share, which with a
+  // score bias (read from global memory) they are earlier.  Two -> four threads, at most 148 items, alone: 16 tokens 1.08 x the time,
+  // 80 tokens 1.03 ... 1.10, 144 tokens 1.00 ... 1.07, 170 tokens 0.93 ... 1.01, 256 tokens 0.91 ... 1.02, in a block of 170 or 197 tokens
+  // 0.93 ... 1.02 (mean 0.99); with bias 16 tokens 1.08, 33 ... 80 tokens 0.97 ... 1.01 on up to 74 items and 1.01 ... 1.03 on 148,
+  // 129 ... 197 tokens 0.75 ... 0.97.
+  const int64_t long_rows = !a.bias ? 160 : (2 * a.items <= ctx->sm_count ? 32 : 128);
+  const int tpr = pack ? 1 : (a.items <= ctx->sm_count && T > long_rows ? 4 : 2);
   const size_t partials = tpr == 4 ? ShortShape<4>::kPartials : ShortShape<2>::kPartials;
   const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + partials + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
   // CTAs per SM: as many as leave room for four copies of the table

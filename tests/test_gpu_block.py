@@ -98,8 +98,29 @@ def test_fused_attention_kernel_serves_short_rows():
     assert c.poll_status() == 0
 
 
-# two tiles per head: at most 148 items take four threads per score row, more take two; remainders of 0, 1, 8, 9 columns for
-# each of the threads
+def _attention_case(g, B, T, d, heads, bias, k_out=8, shift=None):
+    """One attention call against the oracle; shift: both requantisations with this shift (below 33 the kernels take their
+    general arithmetic, as for k_out below 8)."""
+    import dataclasses
+    from ivit_inputs import ExpParams, Scale
+    c = g.ctx()
+    blk = make_block(_Ids(60 + T), 2, B, T, heads * d, heads, heads * d, attn_bias_batches=heads if bias else 0)
+    if k_out != 8:
+        blk = dataclasses.replace(blk, smax=ExpParams(blk.smax.I0, blk.smax.N, 45, k_out),
+                                  pv_scale=Scale(blk.pv_scale.mult, max(31, blk.pv_scale.shift - (8 - k_out))))
+    if shift is not None:
+        blk = dataclasses.replace(blk, **{f: Scale(getattr(blk, f).mult >> (getattr(blk, f).shift - shift), shift)
+                                          for f in ("qk_scale", "pv_scale")})
+    rng = np.random.default_rng(B + T)
+    QKV = np.clip(np.rint(rng.standard_normal((B * T, 3 * heads * d)) * 32), -128, 127).astype(np.int8)
+    got = g.host(c.attention(g.binding.DeviceBlock(blk, "cuda"), torch.from_numpy(QKV).cuda()))
+    want = O.attention(blk, QKV)
+    assert len(np.unique(want)) > 20
+    g.assert_equal(got, want, f"attention of {B} x {T} tokens, {heads} heads of {d}")
+    assert c.poll_status() == 0
+
+
+# launches of at most 148 items take four threads per score row from 161 tokens on (with a bias earlier), others two
 @pytest.mark.parametrize("B,T,D,heads,bias", [(1, 129, 64, 1, False), (2, 144, 128, 2, True), (3, 168, 64, 2, False), (1, 185, 64, 1, True),
                                               (1, 201, 64, 2, False), (2, 217, 192, 3, True), (1, 233, 64, 1, False), (1, 249, 128, 1, True),
                                               (74, 197, 64, 1, False), (75, 197, 64, 1, True), (1, 9, 64, 1, True), (148, 70, 64, 1, False),
@@ -113,6 +134,26 @@ def test_attention_threads_per_row(B, T, D, heads, bias):
     got = c.attention(g.binding.DeviceBlock(blk, "cuda"), torch.from_numpy(QKV).cuda())
     g.assert_equal(g.host(got), O.attention(blk, QKV), "attention")
     assert c.poll_status() == 0
+
+
+# More work items than two CTAs per SM: two threads per score row, several items per CTA (item ring, barrier phases, the next
+# item's bias).  Odd and even numbers of whole 16-column chunks, so that the remaining columns fall to either thread; 1, 8, 9 and
+# 15 of them; both arithmetic forms.
+@pytest.mark.parametrize("bias", [False, True])
+@pytest.mark.parametrize("B,T,k_out,shift", [(160, 145, 8, None), (160, 161, 5, None), (160, 152, 5, None), (160, 168, 8, None),
+                                             (160, 153, 8, 32), (160, 169, 8, None), (160, 159, 8, None), (160, 175, 5, None),
+                                             (310, 81, 8, None), (310, 104, 6, None), (160, 256, 8, 31), (310, 128, 8, None)])
+def test_attention_two_threads_per_row_several_items(B, T, k_out, shift, bias):
+    _attention_case(_g(), B, T, 32, 1, bias, k_out, shift)
+
+
+# At most one item per SM, on both sides of the rule for four threads; whole chunks and remainders for each of the four; shifts
+# below 33 take the general arithmetic
+@pytest.mark.parametrize("B,T,heads,bias", [(1, 20, 2, True), (1, 40, 2, True), (1, 129, 1, True), (2, 130, 2, False), (2, 161, 1, False),
+                                            (2, 170, 1, True), (1, 177, 1, True), (1, 193, 2, False), (1, 197, 2, False), (2, 216, 1, False)])
+@pytest.mark.parametrize("shift", [None, 31, 32])
+def test_attention_few_items(B, T, heads, bias, shift):
+    _attention_case(_g(), B, T, 64, heads, bias, 8, shift)
 
 
 @pytest.mark.parametrize("engine", [0, 1])

@@ -71,8 +71,8 @@ def program(tmp_path_factory):
     return str(d / "t")
 
 
-# four and eight Shiftmax warps: packed windows and single images; few items and more than a phase takes arrivals
+# four, eight and sixteen Shiftmax warps: packed windows and single images; few items and more than a phase takes arrivals
 @pytest.mark.parametrize("scores_out", [0, 1])
-@pytest.mark.parametrize("warps,items,done", [(8, 1, 0), (8, 2, 1), (8, 40, 3), (4, 25, 0), (4, 6, 5)])
+@pytest.mark.parametrize("warps,items,done", [(8, 1, 0), (8, 2, 1), (8, 40, 3), (4, 25, 0), (4, 6, 5), (16, 1, 0)])
 def test_everyone_leaves_after_a_wait_that_ran_out(program, warps, items, done, scores_out):
     assert subprocess.run([program, str(warps), str(items), str(done), str(scores_out)], timeout=60).returncode == 0
