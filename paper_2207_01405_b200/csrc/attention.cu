@@ -1130,8 +1130,9 @@ static int launch_attention_short(ivit_ctx* ctx, const ivit_block_params* p, con
   const int tpr = pack ? 1 : (a.items <= ctx->sm_count && T > long_rows ? 4 : 2);
   const size_t partials = tpr == 4 ? ShortShape<4>::kPartials : ShortShape<2>::kPartials;
   const size_t fixed = 1024 + p_off + (size_t)((a.kpad + 127) / 128) * 128 * 128 + partials + 128 * 4 + 2 * sizeof(AttnItem) + 64 + bias_bytes;
-  // CTAs per SM: as many as leave room for four copies of the table
-  int per_sm = pack ? ShortShape<1>::kCtas : ShortShape<2>::kCtas;
+  // CTAs per SM: as many as leave room for four copies of the table.  (Four threads per row: the CTA is alone on its SM and takes all
+  // of its shared memory, at d = 128 for 32 copies instead of 4: 8 x 197 tokens, two heads 7.2 -> 6.4 us, a block of that 28.0 -> 27.2.)
+  int per_sm = pack ? ShortShape<1>::kCtas : (tpr == 4 ? ShortShape<4>::kCtas : ShortShape<2>::kCtas);
   auto budget = [](int n) { return n == 1 ? (size_t)(227 * 1024) : (size_t)(228 * 1024 / n - 1024); };
   while (per_sm > 1 && fixed + 4 * 1024 > budget(per_sm)) --per_sm;
   if (!fit_table(a, fixed, budget(per_sm))) return IVIT_ERR_UNSUPPORTED;
