@@ -119,8 +119,9 @@ int64_t ivit_ctx_pair_launch_count(const ivit_ctx* ctx);
  * the context, 16 sets at a time, the oldest slot being rebuilt for a 17th.  This counter changes whenever a slot
  * is built or rebuilt.  A CUDA graph that the CALLER captured around library calls holds the addresses of the
  * tables those calls used: it stays valid while this counter keeps the value it had when the capture ended, and
- * must be captured again otherwise (or keep the models that share a context to at most 16 parameter sets).  The
- * library's own graphs (ivit_ctx_set_host_graph) check this themselves. */
+ * must be captured again otherwise (or keep the models that share a context to at most 16 parameter sets).  A
+ * table first needed inside such a capture is built by the graph when it runs, and counts as built from then on: make the
+ * first call of a model outside.  The library's own graphs (ivit_ctx_set_host_graph) check all this themselves. */
 uint64_t ivit_ctx_table_generation(const ivit_ctx* ctx);
 /* Selects the GEMM engine: 0 = tcgen05 tensor-core kernels where the shape
  * qualifies (default), 1 = force the CUDA-core (dp4a) kernels everywhere.

@@ -168,11 +168,9 @@ struct TileCoord {
   int bo, bi, p0, q0;
 };
 
-// Tiles are ordered p-block fastest and every CTA owns a contiguous range of them, so that the tiles a
-// CTA works on in a row share their Q operand (the activation rows of a Dense layer).
-
-// The tiles of one worker (a CTA, or a pair of them): a contiguous range and, when the tiles of a ragged last row block
-// are dealt out by themselves, up to two of those.  They cost a fraction of a whole tile, so the workers that have one
+// The tiles of one worker (a CTA, or a pair of them).  Tiles are ordered p-block fastest and a worker owns a contiguous range of
+// them, so that those it works on in a row share their Q operand (the activation rows of a Dense layer), and, when the tiles of a
+// ragged last row block are dealt out by themselves, up to two of those.  They cost a fraction of a whole tile, so the workers that have one
 // whole tile less take them first (one each, then a second one), then the others take one each.  Without that a ragged
 // block can add a whole round: 12608 rows are 49 blocks of 256 and one of 64, and three channel tiles of 50 blocks on 148
 // workers are 150 tiles, two rounds, instead of 147 tiles and three short ones, one round and a quarter.
